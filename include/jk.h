@@ -179,20 +179,25 @@ int jk_build_batch(jk_handle *h, const double *const *D, int32_t n_dm, int with_
  * with Q_ab at or below it are dropped at init, default 1e-18),
  * "use_graph" (0/1), "use_dmax" (0/1: 0 screens with Dmax := 1),
  * "profile" (0/1: CUDA events around every integral launch, see jk_profile;
- * they become event nodes when the build is captured into a graph),
+ * they become event nodes when the build is captured into a graph; a profiled
+ * build with stats launches every class pair by itself, others launch all class
+ * pairs of the same angular momenta together),
  * "omega" (range separation, Table 1 rys_type of the paper: 0 the Coulomb
  * operator 1/r; w > 0 the long-range erf(w r)/r; w < 0 the short-range
  * erfc(|w| r)/r; the Schwarz factors of 1/r bound both),
  * "prim_eps" (primitive quartets with q_ij q_kl Dmax <= min(prim_eps,
  * cutoff) are skipped; q is the primitive-pair Schwarz factor; default 1e-16),
  * "part_count", "part_index" (a build computes only part part_index of
- * part_count of every class kernel's work; J and K are then partial sums
+ * part_count of every class kernel's work, every part_count-th work item; J and K are then partial sums
  * whose sum over the parts is the full result, i.e. one sum all-reduce
  * combines GPUs that split one batch),
- * "branches" (1..8: class kernels forked over this many streams / graph
- * branches),
+ * "branches" (1..8: at least this many streams / graph branches take the class
+ * kernels' launches; a build that is not profiled spreads them over 8, a
+ * profiled one uses exactly this many),
  * "chunk" (32..65536, default 64: candidate kets per work item of the
- * persistent class kernels; changing it re-plans the work items),
+ * persistent class kernels for classes with one thread per quartet; classes
+ * with G threads per quartet take 1/G of it, at least 4, and systems with more
+ * than 8 million items larger ones; changing it re-plans the work items),
  * "asym64" (0/1, default 0: the FP32 tier evaluates the large-T
  * Gauss-Hermite limit of the Rys roots and weights in FP64 and rounds the
  * result to FP32, instead of evaluating it in FP32),

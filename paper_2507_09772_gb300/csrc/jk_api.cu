@@ -126,9 +126,8 @@ struct KSpec {
         if (kind == 1)
             snprintf(b, sizeof b, "jk_schwarz_kernel<%d,%d,%d,%d,%d,%d,%d,%d,%d>", la, lb, na, nb, ga, gb, gc, gd, gx);
         else
-            snprintf(b, sizeof b, "jk_class_kernel<%d,%d,%d,%d,%d,%d,%d,%d,%d,%d,%d,%d,%d,%d,%d,%d,%s,%d,%d>", la,
-                     lb, lc, ld, na, nb, nc, nd, ga, gb, gc, gd, gx, ndm, doj, dok, fp32 ? "float" : "double", mode,
-                     op);
+            snprintf(b, sizeof b, "jk_class_kernel<%d,%d,%d,%d,%d,%d,%d,%d,%d,%d,%d,%d,%s,%d,%d>", la, lb, lc, ld, ga,
+                     gb, gc, gd, gx, ndm, doj, dok, fp32 ? "float" : "double", mode, op);
         return b;
     }
     int G() const { return ga * gb * gc * gd; }
@@ -201,7 +200,8 @@ uint64_t spec_key(const KSpec &s)
 {
     int major = 0, minor = 0;
     nvrtcVersion(&major, &minor);
-    uint64_t h = fnv(jk_kernel_source, sizeof(jk_kernel_source));
+    static const uint64_t src = fnv(jk_kernel_source, sizeof(jk_kernel_source));
+    uint64_t h = src;
     std::string n = s.name();
     h = fnv(n.data(), n.size(), h);
     for (auto &o : nvrtc_options(s)) h = fnv(o.data(), o.size(), h);
@@ -689,29 +689,54 @@ struct PairClass {
     int *d_beg = nullptr, *d_end = nullptr;
 };
 
+// A class pair (bra class, ket class).
 struct Launch {
     int c1, c2;        // pair classes (bra, ket)
     KSpec spec[2];     // [0] FP64, [1] FP32
     double cost;       // scheduling estimate
-    // nbra + 1 work-item offsets (chunks of kets per bra): [0] with the
-    // handle's chunk, [1] with the chunk of the FP64 tier of two-tier builds
-    long long *d_prefix[2] = {nullptr, nullptr};
-    long long nitems[2] = {0, 0};
     double cand = 0;   // candidate kets summed over the bras (Q_ab Q_cd > JK_ITEM_EPS)
 };
 
-// Kets per work item. A bra pair's candidate kets (those whose Schwarz
-// product can exceed JK_ITEM_EPS with Dmax = 1) are split into chunks of this
-// size; the last chunk always runs to the molecule's last ket.
+// The launches of one tier: the class pairs grouped by kernel (angular
+// momenta and fragment shape), or one by one when the launches are profiled.
+struct LaunchGroup {
+    KSpec spec;
+    int sub0 = 0, nsub = 0;
+    long long cap = 0;   // work items it can have at most
+};
+struct TierPlan {
+    std::vector<LaunchGroup> groups;
+    std::vector<int> launch;             // class pair of every sub
+    JkSub *d_subs = nullptr;
+    int2 *d_blocks = nullptr;            // blocks of jk_plan_kernel
+    int nblocks = 0;
+    JkItem *d_items = nullptr;
+    long long *d_item_off = nullptr;     // per group
+    std::vector<long long> item_off;
+    std::map<int, std::vector<KInfo>> kernels;   // per flag combination, one per group
+    ~TierPlan() { cudaFree(d_subs); cudaFree(d_blocks); cudaFree(d_items); cudaFree(d_item_off); }
+};
+
+// Kets per work item of a class with one thread per quartet; a class whose
+// quartet takes G threads gets proportionally fewer (at least JK_CHUNK_MIN),
+// so that an item is the same number of rounds of a warp: with 64 kets for
+// every class, a (dd|dp) item (18 threads, one quartet per warp at a time) ran
+// 2 ms on its own. Systems whose items would exceed JK_ITEMS_MAX get larger
+// chunks.
 #define JK_CHUNK 64
 // The FP64 tier of a mixed build keeps ~7 % of the candidates; with 512 per
 // item the batched mixed build ran 5 % faster than with 64 (and than 2,048).
 #define JK_CHUNK_HI 512
+#define JK_CHUNK_MIN 4
+#define JK_ITEMS_MAX 8000000LL
 #define JK_ITEM_EPS 1e-15
 
 }  // namespace
 
 #define JK_MAX_BRANCHES 7
+// Streams the launches of a build are spread over unless they are profiled: the
+// tail of one launch is filled by the next ones (21 launches for s, p, d shells).
+#define JK_AUTO_BRANCHES 8
 
 struct jk_handle {
     int device = 0;
@@ -733,8 +758,14 @@ struct jk_handle {
     unsigned long long *d_dmax_mol = nullptr;
     double *d_rys64 = nullptr;
     float *d_rys32 = nullptr;
-    unsigned long long *d_work = nullptr;  // one counter per launch
-    unsigned long long *d_stats = nullptr; // three per launch and tier
+    // counters zeroed at the start of every build, one allocation: per tier and
+    // group the items listed and taken; three statistics per class pair and
+    // tier; the largest |D| per molecule; the routed list lengths
+    unsigned long long *d_zero = nullptr;
+    size_t zero_bytes = 0;
+    unsigned long long *d_ctr = nullptr;   // [2 tiers][class pairs][listed, taken]
+    unsigned long long *d_stats = nullptr; // three per class pair and tier
+    std::map<int, std::unique_ptr<TierPlan>> plans;   // by tier, chunk and merging
     int *d_err = nullptr;
     int *h_err = nullptr;                  // pinned copy of d_err taken after each build without stats
     cudaEvent_t err_ev = nullptr;          // recorded after that copy
@@ -780,18 +811,19 @@ struct jk_handle {
     bool has_router = false;
     unsigned long long *d_logn = nullptr;
     JkRouted *d_rlist = nullptr;           // routed builds: released quartets, per launch segments
-    unsigned long long *d_rcount = nullptr;
+    unsigned long long *d_rcount = nullptr;   // entries the FP64 tier appended, per class pair (in d_zero)
     std::vector<long long> rl_off, rl_cap;
+    long long *d_rl = nullptr;             // offsets, then capacities
     std::vector<long long> rl_need;        // entries each list needed in the last build with stats
     double route_cap = 16777216.0;         // list entries over all launches
     int asym64 = 0;                        // FP32 tier: large-T roots and weights in FP64
-    int chunk = 64;                        // kets per work item
+    int chunk = JK_CHUNK;                  // kets per work item
     // FP32 tier: float-to-double by integer operations (1) or by the
     // conversion instruction (0, measured 11 % faster on the FP32 tier of
     // the batched workload: the integer sequence costs more issue slots than
     // the FP64-pipe instruction it replaces)
     int widen_int = 0;
-    int chunk_hi = 64;                     // ... for the FP64 tier of mixed and routed builds
+    int chunk_hi = JK_CHUNK_HI;            // ... for the FP64 tier of mixed and routed builds
     // bounds compared in FP64 (0: in FP32 when the cutoff is >= 1e-30); FP64
     // costs about 2 % of a mixed build of the batched workload
     int screen64 = 1;
@@ -809,11 +841,11 @@ void free_handle(jk_handle *h)
 {
     if (!h) return;
     for (auto &c : h->classes) { cudaFree(c.d_beg); cudaFree(c.d_end); }
-    for (auto &L : h->launches) { cudaFree(L.d_prefix[0]); cudaFree(L.d_prefix[1]); }
+    h->plans.clear();
     cudaFree(h->d_sh_mol); cudaFree(h->d_mol_sh0); cudaFree(h->d_sh_ao); cudaFree(h->d_sh_nc);
     cudaFree(h->d_pairs); cudaFree(h->d_pp64); cudaFree(h->d_pp32); cudaFree(h->d_mols);
-    cudaFree(h->d_dmax); cudaFree(h->d_dmax32); cudaFree(h->d_dmax_mol); cudaFree(h->d_rys64); cudaFree(h->d_rys32);
-    cudaFree(h->d_work); cudaFree(h->d_stats); cudaFree(h->d_err); cudaFree(h->d_tile_off);
+    cudaFree(h->d_dmax); cudaFree(h->d_dmax32); cudaFree(h->d_rys64); cudaFree(h->d_rys32);
+    cudaFree(h->d_zero); cudaFree(h->d_err); cudaFree(h->d_tile_off);
     if (h->h_mols) cudaFreeHost(h->h_mols);
     if (h->h_err) cudaFreeHost(h->h_err);
     if (h->err_ev) cudaEventDestroy(h->err_ev);
@@ -824,7 +856,7 @@ void free_handle(jk_handle *h)
     cudaFree(h->d_sh_l); cudaFree(h->d_sh_sph); cudaFree(h->d_sh_aou); cudaFree(h->d_c2s_off);
     cudaFree(h->d_c2s); cudaFree(h->d_cart); cudaFree(h->d_sph); cudaFree(h->d_d32);
     cudaFree(h->d_pfeat); cudaFree(h->d_router); cudaFree(h->d_logn);
-    cudaFree(h->d_rlist); cudaFree(h->d_rcount);
+    cudaFree(h->d_rlist); cudaFree(h->d_rl);
     for (auto &g : h->graphs) cudaGraphExecDestroy(g.second.first);
     if (h->cap) cudaStreamDestroy(h->cap);
     for (int b = 0; b < JK_MAX_BRANCHES; ++b) {
@@ -848,48 +880,153 @@ int upload(T **dst, const std::vector<T> &src)
 // shell type order: l first, then nprim
 long type_key(const jk_shell &s) { return (long)s.l * 64 + s.nprim; }
 
-// Work items of every launch: per bra, ceil(candidates / chunk) (at least
-// one), where the candidates are the kets (sorted by Q) with Q_ab Q_cd >
-// JK_ITEM_EPS; the last chunk of a bra runs to the molecule's last ket. Two
-// partitions: `chunk` for every tier but one, `chunk_hi` for the FP64 tier
-// of mixed and routed builds, which keeps only the few candidates above
-// tau32, so that its items still fill whole rounds of a warp. Also the
-// launch's cost estimate (candidates x modelled FLOPs per quartet).
-int plan_items(jk_handle *h, int chunk, int chunk_hi)
+// Cost estimate of every class pair: its candidates (pairs with Q_ab Q_cd >
+// JK_ITEM_EPS; both lists are sorted by Q) times the modelled FLOPs.
+void estimate_costs(jk_handle *h)
 {
     for (auto &L : h->launches) {
         const PairClass &A = h->classes[L.c1], &B = h->classes[L.c2];
-        std::vector<long long> pre(A.n + 1, 0), pre2(A.n + 1, 0);
         double work = 0;
         for (int m = 0; m < h->nmol; ++m) {
-            const int b0 = A.beg[m], b1 = A.end[m];
-            const int k0 = B.beg[m], k1 = B.end[m];
-            for (int bi = b0; bi < b1; ++bi) {
+            int k = B.end[m];   // kets [B.beg, k) pass for the current bra
+            for (int bi = A.beg[m]; bi < A.end[m] && k > B.beg[m]; ++bi) {
                 const double qa = h->h_pairs[A.off + bi].Q;
-                const int kfirst = (L.c1 == L.c2) ? bi : k0;
-                // kets with qa * Q_cd > eps form a prefix of [k0, k1)
-                int lo = k0, hi = k1;
-                while (lo < hi) {
-                    int mid = (lo + hi) / 2;
-                    if (qa * h->h_pairs[B.off + mid].Q > JK_ITEM_EPS) lo = mid + 1; else hi = mid;
-                }
-                long long ncand = std::max(0, lo - kfirst);
-                pre[bi + 1] = std::max(1LL, (ncand + chunk - 1) / chunk);
-                pre2[bi + 1] = std::max(1LL, (ncand + chunk_hi - 1) / chunk_hi);
-                work += (double)ncand;
+                while (k > B.beg[m] && !(qa * h->h_pairs[B.off + k - 1].Q > JK_ITEM_EPS)) --k;
+                work += (double)std::max(0, k - (L.c1 == L.c2 ? bi : B.beg[m]));
             }
         }
-        for (int bi = 0; bi < A.n; ++bi) { pre[bi + 1] += pre[bi]; pre2[bi + 1] += pre2[bi]; }
-        L.nitems[0] = pre[A.n];
-        L.nitems[1] = pre2[A.n];
-        for (int t = 0; t < 2; ++t) { cudaFree(L.d_prefix[t]); L.d_prefix[t] = nullptr; }
-        if (int rc = upload(&L.d_prefix[0], pre)) return rc;
-        if (int rc = upload(&L.d_prefix[1], pre2)) return rc;
         L.cand = work;
         L.cost = work * class_flops(L.spec[0], 1);
     }
-    h->chunk = chunk;
-    h->chunk_hi = chunk_hi;
+}
+
+void drop_graphs(jk_handle *h)
+{
+    for (auto &g : h->graphs) cudaGraphExecDestroy(g.second.first);
+    h->graphs.clear();
+}
+
+// The launches of a tier (t = 0 FP64 shapes, 1 FP32 shapes; hi: the chunk of
+// the FP64 tier of two-tier builds; merge: class pairs that share a kernel in
+// one launch), made on first use and kept until the shapes or chunks change.
+int tier_plan(jk_handle *h, int t, int hi, int merge, TierPlan **out)
+{
+    const int key = t + 2 * hi + 4 * merge;
+    auto it = h->plans.find(key);
+    if (it != h->plans.end()) { *out = it->second.get(); return JK_OK; }
+    std::unique_ptr<TierPlan> P(new TierPlan());
+    // group the class pairs (h->launches is sorted by cost, largest first)
+    std::vector<std::vector<int>> members;
+    std::map<std::string, int> by_kernel;
+    for (size_t l = 0; l < h->launches.size(); ++l) {
+        int g = (int)members.size();
+        if (merge) {
+            auto r = by_kernel.emplace(h->launches[l].spec[t].name(), g);
+            g = r.first->second;
+        }
+        if (g == (int)members.size()) members.emplace_back();
+        members[g].push_back((int)l);
+    }
+    auto prims = [&](int l) {
+        const KSpec &s = h->launches[l].spec[t];
+        return s.na * s.nb * s.nc * s.nd;
+    };
+    std::vector<double> cost(members.size(), 0.0);
+    std::vector<int> gord(members.size());
+    for (size_t g = 0; g < members.size(); ++g) {
+        gord[g] = (int)g;
+        for (int l : members[g]) cost[g] += h->launches[l].cost;
+        // the longest items first
+        std::stable_sort(members[g].begin(), members[g].end(), [&](int x, int y) { return prims(x) > prims(y); });
+    }
+    std::stable_sort(gord.begin(), gord.end(), [&](int x, int y) { return cost[x] > cost[y]; });
+    const long long base = hi ? h->chunk_hi : h->chunk;
+    std::vector<JkSub> subs;
+    std::vector<long long> cap;
+    for (long long f = 1;; f *= 2) {
+        subs.clear();
+        cap.assign(members.size(), 0);
+        P->groups.clear();
+        P->launch.clear();
+        long long total = 0, least = 0;
+        for (size_t k = 0; k < gord.size(); ++k) {
+            const auto &mem = members[gord[k]];
+            LaunchGroup G;
+            G.spec = h->launches[mem[0]].spec[t];
+            G.sub0 = (int)subs.size();
+            G.nsub = (int)mem.size();
+            const int ngw = G.spec.G() <= 32 ? 32 / G.spec.G() : 1;
+            for (int l : mem) {
+                const Launch &L = h->launches[l];
+                const PairClass &A = h->classes[L.c1], &B = h->classes[L.c2];
+                JkSub S;
+                memset(&S, 0, sizeof S);
+                S.bra = h->d_pairs + A.off;
+                S.ket = h->d_pairs + B.off;
+                S.ket_beg = B.d_beg;
+                S.ket_end = B.d_end;
+                S.bra_feat = h->d_pfeat + A.off;
+                S.ket_feat = h->d_pfeat + B.off;
+                S.nbra = A.n;
+                S.same_class = L.c1 == L.c2 ? 1 : 0;
+                S.nab = L.spec[t].na * L.spec[t].nb;
+                S.ncd = L.spec[t].nc * L.spec[t].nd;
+                const long long c = std::min<long long>(1 << 24, std::max<long long>(JK_CHUNK_MIN, base * ngw / 32) * f);
+                S.chunk = (int)c;
+                S.group = (int)k;
+                S.launch = l;
+                for (int m = 0; m < h->nmol; ++m) {
+                    const long long nb = A.end[m] - A.beg[m], nk = B.end[m] - B.beg[m];
+                    // same class: bra i has nk - i kets
+                    const long long q = nk / c, r = nk % c;
+                    G.cap += S.same_class ? c * q * (q + 1) / 2 + r * (q + 1) : nb * ((nk + c - 1) / c);
+                    if (nk > 0) least += nb;
+                }
+                subs.push_back(S);
+                P->launch.push_back(l);
+            }
+            total += G.cap;
+            P->groups.push_back(G);
+        }
+        if (total <= JK_ITEMS_MAX + least || f >= (1 << 20)) break;
+    }
+    std::vector<int2> blocks;
+    for (size_t k = 0; k < subs.size(); ++k)
+        for (int i = 0; i < subs[k].nbra; i += 256) blocks.push_back(make_int2((int)k, i));
+    long long tot = 0;
+    for (auto &G : P->groups) { P->item_off.push_back(tot); tot += G.cap; }
+    P->nblocks = (int)blocks.size();
+    int rc;
+    if ((rc = upload(&P->d_subs, subs)) || (rc = upload(&P->d_blocks, blocks)) || (rc = upload(&P->d_item_off, P->item_off)))
+        return rc;
+    CK(cudaMalloc(&P->d_items, sizeof(JkItem) * (size_t)std::max(tot, 1LL)));
+    *out = P.get();
+    h->plans[key] = std::move(P);
+    return JK_OK;
+}
+
+// The kernels of a plan's groups for one flag combination, looked up once.
+int plan_kernels(jk_handle *h, TierPlan *P, int ndm, int doj, int dok, int mode, int op, std::vector<KInfo> **out)
+{
+    const int key = ndm | doj << 3 | dok << 4 | mode << 5 | op << 7;
+    auto it = P->kernels.find(key);
+    if (it == P->kernels.end()) {
+        std::vector<KSpec> specs;
+        for (auto &G : P->groups) {
+            KSpec s = G.spec;
+            s.ndm = ndm; s.doj = doj; s.dok = dok; s.op = op;
+            // a quartet split over CTAs is screened by each of them, so it is
+            // never routed: its band stays in FP64
+            s.mode = mode == 1 && s.gx > 1 ? 0 : mode;
+            specs.push_back(s);
+        }
+        std::vector<KInfo> ki;
+        auto tc = std::chrono::steady_clock::now();
+        if (int rc = ensure_kernels(specs, ki)) return rc;
+        h->compile_ms += std::chrono::duration<double, std::milli>(std::chrono::steady_clock::now() - tc).count();
+        it = P->kernels.emplace(key, ki).first;
+    }
+    *out = &it->second;
     return JK_OK;
 }
 
@@ -1258,7 +1395,7 @@ int init_impl(int32_t nmol, const int32_t *mol_shell_off, const jk_shell *shells
             }
             h->launches.push_back(L);
         }
-    if ((rc = plan_items(h.get(), JK_CHUNK, JK_CHUNK_HI))) return rc;
+    estimate_costs(h.get());
     std::stable_sort(h->launches.begin(), h->launches.end(), [](const Launch &x, const Launch &y) { return x.cost > y.cost; });
 
     // ---- per-build scratch
@@ -1280,11 +1417,18 @@ int init_impl(int32_t nmol, const int32_t *mol_shell_off, const jk_shell *shells
     if ((rc = upload(&h->d_tile_off, toff))) return rc;
     CK(cudaMalloc(&h->d_dmax, sizeof(double) * dtot));
     CK(cudaMalloc(&h->d_dmax32, sizeof(float) * dtot));
-    CK(cudaMalloc(&h->d_dmax_mol, sizeof(unsigned long long) * nmol));
     CK(cudaMalloc(&h->d_mols, sizeof(JkMol) * nmol));
-    const size_t nl = h->launches.size() * 3;   // FP64, FP32 and the routed list kernel
-    CK(cudaMalloc(&h->d_work, sizeof(unsigned long long) * nl));
-    CK(cudaMalloc(&h->d_stats, sizeof(unsigned long long) * 3 * nl));
+    {
+        // class pairs x (2 tiers x (listed, taken) + 3 tiers (FP64, FP32, routed
+        // list) x 3 statistics + routed count), then the molecules' largest |D|
+        const size_t nl = h->launches.size(), n = nl * (4 + 9 + 1) + nmol;
+        h->zero_bytes = sizeof(unsigned long long) * n;
+        CK(cudaMalloc(&h->d_zero, h->zero_bytes));
+        h->d_ctr = h->d_zero;
+        h->d_stats = h->d_zero + 4 * nl;
+        h->d_rcount = h->d_stats + 9 * nl;
+        h->d_dmax_mol = h->d_rcount + nl;
+    }
     CK(cudaMalloc(&h->d_err, sizeof(int)));
     CK(cudaMemset(h->d_err, 0, sizeof(int)));
     if (h->spherical) {
@@ -1377,32 +1521,28 @@ int build_impl(jk_handle *h, const double *const *D, int32_t ndm, int with_j, in
     cudaStream_t st = (cudaStream_t)stream;
     if (int prc = poll_device_error(h, false)) return prc;
 
-    // kernels for this combination
-    std::vector<KSpec> specs;
-    std::vector<int> lidx, tier;
-    // tier 0 FP64, 1 FP32; routed builds add tier 2, the FP32 list kernel
-    // of the quartets the router released from the FP64 tier (the router
-    // itself runs in the FP64 tier only)
+    // launches and kernels for this combination. Tier 0 FP64, 1 FP32; routed
+    // builds add tier 2, the FP32 list kernel of the quartets the router
+    // released from the FP64 tier (the router itself runs in the FP64 tier only)
     const bool routed = mode == JK_PREC_MIXED_ROUTED;
-    for (size_t i = 0; i < h->launches.size(); ++i) {
-        for (int t = 0; t < 3; ++t) {
-            const bool two = mode == JK_PREC_MIXED || routed;
-            bool use = (t == 0) ? (mode == JK_PREC_FP64 || two) : (t == 1 ? (mode == JK_PREC_FP32 || two) : routed);
-            if (!use) continue;
-            KSpec s = h->launches[i].spec[t == 0 ? 0 : 1];
-            s.ndm = ndm; s.doj = with_j ? 1 : 0; s.dok = with_k ? 1 : 0;
-            s.mode = logs ? 2 : (routed ? (t == 0 ? 1 : (t == 2 ? 3 : 0)) : 0);
-            s.op = h->omega == 0.0 ? 0 : (h->omega > 0.0 ? 1 : 2);
-            specs.push_back(s);
-            lidx.push_back((int)i);
-            tier.push_back(t);
-        }
+    const bool two = mode == JK_PREC_MIXED || routed;
+    const bool prof = h->profile && stats;
+    const int merge = prof ? 0 : 1;
+    const int op = h->omega == 0.0 ? 0 : (h->omega > 0.0 ? 1 : 2);
+    struct Tier { int t; TierPlan *P; std::vector<KInfo> *ki; };
+    std::vector<Tier> tiers;
+    int rc;
+    for (int t = 0; t < 3; ++t) {
+        const bool use = (t == 0) ? (mode == JK_PREC_FP64 || two) : (t == 1 ? (mode == JK_PREC_FP32 || two) : routed);
+        if (!use) continue;
+        Tier T{t, nullptr, nullptr};
+        if ((rc = tier_plan(h, t == 0 ? 0 : 1, t == 0 && two ? 1 : 0, merge, &T.P))) return rc;
+        const int kmode = logs ? 2 : (routed ? (t == 0 ? 1 : (t == 2 ? 3 : 0)) : 0);
+        if ((rc = plan_kernels(h, T.P, ndm, with_j ? 1 : 0, with_k ? 1 : 0, kmode, op, &T.ki))) return rc;
+        tiers.push_back(T);
     }
-    std::vector<KInfo> ki;
-    auto tc = std::chrono::steady_clock::now();
-    int rc = ensure_kernels(specs, ki);
-    if (rc) return rc;
-    h->compile_ms += std::chrono::duration<double, std::milli>(std::chrono::steady_clock::now() - tc).count();
+    size_t nlaunch_class = 0;
+    for (auto &T : tiers) nlaunch_class += T.P->groups.size();
 
     // Cartesian scratch for spherical molecules (3 x ndm x nao_c^2 each)
     if (h->spherical && h->cart_ndm < (size_t)ndm) {
@@ -1440,8 +1580,8 @@ int build_impl(jk_handle *h, const double *const *D, int32_t ndm, int with_j, in
         for (size_t i = 0; i < h->rl_need.size(); ++i) grow = grow || h->rl_need[i] > h->rl_cap[i];
     if (routed && (!h->d_rlist || grow)) {
         CK(cudaStreamSynchronize(st));
-        cudaFree(h->d_rlist); cudaFree(h->d_rcount);
-        h->d_rlist = nullptr; h->d_rcount = nullptr;
+        cudaFree(h->d_rlist); cudaFree(h->d_rl);
+        h->d_rlist = nullptr; h->d_rl = nullptr;
         double tc2 = 0;
         for (auto &L : h->launches) tc2 += L.cand;
         std::vector<long long> cap(h->launches.size());
@@ -1460,7 +1600,9 @@ int build_impl(jk_handle *h, const double *const *D, int32_t ndm, int with_j, in
             tot += h->rl_cap[i];
         }
         CK(cudaMalloc(&h->d_rlist, sizeof(JkRouted) * (size_t)std::max(tot, 1LL)));
-        CK(cudaMalloc(&h->d_rcount, sizeof(unsigned long long) * std::max<size_t>(h->launches.size(), 1)));
+        std::vector<long long> rl(h->rl_off);
+        rl.insert(rl.end(), h->rl_cap.begin(), h->rl_cap.end());
+        if ((rc = upload(&h->d_rl, rl))) return rc;
         ++h->cart_gen;
     }
     // per-molecule descriptors
@@ -1508,15 +1650,14 @@ int build_impl(jk_handle *h, const double *const *D, int32_t ndm, int with_j, in
         max_nsh = std::max(max_nsh, h->mol_sh0[m + 1] - h->mol_sh0[m]);
         max_nao = std::max(max_nao, h->nao_cart[m]);
     }
-    const size_t nl = h->launches.size() * 3;   // counters per launch and tier (incl. the routed list tier)
+    const size_t nl = h->launches.size();
     const double inf = INFINITY;
-    const bool prof = h->profile && stats;
-    if (prof && h->prof_ev.size() < 2 * specs.size()) {
+    if (prof && h->prof_ev.size() < 2 * nlaunch_class) {
         size_t have = h->prof_ev.size();
-        h->prof_ev.resize(2 * specs.size());
+        h->prof_ev.resize(2 * nlaunch_class);
         for (size_t e = have; e < h->prof_ev.size(); ++e) CK(cudaEventCreate(&h->prof_ev[e]));
     }
-    const int nbranch = std::max(1, std::min(h->branches, JK_MAX_BRANCHES + 1));
+    const int nbranch = prof ? h->branches : std::max(h->branches, JK_AUTO_BRANCHES);
     int nlaunch_aux = 0;
 
     // Everything a build does on the device, in order, on stream s (and, for
@@ -1540,10 +1681,7 @@ int build_impl(jk_handle *h, const double *const *D, int32_t ndm, int with_j, in
             CK(cudaGetLastError());
             ++nlaunch_aux;
         }
-        CK(cudaMemsetAsync(h->d_work, 0, sizeof(unsigned long long) * nl, s0));
-        CK(cudaMemsetAsync(h->d_stats, 0, sizeof(unsigned long long) * 3 * nl, s0));
-        CK(cudaMemsetAsync(h->d_dmax_mol, 0, sizeof(unsigned long long) * h->nmol, s0));
-        if (routed) CK(cudaMemsetAsync(h->d_rcount, 0, sizeof(unsigned long long) * h->launches.size(), s0));
+        CK(cudaMemsetAsync(h->d_zero, 0, h->zero_bytes, s0));
         jk_dmax_kernel<<<h->nshell, 128, 0, s0>>>(h->d_mols, h->d_sh_mol, h->d_mol_sh0, h->d_sh_ao, h->d_sh_nc, ndm,
                                                   h->d_dmax, h->d_dmax32, h->d_dmax_mol, h->d_err);
         CK(cudaGetLastError());
@@ -1555,107 +1693,131 @@ int build_impl(jk_handle *h, const double *const *D, int32_t ndm, int with_j, in
             CK(cudaGetLastError());
             ++nlaunch_aux;
         }
-        if (nbranch > 1) {
+        const double tau = std::max(cutoff, h->tau32);
+        const double band_hi = tau * h->router_band;
+        // screening: FP32 bounds with the FP64 rule kept exact (2, the
+        // default), plain FP32 (1, option screen64 = 0), or FP64 (0, for
+        // cutoffs below the FP32 range). One choice for every launch of the
+        // build, so that the tiers of a mixed build compare the same bounds in
+        // the same precision
+        const int scr32 = cutoff >= 1e-30 ? (h->screen64 ? 2 : 1) : 0;
+        // bounds of the tiers; in a routed build the FP32 tier keeps the Schwarz
+        // split, the band goes to the FP64 tier, which routes it (tier 2 reads
+        // its lists)
+        auto lo_of = [&](int t) { return two && t == 0 ? tau : cutoff; };
+        auto hi_of = [&](int t) { return two && t != 0 ? tau : inf; };
+        {
+            JkPlanArgs pa;
+            memset(&pa, 0, sizeof pa);
+            pa.dmax_mol = reinterpret_cast<const double *>(h->d_dmax_mol);
+            pa.use_dmax = h->use_dmax;
+            pa.scr32 = scr32;
+            pa.part_index = h->part_index;
+            pa.part_count = h->part_count;
+            int np = 0, nblk = 1;
+            for (auto &T : tiers) {
+                if (T.t == 2) continue;
+                JkPlanTier &q = pa.tier[np++];
+                q.subs = T.P->d_subs;
+                q.blocks = T.P->d_blocks;
+                q.nblocks = T.P->nblocks;
+                q.items = T.P->d_items;
+                q.item_off = T.P->d_item_off;
+                q.nitems = h->d_ctr + (size_t)T.t * 2 * nl;
+                q.lo = lo_of(T.t);
+                q.lo32 = (float)q.lo;
+                nblk = std::max(nblk, q.nblocks);
+            }
+            jk_plan_kernel<<<dim3((unsigned)nblk, np), 256, 0, s0>>>(pa);
+            CK(cudaGetLastError());
+            ++nlaunch_aux;
+        }
+        auto fork = [&]() -> int {
+            if (nbranch < 2) return JK_OK;
             CK(cudaEventRecord(h->ev_fork, s0));
             for (int b = 1; b < nbranch; ++b) CK(cudaStreamWaitEvent(h->side[b - 1], h->ev_fork, 0));
-        }
-        for (size_t k = 0; k < specs.size(); ++k) {
-            // a routed class pair keeps its three launches on one stream (the
-            // list kernel reads what the FP64 launch wrote)
-            const size_t br = routed ? (size_t)lidx[k] : k;
-            cudaStream_t sk = (nbranch > 1 && br % nbranch) ? h->side[br % nbranch - 1] : s0;
-            const Launch &L = h->launches[lidx[k]];
-            const PairClass &A = h->classes[L.c1], &B = h->classes[L.c2];
-            JkClassArgs a;
-            // bra and ket indices are relative to the base of their pair class
-            a.bra = h->d_pairs + A.off;
-            a.ket = h->d_pairs + B.off;
-            a.ket_beg = B.d_beg;
-            a.ket_end = B.d_end;
-            a.pp64 = h->d_pp64;
-            a.pp32 = h->d_pp32;
-            a.mols = h->d_mols;
-            a.dmax = h->d_dmax;
-            a.dmax32 = h->d_dmax32;
-            a.dmax_mol = reinterpret_cast<const double *>(h->d_dmax_mol);
-            a.rys64 = h->d_rys64;
-            a.rys32 = h->d_rys32;
-            const int slot = lidx[k] * 3 + tier[k];
-            a.work = h->d_work + slot;
-            a.stats = h->d_stats + 3 * slot;
-            a.err = h->d_err;
-            const double tau = std::max(cutoff, h->tau32);
-            const double band_hi = tau * h->router_band;
-            if (mode == JK_PREC_MIXED) {
-                if (tier[k] == 0) { a.lo = tau; a.hi = inf; }
-                else { a.lo = cutoff; a.hi = tau; }
-            } else if (mode == JK_PREC_MIXED_ROUTED) {
-                // the FP32 tier keeps the Schwarz split; the band goes to the
-                // FP64 tier, which routes it (tier 2 reads its list)
-                if (tier[k] == 0) { a.lo = tau; a.hi = inf; }
-                else { a.lo = cutoff; a.hi = tau; }
-            } else {
-                a.lo = cutoff; a.hi = inf;
-            }
-            a.bra_feat = h->d_pfeat + A.off;
-            a.ket_feat = h->d_pfeat + B.off;
-            a.router = h->d_router;
-            a.tau = tau;
-            a.band_hi = band_hi;
-            // FP32 screening unless the cutoff is below the FP32 range; one
-            // choice for every launch of the build, so that the tiers of a
-            // mixed build compare the same bounds in the same precision
-            // screening: FP32 bounds with the FP64 rule kept exact (2, the
-            // default), plain FP32 (1, option screen64 = 0), or FP64 (0, for
-            // cutoffs below the FP32 range)
-            a.scr32 = cutoff >= 1e-30 ? (h->screen64 ? 2 : 1) : 0;
-            a.lo32 = (float)a.lo;
-            a.hi32 = std::isinf(a.hi) ? INFINITY : (float)a.hi;
-            a.tau32 = (float)tau;
-            a.band_hi32 = (float)band_hi;
-            a.tier = tier[k] == 0 ? 0 : 1;
-            a.rlist = routed ? h->d_rlist + h->rl_off[lidx[k]] : nullptr;
-            a.rcount = routed ? h->d_rcount + lidx[k] : nullptr;
-            a.rcap = routed ? h->rl_cap[lidx[k]] : 0;
-            a.asym64 = h->asym64;
-            a.widen_int = h->widen_int;
-            a.log_x = logs ? logs->x : nullptr;
-            a.log_y = logs ? logs->y : nullptr;
-            a.log_n = h->d_logn;
-            a.log_cap = logs ? logs->cap : 0;
-            a.nbra = A.n;
-            const int pi = (tier[k] == 0 && (mode == JK_PREC_MIXED || routed)) ? 1 : 0;
-            a.item_prefix = L.d_prefix[pi];
-            const long long nunits = L.nitems[pi] * specs[k].gx;   // work items x slabs
-            a.item_lo = nunits * h->part_index / h->part_count;
-            a.item_hi = nunits * (h->part_index + 1) / h->part_count;
-            a.chunk = pi ? h->chunk_hi : h->chunk;
-            a.prim_eps = std::min(cutoff, h->prim_eps);
-            a.prim_eps32 = (float)a.prim_eps;
-            a.omega = std::fabs(h->omega);
-            a.same_class = (L.c1 == L.c2) ? 1 : 0;
-            a.with_j = with_j ? 1 : 0;
-            a.with_k = with_k ? 1 : 0;
-            a.use_dmax = h->use_dmax;
-            a.ndm = ndm;
-            int grid = std::max(1, ki[k].blocks_per_sm) * h->num_sms;
-            const long long units = specs[k].G() <= 32 ? 4 : 1;   // work items in flight per CTA
-            long long need = (a.item_hi - a.item_lo + units - 1) / units;
-            if (need < grid) grid = (int)std::max(1LL, need);
-            void *params[] = {&a};
-            // External records become event nodes when captured into a graph
-            if (prof) CK(cudaEventRecordWithFlags(h->prof_ev[2 * k], sk, rec_flags));
-            CUresult r = drv().launchKernel(ki[k].fn, grid, 1, 1, specs[k].block(), 1, 1, (unsigned)ki[k].smem,
-                                            (CUstream)sk, params, nullptr);
-            if (r != CUDA_SUCCESS) return fail(JK_ERR_CUDA, "launch of %s failed: %d", specs[k].name().c_str(), (int)r);
-            if (prof) CK(cudaEventRecordWithFlags(h->prof_ev[2 * k + 1], sk, rec_flags));
-        }
-        if (nbranch > 1) {
+            return JK_OK;
+        };
+        auto join = [&]() -> int {
             for (int b = 1; b < nbranch; ++b) {
                 CK(cudaEventRecord(h->ev_join[b - 1], h->side[b - 1]));
                 CK(cudaStreamWaitEvent(s0, h->ev_join[b - 1], 0));
             }
+            return JK_OK;
+        };
+        if (int e = fork()) return e;
+        size_t k = 0;   // launch number
+        for (auto &T : tiers) {
+            if (T.t == 2) {
+                // the list kernels read what every FP64 launch wrote
+                if (int e = join()) return e;
+                if (int e = fork()) return e;
+            }
+            for (size_t g = 0; g < T.P->groups.size(); ++g, ++k) {
+                const LaunchGroup &G = T.P->groups[g];
+                const KInfo &ki = (*T.ki)[g];
+                cudaStream_t sk = k % nbranch ? h->side[k % nbranch - 1] : s0;
+                JkClassArgs a;
+                memset(&a, 0, sizeof a);
+                a.subs = T.P->d_subs + (T.t == 2 ? G.sub0 : 0);   // items index the plan's whole table
+                a.nsub = G.nsub;
+                a.items = T.P->d_items + T.P->item_off[g];
+                unsigned long long *ctr = h->d_ctr + (size_t)(T.t == 0 ? 0 : 1) * 2 * nl;
+                a.nitems = ctr + g;
+                a.work = ctr + nl + g;
+                a.pp64 = h->d_pp64;
+                a.pp32 = h->d_pp32;
+                a.mols = h->d_mols;
+                a.dmax = h->d_dmax;
+                a.dmax32 = h->d_dmax32;
+                a.dmax_mol = reinterpret_cast<const double *>(h->d_dmax_mol);
+                a.rys64 = h->d_rys64;
+                a.rys32 = h->d_rys32;
+                a.stats = h->d_stats + 3 * T.t;
+                a.stat_stride = 9;
+                a.err = h->d_err;
+                a.lo = lo_of(T.t);
+                a.hi = hi_of(T.t);
+                a.router = h->d_router;
+                a.tau = tau;
+                a.band_hi = band_hi;
+                a.scr32 = scr32;
+                a.lo32 = (float)a.lo;
+                a.hi32 = std::isinf(a.hi) ? INFINITY : (float)a.hi;
+                a.tau32 = (float)tau;
+                a.band_hi32 = (float)band_hi;
+                a.tier = T.t == 0 ? 0 : 1;
+                a.rlist = routed ? h->d_rlist : nullptr;
+                a.rcount = h->d_rcount;
+                a.roff = routed ? h->d_rl : nullptr;
+                a.rcap = routed ? h->d_rl + nl : nullptr;
+                a.asym64 = h->asym64;
+                a.widen_int = h->widen_int;
+                a.log_x = logs ? logs->x : nullptr;
+                a.log_y = logs ? logs->y : nullptr;
+                a.log_n = h->d_logn;
+                a.log_cap = logs ? logs->cap : 0;
+                a.prim_eps = std::min(cutoff, h->prim_eps);
+                a.prim_eps32 = (float)a.prim_eps;
+                a.omega = std::fabs(h->omega);
+                a.with_j = with_j ? 1 : 0;
+                a.with_k = with_k ? 1 : 0;
+                a.use_dmax = h->use_dmax;
+                a.ndm = ndm;
+                int grid = std::max(1, ki.blocks_per_sm) * h->num_sms;
+                const long long units = G.spec.G() <= 32 ? 4 : 1;   // work items in flight per CTA
+                const long long need = T.t == 2 ? grid : (G.cap * G.spec.gx + units - 1) / units;
+                if (need < grid) grid = (int)std::max(1LL, need);
+                void *params[] = {&a};
+                // External records become event nodes when captured into a graph
+                if (prof) CK(cudaEventRecordWithFlags(h->prof_ev[2 * k], sk, rec_flags));
+                CUresult r = drv().launchKernel(ki.fn, grid, 1, 1, G.spec.block(), 1, 1, (unsigned)ki.smem, (CUstream)sk,
+                                                params, nullptr);
+                if (r != CUDA_SUCCESS) return fail(JK_ERR_CUDA, "launch of %s failed: %d", G.spec.name().c_str(), (int)r);
+                if (prof) CK(cudaEventRecordWithFlags(h->prof_ev[2 * k + 1], sk, rec_flags));
+            }
         }
+        if (int e = join()) return e;
         if (h->ntiles > 0) {
             dim3 grid((unsigned)h->ntiles, ndm, 2);
             jk_symmetrize_kernel<<<grid, dim3(32, 8), 0, s0>>>(h->d_mols, h->d_tile_off, h->nmol, ndm, with_j, with_k);
@@ -1710,47 +1872,54 @@ int build_impl(jk_handle *h, const double *const *D, int32_t ndm, int with_j, in
         CK(cudaStreamSynchronize(st));
         float ms = 0;
         CK(cudaEventElapsedTime(&ms, h->ev0, h->ev1));
-        std::vector<unsigned long long> cnt(3 * nl);
-        CK(cudaMemcpy(cnt.data(), h->d_stats, sizeof(unsigned long long) * 3 * nl, cudaMemcpyDeviceToHost));
+        std::vector<unsigned long long> cnt(9 * nl);
+        CK(cudaMemcpy(cnt.data(), h->d_stats, sizeof(unsigned long long) * cnt.size(), cudaMemcpyDeviceToHost));
         int err = 0;
         CK(cudaMemcpy(&err, h->d_err, sizeof(int), cudaMemcpyDeviceToHost));
         if (routed) {
-            std::vector<unsigned long long> rc2(h->launches.size());
-            CK(cudaMemcpy(rc2.data(), h->d_rcount, sizeof(unsigned long long) * rc2.size(), cudaMemcpyDeviceToHost));
+            std::vector<unsigned long long> rc2(nl);
+            CK(cudaMemcpy(rc2.data(), h->d_rcount, sizeof(unsigned long long) * nl, cudaMemcpyDeviceToHost));
             h->rl_need.assign(rc2.begin(), rc2.end());
         }
         memset(stats, 0, sizeof(*stats));
         int64_t routed_fp32 = 0;
         stats->ms = ms;
-        stats->kernel_launches = (int64_t)specs.size() + nlaunch_aux;
+        stats->kernel_launches = (int64_t)nlaunch_class + nlaunch_aux;
         if (prof) { h->prof.clear(); h->prof_slot.clear(); }
-        for (size_t k = 0; k < specs.size(); ++k) {
-            const int slot = lidx[k] * 3 + tier[k];
-            unsigned long long nq = cnt[3 * slot], np = cnt[3 * slot + 1];
-            if (tier[k] == 0) stats->quartets_fp64 += (int64_t)nq;
-            else stats->quartets_fp32 += (int64_t)nq;
-            if (tier[k] == 2) routed_fp32 += (int64_t)nq;
-            stats->prim_quartets += (int64_t)np;
-            stats->flops_model += flops_of(specs[k], ndm, nq, np);
-            if (prof) {
-                jk_launch_prof p;
-                const KSpec &x = specs[k];
-                p.la = x.la; p.lb = x.lb; p.lc = x.lc; p.ld = x.ld;
-                p.na = x.na; p.nb = x.nb; p.nc = x.nc; p.nd = x.nd;
-                p.tier = tier[k] == 0 ? 0 : 1;
-                p.threads_per_quartet = x.G();
-                p.regs = ki[k].regs;
-                p.local_bytes = ki[k].local_bytes;
-                p.quartets = (int64_t)nq;
-                p.prim_quartets = (int64_t)np;
-                float lm = 0;
-                CK(cudaEventElapsedTime(&lm, h->prof_ev[2 * k], h->prof_ev[2 * k + 1]));
-                p.ms = lm;
-                p.flops_model = flops_of(x, ndm, nq, np);
-                h->prof.push_back(p);
-                h->prof_slot.push_back(slot);
+        size_t k = 0;   // launch number
+        for (auto &T : tiers)
+            for (size_t g = 0; g < T.P->groups.size(); ++g, ++k) {
+                const LaunchGroup &G = T.P->groups[g];
+                for (int i = G.sub0; i < G.sub0 + G.nsub; ++i) {
+                    const int l = T.P->launch[i], slot = l * 3 + T.t;
+                    KSpec x = h->launches[l].spec[T.t == 0 ? 0 : 1];
+                    x.op = op;
+                    const unsigned long long nq = cnt[3 * slot], np = cnt[3 * slot + 1];
+                    if (T.t == 0) stats->quartets_fp64 += (int64_t)nq;
+                    else stats->quartets_fp32 += (int64_t)nq;
+                    if (T.t == 2) routed_fp32 += (int64_t)nq;
+                    stats->prim_quartets += (int64_t)np;
+                    stats->flops_model += flops_of(x, ndm, nq, np);
+                    if (prof) {   // one class pair per launch
+                        const KInfo &ki = (*T.ki)[g];
+                        jk_launch_prof p;
+                        p.la = x.la; p.lb = x.lb; p.lc = x.lc; p.ld = x.ld;
+                        p.na = x.na; p.nb = x.nb; p.nc = x.nc; p.nd = x.nd;
+                        p.tier = T.t == 0 ? 0 : 1;
+                        p.threads_per_quartet = x.G();
+                        p.regs = ki.regs;
+                        p.local_bytes = ki.local_bytes;
+                        p.quartets = (int64_t)nq;
+                        p.prim_quartets = (int64_t)np;
+                        float lm = 0;
+                        CK(cudaEventElapsedTime(&lm, h->prof_ev[2 * k], h->prof_ev[2 * k + 1]));
+                        p.ms = lm;
+                        p.flops_model = flops_of(x, ndm, nq, np);
+                        h->prof.push_back(p);
+                        h->prof_slot.push_back(slot);
+                    }
+                }
             }
-        }
         stats->quartets_routed = routed_fp32;
         h->err_pending = false;
         if (err) return device_error(h, err, "this build");
@@ -1886,7 +2055,7 @@ int tune_impl(jk_handle *h, const double *const *D, int32_t ndm, int with_j, int
     std::vector<Item> items;
     for (size_t l = 0; l < h->launches.size(); ++l) {
         const Launch &L = h->launches[l];
-        if (L.nitems[0] == 0 || L.cost < min_share * total) continue;
+        if (L.cost < min_share * total) continue;
         for (int t : tiers) {
             Item it;
             it.l = (int)l;
@@ -1928,6 +2097,8 @@ int tune_impl(jk_handle *h, const double *const *D, int32_t ndm, int with_j, int
     int rc = JK_OK;
     for (size_t r = 0; r < nround && rc == JK_OK; ++r) {
         for (auto &it : items) h->launches[it.l].spec[it.t] = it.c[std::min(r, it.c.size() - 1)];
+        cudaDeviceSynchronize();
+        h->plans.clear();
         std::vector<double> tm(items.size(), INFINITY);
         for (int rep2 = 0; rep2 < 2 && rc == JK_OK; ++rep2) {
             jk_stats st;
@@ -1959,8 +2130,9 @@ int tune_impl(jk_handle *h, const double *const *D, int32_t ndm, int with_j, int
         before += it.first;
         after += it.best;
     }
-    for (auto &g : h->graphs) cudaGraphExecDestroy(g.second.first);
-    h->graphs.clear();
+    cudaDeviceSynchronize();
+    drop_graphs(h);
+    h->plans.clear();
     if (rc) return rc;
     tune_store(h->device, chosen);
     if (rep) {
@@ -2095,9 +2267,10 @@ int jk_set_option(jk_handle *h, const char *key, double value)
         const int c0 = k == "chunk" ? (int)value : h->chunk, c1 = k == "chunk" ? h->chunk_hi : (int)value;
         if (c0 != h->chunk || c1 != h->chunk_hi) {
             cudaDeviceSynchronize();
-            for (auto &g : h->graphs) cudaGraphExecDestroy(g.second.first);
-            h->graphs.clear();
-            if (int rc = plan_items(h, c0, c1)) return rc;
+            drop_graphs(h);
+            h->plans.clear();
+            h->chunk = c0;
+            h->chunk_hi = c1;
         }
     }
     else if (k == "screen64") h->screen64 = value != 0;
@@ -2105,11 +2278,10 @@ int jk_set_option(jk_handle *h, const char *key, double value)
         if (!(value >= 1 && value <= 1e9)) return fail(JK_ERR_ARG, "route_cap must be in [1, 1e9]");
         if (value != h->route_cap) {
             cudaDeviceSynchronize();
-            cudaFree(h->d_rlist); cudaFree(h->d_rcount);
-            h->d_rlist = nullptr; h->d_rcount = nullptr;
+            cudaFree(h->d_rlist); cudaFree(h->d_rl);
+            h->d_rlist = nullptr; h->d_rl = nullptr;
             h->rl_cap.clear(); h->rl_need.clear();
-            for (auto &g : h->graphs) cudaGraphExecDestroy(g.second.first);
-            h->graphs.clear();
+            drop_graphs(h);
         }
         h->route_cap = value;
     }
@@ -2203,8 +2375,7 @@ int jk_router_load(jk_handle *h, const jk_router_blob *w)
     router_dev_from_blob(*w, d);
     CK(cudaMemcpy(h->d_router, &d, sizeof d, cudaMemcpyHostToDevice));
     h->has_router = true;
-    for (auto &g : h->graphs) cudaGraphExecDestroy(g.second.first);
-    h->graphs.clear();
+    drop_graphs(h);
     return JK_OK;
 }
 

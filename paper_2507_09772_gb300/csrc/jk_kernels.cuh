@@ -1,7 +1,9 @@
 // Integral kernels of the JK build, compiled at run time by NVRTC for
-// sm_103a, one instantiation per (l_a, l_b, l_c, l_d, n_a, n_b, n_c, n_d)
-// class and per fragmentation, density count, J/K flags and precision
-// (the static parameters of Table 1 of the paper). The library prepends
+// sm_103a, one instantiation per (l_a, l_b, l_c, l_d), fragmentation,
+// density count, J/K flags and precision (the static parameters of Table 1 of
+// the paper, except the primitive counts, which are loop limits read from the
+// class pair: one launch then runs every class pair of the same angular
+// momenta, see the class kernel). The library prepends
 // jk_types.h and the generated rys_params.cuh.
 //
 // Method (Sec. 2 of the paper):
@@ -335,10 +337,9 @@ __device__ __forceinline__ void jk_op_root(R Tt, R rho, R pref, double omega, in
     }
 }
 
-template <int LA, int LB, int LC, int LD, int NPA, int NPB, int NPC, int NPD,
-          int GA, int GB, int GC, int GD, typename R, int OP = 0,
+template <int LA, int LB, int LC, int LD, int GA, int GB, int GC, int GD, typename R, int OP = 0,
           int NT = JkShape<LA, LB, LC, LD, GA, GB, GC, GD, OP>::G>
-__device__ __forceinline__ int jk_quartet(const JkPair &bra, const JkPair &ket, float qthr, double omega, int a64,
+__device__ __forceinline__ int jk_quartet(const JkPair &bra, const JkPair &ket, int nab, int ncd, float qthr, double omega, int a64,
                                            const typename JkPP<R>::T *__restrict__ pp,
                                            const R *__restrict__ rys, R *grp, unsigned gmask, int tg, bool act,
                                            const JkOffsets<JkShape<LA, LB, LC, LD, GA, GB, GC, GD, OP>> &off,
@@ -363,11 +364,12 @@ __device__ __forceinline__ int jk_quartet(const JkPair &bra, const JkPair &ket, 
     const float qb0 = jk_pp_q(bpp[0]);
     int nprim = 0;
 #pragma unroll 1
-    for (int kl = 0; kl < NPC * NPD; ++kl) {
+    for (int kl = 0; kl < ncd; ++kl) {
         const PPT kp = kpp[kl];
         const float qk = jk_pp_q(kp);
         if (qb0 * qk <= qthf) break;
-        for (int ij = 0; ij < NPA * NPB; ++ij) {
+#pragma unroll 1
+        for (int ij = 0; ij < nab; ++ij) {
             const PPT bp = bpp[ij];
             if (jk_pp_q(bp) * qk <= qthf) break;
             ++nprim;
@@ -476,35 +478,36 @@ template <> __device__ __forceinline__ const float *jk_rys<float>(const JkClassA
 // kernel (MODE 3) of the class pair. Returns whether this lane's quartet was
 // listed; a quartet that finds the list full stays in FP64. All 32 lanes of
 // the warp call it.
-__device__ __forceinline__ bool jk_route_out(const JkClassArgs &args, bool rel, int item, int j, float dq)
+__device__ __forceinline__ bool jk_route_out(const JkClassArgs &args, int launch, bool rel, int item, int j, float dq)
 {
     const unsigned m = __ballot_sync(0xffffffffu, rel);
     if (!m) return false;
     const int lane = threadIdx.x & 31, first = __ffs(m) - 1;
     unsigned long long base = 0;
-    if (lane == first) base = atomicAdd(args.rcount, (unsigned long long)__popc(m));
+    if (lane == first) base = atomicAdd(args.rcount + launch, (unsigned long long)__popc(m));
     base = __shfl_sync(0xffffffffu, base, first);
     const long long pos = (long long)base + __popc(m & ((1u << lane) - 1u));
-    const bool listed = rel && pos < args.rcap;
+    const bool listed = rel && pos < args.rcap[launch];
     if (listed) {
         JkRouted e;
         e.item = item; e.ket = j; e.dmq = dq; e.pad = 0;
-        args.rlist[pos] = e;
+        args.rlist[args.roff[launch] + pos] = e;
     }
     return listed;
 }
 
 // ------------------------------------------------- screening of a candidate
 template <int MODE>
-__device__ __forceinline__ void jk_screen_bound(const JkClassArgs &args, const JkPair &bra, const JkMol &mol,
+__device__ __forceinline__ void jk_screen_bound(const JkClassArgs &args, const JkPair *__restrict__ kets,
+                                                const JkPair &bra, const JkMol &mol,
                                                 const double *dmx, double dmol, float dmol32, int j, int ke,
                                                 bool &sig, bool &stop, bool &band, float &dmq, float &Bout);
 // Keep (bra, ket j) iff lo < Q_ab Q_cd Dmax <= hi; `stop` when even the
 // molecule's largest density element cannot lift this ket (and every later
 // one, kets being sorted by Q) above lo.
 template <int MODE>
-__device__ __forceinline__ void jk_screen(const JkClassArgs &args, const JkPair &bra, const JkPairFeat &braf,
-                                          const JkMol &mol, const double *dmx, double dmol, float dmol32, int item,
+__device__ __forceinline__ void jk_screen(const JkClassArgs &args, const JkSub &sub, const JkPair &bra,
+                                          const JkPairFeat &braf, const JkMol &mol, const double *dmx, double dmol, float dmol32, int item,
                                           int j, int ke, bool &sig, bool &stop, bool &band, float &dmq,
                                           unsigned short *rsm)
 {
@@ -513,16 +516,16 @@ __device__ __forceinline__ void jk_screen(const JkClassArgs &args, const JkPair 
     band = false;
     dmq = 1.0f;
     float B = 0.0f;
-    jk_screen_bound<MODE>(args, bra, mol, dmx, dmol, dmol32, j, ke, sig, stop, band, dmq, B);
+    jk_screen_bound<MODE>(args, sub.ket, bra, mol, dmx, dmol, dmol32, j, ke, sig, stop, band, dmq, B);
     if (MODE == 1) {
         // learned router for the band candidates, all lanes together on the
         // tensor cores; `band` then marks the quartets released to FP32
         bool listed = false;
         if (__ballot_sync(0xffffffffu, band)) {
-            const JkPairFeat kf = band ? args.ket_feat[j] : braf;
+            const JkPairFeat kf = band ? sub.ket_feat[j] : braf;
             const bool to32 = jk_router_to_fp32_warp(args.router, braf, kf, band ? B : 2.0f * args.tau32,
                                                      band ? dmq : 1.0f, args.tau32, rsm);
-            listed = jk_route_out(args, band && to32, item, j, dmq);
+            listed = jk_route_out(args, sub.launch, band && to32, item, j, dmq);
             if (band) sig = !listed;
         }
         band = listed;
@@ -538,12 +541,13 @@ __device__ __forceinline__ bool jk_near(float x, float y)
 }
 
 template <int MODE>
-__device__ __forceinline__ void jk_screen_bound(const JkClassArgs &args, const JkPair &bra, const JkMol &mol,
+__device__ __forceinline__ void jk_screen_bound(const JkClassArgs &args, const JkPair *__restrict__ kets,
+                                                const JkPair &bra, const JkMol &mol,
                                                 const double *dmx, double dmol, float dmol32, int j, int ke,
                                                 bool &sig, bool &stop, bool &band, float &dmq, float &Bout)
 {
     if (j >= ke) return;
-    const JkPair &kt = args.ket[j];
+    const JkPair &kt = kets[j];
     if (args.scr32) {
         // FP32 bounds: a handful of FP32 operations per candidate instead of
         // FP64-pipe work (an FP64 instruction costs the FP32 tier 64 FP32
@@ -789,28 +793,37 @@ __device__ __forceinline__ void jk_flush_jab(R (&jab)[NDM][FA][FB], const JkMol 
                     jk_red_add(mol.J + m * nn + (long long)(a0 + ia) * mol.nao + b0 + ib, jk_wide(jab[m][ia][ib], wi));
 }
 
-// Work item t -> bra pair i (binary search in the item prefix) and the ket
-// range of its chunk. The last chunk of a bra runs to the molecule's last
-// ket, so the partition covers every candidate whatever the estimate was.
-__device__ __forceinline__ int jk_item_bra(const JkClassArgs &args, long long t)
+// Counters of a warp (or CTA) for the class pair it works on, added to the
+// class pair's statistics when it moves to another one.
+struct JkCount {
+    unsigned long long nq, nprim, nband;
+};
+__device__ __forceinline__ void jk_count_flush(const JkClassArgs &args, int launch, JkCount &c)
 {
-    int lo = 0, hi = args.nbra - 1;
-    while (lo < hi) {
-        const int mid = (lo + hi + 1) >> 1;
-        if (__ldg(args.item_prefix + mid) <= t) lo = mid; else hi = mid - 1;
+    if (launch >= 0 && (c.nq || c.nband)) {
+        unsigned long long *st = args.stats + (long long)launch * args.stat_stride;
+        atomicAdd(st, c.nq);
+        atomicAdd(st + 1, c.nprim);
+        if (c.nband) atomicAdd(st + 2, c.nband);
     }
-    return lo;
+    c.nq = c.nprim = c.nband = 0;
 }
 
 // ------------------------------------------------------- the class kernel
-// Persistent: warps (or, for groups of more than 32 threads, whole CTAs)
-// take work items from a global counter until none are left. A group of
-// more than 256 threads (the largest classes, e.g. (gg|gg)) is split over
-// X CTAs: work item t is slab t % X of quartet item t / X, each CTA builds
-// the roots and 2D tables itself and evaluates the elements of its G / X
-// threads.
-template <int LA, int LB, int LC, int LD, int NPA, int NPB, int NPC, int NPD,
-          int GA, int GB, int GC, int GD, int X, int NDM, int DOJ, int DOK, typename R, int MODE, int OP>
+// One launch runs every class pair of the same angular momenta and fragment
+// shape. Persistent: warps (or, for groups of more than 32 threads, whole
+// CTAs) take work items, a bra pair and a range of its kets, from the list
+// that jk_plan_kernel wrote for this build, the first by their own index and
+// the next ones from a counter. A group of more than 256 threads (the largest
+// classes, e.g. (gg|gg)) is split over X CTAs: work unit t is slab t % X of
+// item t / X, each CTA builds the roots and 2D tables itself and evaluates
+// the elements of its G / X threads.
+//
+// Why class pairs share a launch: a 6-31G*-shaped basis has 231 class pairs
+// (21 angular momenta); launched one by one, most of them were too small to
+// fill the GPU and ended in a tail of a few long items each.
+template <int LA, int LB, int LC, int LD, int GA, int GB, int GC, int GD, int X, int NDM, int DOJ, int DOK,
+          typename R, int MODE, int OP>
 __global__ void __launch_bounds__(JkShape<LA, LB, LC, LD, GA, GB, GC, GD>::G <= 32 ? 128
                                   : ((JkShape<LA, LB, LC, LD, GA, GB, GC, GD>::G / X + 31) / 32) * 32)
 jk_class_kernel(const JkClassArgs args)
@@ -822,6 +835,8 @@ jk_class_kernel(const JkClassArgs args)
     const int lane = threadIdx.x & 31;
     const typename JkPP<R>::T *pp = jk_pp<R>(args);
     const R *rys = jk_rys<R>(args);
+    const long long nitems = MODE == 3 ? 0 : (long long)*args.nitems;
+    if (MODE != 3 && (long long)blockIdx.x * (G <= 32 ? 4 : 1) >= nitems * X) return;
     // The FP32 tier reads its Rys table from shared memory: lanes gather
     // coefficients of unrelated intervals, which from global memory costs one
     // L1 wavefront per lane and load. Only this class's N-root table, copied
@@ -838,6 +853,8 @@ jk_class_kernel(const JkClassArgs args)
         rys = reinterpret_cast<const R *>(jk_smem_raw);
         smem_groups = reinterpret_cast<R *>(jk_smem_raw) + NT;
     }
+    JkCount cnt = {0, 0, 0};
+    int cur = -1;   // class pair the counters belong to
 
     static_assert(X == 1 || (G > 32 && G % X == 0), "a split group spans whole CTAs");
     if constexpr (G <= 32) {
@@ -859,77 +876,89 @@ jk_class_kernel(const JkClassArgs args)
         const int gd = tg % GD, gc = (tg / GD) % GC, gb = (tg / (GD * GC)) % GB, ga = tg / (GD * GC * GB);
         JkOffsets<S> off;
         jk_make_offsets<LA, LB, LC, LD, GA, GB, GC, GD, S>(ga, gb, gc, gd, off);
+        const long long nw = (long long)gridDim.x * 4, w0 = (long long)blockIdx.x * 4 + wib;
         if constexpr (MODE == 3) {
             // FP32 list kernel of a routed build: the band quartets the FP64
             // tier released, one per group; each bra's J block is flushed on
-            // its own (the quartets of a warp belong to unrelated bras)
-            const long long n = min((long long)*args.rcount, args.rcap);
-            unsigned long long nq = 0, nprim = 0;
-            for (;;) {
-                long long t = 0;
-                if (lane == 0) t = (long long)atomicAdd(args.work, (unsigned long long)NGW);
-                t = __shfl_sync(0xffffffffu, t, 0);
-                if (t >= n) break;
-                const long long e = t + gw;
-                if (active && e < n) {
-                    const JkRouted rq = args.rlist[e];
-                    const JkPair bra = args.bra[rq.item];
-                    const JkPair ket = args.ket[rq.ket];
-                    const JkMol mol = args.mols[bra.mol];
-                    R T[S::EPT];
+            // its own (the quartets of a warp belong to unrelated bras). Each
+            // class pair's list is dealt to the warps in turn, the next one
+            // from where the last ended.
+            long long dealt = 0;
+            for (int isub = 0; isub < args.nsub; ++isub) {
+                const JkSub &sub = args.subs[isub];
+                const int launch = sub.launch;
+                const long long n = min((long long)args.rcount[launch], args.rcap[launch]);
+                if (n <= 0) continue;
+                const long long rounds = (n + NGW - 1) / NGW;
+                long long r = w0 - dealt % nw;
+                if (r < 0) r += nw;
+                dealt += rounds;
+                const JkRouted *list = args.rlist + args.roff[launch];
+                for (; r < rounds; r += nw) {
+                    const long long e = r * NGW + gw;
+                    if (active && e < n) {
+                        const JkRouted rq = list[e];
+                        const JkPair bra = sub.bra[rq.item];
+                        const JkPair ket = sub.ket[rq.ket];
+                        const JkMol mol = args.mols[bra.mol];
+                        R T[S::EPT];
 #pragma unroll
-                    for (int k = 0; k < S::EPT; ++k) T[k] = (R)0;
-                    const int np = jk_quartet<LA, LB, LC, LD, NPA, NPB, NPC, NPD, GA, GB, GC, GD, R, OP>(
-                        bra, ket, __fdiv_rn(args.prim_eps32, rq.dmq), args.omega, args.asym64, pp, rys, grp, gmask,
-                        tg, true, off, T);
-                    R f = (R)1;
-                    if (bra.a == bra.b) f *= (R)0.5;
-                    if (ket.a == ket.b) f *= (R)0.5;
-                    if (args.same_class && rq.ket == rq.item) f *= (R)0.5;
-                    R jab[NDM][FA][FB];
+                        for (int k = 0; k < S::EPT; ++k) T[k] = (R)0;
+                        const int np = jk_quartet<LA, LB, LC, LD, GA, GB, GC, GD, R, OP>(
+                            bra, ket, sub.nab, sub.ncd, __fdiv_rn(args.prim_eps32, rq.dmq), args.omega, args.asym64,
+                            pp, rys, grp, gmask, tg, true, off, T);
+                        R f = (R)1;
+                        if (bra.a == bra.b) f *= (R)0.5;
+                        if (ket.a == ket.b) f *= (R)0.5;
+                        if (sub.same_class && rq.ket == rq.item) f *= (R)0.5;
+                        R jab[NDM][FA][FB];
 #pragma unroll
-                    for (int m = 0; m < NDM; ++m)
+                        for (int m = 0; m < NDM; ++m)
 #pragma unroll
-                        for (int i = 0; i < FA; ++i)
+                            for (int i = 0; i < FA; ++i)
 #pragma unroll
-                            for (int jj = 0; jj < FB; ++jj) jab[m][i][jj] = (R)0;
-                    const int a0 = bra.a_ao + ga * FA, b0 = bra.b_ao + gb * FB;
-                    jk_contract<FA, FB, FC, FD, NDM, DOJ, DOK, R>(T, f, mol, a0, b0, ket.a_ao + gc * FC,
-                                                                 ket.b_ao + gd * FD, jab, args.widen_int);
-                    if (DOJ) jk_flush_jab<FA, FB, NDM, R>(jab, mol, a0, b0, args.widen_int);
-                    if (tg == 0) { ++nq; nprim += np; }
+                                for (int jj = 0; jj < FB; ++jj) jab[m][i][jj] = (R)0;
+                        const int a0 = bra.a_ao + ga * FA, b0 = bra.b_ao + gb * FB;
+                        jk_contract<FA, FB, FC, FD, NDM, DOJ, DOK, R>(T, f, mol, a0, b0, ket.a_ao + gc * FC,
+                                                                     ket.b_ao + gd * FD, jab, args.widen_int);
+                        if (DOJ) jk_flush_jab<FA, FB, NDM, R>(jab, mol, a0, b0, args.widen_int);
+                        if (tg == 0) { ++cnt.nq; cnt.nprim += np; }
+                    }
                 }
-            }
-            for (int o = 16; o > 0; o >>= 1) {
-                nq += __shfl_xor_sync(0xffffffffu, nq, o);
-                nprim += __shfl_xor_sync(0xffffffffu, nprim, o);
-            }
-            if (lane == 0 && nq) {
-                atomicAdd(args.stats, nq);
-                atomicAdd(args.stats + 1, nprim);
+                for (int o = 16; o > 0; o >>= 1) {
+                    cnt.nq += __shfl_xor_sync(0xffffffffu, cnt.nq, o);
+                    cnt.nprim += __shfl_xor_sync(0xffffffffu, cnt.nprim, o);
+                }
+                if (lane == 0) jk_count_flush(args, launch, cnt);
+                cnt.nq = cnt.nprim = 0;
             }
             return;
         }
-        for (;;) {
-            long long t = 0;
-            if (lane == 0) t = args.item_lo + (long long)atomicAdd(args.work, 1ull);
-            t = __shfl_sync(0xffffffffu, t, 0);
-            if (t >= args.item_hi) break;
-            const int item = jk_item_bra(args, t);
-            const int ch = (int)(t - __ldg(args.item_prefix + item));
-            const int nch = (int)(__ldg(args.item_prefix + item + 1) - __ldg(args.item_prefix + item));
-            const JkPair bra = args.bra[item];
+        // the FP32 tier's items are short: the next ticket is drawn while this
+        // one runs (an FP64 item hides the counter's latency itself, and a
+        // ticket held back by a long item would lengthen the launch's tail)
+        constexpr bool AHEAD = JkIsFloat<R>::v;
+        long long t = w0;
+        while (t < nitems) {
+            unsigned long long nx = 0;
+            if (AHEAD && lane == 0) nx = atomicAdd(args.work, 1ull);
+            const JkItem wi = args.items[t];
+            const JkSub &sub = args.subs[wi.sub];
+            const JkPair *__restrict__ kets = sub.ket;
+            const int item = wi.bra, nab = sub.nab, ncd = sub.ncd, same_class = sub.same_class;
+            const int kb = wi.kb, ke = wi.ke;
+            if (sub.launch != cur) {
+                if (lane == 0) jk_count_flush(args, cur, cnt);
+                cur = sub.launch;
+            }
+            const JkPair bra = sub.bra[item];
             const JkMol mol = args.mols[bra.mol];
-            const int kb0 = args.same_class ? item : args.ket_beg[bra.mol];
-            const int kend = args.ket_end[bra.mol];
-            const int kb = min(kend, kb0 + ch * args.chunk);
-            const int ke = (ch == nch - 1) ? kend : min(kend, kb + args.chunk);
             const double *dmx = args.dmax + mol.dmax_off;
             const double dmol = args.use_dmax ? args.dmax_mol[bra.mol] : 1.0;
             const float dmol32 = (float)dmol;
             const int a0 = bra.a_ao + ga * FA, b0 = bra.b_ao + gb * FB;
             JkPairFeat braf;
-            if (MODE != 0) braf = args.bra_feat[item];
+            if (MODE != 0) braf = sub.bra_feat[item];
             R jab[NDM][FA][FB];
 #pragma unroll
             for (int m = 0; m < NDM; ++m)
@@ -937,7 +966,7 @@ jk_class_kernel(const JkClassArgs args)
                 for (int i = 0; i < FA; ++i)
 #pragma unroll
                     for (int j = 0; j < FB; ++j) jab[m][i][j] = (R)0;
-            unsigned long long nq = 0, nband = 0, nprim = 0;
+            int nq = 0, nband = 0, nprim = 0;
             // significant kets wait in a per-warp queue (in scan order) until
             // a round can give every group of the warp one; partial rounds
             // only at the end of the item
@@ -948,7 +977,7 @@ jk_class_kernel(const JkClassArgs args)
             for (int base = kb; base < ke; base += 32) {
                 bool sig = false, stop = false, band = false;
                 float dmq = 1.0f, B = 0.0f;
-                jk_screen_bound<MODE>(args, bra, mol, dmx, dmol, dmol32, base + lane, ke, sig, stop, band, dmq, B);
+                jk_screen_bound<MODE>(args, kets, bra, mol, dmx, dmol, dmol32, base + lane, ke, sig, stop, band, dmq, B);
                 const unsigned lt = (1u << lane) - 1u;
                 const bool def = sig && !band;   // decided by the bounds alone
                 const unsigned mdef = __ballot_sync(0xffffffffu, def);
@@ -981,11 +1010,11 @@ jk_class_kernel(const JkClassArgs args)
                         const int j = mine ? s_bk[wib][lane] : 0;
                         const float dj = mine ? s_bd[wib][lane] : 1.0f;
                         const float bj = mine ? s_bb[wib][lane] : 2.0f * args.tau32;
-                        const JkPairFeat kf = mine ? args.ket_feat[j] : braf;
+                        const JkPairFeat kf = mine ? sub.ket_feat[j] : braf;
                         const bool to32 = jk_router_to_fp32_warp(args.router, braf, kf, bj, dj, args.tau32, rsm);
                         // released quartets go to the FP32 list kernel; the
                         // rest of the band stays here, in FP64
-                        const bool listed = jk_route_out(args, mine && to32, item, j, dj);
+                        const bool listed = jk_route_out(args, cur, mine && to32, item, j, dj);
                         const bool keep = mine && !listed;
                         const unsigned mk = __ballot_sync(0xffffffffu, keep);
                         nq += __popc(mk);
@@ -1017,19 +1046,18 @@ jk_class_kernel(const JkClassArgs args)
                         dmk = s_qd[wib][gw];
                     }
                     if (myket >= 0) {
-                        const JkPair ket = args.ket[myket];
+                        const JkPair ket = kets[myket];
                         R T[S::EPT];
 #pragma unroll
                         for (int k = 0; k < S::EPT; ++k) T[k] = (R)0;
-                        const int np = jk_quartet<LA, LB, LC, LD, NPA, NPB, NPC, NPD, GA, GB, GC, GD, R, OP>(
-                            bra, ket, __fdiv_rn(args.prim_eps32, dmk), args.omega, args.asym64, pp, rys, grp, gmask,
-                            tg, true,
-                            off, T);
+                        const int np = jk_quartet<LA, LB, LC, LD, GA, GB, GC, GD, R, OP>(
+                            bra, ket, nab, ncd, __fdiv_rn(args.prim_eps32, dmk), args.omega, args.asym64, pp, rys, grp,
+                            gmask, tg, true, off, T);
                         if (tg == 0) nprim += np;
                         R f = (R)1;
                         if (bra.a == bra.b) f *= (R)0.5;
                         if (ket.a == ket.b) f *= (R)0.5;
-                        if (args.same_class && myket == item) f *= (R)0.5;
+                        if (same_class && myket == item) f *= (R)0.5;
                         jk_contract<FA, FB, FC, FD, NDM, DOJ, DOK, R>(T, f, mol, a0, b0, ket.a_ao + gc * FC,
                                                                      ket.b_ao + gd * FD, jab, args.widen_int);
                         if (MODE == 2) {
@@ -1038,7 +1066,7 @@ jk_class_kernel(const JkClassArgs args)
                             for (int k = 0; k < S::EPT; ++k) tm = fmax(tm, fabs((double)T[k]));
                             for (int q = 0; q < G; ++q) tm = fmax(tm, __shfl_sync(gmask, tm, (gw * G + q) & 31));
                             if (tg == 0)
-                                jk_log_sample(args, bra, ket, braf, args.ket_feat[myket],
+                                jk_log_sample(args, bra, ket, braf, sub.ket_feat[myket],
                                               jk_quartet_dmax(args, bra, ket, mol, dmx), tm);
                         }
                     }
@@ -1056,13 +1084,13 @@ jk_class_kernel(const JkClassArgs args)
                 if (last) break;
             }
             if (DOJ && active) jk_flush_jab<FA, FB, NDM, R>(jab, mol, a0, b0, args.widen_int);
-            for (int o = 16; o > 0; o >>= 1) nprim += __shfl_xor_sync(0xffffffffu, nprim, o);
-            if (lane == 0 && nq) {
-                atomicAdd(args.stats, nq);
-                atomicAdd(args.stats + 1, nprim);
-                if (nband) atomicAdd(args.stats + 2, nband);
-            }
+            cnt.nq += nq;
+            cnt.nband += nband;
+            cnt.nprim += __reduce_add_sync(0xffffffffu, (unsigned)nprim);
+            if (!AHEAD && lane == 0) nx = atomicAdd(args.work, 1ull);
+            t = nw + (long long)__shfl_sync(0xffffffffu, nx, 0);
         }
+        if (lane == 0) jk_count_flush(args, cur, cnt);
     } else {
         // one group (or one of its X slabs) per CTA of round_up(G / X, 32) threads
         constexpr int NTC = G / X;
@@ -1080,65 +1108,63 @@ jk_class_kernel(const JkClassArgs args)
         jk_make_offsets<LA, LB, LC, LD, GA, GB, GC, GD, S>(ga, gb, gc, gd, off);
         if constexpr (MODE == 3) {
             // FP32 list kernel of a routed build: one released quartet (or one
-            // of its X slabs) per CTA at a time
-            const long long n = min((long long)*args.rcount, args.rcap);
-            unsigned long long nq = 0, nprim = 0;
-            for (;;) {
-                if (threadIdx.x == 0) s_item = (long long)atomicAdd(args.work, 1ull);
-                __syncthreads();
-                const long long tt = s_item;
-                __syncthreads();
-                if (tt >= n * X) break;
-                const long long e = X == 1 ? tt : tt / X;
-                const int slab = (int)(tt - e * X);
-                if constexpr (X > 1) {
-                    const int tgl = slab * NTC + tgc;
-                    gd = tgl % GD; gc = (tgl / GD) % GC; gb = (tgl / (GD * GC)) % GB; ga = tgl / (GD * GC * GB);
-                    jk_make_offsets<LA, LB, LC, LD, GA, GB, GC, GD, S>(ga, gb, gc, gd, off);
+            // of its X slabs) per CTA at a time, dealt as in the warp path
+            long long dealt = 0;
+            for (int isub = 0; isub < args.nsub; ++isub) {
+                const JkSub &sub = args.subs[isub];
+                const int launch = sub.launch;
+                const long long n = min((long long)args.rcount[launch], args.rcap[launch]) * X;
+                if (n <= 0) continue;
+                long long tt = (long long)blockIdx.x - dealt % gridDim.x;
+                if (tt < 0) tt += gridDim.x;
+                dealt += n;
+                const JkRouted *list = args.rlist + args.roff[launch];
+                for (; tt < n; tt += gridDim.x) {
+                    const long long e = X == 1 ? tt : tt / X;
+                    const int slab = (int)(tt - e * X);
+                    if constexpr (X > 1) {
+                        const int tgl = slab * NTC + tgc;
+                        gd = tgl % GD; gc = (tgl / GD) % GC; gb = (tgl / (GD * GC)) % GB; ga = tgl / (GD * GC * GB);
+                        jk_make_offsets<LA, LB, LC, LD, GA, GB, GC, GD, S>(ga, gb, gc, gd, off);
+                    }
+                    const JkRouted rq = list[e];
+                    const JkPair bra = sub.bra[rq.item];
+                    const JkPair ket = sub.ket[rq.ket];
+                    const JkMol mol = args.mols[bra.mol];
+                    R T[S::EPT];
+#pragma unroll
+                    for (int k = 0; k < S::EPT; ++k) T[k] = (R)0;
+                    const int np = jk_quartet<LA, LB, LC, LD, GA, GB, GC, GD, R, OP, NTC>(
+                        bra, ket, sub.nab, sub.ncd, __fdiv_rn(args.prim_eps32, rq.dmq), args.omega, args.asym64, pp,
+                        rys, grp, 0u, tg, act, off, T);
+                    if (act) {
+                        R f = (R)1;
+                        if (bra.a == bra.b) f *= (R)0.5;
+                        if (ket.a == ket.b) f *= (R)0.5;
+                        if (sub.same_class && rq.ket == rq.item) f *= (R)0.5;
+                        R jab[NDM][FA][FB];
+#pragma unroll
+                        for (int m = 0; m < NDM; ++m)
+#pragma unroll
+                            for (int i = 0; i < FA; ++i)
+#pragma unroll
+                                for (int jj = 0; jj < FB; ++jj) jab[m][i][jj] = (R)0;
+                        const int a0 = bra.a_ao + ga * FA, b0 = bra.b_ao + gb * FB;
+                        jk_contract<FA, FB, FC, FD, NDM, DOJ, DOK, R>(T, f, mol, a0, b0, ket.a_ao + gc * FC,
+                                                                     ket.b_ao + gd * FD, jab, args.widen_int);
+                        if (DOJ) jk_flush_jab<FA, FB, NDM, R>(jab, mol, a0, b0, args.widen_int);
+                    }
+                    if (slab == 0) { ++cnt.nq; cnt.nprim += np; }
+                    // every thread is done with this entry's shared tables
+                    __syncthreads();
                 }
-                const JkRouted rq = args.rlist[e];
-                const JkPair bra = args.bra[rq.item];
-                const JkPair ket = args.ket[rq.ket];
-                const JkMol mol = args.mols[bra.mol];
-                R T[S::EPT];
-#pragma unroll
-                for (int k = 0; k < S::EPT; ++k) T[k] = (R)0;
-                const int np = jk_quartet<LA, LB, LC, LD, NPA, NPB, NPC, NPD, GA, GB, GC, GD, R, OP, NTC>(
-                    bra, ket, __fdiv_rn(args.prim_eps32, rq.dmq), args.omega, args.asym64, pp, rys, grp, 0u, tg, act,
-                    off, T);
-                if (act) {
-                    R f = (R)1;
-                    if (bra.a == bra.b) f *= (R)0.5;
-                    if (ket.a == ket.b) f *= (R)0.5;
-                    if (args.same_class && rq.ket == rq.item) f *= (R)0.5;
-                    R jab[NDM][FA][FB];
-#pragma unroll
-                    for (int m = 0; m < NDM; ++m)
-#pragma unroll
-                        for (int i = 0; i < FA; ++i)
-#pragma unroll
-                            for (int jj = 0; jj < FB; ++jj) jab[m][i][jj] = (R)0;
-                    const int a0 = bra.a_ao + ga * FA, b0 = bra.b_ao + gb * FB;
-                    jk_contract<FA, FB, FC, FD, NDM, DOJ, DOK, R>(T, f, mol, a0, b0, ket.a_ao + gc * FC,
-                                                                 ket.b_ao + gd * FD, jab, args.widen_int);
-                    if (DOJ) jk_flush_jab<FA, FB, NDM, R>(jab, mol, a0, b0, args.widen_int);
-                }
-                if (slab == 0) { ++nq; nprim += np; }
-                // every thread is done with this entry's shared tables
-                __syncthreads();
-            }
-            if (threadIdx.x == 0 && nq) {
-                atomicAdd(args.stats, nq);
-                atomicAdd(args.stats + 1, nprim);
+                if (threadIdx.x == 0) jk_count_flush(args, launch, cnt);
+                cnt.nq = cnt.nprim = 0;
             }
             return;
         }
-        for (;;) {
-            if (threadIdx.x == 0) s_item = args.item_lo + (long long)atomicAdd(args.work, 1ull);
-            __syncthreads();
-            const long long tt = s_item;
-            __syncthreads();
-            if (tt >= args.item_hi) break;
+        long long tt = blockIdx.x;
+        while (tt < nitems * X) {
             const long long t = X == 1 ? tt : tt / X;
             const int slab = (int)(tt - t * X);
             if constexpr (X > 1) {
@@ -1147,21 +1173,22 @@ jk_class_kernel(const JkClassArgs args)
                 gd = tgl % GD; gc = (tgl / GD) % GC; gb = (tgl / (GD * GC)) % GB; ga = tgl / (GD * GC * GB);
                 jk_make_offsets<LA, LB, LC, LD, GA, GB, GC, GD, S>(ga, gb, gc, gd, off);
             }
-            const int item = jk_item_bra(args, t);
-            const int ch = (int)(t - __ldg(args.item_prefix + item));
-            const int nch = (int)(__ldg(args.item_prefix + item + 1) - __ldg(args.item_prefix + item));
-            const JkPair bra = args.bra[item];
+            const JkItem wi = args.items[t];
+            const JkSub &sub = args.subs[wi.sub];
+            const int item = wi.bra, nab = sub.nab, ncd = sub.ncd, same_class = sub.same_class;
+            const int kb = wi.kb, ke = wi.ke;
+            if (sub.launch != cur) {
+                if (threadIdx.x == 0) jk_count_flush(args, cur, cnt);
+                cur = sub.launch;
+            }
+            const JkPair bra = sub.bra[item];
             const JkMol mol = args.mols[bra.mol];
-            const int kb0 = args.same_class ? item : args.ket_beg[bra.mol];
-            const int kend = args.ket_end[bra.mol];
-            const int kb = min(kend, kb0 + ch * args.chunk);
-            const int ke = (ch == nch - 1) ? kend : min(kend, kb + args.chunk);
             const double *dmx = args.dmax + mol.dmax_off;
             const double dmol = args.use_dmax ? args.dmax_mol[bra.mol] : 1.0;
             const float dmol32 = (float)dmol;
             const int a0 = bra.a_ao + ga * FA, b0 = bra.b_ao + gb * FB;
             JkPairFeat braf;
-            if (MODE != 0) braf = args.bra_feat[item];
+            if (MODE != 0) braf = sub.bra_feat[item];
             R jab[NDM][FA][FB];
 #pragma unroll
             for (int m = 0; m < NDM; ++m)
@@ -1174,8 +1201,8 @@ jk_class_kernel(const JkClassArgs args)
                 if (threadIdx.x < 32) {
                     bool sig, stop, band;
                     float dmq;
-                    jk_screen<MODE>(args, bra, braf, mol, dmx, dmol, dmol32, item, base + lane, ke, sig, stop, band, dmq,
-                                    s_rsm);
+                    jk_screen<MODE>(args, sub, bra, braf, mol, dmx, dmol, dmol32, item, base + lane, ke, sig, stop, band,
+                                    dmq, s_rsm);
                     s_dm[lane] = dmq;
                     const unsigned msk = __ballot_sync(0xffffffffu, sig);
                     const int anystop = __any_sync(0xffffffffu, stop);
@@ -1190,20 +1217,19 @@ jk_class_kernel(const JkClassArgs args)
                 while (mask) {
                     const int myket = base + __ffs(mask) - 1;
                     mask &= mask - 1;
-                    const JkPair ket = args.ket[myket];
+                    const JkPair ket = sub.ket[myket];
                     R T[S::EPT];
 #pragma unroll
                     for (int k = 0; k < S::EPT; ++k) T[k] = (R)0;
-                    const int np = jk_quartet<LA, LB, LC, LD, NPA, NPB, NPC, NPD, GA, GB, GC, GD, R, OP, NTC>(
-                        bra, ket, __fdiv_rn(args.prim_eps32, s_dm[myket - base]), args.omega, args.asym64, pp, rys,
-                        grp, 0u, tg,
-                        act, off, T);
+                    const int np = jk_quartet<LA, LB, LC, LD, GA, GB, GC, GD, R, OP, NTC>(
+                        bra, ket, nab, ncd, __fdiv_rn(args.prim_eps32, s_dm[myket - base]), args.omega, args.asym64, pp,
+                        rys, grp, 0u, tg, act, off, T);
                     nprim += np;
                     if (act) {
                         R f = (R)1;
                         if (bra.a == bra.b) f *= (R)0.5;
                         if (ket.a == ket.b) f *= (R)0.5;
-                        if (args.same_class && myket == item) f *= (R)0.5;
+                        if (same_class && myket == item) f *= (R)0.5;
                         jk_contract<FA, FB, FC, FD, NDM, DOJ, DOK, R>(T, f, mol, a0, b0, ket.a_ao + gc * FC,
                                                                      ket.b_ao + gd * FD, jab, args.widen_int);
                     }
@@ -1219,7 +1245,7 @@ jk_class_kernel(const JkClassArgs args)
                         __syncthreads();
                         if (threadIdx.x == 0) {
                             for (int w = 1; w < (int)(blockDim.x >> 5); ++w) tm = fmax(tm, s_tm[w]);
-                            jk_log_sample(args, bra, ket, braf, args.ket_feat[myket],
+                            jk_log_sample(args, bra, ket, braf, sub.ket_feat[myket],
                                           jk_quartet_dmax(args, bra, ket, mol, dmx), tm);
                         }
                         __syncthreads();
@@ -1232,12 +1258,13 @@ jk_class_kernel(const JkClassArgs args)
                 if (stop) break;
             }
             if (DOJ && act) jk_flush_jab<FA, FB, NDM, R>(jab, mol, a0, b0, args.widen_int);
-            if (threadIdx.x == 0 && nq && slab == 0) {
-                atomicAdd(args.stats, nq);
-                atomicAdd(args.stats + 1, nprim);
-                if (nband) atomicAdd(args.stats + 2, nband);
-            }
+            if (slab == 0) { cnt.nq += nq; cnt.nprim += nprim; cnt.nband += nband; }
+            if (threadIdx.x == 0) s_item = (long long)gridDim.x + (long long)atomicAdd(args.work, 1ull);
+            __syncthreads();
+            tt = s_item;
+            __syncthreads();
         }
+        if (threadIdx.x == 0) jk_count_flush(args, cur, cnt);
     }
 }
 
@@ -1280,7 +1307,7 @@ jk_schwarz_kernel(const JkSchwarzArgs args)
                 double T[S::EPT];
 #pragma unroll
                 for (int k = 0; k < S::EPT; ++k) T[k] = 0.0;
-                jk_quartet<LA, LB, LA, LB, NPA, NPB, NPA, NPB, GA, GB, GC, GD, double>(pr, pr, -1.0f, 0.0, 0, args.pp64, args.rys64, grp, gmask, tg, true, off, T);
+                jk_quartet<LA, LB, LA, LB, GA, GB, GC, GD, double>(pr, pr, NPA * NPB, NPA * NPB, -1.0f, 0.0, 0, args.pp64, args.rys64, grp, gmask, tg, true, off, T);
                 if (ga == gc && gb == gd) {
 #pragma unroll
                     for (int ia = 0; ia < FA; ++ia)
@@ -1315,8 +1342,8 @@ jk_schwarz_kernel(const JkSchwarzArgs args)
             double T[S::EPT];
 #pragma unroll
             for (int k = 0; k < S::EPT; ++k) T[k] = 0.0;
-            jk_quartet<LA, LB, LA, LB, NPA, NPB, NPA, NPB, GA, GB, GC, GD, double, 0, NTC>(
-                pr, pr, -1.0f, 0.0, 0, args.pp64, args.rys64, grp, 0u, tg, act, off, T);
+            jk_quartet<LA, LB, LA, LB, GA, GB, GC, GD, double, 0, NTC>(
+                pr, pr, NPA * NPB, NPA * NPB, -1.0f, 0.0, 0, args.pp64, args.rys64, grp, 0u, tg, act, off, T);
             double mx = 0.0;
             if (act && ga == gc && gb == gd) {
 #pragma unroll

@@ -59,22 +59,47 @@ struct JkMol {
 struct JkRouterDev;
 struct JkPairFeat;
 
+// One class pair (bra pair class, ket pair class) of a launch. A launch runs
+// every class pair that shares a kernel (angular momenta and fragment shape),
+// whatever its primitive counts.
+struct JkSub {
+    const JkPair *bra;           // pairs of the bra class
+    const JkPair *ket;           // pairs of the ket class
+    const int *ket_beg;          // per molecule: first ket index in the ket class
+    const int *ket_end;          // per molecule: one past the last
+    const JkPairFeat *bra_feat;  // aligned with bra / ket
+    const JkPairFeat *ket_feat;
+    int nbra;
+    int same_class;              // ket class == bra class: ket index >= bra index
+    int nab, ncd;                // primitive pairs of a bra / ket pair
+    int chunk;                   // kets per work item
+    int group;                   // launch it belongs to
+    int launch;                  // class pair index: statistics, routed lists
+    int pad;
+};
+
+// A work item: the candidates [kb, ke) of the ket class for one bra pair.
+struct alignas(16) JkItem {
+    int sub, bra, kb, ke;
+};
+
 // A band quartet the learned router released from the FP64 tier: bra pair
-// `item` of the launch's bra class, ket pair `ket` of its ket class, and the
-// density factor its screening used. The FP32 list kernel (MODE 3) of the
-// same class pair evaluates it.
+// `item` of the class pair's bra class, ket pair `ket` of its ket class, and
+// the density factor its screening used. The FP32 list kernel (MODE 3) of
+// the class pair evaluates it.
 struct alignas(16) JkRouted {
     int item, ket;
     float dmq;
     int pad;
 };
 
-// Arguments of one class-pair launch (passed by value).
+// Arguments of one launch (passed by value).
 struct JkClassArgs {
-    const JkPair *bra;           // pairs of the bra class
-    const JkPair *ket;           // pairs of the ket class
-    const int *ket_beg;          // per molecule: first ket index in the ket class
-    const int *ket_end;          // per molecule: one past the last
+    const JkSub *subs;           // the class pairs of the launch
+    int nsub;
+    const JkItem *items;         // work items, listed per build by jk_plan_kernel
+    const unsigned long long *nitems;
+    unsigned long long *work;    // work counter (zeroed before the launch)
     const JkPrimPair64 *pp64;
     const JkPrimPair32 *pp32;
     const JkMol *mols;
@@ -83,13 +108,10 @@ struct JkClassArgs {
     const double *dmax_mol;      // per molecule: max over its table
     const double *rys64;         // FP64 Rys tables
     const float *rys32;          // FP32 Rys tables
-    unsigned long long *work;    // work counter (zeroed before the launch)
-    const long long *item_prefix;  // nbra + 1: first work item of each bra pair
-    long long item_lo, item_hi;  // this build's share of the items [lo, hi) (partitioned builds)
-    int chunk;                   // kets per work item (the last item of a bra runs to ket_end)
     double prim_eps;             // skip primitive quartets with q_ij q_kl Dmax <= prim_eps
     double omega;                // |w| of the range-separated operator (OP 1, 2)
-    unsigned long long *stats;   // [0] quartets, [1] primitive quartets, [2] routed band quartets
+    unsigned long long *stats;   // per class pair (stride stat_stride): [0] quartets, [1] primitive quartets, [2] routed
+    int stat_stride;
     int *err;                    // device error word
     double lo, hi;               // keep a quartet iff lo < Q_ab Q_cd Dmax <= hi
     // FP32 screening (scr32 = 1, used when the build's cutoff is >= 1e-30 so
@@ -97,14 +119,10 @@ struct JkClassArgs {
     // the band in FP32; every tier of a build evaluates them identically
     int scr32;
     float lo32, hi32, tau32, band_hi32, prim_eps32;
-    int nbra;
-    int same_class;              // ket class == bra class: ket index >= bra index
     int with_j, with_k;          // which outputs (and density blocks) to use
     int use_dmax;                // 0: screen with Dmax := 1
     int ndm;
     // learned router (MODE 1) and label logging (MODE 2)
-    const JkPairFeat *bra_feat;  // aligned with bra / ket
-    const JkPairFeat *ket_feat;
     const JkRouterDev *router;
     double tau;                  // band (tau, band_hi]
     double band_hi;
@@ -114,12 +132,13 @@ struct JkClassArgs {
     unsigned long long *log_n;   // MODE 2: samples written (may exceed log_cap)
     long long log_cap;
     // routed builds: the FP64 tier (MODE 1) appends the band quartets the
-    // router releases to this launch's list (while it has room; a quartet
-    // that finds it full stays in FP64); the FP32 list kernel (MODE 3) of the
-    // class pair evaluates min(*rcount, rcap) entries
+    // router releases to their class pair's list (rlist + roff[launch], while
+    // it has room: rcap[launch]; a quartet that finds it full stays in FP64);
+    // the FP32 list kernel (MODE 3) evaluates min(rcount[launch], rcap[launch])
+    // entries of each of its class pairs
     JkRouted *rlist;
     unsigned long long *rcount;
-    long long rcap;
+    const long long *roff, *rcap;
     // 1: the FP32 tier evaluates the large-T (Gauss-Hermite) roots and
     // weights in FP64 and rounds them to FP32
     int asym64;

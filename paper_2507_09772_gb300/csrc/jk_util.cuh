@@ -145,6 +145,90 @@ __global__ void jk_fma_probe_kernel(int iters, T seed, T *sink)
     if (r == (T)-12345.678) sink[0] = r;
 }
 
+// Work items of one tier of a build: for every bra pair of every class pair,
+// the kets (sorted by Q) whose Schwarz product with the bra and the molecule's
+// largest density element can exceed the tier's lower bound, cut into chunks.
+struct JkPlanTier {
+    const JkSub *subs;
+    const int2 *blocks;            // per block: class pair, first bra
+    int nblocks;
+    JkItem *items;
+    const long long *item_off;     // per launch group: where its items start
+    unsigned long long *nitems;    // per launch group (zeroed before)
+    double lo;
+    float lo32;
+};
+struct JkPlanArgs {
+    JkPlanTier tier[2];
+    const double *dmax_mol;
+    int use_dmax, scr32;
+    int part_index, part_count;
+};
+
+// One thread per bra pair: the ket prefix by binary search, then the chunks
+// appended to the launch group's list (one counter update per warp; the
+// blocks run the class pairs with the longest items first, and so, roughly,
+// does the list). Listing the items per build, from this build's density and
+// thresholds, instead of once from Q alone leaves no empty items: in the FP64
+// tier of a mixed build most (bra, chunk) combinations have no candidate. A
+// partitioned build keeps every part_count-th chunk, counted so that the
+// choice depends on the pair indices only. The FP32 bound is taken 4e-6 low
+// (it carries at most four roundings, 2.4e-7), so no candidate is lost; the
+// class kernels decide each one exactly.
+__global__ void __launch_bounds__(256) jk_plan_kernel(const JkPlanArgs args)
+{
+    const JkPlanTier T = blockIdx.y == 0 ? args.tier[0] : args.tier[1];
+    if ((int)blockIdx.x >= T.nblocks) return;
+    const int2 blk = T.blocks[blockIdx.x];
+    const JkSub &S = T.subs[blk.x];
+    const int i = blk.y + threadIdx.x, lane = threadIdx.x & 31;
+    int k0 = 0, n = 0;
+    if (i < S.nbra) {
+        const JkPair &b = S.bra[i];
+        const int m = b.mol;
+        k0 = S.same_class ? i : S.ket_beg[m];
+        int lo = k0, hi = S.ket_end[m];
+        const double dm = args.use_dmax ? args.dmax_mol[m] : 1.0;
+        if (args.scr32) {
+            const float f = b.Qf * (float)dm, thr = T.lo32 * (1.0f - 4e-6f);
+            while (lo < hi) {
+                const int mid = (lo + hi) >> 1;
+                if (f * S.ket[mid].Qf > thr) lo = mid + 1; else hi = mid;
+            }
+        } else {
+            while (lo < hi) {
+                const int mid = (lo + hi) >> 1;
+                if ((b.Q * S.ket[mid].Q) * dm > T.lo) lo = mid + 1; else hi = mid;
+            }
+        }
+        n = lo - k0;
+    }
+    const int c = S.chunk, nch = (n + c - 1) / c;
+    // chunks of this part: c0, c0 + part_count, ...
+    const int c0 = (args.part_index + args.part_count - (i + S.launch) % args.part_count) % args.part_count;
+    const int mine = nch > c0 ? (nch - c0 + args.part_count - 1) / args.part_count : 0;
+    int pre = mine;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const int v = __shfl_up_sync(0xffffffffu, pre, o);
+        if (lane >= o) pre += v;
+    }
+    const int tot = __shfl_sync(0xffffffffu, pre, 31);
+    unsigned long long base = 0;
+    if (lane == 31 && tot) base = atomicAdd(T.nitems + S.group, (unsigned long long)tot);
+    base = __shfl_sync(0xffffffffu, base, 31);
+    JkItem *out = T.items + T.item_off[S.group] + base + (pre - mine);
+    for (int k = 0; k < mine; ++k) {
+        const int kb = k0 + (c0 + k * args.part_count) * c;
+        JkItem it;
+        it.sub = blk.x;
+        it.bra = i;
+        it.kb = kb;
+        it.ke = min(k0 + n, kb + c);
+        out[k] = it;
+    }
+}
+
 // Zero the J/K accumulators of every molecule (pointers read from the
 // device descriptors, so a captured graph stays valid when they change).
 __global__ void jk_zero_kernel(const JkMol *__restrict__ mols, int ndm)
