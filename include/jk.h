@@ -191,9 +191,8 @@ int jk_build_batch(jk_handle *h, const double *const *D, int32_t n_dm, int with_
  * part_count of every class kernel's work, every part_count-th work item; J and K are then partial sums
  * whose sum over the parts is the full result, i.e. one sum all-reduce
  * combines GPUs that split one batch),
- * "branches" (1..8: at least this many streams / graph branches take the class
- * kernels' launches; a build that is not profiled spreads them over 8, a
- * profiled one uses exactly this many),
+ * "branches" (1..8: streams / graph branches of a profiled build's class
+ * kernels; other builds spread them over 24),
  * "chunk" (32..65536, default 64: candidate kets per work item of the
  * persistent class kernels for classes with one thread per quartet; classes
  * with G threads per quartet take 1/G of it, at least 4, and systems with more
@@ -211,6 +210,14 @@ int jk_build_batch(jk_handle *h, const double *const *D, int32_t n_dm, int with_
  * in FP32 and is redone in FP64 when the two sides are within a relative
  * 2e-6 of each other; 0 keeps the plain FP32 compare when the cutoff is
  * >= 1e-30),
+ * "split" (0..1, default 1/8192: FP64-tier quartets whose bound Q_ab Q_cd Dmax
+ * is at most split x max Q^2 x max |D| of their molecule, and in mixed and
+ * routed builds at least those up to 4,096 tau32, are evaluated in pairs of FP32
+ * numbers (48 bits, relative error about 1e-14, 1e-12 at worst for the tightest
+ * functions), which the GPU does several times faster; the error this adds is
+ * below the one the result has from the cutoff. They count as FP64 quartets.
+ * 0: FP64 instructions for every FP64-tier quartet, as for cutoffs below 1e-30
+ * and for bases with exponents outside (1e-6, 1e8)),
  * "route_cap" (default 16777216: initial entries of the per-class-pair lists
  * of quartets the router releases from the FP64 tier, shared out by
  * candidate count; a list that overflowed in a build with stats is grown
@@ -313,7 +320,7 @@ int jk_profile(jk_handle *h, jk_launch_prof *out, int32_t max, int32_t *n);
 int jk_measure_peak(int32_t which, double ms, double *flops_per_s);
 
 /* Ahead-of-time compilation of one class kernel (angular momenta la..ld,
- * primitive counts na..nd, n_dm, flags, fp32 = 1 for the FP32 tier, mode 0
+ * primitive counts na..nd, n_dm, flags, fp32 = 1 for the FP32 tier, 2 for the two-float form of the FP64 tier, mode 0
  * plain / 1 routed FP64 tier (runs the router on its band) / 2 router-label
  * logging (FP64) / 3 routed FP32 list kernel (the quartets mode 1 released),
  * op 0 1/r / 1 erf / 2 erfc) into

@@ -104,7 +104,7 @@ Driver &drv()
     return d;
 }
 
-static_assert(sizeof(JkPair) == 96 && sizeof(JkPrimPair64) == 96 && sizeof(JkPrimPair32) == 48 &&
+static_assert(sizeof(JkPair) == 96 && sizeof(JkPrimPair64) == 96 && sizeof(JkPrimPair32) == 48 && sizeof(JkPrimPairDf) == 80 &&
                   sizeof(JkPairFeat) == 32,
               "record sizes are part of the device layout");
 
@@ -116,7 +116,8 @@ struct KSpec {
     int la = 0, lb = 0, lc = 0, ld = 0, na = 1, nb = 1, nc = 1, nd = 1;
     int ga = 1, gb = 1, gc = 1, gd = 1;
     int gx = 1;    // CTAs one group is split over (groups of more than 256 threads)
-    int ndm = 1, doj = 1, dok = 1, fp32 = 0;
+    int ndm = 1, doj = 1, dok = 1;
+    int fp32 = 0;  // 0 FP64, 1 FP32, 2 two floats (the split tier)
     int mode = 0;  // 0 plain, 1 routed (learned router in the band), 2 label logging
     int op = 0;    // 0 1/r, 1 erf(w r)/r, 2 erfc(w r)/r
 
@@ -127,7 +128,7 @@ struct KSpec {
             snprintf(b, sizeof b, "jk_schwarz_kernel<%d,%d,%d,%d,%d,%d,%d,%d,%d>", la, lb, na, nb, ga, gb, gc, gd, gx);
         else
             snprintf(b, sizeof b, "jk_class_kernel<%d,%d,%d,%d,%d,%d,%d,%d,%d,%d,%d,%d,%s,%d,%d>", la, lb, lc, ld, ga,
-                     gb, gc, gd, gx, ndm, doj, dok, fp32 ? "float" : "double", mode, op);
+                     gb, gc, gd, gx, ndm, doj, dok, fp32 == 2 ? "jkdf" : (fp32 ? "float" : "double"), mode, op);
         return b;
     }
     int G() const { return ga * gb * gc * gd; }
@@ -137,18 +138,20 @@ struct KSpec {
     // G <= 32: four warps, each holding 32/G groups; G > 32: one group (or
     // one of its gx slabs) per CTA
     int block() const { return G() <= 32 ? 128 : ((G() / gx + 31) / 32) * 32; }
-    // FP32 class kernels keep their N-root Rys table in shared memory
+    // FP32 and two-float class kernels keep their N-root Rys table in shared memory
     size_t rys_table_bytes() const
     {
         if (kind != 0 || !fp32) return 0;
         const int n = (la + lb + lc + ld) / 2 + 1;
+        // two-float tables: staged up to JK_DF_STAGE = 3 roots
+        if (fp32 == 2) return n <= 3 ? (size_t)rys64_nint_host[n] * (32 * n + 4) * sizeof(float) : 0;
         // per interval 2 n functions x 8 coefficients, padded by 4 floats
         return (size_t)rys32_nint_host[n] * (2 * n * (rys32_deg_host + 1) + 4) * sizeof(float);
     }
     size_t smem_bytes() const
     {
         const size_t groups = G() <= 32 ? (size_t)4 * (32 / G()) : 1;
-        return rys_table_bytes() + groups * smem_group_reals() * (fp32 ? 4 : 8);
+        return rys_table_bytes() + groups * smem_group_reals() * (fp32 == 1 ? 4 : 8);
     }
     int groups_per_cta() const { return G() <= 32 ? 4 * (32 / G()) : 1; }
 };
@@ -473,7 +476,7 @@ void choose_fragments(KSpec &s, bool symmetric)
     const int reg_cap = 48;                   // per-thread fragment budget (reals)
     const int gmax = symmetric ? 1024 : 256;  // threads per quartet in one CTA
     const int gsplit = 256;                   // threads per CTA of a group split over CTAs
-    const int g1_cap = s.fp32 ? 128 : 64;     // register-mode budget: fragment + 3 tables
+    const int g1_cap = s.fp32 == 1 ? 128 : 64;     // register-mode budget: fragment + 3 tables
     s.gx = 1;
     if (ne + 3 * ni <= g1_cap) { s.ga = s.gb = s.gc = s.gd = 1; return; }
     // CTAs for a group of g threads: 1 if it fits one CTA, else the fewest
@@ -526,7 +529,7 @@ std::vector<KSpec> fragment_candidates(const KSpec &s0, int maxc)
     std::vector<KSpec> out{s0};
     const int nf[4] = {ncart(s0.la), ncart(s0.lb), ncart(s0.lc), ncart(s0.ld)};
     const int ne = nf[0] * nf[1] * nf[2] * nf[3];
-    const int g1_cap = s0.fp32 ? 128 : 64;
+    const int g1_cap = s0.fp32 == 1 ? 128 : 64;
     auto push = [&](int a, int b, int c, int d) {
         if ((int)out.size() >= maxc) return;
         for (auto &x : out)
@@ -692,7 +695,7 @@ struct PairClass {
 // A class pair (bra class, ket class).
 struct Launch {
     int c1, c2;        // pair classes (bra, ket)
-    KSpec spec[2];     // [0] FP64, [1] FP32
+    KSpec spec[3];     // [0] FP64, [1] FP32, [2] two floats
     double cost;       // scheduling estimate
     double cand = 0;   // candidate kets summed over the bras (Q_ab Q_cd > JK_ITEM_EPS)
 };
@@ -729,14 +732,31 @@ struct TierPlan {
 #define JK_CHUNK_HI 512
 #define JK_CHUNK_MIN 4
 #define JK_ITEMS_MAX 8000000LL
+// Small systems: an item is a serial chain of primitive quartets, about
+// JK_LAT_* seconds per modelled FLOP of a lane when few warps share an SM
+// ((ss|ss) of six-primitive s shells: 1,296 primitive quartets, 1.8 ms). Where
+// the chain would exceed both JK_CHAIN_MIN and a quarter of the build's
+// estimated time (modelled FLOPs at JK_RATE_*), the chunk goes down to one
+// round of the warp, then the bra's primitive pairs are shared out over
+// several items, each of which contracts its part with the density by itself.
+#define JK_CHAIN_MIN 30e-6
+static const double JK_LAT[3] = {20e-9, 5e-9, 20e-9};      // FP64, FP32, two floats
+static const double JK_RATE[3] = {0.8e12, 6e12, 2e12};
 #define JK_ITEM_EPS 1e-15
+// Quartets of the FP64 tier whose bound is at most JK_SPLIT x (max Q)^2 x
+// max |D| are evaluated in two-float arithmetic (relative error about 1e-14),
+// the few above it, which carry the result, in FP64 instructions.
+#define JK_SPLIT (1.0 / 8192)
+#define JK_SPLIT_TAU 4096.0
 
 }  // namespace
 
-#define JK_MAX_BRANCHES 7
+#define JK_MAX_BRANCHES 7        // option "branches" less one
 // Streams the launches of a build are spread over unless they are profiled: the
-// tail of one launch is filled by the next ones (21 launches for s, p, d shells).
-#define JK_AUTO_BRANCHES 8
+// tail of one launch is filled by the next ones (s, p, d shells: 21 per tier; s
+// to f: 55). 45 functions in FP64: 1.74 ms on 4 streams, 1.17 on 8, 0.98 on 14,
+// 0.76 on 24; 8 molecules 280, 282, 286, 279 ms; 24 mixed 314, 314, 317, 300.
+#define JK_SIDE_STREAMS 23
 
 struct jk_handle {
     int device = 0;
@@ -745,6 +765,7 @@ struct jk_handle {
     std::vector<jk_shell> shells;
     std::vector<int> mol_sh0;              // nmol + 1
     std::vector<int> nao_cart, nao_user;   // per molecule
+    std::vector<double> mol_qmax2;         // largest Q squared
     std::vector<int> sh_ao_cart;           // molecule-local Cartesian AO offset per shell
     bool spherical = false;
     // device
@@ -752,18 +773,19 @@ struct jk_handle {
     JkPair *d_pairs = nullptr;
     JkPrimPair64 *d_pp64 = nullptr;
     JkPrimPair32 *d_pp32 = nullptr;
+    JkPrimPairDf *d_ppdf = nullptr;
     JkMol *d_mols = nullptr;
     double *d_dmax = nullptr;
     float *d_dmax32 = nullptr;
     unsigned long long *d_dmax_mol = nullptr;
     double *d_rys64 = nullptr;
-    float *d_rys32 = nullptr;
+    float *d_rys32 = nullptr, *d_rysdf = nullptr;
     // counters zeroed at the start of every build, one allocation: per tier and
     // group the items listed and taken; three statistics per class pair and
     // tier; the largest |D| per molecule; the routed list lengths
     unsigned long long *d_zero = nullptr;
     size_t zero_bytes = 0;
-    unsigned long long *d_ctr = nullptr;   // [2 tiers][class pairs][listed, taken]
+    unsigned long long *d_ctr = nullptr;   // [FP64, FP32, split][class pairs][listed, taken]
     unsigned long long *d_stats = nullptr; // three per class pair and tier
     std::map<int, std::unique_ptr<TierPlan>> plans;   // by tier, chunk and merging
     int *d_err = nullptr;
@@ -791,7 +813,7 @@ struct jk_handle {
     double init_ms = 0, compile_ms = 0;
     std::vector<cudaEvent_t> prof_ev;      // two per launch slot
     std::vector<jk_launch_prof> prof;
-    std::vector<int> prof_slot;            // launch * 3 + tier of each prof record
+    std::vector<int> prof_slot;            // launch * 4 + tier of each prof record
     // spherical molecules: Cartesian scratch copies of D, J, K
     std::vector<char> mol_sph;             // per molecule
     std::vector<int> sh_ao_user;           // molecule-local AO offset in the caller's basis
@@ -803,7 +825,8 @@ struct jk_handle {
     JkSphMol *d_sph = nullptr, *h_sph = nullptr;  // [0, nmol): to Cartesian, [nmol, 2 nmol): back
     size_t cart_gen = 0;                   // bumps when the scratch moves (invalidates graphs)
     float *d_d32 = nullptr;                // FP32 copies of D for the FP32 tier: ndm x nao_c^2 per molecule
-    size_t d32_ndm = 0;
+    float2 *d_d2 = nullptr;                // ... as two floats for the split tier
+    size_t d32_ndm = 0, d2_ndm = 0;
     std::vector<size_t> d32_off;
     // learned router
     JkPairFeat *d_pfeat = nullptr;         // aligned with d_pairs
@@ -816,6 +839,8 @@ struct jk_handle {
     long long *d_rl = nullptr;             // offsets, then capacities
     std::vector<long long> rl_need;        // entries each list needed in the last build with stats
     double route_cap = 16777216.0;         // list entries over all launches
+    double split = JK_SPLIT;               // split threshold; 0: every quartet of the FP64 tier in FP64 instructions
+    bool df_ok = true;                     // the basis stays far inside the FP32 range
     int asym64 = 0;                        // FP32 tier: large-T roots and weights in FP64
     int chunk = JK_CHUNK;                  // kets per work item
     // FP32 tier: float-to-double by integer operations (1) or by the
@@ -830,8 +855,8 @@ struct jk_handle {
     // graphs and branch streams
     int branches = 1;
     cudaStream_t cap = nullptr;
-    cudaStream_t side[JK_MAX_BRANCHES] = {};
-    cudaEvent_t ev_fork = nullptr, ev_join[JK_MAX_BRANCHES] = {};
+    cudaStream_t side[JK_SIDE_STREAMS] = {};
+    cudaEvent_t ev_fork = nullptr, ev_join[JK_SIDE_STREAMS] = {};
     std::map<std::string, std::pair<cudaGraphExec_t, int>> graphs;
 };
 
@@ -843,7 +868,7 @@ void free_handle(jk_handle *h)
     for (auto &c : h->classes) { cudaFree(c.d_beg); cudaFree(c.d_end); }
     h->plans.clear();
     cudaFree(h->d_sh_mol); cudaFree(h->d_mol_sh0); cudaFree(h->d_sh_ao); cudaFree(h->d_sh_nc);
-    cudaFree(h->d_pairs); cudaFree(h->d_pp64); cudaFree(h->d_pp32); cudaFree(h->d_mols);
+    cudaFree(h->d_pairs); cudaFree(h->d_pp64); cudaFree(h->d_pp32); cudaFree(h->d_ppdf); cudaFree(h->d_rysdf); cudaFree(h->d_d2); cudaFree(h->d_mols);
     cudaFree(h->d_dmax); cudaFree(h->d_dmax32); cudaFree(h->d_rys64); cudaFree(h->d_rys32);
     cudaFree(h->d_zero); cudaFree(h->d_err); cudaFree(h->d_tile_off);
     if (h->h_mols) cudaFreeHost(h->h_mols);
@@ -859,7 +884,7 @@ void free_handle(jk_handle *h)
     cudaFree(h->d_rlist); cudaFree(h->d_rl);
     for (auto &g : h->graphs) cudaGraphExecDestroy(g.second.first);
     if (h->cap) cudaStreamDestroy(h->cap);
-    for (int b = 0; b < JK_MAX_BRANCHES; ++b) {
+    for (int b = 0; b < JK_SIDE_STREAMS; ++b) {
         if (h->side[b]) cudaStreamDestroy(h->side[b]);
         if (h->ev_join[b]) cudaEventDestroy(h->ev_join[b]);
     }
@@ -906,12 +931,14 @@ void drop_graphs(jk_handle *h)
     h->graphs.clear();
 }
 
-// The launches of a tier (t = 0 FP64 shapes, 1 FP32 shapes; hi: the chunk of
+// The launches of a tier (t = 0 FP64 shapes, 1 FP32, 2 two-float; hi: the chunk of
 // the FP64 tier of two-tier builds; merge: class pairs that share a kernel in
-// one launch), made on first use and kept until the shapes or chunks change.
-int tier_plan(jk_handle *h, int t, int hi, int merge, TierPlan **out)
+// one launch; whole: items never share a quartet's primitives, for the kernels
+// that log or route quartets), made on first use and kept until the shapes or
+// chunks change.
+int tier_plan(jk_handle *h, int t, int hi, int merge, int whole, TierPlan **out)
 {
-    const int key = t + 2 * hi + 4 * merge;
+    const int key = t + 4 * hi + 8 * merge + 16 * whole;
     auto it = h->plans.find(key);
     if (it != h->plans.end()) { *out = it->second.get(); return JK_OK; }
     std::unique_ptr<TierPlan> P(new TierPlan());
@@ -941,6 +968,10 @@ int tier_plan(jk_handle *h, int t, int hi, int merge, TierPlan **out)
     }
     std::stable_sort(gord.begin(), gord.end(), [&](int x, int y) { return cost[x] > cost[y]; });
     const long long base = hi ? h->chunk_hi : h->chunk;
+    double total_cost = 0;
+    for (auto &L : h->launches) total_cost += L.cost;
+    const double kept = hi ? 0.3 : 1.0;   // share of the candidates the tier evaluates
+    const double chain_max = std::max(JK_CHAIN_MIN, 0.25 * kept * total_cost / JK_RATE[t]) / JK_LAT[t];
     std::vector<JkSub> subs;
     std::vector<long long> cap;
     for (long long f = 1;; f *= 2) {
@@ -971,7 +1002,16 @@ int tier_plan(jk_handle *h, int t, int hi, int merge, TierPlan **out)
                 S.same_class = L.c1 == L.c2 ? 1 : 0;
                 S.nab = L.spec[t].na * L.spec[t].nb;
                 S.ncd = L.spec[t].nc * L.spec[t].nd;
-                const long long c = std::min<long long>(1 << 24, std::max<long long>(JK_CHUNK_MIN, base * ngw / 32) * f);
+                KSpec one = L.spec[t];
+                one.na = one.nb = one.nc = one.nd = 1;
+                // modelled FLOPs of a lane per round, at most
+                const double round = class_flops(one, 1) / one.G() * S.nab * S.ncd;
+                long long c = std::max<long long>(JK_CHUNK_MIN, base * ngw / 32);
+                while (c > ngw && round * std::max(1.0, kept * c / ngw) > chain_max) c = (c + 1) / 2;
+                S.split = 1;
+                if (!whole)
+                    S.split = (int)std::min<double>(S.nab, std::max(1.0, std::ceil(round * std::max(1.0, kept * c / ngw) / chain_max)));
+                c = std::min<long long>(1 << 24, c * f);
                 S.chunk = (int)c;
                 S.group = (int)k;
                 S.launch = l;
@@ -979,8 +1019,8 @@ int tier_plan(jk_handle *h, int t, int hi, int merge, TierPlan **out)
                     const long long nb = A.end[m] - A.beg[m], nk = B.end[m] - B.beg[m];
                     // same class: bra i has nk - i kets
                     const long long q = nk / c, r = nk % c;
-                    G.cap += S.same_class ? c * q * (q + 1) / 2 + r * (q + 1) : nb * ((nk + c - 1) / c);
-                    if (nk > 0) least += nb;
+                    G.cap += S.split * (S.same_class ? c * q * (q + 1) / 2 + r * (q + 1) : nb * ((nk + c - 1) / c));
+                    if (nk > 0) least += nb * S.split;
                 }
                 subs.push_back(S);
                 P->launch.push_back(l);
@@ -1156,8 +1196,10 @@ int init_impl(int32_t nmol, const int32_t *mol_shell_off, const jk_shell *shells
         return rc;
     CK(cudaMalloc(&h->d_pp64, sizeof(JkPrimPair64) * npp));
     CK(cudaMalloc(&h->d_pp32, sizeof(JkPrimPair32) * npp));
+    CK(cudaMalloc(&h->d_ppdf, sizeof(JkPrimPairDf) * npp));
     jk_pairdata_kernel<<<(unsigned)((ncand + 127) / 128), 128>>>((int)ncand, d_ca, d_cb, d_cpp, d_atom, d_np, d_prim,
-                                                                  d_coords, d_exps, d_coeffs, h->d_pp64, h->d_pp32);
+                                                                  d_coords, d_exps, d_coeffs, h->d_pp64, h->d_pp32,
+                                                                  h->d_ppdf);
     CK(cudaGetLastError());
 
     // ---- Rys tables
@@ -1165,7 +1207,25 @@ int init_impl(int32_t nmol, const int32_t *mol_shell_off, const jk_shell *shells
         std::vector<double> t64(rys_table64, rys_table64 + rys_table64_size);
         std::vector<float> t32(rys_table32_size);
         for (size_t i = 0; i < rys_table32_size; ++i) t32[i] = (float)rys_table32_src[i];
-        if ((rc = upload(&h->d_rys64, t64)) || (rc = upload(&h->d_rys32, t32))) return rc;
+        // two-float tables from the FP64 ones (per function c0..c5, then c6..c9
+        // as floats), intervals padded by four floats
+        std::vector<float> tdf;
+        size_t o = 0;
+        for (int n = 1; n < (int)(sizeof rys64_nint_host / sizeof rys64_nint_host[0]); ++n)
+            for (int k = 0; k < rys64_nint_host[n]; ++k) {
+                for (int f = 0; f < 2 * n; ++f, o += 8) {
+                    for (int i = 0; i < 6; ++i) {
+                        const float hi = (float)t64[o + i];
+                        tdf.push_back(hi);
+                        tdf.push_back((float)(t64[o + i] - (double)hi));
+                    }
+                    float tail[4];
+                    memcpy(tail, &t64[o + 6], sizeof tail);
+                    tdf.insert(tdf.end(), tail, tail + 4);
+                }
+                tdf.insert(tdf.end(), 4, 0.0f);
+            }
+        if ((rc = upload(&h->d_rys64, t64)) || (rc = upload(&h->d_rys32, t32)) || (rc = upload(&h->d_rysdf, tdf))) return rc;
     }
 
     // ---- JkPair records for the candidates (unsorted), Schwarz per class
@@ -1179,7 +1239,7 @@ int init_impl(int32_t nmol, const int32_t *mol_shell_off, const jk_shell *shells
         const double *A = coords + 3 * shells[a].atom, *B = coords + 3 * shells[b].atom;
         p.ABx = A[0] - B[0]; p.ABy = A[1] - B[1]; p.ABz = A[2] - B[2];
         p.ABxf = (float)p.ABx; p.AByf = (float)p.ABy; p.ABzf = (float)p.ABz;
-        p.pad0 = 0; p.pad1 = 0.0;
+        p.ABxl = (float)(p.ABx - (double)p.ABxf); p.AByl = (float)(p.ABy - (double)p.AByf); p.ABzl = (float)(p.ABz - (double)p.ABzf);
         p.Q = 0; p.Qf = 0.f; p.padf = 0.f;
     }
     JkPair *d_cp = nullptr;
@@ -1265,7 +1325,8 @@ int init_impl(int32_t nmol, const int32_t *mol_shell_off, const jk_shell *shells
         int *d_cnt = nullptr;
         JkPrimPair64 *n64 = nullptr;
         JkPrimPair32 *n32 = nullptr;
-        auto cl2 = [&]() { cudaFree(d_pseudo); cudaFree(d_qp); cudaFree(d_cnt); cudaFree(n64); cudaFree(n32); };
+        JkPrimPairDf *ndf = nullptr;
+        auto cl2 = [&]() { cudaFree(d_pseudo); cudaFree(d_qp); cudaFree(d_cnt); cudaFree(n64); cudaFree(n32); cudaFree(ndf); };
         struct G3 { std::function<void()> f; ~G3() { f(); } } g3{cl2};
         if ((rc = upload(&d_pseudo, pseudo))) return rc;
         CK(cudaMalloc(&d_qp, sizeof(double) * npp));
@@ -1295,12 +1356,14 @@ int init_impl(int32_t nmol, const int32_t *mol_shell_off, const jk_shell *shells
         if ((rc = upload(&d_cnt, cnt))) return rc;
         CK(cudaMalloc(&n64, sizeof(JkPrimPair64) * npp));
         CK(cudaMalloc(&n32, sizeof(JkPrimPair32) * npp));
+        CK(cudaMalloc(&ndf, sizeof(JkPrimPairDf) * npp));
         jk_primsort_kernel<<<(unsigned)((ncand + 127) / 128), 128>>>((int)ncand, d_cpp, d_cnt, d_qp, h->d_pp64,
-                                                                      h->d_pp32, n64, n32);
+                                                                      h->d_pp32, h->d_ppdf, n64, n32, ndf);
         CK(cudaGetLastError());
         CK(cudaDeviceSynchronize());
         std::swap(h->d_pp64, n64);
         std::swap(h->d_pp32, n32);
+        std::swap(h->d_ppdf, ndf);
     }
 
     // ---- prune, group by (class, molecule), sort by Q descending
@@ -1318,6 +1381,14 @@ int init_impl(int32_t nmol, const int32_t *mol_shell_off, const jk_shell *shells
         h->h_pairs[k].Q = q[order[k]];
         h->h_pairs[k].Qf = (float)q[order[k]];
     }
+    h->mol_qmax2.assign(nmol, 0.0);
+    for (auto &p : h->h_pairs) h->mol_qmax2[p.mol] = std::max(h->mol_qmax2[p.mol], p.Q * p.Q);
+    // two floats need every intermediate well inside the FP32 range
+    for (int i = 0; i < nprim_total; ++i) {
+        const double c = std::fabs(coeffs[i]);
+        h->df_ok = h->df_ok && exps[i] > 1e-6 && exps[i] < 1e8 && c < 1e8 && (c == 0 || c > 1e-8);
+    }
+    for (int i = 0; i < 3 * natm; ++i) h->df_ok = h->df_ok && std::fabs(coords[i]) < 1e5;
     size_t k0 = 0;
     while (k0 < order.size()) {
         size_t k1 = k0;
@@ -1384,7 +1455,7 @@ int init_impl(int32_t nmol, const int32_t *mol_shell_off, const jk_shell *shells
             Launch L;
             L.c1 = i; L.c2 = j;
             const PairClass &A = h->classes[i], &B = h->classes[j];
-            for (int t = 0; t < 2; ++t) {
+            for (int t = 0; t < 3; ++t) {
                 KSpec &s = L.spec[t];
                 s.kind = 0;
                 s.la = A.la; s.lb = A.lb; s.lc = B.la; s.ld = B.lb;
@@ -1419,14 +1490,14 @@ int init_impl(int32_t nmol, const int32_t *mol_shell_off, const jk_shell *shells
     CK(cudaMalloc(&h->d_dmax32, sizeof(float) * dtot));
     CK(cudaMalloc(&h->d_mols, sizeof(JkMol) * nmol));
     {
-        // class pairs x (2 tiers x (listed, taken) + 3 tiers (FP64, FP32, routed
-        // list) x 3 statistics + routed count), then the molecules' largest |D|
-        const size_t nl = h->launches.size(), n = nl * (4 + 9 + 1) + nmol;
+        // class pairs x (3 tiers x (listed, taken) + 4 tiers (FP64, FP32, routed
+        // list, split) x 3 statistics + routed count), then the molecules' largest |D|
+        const size_t nl = h->launches.size(), n = nl * (6 + 12 + 1) + nmol;
         h->zero_bytes = sizeof(unsigned long long) * n;
         CK(cudaMalloc(&h->d_zero, h->zero_bytes));
         h->d_ctr = h->d_zero;
-        h->d_stats = h->d_zero + 4 * nl;
-        h->d_rcount = h->d_stats + 9 * nl;
+        h->d_stats = h->d_zero + 6 * nl;
+        h->d_rcount = h->d_stats + 12 * nl;
         h->d_dmax_mol = h->d_rcount + nl;
     }
     CK(cudaMalloc(&h->d_err, sizeof(int)));
@@ -1456,7 +1527,7 @@ int init_impl(int32_t nmol, const int32_t *mol_shell_off, const jk_shell *shells
     CK(cudaEventCreate(&h->ev1));
     CK(cudaStreamCreateWithFlags(&h->cap, cudaStreamNonBlocking));
     CK(cudaEventCreateWithFlags(&h->ev_fork, cudaEventDisableTiming));
-    for (int b = 0; b < JK_MAX_BRANCHES; ++b) {
+    for (int b = 0; b < JK_SIDE_STREAMS; ++b) {
         CK(cudaStreamCreateWithFlags(&h->side[b], cudaStreamNonBlocking));
         CK(cudaEventCreateWithFlags(&h->ev_join[b], cudaEventDisableTiming));
     }
@@ -1521,23 +1592,30 @@ int build_impl(jk_handle *h, const double *const *D, int32_t ndm, int with_j, in
     cudaStream_t st = (cudaStream_t)stream;
     if (int prc = poll_device_error(h, false)) return prc;
 
-    // launches and kernels for this combination. Tier 0 FP64, 1 FP32; routed
-    // builds add tier 2, the FP32 list kernel of the quartets the router
-    // released from the FP64 tier (the router itself runs in the FP64 tier only)
+    // launches and kernels for this combination. Tier 0 FP64, 1 FP32, 3 split
+    // (the part of the FP64 tier below the split threshold, in two floats);
+    // routed builds add tier 2, the FP32 list kernel of the quartets the router
+    // released from the FP64 and split tiers (the router runs in those only)
     const bool routed = mode == JK_PREC_MIXED_ROUTED;
     const bool two = mode == JK_PREC_MIXED || routed;
     const bool prof = h->profile && stats;
     const int merge = prof ? 0 : 1;
     const int op = h->omega == 0.0 ? 0 : (h->omega > 0.0 ? 1 : 2);
+    const bool use32 = mode != JK_PREC_FP64;
+    const bool usedf = mode != JK_PREC_FP32 && h->split > 0 && h->df_ok && !logs && cutoff >= 1e-30;
+    static const int spec_of[4] = {0, 1, 1, 2}, ctr_of[4] = {0, 1, 1, 2};
     struct Tier { int t; TierPlan *P; std::vector<KInfo> *ki; };
     std::vector<Tier> tiers;
     int rc;
-    for (int t = 0; t < 3; ++t) {
-        const bool use = (t == 0) ? (mode == JK_PREC_FP64 || two) : (t == 1 ? (mode == JK_PREC_FP32 || two) : routed);
+    for (int t : {0, 3, 1, 2}) {   // the FP64 tier's long chains first
+        const bool use = t == 0 ? mode != JK_PREC_FP32 : (t == 1 ? use32 : (t == 2 ? routed : usedf));
         if (!use) continue;
         Tier T{t, nullptr, nullptr};
-        if ((rc = tier_plan(h, t == 0 ? 0 : 1, t == 0 && two ? 1 : 0, merge, &T.P))) return rc;
-        const int kmode = logs ? 2 : (routed ? (t == 0 ? 1 : (t == 2 ? 3 : 0)) : 0);
+        // tiers that keep few of the candidates they scan take longer items
+        const int hi = (t == 0 && (two || usedf)) || (t == 3 && two) ? 1 : 0;
+        const int whole = logs || (routed && t != 1) ? 1 : 0;
+        if ((rc = tier_plan(h, spec_of[t], hi, merge, t == 2 ? 0 : whole, &T.P))) return rc;
+        const int kmode = logs ? 2 : (routed ? (t == 2 ? 3 : (t == 1 ? 0 : 1)) : 0);
         if ((rc = plan_kernels(h, T.P, ndm, with_j ? 1 : 0, with_k ? 1 : 0, kmode, op, &T.ki))) return rc;
         tiers.push_back(T);
     }
@@ -1557,17 +1635,27 @@ int build_impl(jk_handle *h, const double *const *D, int32_t ndm, int with_j, in
         h->cart_ndm = ndm;
         ++h->cart_gen;
     }
-    // FP32 copies of the densities when the FP32 tier runs
-    const bool use32 = mode != JK_PREC_FP64;
-    if (use32 && h->d32_ndm < (size_t)ndm) {
+    // copies of the densities for the FP32 and split tiers
+    if ((use32 && h->d32_ndm < (size_t)ndm) || (usedf && h->d2_ndm < (size_t)ndm)) {
         CK(cudaStreamSynchronize(st));
-        cudaFree(h->d_d32);
-        h->d_d32 = nullptr;
         h->d32_off.assign(h->nmol, 0);
+        const size_t n = std::max({h->d32_ndm, h->d2_ndm, (size_t)ndm});
         size_t tot = 0;
-        for (int m = 0; m < h->nmol; ++m) { h->d32_off[m] = tot; tot += (size_t)ndm * h->nao_cart[m] * h->nao_cart[m]; }
-        CK(cudaMalloc(&h->d_d32, sizeof(float) * std::max<size_t>(tot, 1)));
-        h->d32_ndm = ndm;
+        for (int m = 0; m < h->nmol; ++m) { h->d32_off[m] = tot; tot += n * h->nao_cart[m] * h->nao_cart[m]; }
+        if (use32 || h->d_d32) {
+            cudaFree(h->d_d32);
+            h->d_d32 = nullptr;
+            h->d32_ndm = 0;
+            CK(cudaMalloc(&h->d_d32, sizeof(float) * std::max<size_t>(tot, 1)));
+            h->d32_ndm = n;
+        }
+        if (usedf || h->d_d2) {
+            cudaFree(h->d_d2);
+            h->d_d2 = nullptr;
+            h->d2_ndm = 0;
+            CK(cudaMalloc(&h->d_d2, sizeof(float2) * std::max<size_t>(tot, 1)));
+            h->d2_ndm = n;
+        }
         ++h->cart_gen;
     }
     // routed builds: one list per class pair for the quartets the router
@@ -1636,6 +1724,8 @@ int build_impl(jk_handle *h, const double *const *D, int32_t ndm, int with_j, in
             }
         }
         x.D32 = use32 ? h->d_d32 + h->d32_off[m] : nullptr;
+        x.D2 = usedf ? h->d_d2 + h->d32_off[m] : nullptr;
+        x.qmax2 = h->mol_qmax2[m];
         x.nsh = h->mol_sh0[m + 1] - h->mol_sh0[m];
         x.dmax_off = off;
         off += (long long)x.nsh * x.nsh;
@@ -1657,7 +1747,8 @@ int build_impl(jk_handle *h, const double *const *D, int32_t ndm, int with_j, in
         h->prof_ev.resize(2 * nlaunch_class);
         for (size_t e = have; e < h->prof_ev.size(); ++e) CK(cudaEventCreate(&h->prof_ev[e]));
     }
-    const int nbranch = prof ? h->branches : std::max(h->branches, JK_AUTO_BRANCHES);
+    const int nbranch = prof ? h->branches
+                             : std::min(JK_SIDE_STREAMS + 1, (int)nlaunch_class);
     int nlaunch_aux = 0;
 
     // Everything a build does on the device, in order, on stream s (and, for
@@ -1686,7 +1777,7 @@ int build_impl(jk_handle *h, const double *const *D, int32_t ndm, int with_j, in
                                                   h->d_dmax, h->d_dmax32, h->d_dmax_mol, h->d_err);
         CK(cudaGetLastError());
         ++nlaunch_aux;
-        if (use32) {
+        if (use32 || usedf) {
             long long per = (long long)ndm * max_nao * max_nao;
             dim3 g((unsigned)std::min<long long>((per + 255) / 256, 4096), h->nmol);
             jk_d32_kernel<<<g, 256, 0, s0>>>(h->d_mols, ndm);
@@ -1704,12 +1795,20 @@ int build_impl(jk_handle *h, const double *const *D, int32_t ndm, int with_j, in
         // bounds of the tiers; in a routed build the FP32 tier keeps the Schwarz
         // split, the band goes to the FP64 tier, which routes it (tier 2 reads
         // its lists)
-        auto lo_of = [&](int t) { return two && t == 0 ? tau : cutoff; };
-        auto hi_of = [&](int t) { return two && t != 0 ? tau : inf; };
+        auto lo_of = [&](int t) { return two && (t == 0 || t == 3) ? tau : cutoff; };
+        auto hi_of = [&](int t) { return two && (t == 1 || t == 2) ? tau : inf; };
+        // the split threshold divides the FP64 tier's range (per molecule); a
+        // build with an FP32 tier (relative error 6e-8 up to tau) takes two
+        // floats (1e-12 at worst) up to 4,096 tau, a sixteenth of that error
+        const double split_min = two ? JK_SPLIT_TAU * tau : 0.0;
+        auto side_of = [&](int t) { return !usedf ? 0 : (t == 0 ? 1 : (t == 3 ? -1 : 0)); };
         {
             JkPlanArgs pa;
             memset(&pa, 0, sizeof pa);
             pa.dmax_mol = reinterpret_cast<const double *>(h->d_dmax_mol);
+            pa.mols = h->d_mols;
+            pa.split = h->split;
+            pa.split_min = split_min;
             pa.use_dmax = h->use_dmax;
             pa.scr32 = scr32;
             pa.part_index = h->part_index;
@@ -1723,9 +1822,9 @@ int build_impl(jk_handle *h, const double *const *D, int32_t ndm, int with_j, in
                 q.nblocks = T.P->nblocks;
                 q.items = T.P->d_items;
                 q.item_off = T.P->d_item_off;
-                q.nitems = h->d_ctr + (size_t)T.t * 2 * nl;
+                q.nitems = h->d_ctr + (size_t)ctr_of[T.t] * 2 * nl;
                 q.lo = lo_of(T.t);
-                q.lo32 = (float)q.lo;
+                q.split_side = side_of(T.t);
                 nblk = std::max(nblk, q.nblocks);
             }
             jk_plan_kernel<<<dim3((unsigned)nblk, np), 256, 0, s0>>>(pa);
@@ -1762,19 +1861,24 @@ int build_impl(jk_handle *h, const double *const *D, int32_t ndm, int with_j, in
                 a.subs = T.P->d_subs + (T.t == 2 ? G.sub0 : 0);   // items index the plan's whole table
                 a.nsub = G.nsub;
                 a.items = T.P->d_items + T.P->item_off[g];
-                unsigned long long *ctr = h->d_ctr + (size_t)(T.t == 0 ? 0 : 1) * 2 * nl;
+                unsigned long long *ctr = h->d_ctr + (size_t)ctr_of[T.t] * 2 * nl;
                 a.nitems = ctr + g;
                 a.work = ctr + nl + g;
                 a.pp64 = h->d_pp64;
                 a.pp32 = h->d_pp32;
+                a.ppdf = h->d_ppdf;
                 a.mols = h->d_mols;
                 a.dmax = h->d_dmax;
                 a.dmax32 = h->d_dmax32;
                 a.dmax_mol = reinterpret_cast<const double *>(h->d_dmax_mol);
                 a.rys64 = h->d_rys64;
                 a.rys32 = h->d_rys32;
+                a.rysdf = h->d_rysdf;
+                a.split = h->split;
+                a.split_min = split_min;
+                a.split_side = side_of(T.t);
                 a.stats = h->d_stats + 3 * T.t;
-                a.stat_stride = 9;
+                a.stat_stride = 12;
                 a.err = h->d_err;
                 a.lo = lo_of(T.t);
                 a.hi = hi_of(T.t);
@@ -1786,7 +1890,7 @@ int build_impl(jk_handle *h, const double *const *D, int32_t ndm, int with_j, in
                 a.hi32 = std::isinf(a.hi) ? INFINITY : (float)a.hi;
                 a.tau32 = (float)tau;
                 a.band_hi32 = (float)band_hi;
-                a.tier = T.t == 0 ? 0 : 1;
+                a.tier = T.t == 0 || T.t == 3 ? 0 : 1;
                 a.rlist = routed ? h->d_rlist : nullptr;
                 a.rcount = h->d_rcount;
                 a.roff = routed ? h->d_rl : nullptr;
@@ -1844,8 +1948,8 @@ int build_impl(jk_handle *h, const double *const *D, int32_t ndm, int with_j, in
                  cutoff, h->tau32, h->router_band, h->use_dmax, nbranch, h->cart_gen, prof ? 1 : 0, h->part_index,
                  h->part_count, h->prim_eps, h->asym64, h->screen64 + 2 * h->widen_int);
         std::string key = keyb;
-        char ob[40];
-        snprintf(ob, sizeof ob, "/%a", h->omega);
+        char ob[80];
+        snprintf(ob, sizeof ob, "/%a/%a", h->omega, h->split);
         key += ob;
         auto it = h->graphs.find(key);
         if (it == h->graphs.end()) {
@@ -1872,7 +1976,7 @@ int build_impl(jk_handle *h, const double *const *D, int32_t ndm, int with_j, in
         CK(cudaStreamSynchronize(st));
         float ms = 0;
         CK(cudaEventElapsedTime(&ms, h->ev0, h->ev1));
-        std::vector<unsigned long long> cnt(9 * nl);
+        std::vector<unsigned long long> cnt(12 * nl);
         CK(cudaMemcpy(cnt.data(), h->d_stats, sizeof(unsigned long long) * cnt.size(), cudaMemcpyDeviceToHost));
         int err = 0;
         CK(cudaMemcpy(&err, h->d_err, sizeof(int), cudaMemcpyDeviceToHost));
@@ -1891,11 +1995,11 @@ int build_impl(jk_handle *h, const double *const *D, int32_t ndm, int with_j, in
             for (size_t g = 0; g < T.P->groups.size(); ++g, ++k) {
                 const LaunchGroup &G = T.P->groups[g];
                 for (int i = G.sub0; i < G.sub0 + G.nsub; ++i) {
-                    const int l = T.P->launch[i], slot = l * 3 + T.t;
-                    KSpec x = h->launches[l].spec[T.t == 0 ? 0 : 1];
+                    const int l = T.P->launch[i], slot = l * 4 + T.t;
+                    KSpec x = h->launches[l].spec[spec_of[T.t]];
                     x.op = op;
                     const unsigned long long nq = cnt[3 * slot], np = cnt[3 * slot + 1];
-                    if (T.t == 0) stats->quartets_fp64 += (int64_t)nq;
+                    if (T.t == 0 || T.t == 3) stats->quartets_fp64 += (int64_t)nq;
                     else stats->quartets_fp32 += (int64_t)nq;
                     if (T.t == 2) routed_fp32 += (int64_t)nq;
                     stats->prim_quartets += (int64_t)np;
@@ -1905,7 +2009,7 @@ int build_impl(jk_handle *h, const double *const *D, int32_t ndm, int with_j, in
                         jk_launch_prof p;
                         p.la = x.la; p.lb = x.lb; p.lc = x.lc; p.ld = x.ld;
                         p.na = x.na; p.nb = x.nb; p.nc = x.nc; p.nd = x.nd;
-                        p.tier = T.t == 0 ? 0 : 1;
+                        p.tier = T.t == 0 || T.t == 3 ? 0 : 1;
                         p.threads_per_quartet = x.G();
                         p.regs = ki.regs;
                         p.local_bytes = ki.local_bytes;
@@ -2041,9 +2145,11 @@ int tune_impl(jk_handle *h, const double *const *D, int32_t ndm, int with_j, int
     if (ndm < 1 || ndm > JK_NDM_MAX) return fail(JK_ERR_ARG, "bad n_dm");
     const auto t0 = std::chrono::steady_clock::now();
     const bool two = mode == JK_PREC_MIXED || mode == JK_PREC_MIXED_ROUTED;
-    std::vector<int> tiers;
+    const bool usedf = mode != JK_PREC_FP32 && h->split > 0 && h->df_ok && cutoff >= 1e-30;
+    std::vector<int> tiers;   // shapes: FP64, FP32, two floats
     if (mode == JK_PREC_FP64 || two) tiers.push_back(0);
     if (mode == JK_PREC_FP32 || two) tiers.push_back(1);
+    if (usedf) tiers.push_back(2);
     double total = 0;
     for (auto &L : h->launches) total += L.cost;
     struct Item {
@@ -2071,7 +2177,7 @@ int tune_impl(jk_handle *h, const double *const *D, int32_t ndm, int with_j, int
         for (auto &it : items)
             for (auto c : it.c) {
                 c.ndm = ndm; c.doj = with_j ? 1 : 0; c.dok = with_k ? 1 : 0;
-                c.mode = (mode == JK_PREC_MIXED_ROUTED && it.t == 0) ? 1 : 0;
+                c.mode = (mode == JK_PREC_MIXED_ROUTED && it.t != 1) ? 1 : 0;
                 c.op = h->omega == 0.0 ? 0 : (h->omega > 0.0 ? 1 : 2);
                 all.push_back(c);
             }
@@ -2089,7 +2195,7 @@ int tune_impl(jk_handle *h, const double *const *D, int32_t ndm, int with_j, int
     size_t nround = 0;
     for (auto &it : items) nround = std::max(nround, it.c.size());
     std::map<int, int> by_slot;
-    for (size_t i = 0; i < items.size(); ++i) by_slot[items[i].l * 3 + items[i].t] = (int)i;
+    for (size_t i = 0; i < items.size(); ++i) by_slot[items[i].l * 4 + (items[i].t == 2 ? 3 : items[i].t)] = (int)i;
     const int o_prof = h->profile, o_branches = h->branches, o_graph = h->use_graph;
     h->profile = 1;
     h->branches = 1;
@@ -2260,6 +2366,10 @@ int jk_set_option(jk_handle *h, const char *key, double value)
         if (!(value >= 1 && value <= JK_MAX_BRANCHES + 1)) return fail(JK_ERR_ARG, "branches must be in [1, %d]", JK_MAX_BRANCHES + 1);
         h->branches = (int)value;
     }
+    else if (k == "split") {
+        if (!(value >= 0 && value <= 1)) return fail(JK_ERR_ARG, "split must be in [0, 1]");
+        h->split = value;
+    }
     else if (k == "asym64") h->asym64 = value != 0;
     else if (k == "widen_int") h->widen_int = value != 0;
     else if (k == "chunk" || k == "chunk_fp64tier") {
@@ -2304,6 +2414,7 @@ int jk_get_option(jk_handle *h, const char *key, double *value)
     else if (k == "prim_eps") *value = h->prim_eps;
     else if (k == "omega") *value = h->omega;
     else if (k == "part_index") *value = h->part_index;
+    else if (k == "split") *value = h->split;
     else if (k == "asym64") *value = h->asym64;
     else if (k == "widen_int") *value = h->widen_int;
     else if (k == "chunk") *value = h->chunk;
@@ -2599,12 +2710,13 @@ int jk_compile_class(int32_t la, int32_t lb, int32_t lc, int32_t ld, int32_t na,
         nd > JK_NPRIM_MAX)
         return fail(JK_ERR_UNSUPPORTED, "primitive count out of range");
     if (n_dm < 1 || n_dm > JK_NDM_MAX || (!with_j && !with_k)) return fail(JK_ERR_ARG, "bad n_dm or flags");
-    if (mode < 0 || mode > 3 || (mode == 2 && fp32) || (mode == 3 && !fp32)) return fail(JK_ERR_ARG, "bad mode");
+    if (fp32 != 2) fp32 = fp32 ? 1 : 0;
+    if (mode < 0 || mode > 3 || (mode == 2 && fp32) || (mode == 3 && fp32 != 1)) return fail(JK_ERR_ARG, "bad mode");
     if (op < 0 || op > 2) return fail(JK_ERR_ARG, "bad op");
     KSpec s;
     s.kind = 0;
     s.la = la; s.lb = lb; s.lc = lc; s.ld = ld; s.na = na; s.nb = nb; s.nc = nc; s.nd = nd;
-    s.ndm = n_dm; s.doj = with_j ? 1 : 0; s.dok = with_k ? 1 : 0; s.fp32 = fp32 ? 1 : 0;
+    s.ndm = n_dm; s.doj = with_j ? 1 : 0; s.dok = with_k ? 1 : 0; s.fp32 = fp32;
     s.mode = mode;
     s.op = op;
     choose_fragments(s, false);
@@ -2621,7 +2733,8 @@ int jk_compile_basis(const jk_shell *shells, int32_t nshell, int32_t n_dm, int32
 {
     if (!shells || nshell < 1) return fail(JK_ERR_ARG, "no shells");
     if (n_dm < 1 || n_dm > JK_NDM_MAX || (!with_j && !with_k)) return fail(JK_ERR_ARG, "bad n_dm or flags");
-    if (mode < 0 || mode > 3 || (mode == 2 && fp32) || (mode == 3 && !fp32)) return fail(JK_ERR_ARG, "bad mode");
+    if (fp32 != 2) fp32 = fp32 ? 1 : 0;
+    if (mode < 0 || mode > 3 || (mode == 2 && fp32) || (mode == 3 && fp32 != 1)) return fail(JK_ERR_ARG, "bad mode");
     // shell types (l, nprim) -> pair classes (larger type first) -> class pairs
     std::vector<std::pair<int, int>> types;
     for (int i = 0; i < nshell; ++i) {
@@ -2655,7 +2768,7 @@ int jk_compile_basis(const jk_shell *shells, int32_t nshell, int32_t n_dm, int32
             s.lc = types[pcs[j].first].first; s.ld = types[pcs[j].second].first;
             s.na = types[pcs[i].first].second; s.nb = types[pcs[i].second].second;
             s.nc = types[pcs[j].first].second; s.nd = types[pcs[j].second].second;
-            s.ndm = n_dm; s.doj = with_j ? 1 : 0; s.dok = with_k ? 1 : 0; s.fp32 = fp32 ? 1 : 0; s.mode = mode;
+            s.ndm = n_dm; s.doj = with_j ? 1 : 0; s.dok = with_k ? 1 : 0; s.fp32 = fp32; s.mode = mode;
             choose_fragments(s, false);
             specs.push_back(s);
         }

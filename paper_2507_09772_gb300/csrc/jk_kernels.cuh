@@ -44,11 +44,103 @@ __device__ constexpr int jk_cart_exp(int l, int idx, int axis)
     return 0;
 }
 
+// ------------------------------------------------- two-float arithmetic
+// The split tier evaluates its quartets in pairs of floats (value h + l, 48
+// bits). GB300 has 64 FP32 lanes per FP64 lane: one FP64 instruction holds the
+// SM's FP64 pipe for as long as 64 FP32 instructions take to issue, a
+// two-float product takes 4 to 7 of them and a sum 8 to 11 (measured: 2,400
+// G/s two-float multiply-adds against 502 G/s DFMA). The algorithms are the
+// error-free transformations of Dekker (Numer. Math. 18, 1971) and Knuth (The
+// Art of Computer Programming 2, 4.2.2); the explicitly rounded intrinsics keep
+// the compiler from contracting them. "Loose" results may carry an l of a few
+// ulp of h; jk_norm brings it back below half an ulp.
+struct jkdf {
+    float h, l;
+};
+__device__ __forceinline__ jkdf jk_norm(jkdf a)
+{
+    const float s = __fadd_rn(a.h, a.l);
+    return {s, __fadd_rn(a.l, -__fadd_rn(s, -a.h))};
+}
+// product (loose): h l' and l h' included, l l' (2^-48 of the result) dropped
+__device__ __forceinline__ jkdf jk_mul(jkdf a, jkdf b)
+{
+    const float p = __fmul_rn(a.h, b.h);
+    float e = __fmaf_rn(a.h, b.h, -p);
+    e = __fmaf_rn(a.h, b.l, e);
+    return {p, __fmaf_rn(a.l, b.h, e)};
+}
+// sum (loose)
+__device__ __forceinline__ jkdf jk_add(jkdf a, jkdf b)
+{
+    const float s = __fadd_rn(a.h, b.h), t = __fadd_rn(s, -a.h);
+    const float e = __fadd_rn(__fadd_rn(a.h, -__fadd_rn(s, -t)), __fadd_rn(b.h, -t));
+    return {s, __fadd_rn(e, __fadd_rn(a.l, b.l))};
+}
+__device__ __forceinline__ jkdf jk_neg(jkdf a) { return {-a.h, -a.l}; }
+__device__ __forceinline__ jkdf jk_sub(jkdf a, jkdf b) { return jk_add(a, jk_neg(b)); }
+// v += a b (loose)
+__device__ __forceinline__ void jk_acc(jkdf &v, jkdf a, jkdf b) { v = jk_add(v, jk_mul(a, b)); }
+__device__ __forceinline__ void jk_addto(jkdf &v, jkdf a) { v = jk_add(v, a); }
+// times an exactly representable power of two
+__device__ __forceinline__ jkdf jk_scale(jkdf a, float s) { return {__fmul_rn(a.h, s), __fmul_rn(a.l, s)}; }
+// times a small integer (loose)
+__device__ __forceinline__ jkdf jk_int(int n, jkdf a)
+{
+    if (n == 1) return a;
+    const float p = __fmul_rn(a.h, (float)n);
+    return {p, __fmaf_rn((float)n, a.l, __fmaf_rn((float)n, a.h, -p))};
+}
+template <typename R> struct JkConst {
+    __device__ static __forceinline__ R get(double c) { return (R)c; }
+};
+template <> struct JkConst<jkdf> {   // compile-time constants only
+    __device__ static __forceinline__ jkdf get(double c) { return {(float)c, (float)(c - (double)(float)c)}; }
+};
+// 1 / sqrt(x): the FP32 estimate y and its residual r = 1 - x y^2 in two
+// floats, y (1 + r/2 + 3 r^2 / 8) (normalised)
+__device__ __forceinline__ jkdf jk_rsqrt(jkdf x)
+{
+    const float y = rsqrtf(x.h);
+    const float p = __fmul_rn(y, y), e = __fmaf_rn(y, y, -p);
+    const jkdf m = jk_mul(x, jkdf{p, e});
+    const float r = __fadd_rn(__fadd_rn(1.0f, -m.h), -m.l);   // m.h is within an ulp or two of 1: exact difference
+    const float c = __fmaf_rn(__fmul_rn(0.375f, r), r, __fmul_rn(0.5f, r));
+    const float q = __fmul_rn(y, c);
+    const float s = __fadd_rn(y, q);
+    return {s, __fadd_rn(q, -__fadd_rn(s, -y))};
+}
+// the same names for the machine types
+template <typename T> __device__ __forceinline__ T jk_norm(T a) { return a; }
+template <typename T> __device__ __forceinline__ T jk_mul(T a, T b) { return a * b; }
+template <typename T> __device__ __forceinline__ T jk_add(T a, T b) { return a + b; }
+template <typename T> __device__ __forceinline__ T jk_sub(T a, T b) { return a - b; }
+template <typename T> __device__ __forceinline__ T jk_neg(T a) { return -a; }
+template <typename T> __device__ __forceinline__ void jk_acc(T &v, T a, T b) { v += a * b; }
+template <typename T> __device__ __forceinline__ void jk_addto(T &v, T a) { v += a; }
+template <typename T> __device__ __forceinline__ T jk_scale(T a, float s) { return a * (T)s; }
+template <typename T> __device__ __forceinline__ T jk_int(int n, T a) { return T(n) * a; }
+
+// Primitive-pair records by arithmetic, and their fields.
 template <typename R> struct JkPP;
 template <> struct JkPP<double> { typedef JkPrimPair64 T; };
 template <> struct JkPP<float> { typedef JkPrimPair32 T; };
+template <> struct JkPP<jkdf> { typedef JkPrimPairDf T; };
 __device__ __forceinline__ float jk_pp_q(const JkPrimPair64 &r) { return r.qf; }
 __device__ __forceinline__ float jk_pp_q(const JkPrimPair32 &r) { return r.q; }
+__device__ __forceinline__ float jk_pp_q(const JkPrimPairDf &r) { return r.q; }
+template <typename R> struct JkPrim {
+    R Px, Py, Pz, p, PAx, PAy, PAz, K, inv2p;
+};
+template <typename R, typename T> __device__ __forceinline__ JkPrim<R> jk_prim(const T &r)
+{
+    return {r.Px, r.Py, r.Pz, r.p, r.PAx, r.PAy, r.PAz, r.K, r.inv2p};
+}
+template <> __device__ __forceinline__ JkPrim<jkdf> jk_prim<jkdf, JkPrimPairDf>(const JkPrimPairDf &r)
+{
+    return {{r.Pxh, r.Pxl}, {r.Pyh, r.Pyl}, {r.Pzh, r.Pzl}, {r.ph, r.pl}, {r.PAxh, r.PAxl}, {r.PAyh, r.PAyl},
+            {r.PAzh, r.PAzl}, {r.Kh, r.Kl}, {r.i2ph, r.i2pl}};
+}
 
 __device__ __forceinline__ double jk_rsqrt(double x) { return rsqrt(x); }
 
@@ -61,6 +153,10 @@ __device__ __forceinline__ void jk_pair_ab(const JkPair &p, double &x, double &y
 __device__ __forceinline__ void jk_pair_ab(const JkPair &p, float &x, float &y, float &z)
 {
     x = p.ABxf; y = p.AByf; z = p.ABzf;
+}
+__device__ __forceinline__ void jk_pair_ab(const JkPair &p, jkdf &x, jkdf &y, jkdf &z)
+{
+    x = {p.ABxf, p.ABxl}; y = {p.AByf, p.AByl}; z = {p.ABzf, p.ABzl};
 }
 
 // An FP32 tier contribution widened to FP64 for the FP64 atomics into J and
@@ -92,6 +188,16 @@ __device__ __forceinline__ double jk_to_f64(float x)
 }
 // wi = 0: the conversion instruction instead (for comparison)
 __device__ __forceinline__ double jk_wide(float x, int wi) { return wi ? jk_to_f64(x) : (double)x; }
+// Two floats to FP64: both halves by integer operations (a conversion is an
+// FP64-pipe instruction; here the pipe is left with the one sum). A half below
+// the normal FP32 range (1.2e-38) counts as zero.
+__device__ __forceinline__ double jk_to_f64_normal(float x)
+{
+    const unsigned u = __float_as_uint(x), m = u & 0x7fffffffu;
+    const unsigned hi = (u & 0x80000000u) | ((m >> 3) + 0x38000000u);
+    return m < 0x00800000u ? 0.0 : __hiloint2double((int)hi, (int)(m << 29));
+}
+__device__ __forceinline__ double jk_wide(jkdf x, int) { return jk_to_f64_normal(x.h) + jk_to_f64_normal(x.l); }
 __device__ __forceinline__ float jk_rsqrt(float x) { return rsqrtf(x); }
 
 // ----------------------------------------------------- Rys roots, weights
@@ -166,35 +272,90 @@ __device__ __forceinline__ void jk_rys_one(float T, int r, const float *__restri
     w = aw;
 }
 
+// Two floats: `tab` holds per interval, for each of the 2 N functions, c0..c5
+// as (h, l) pairs and c6..c9 (below 2e-7 of c0) as floats, 16 floats, and four
+// floats of padding. 71 FP32 instructions per function, where the FP64
+// evaluation holds the FP64 pipe as long as about 1,000 take.
+__device__ __forceinline__ jkdf jk_rys_poly_df(const float4 *__restrict__ c, jkdf x)
+{
+    const float4 c01 = c[0], c23 = c[1], c45 = c[2], t = c[3];
+    const float f = __fmaf_rn(__fmaf_rn(__fmaf_rn(t.w, x.h, t.z), x.h, t.y), x.h, t.x);
+    jkdf a = jk_add(jkdf{c45.z, c45.w}, jkdf{__fmul_rn(f, x.h), 0.0f});
+    a = jk_add(jk_mul(a, x), jkdf{c45.x, c45.y});
+    a = jk_add(jk_mul(a, x), jkdf{c23.z, c23.w});
+    a = jk_add(jk_mul(a, x), jkdf{c23.x, c23.y});
+    a = jk_add(jk_mul(a, x), jkdf{c01.z, c01.w});
+    a = jk_add(jk_mul(jk_norm(a), x), jkdf{c01.x, c01.y});
+    return jk_norm(a);
+}
+template <int N>
+__device__ __forceinline__ void jk_rys_one(jkdf T, int r, const float *__restrict__ tab, jkdf &u, jkdf &w, int)
+{
+    if (T.h >= (float)(rys64_nint_c[N] * RYS64_H)) {
+        const jkdf s = jk_rsqrt(T);
+        const jkdf s2 = jk_norm(jk_mul(s, s));
+        const float4 g = rys_ghdf[rys_gh_offset[N - 1] / 2 + r];
+        u = jk_norm(jk_mul(jkdf{g.x, g.y}, s2));
+        w = jk_norm(jk_mul(jkdf{g.z, g.w}, s));
+        return;
+    }
+    const int k = min((int)(T.h * (float)RYS64_INVH), rys64_nint_c[N] - 1);
+    // x = (2 / H) T - (2 k + 1), 2 / H a power of two
+    const jkdf x = jk_norm(jk_add(jk_scale(T, (float)(2.0 * RYS64_INVH)), jkdf{-(float)(2 * k + 1), 0.0f}));
+    const float4 *c = reinterpret_cast<const float4 *>(tab + k * (32 * N + 4) + r * 16);
+    u = jk_rys_poly_df(c, x);
+    w = jk_rys_poly_df(c + 4 * N, x);
+}
+
 template <typename R> struct JkIsFloat { static constexpr bool v = false; };
 template <> struct JkIsFloat<float> { static constexpr bool v = true; };
+template <typename R> struct JkIsDf { static constexpr bool v = false; };
+template <> struct JkIsDf<jkdf> { static constexpr bool v = true; };
+template <typename R> struct JkTab { typedef R T; };     // element type of the Rys tables
+template <> struct JkTab<jkdf> { typedef float T; };
 
 // Floats of the FP32 Rys table of the N-root rule in its shared-memory
 // layout (intervals padded from 16 N to 16 N + 4 floats).
 template <int N> struct JkRysTab32 { static constexpr int n = rys32_nint_c[N] * (16 * N + 4); };
+// Two-float tables are staged up to three roots (12, 26, 42 KB); above, the
+// few threads of a group that evaluate roots read them through L1.
+#define JK_DF_STAGE 3
+template <int N> struct JkRysTabDf { static constexpr int n = N <= JK_DF_STAGE ? rys64_nint_c[N] * (32 * N + 4) : 0; };
 
 // --------------------------------------------------------- 2D integrals
 // One direction, one root: vertical recurrence on (n on A, m on C) up to
 // (LA+LB, LC+LD), then horizontal transfers to (a, b, c, d). Output layout
 // out[((a*(LB+1) + b)*(LC+1) + c)*(LD+1) + d].
-template <int LA, int LB, int LC, int LD, typename R>
+// UNIT: i00 is 1 (the x and y directions; z carries the weight).
+template <int LA, int LB, int LC, int LD, bool UNIT, typename R>
 __device__ __forceinline__ void jk_build_2d(R c00, R c00p, R b10, R b01, R b00, R i00,
                                             R ab, R cd, R *__restrict__ out)
 {
     constexpr int NA = LA + LB, NC = LC + LD;
     R V[NA + 1][NC + 1];
     V[0][0] = i00;
-    if (NA > 0) V[1][0] = c00 * i00;
+    if (NA > 0) V[1][0] = UNIT ? c00 : jk_norm(jk_mul(c00, i00));
 #pragma unroll
-    for (int n = 1; n < NA; ++n) V[n + 1][0] = c00 * V[n][0] + R(n) * b10 * V[n - 1][0];
+    for (int n = 1; n < NA; ++n) {
+        R v = jk_mul(c00, V[n][0]);
+        if (UNIT && n == 1) jk_addto(v, b10);
+        else jk_acc(v, jk_int(n, b10), V[n - 1][0]);
+        V[n + 1][0] = jk_norm(v);
+    }
 #pragma unroll
     for (int m = 0; m < NC; ++m) {
 #pragma unroll
         for (int n = 0; n <= NA; ++n) {
-            R v = c00p * V[n][m];
-            if (m > 0) v += R(m) * b01 * V[n][m - 1];
-            if (n > 0) v += R(n) * b00 * V[n - 1][m];
-            V[n][m + 1] = v;
+            R v = UNIT && m == 0 && n == 0 ? c00p : jk_mul(c00p, V[n][m]);
+            if (m > 0) {
+                if (UNIT && m == 1 && n == 0) jk_addto(v, b01);
+                else jk_acc(v, jk_int(m, b01), V[n][m - 1]);
+            }
+            if (n > 0) {
+                if (UNIT && n == 1 && m == 0) jk_addto(v, b00);
+                else jk_acc(v, jk_int(n, b00), V[n - 1][m]);
+            }
+            V[n][m + 1] = jk_norm(v);
         }
     }
     // bra transfer A -> B: H[a][b] = H[a+1][b-1] + AB H[a][b-1]
@@ -207,7 +368,12 @@ __device__ __forceinline__ void jk_build_2d(R c00, R c00p, R b10, R b01, R b00, 
 #pragma unroll
         for (int b = 1; b <= LB; ++b)
 #pragma unroll
-            for (int a = 0; a <= NA - b; ++a) t[a][b] = t[a + 1][b - 1] + ab * t[a][b - 1];
+            for (int a = 0; a <= NA - b; ++a) {
+                R v = t[a + 1][b - 1];
+                if (UNIT && m == 0 && a == 0 && b == 1) jk_addto(v, ab);
+                else jk_acc(v, ab, t[a][b - 1]);
+                t[a][b] = jk_norm(v);
+            }
 #pragma unroll
         for (int a = 0; a <= LA; ++a)
 #pragma unroll
@@ -224,7 +390,12 @@ __device__ __forceinline__ void jk_build_2d(R c00, R c00p, R b10, R b01, R b00, 
 #pragma unroll
             for (int d = 1; d <= LD; ++d)
 #pragma unroll
-                for (int c = 0; c <= NC - d; ++c) s[c][d] = s[c + 1][d - 1] + cd * s[c][d - 1];
+                for (int c = 0; c <= NC - d; ++c) {
+                    R v = s[c + 1][d - 1];
+                    if (UNIT && a == 0 && b == 0 && c == 0 && d == 1) jk_addto(v, cd);
+                    else jk_acc(v, cd, s[c][d - 1]);
+                    s[c][d] = jk_norm(v);
+                }
 #pragma unroll
             for (int c = 0; c <= LC; ++c)
 #pragma unroll
@@ -319,29 +490,30 @@ __device__ __forceinline__ void jk_group_sync(unsigned gmask)
 // for OP 2 set 1 is the erf part with negated weight. Returns u and w * pref.
 template <int NR, int OP, typename R>
 __device__ __forceinline__ void jk_op_root(R Tt, R rho, R pref, double omega, int a64, int r,
-                                           const R *__restrict__ rys, R &u, R &wp)
+                                           const typename JkTab<R>::T *__restrict__ rys, R &u, R &wp)
 {
     R uu, ww;
     if (OP == 0 || (OP == 2 && r < NR)) {
         jk_rys_one<NR>(Tt, r, rys, uu, ww, a64);
         u = uu;
-        wp = ww * pref;
+        wp = jk_norm(jk_mul(ww, pref));
     } else {
         // theta = w^2 / (w^2 + rho), sqrt(theta) = w / sqrt(w^2 + rho)
-        const R om = (R)omega;
-        const R rd = jk_rsqrt(om * om + rho);
-        const R st = om * rd, th = st * st;
-        jk_rys_one<NR>(th * Tt, OP == 2 ? r - NR : r, rys, uu, ww, a64);
-        u = th * uu;
-        wp = (OP == 2 ? -st : st) * ww * pref;
+        const R om = JkConst<R>::get(omega);
+        const R rd = jk_rsqrt(jk_norm(jk_add(jk_mul(om, om), rho)));
+        const R st = jk_norm(jk_mul(om, rd)), th = jk_norm(jk_mul(st, st));
+        jk_rys_one<NR>(jk_norm(jk_mul(th, Tt)), OP == 2 ? r - NR : r, rys, uu, ww, a64);
+        u = jk_norm(jk_mul(th, uu));
+        wp = jk_norm(jk_mul(jk_norm(jk_mul(OP == 2 ? jk_neg(st) : st, ww)), pref));
     }
 }
 
 template <int LA, int LB, int LC, int LD, int GA, int GB, int GC, int GD, typename R, int OP = 0,
           int NT = JkShape<LA, LB, LC, LD, GA, GB, GC, GD, OP>::G>
-__device__ __forceinline__ int jk_quartet(const JkPair &bra, const JkPair &ket, int nab, int ncd, float qthr, double omega, int a64,
+__device__ __forceinline__ int jk_quartet(const JkPair &bra, const JkPair &ket, int ab0, int dab, int nab, int ncd, float qthr, double omega, int a64,
                                            const typename JkPP<R>::T *__restrict__ pp,
-                                           const R *__restrict__ rys, R *grp, unsigned gmask, int tg, bool act,
+                                           const typename JkTab<R>::T *__restrict__ rys, R *grp, unsigned gmask,
+                                           int tg, bool act,
                                            const JkOffsets<JkShape<LA, LB, LC, LD, GA, GB, GC, GD, OP>> &off,
                                            R (&T)[JkShape<LA, LB, LC, LD, GA, GB, GC, GD, OP>::EPT])
 {
@@ -361,39 +533,53 @@ __device__ __forceinline__ int jk_quartet(const JkPair &bra, const JkPair &ket, 
     // record per lane and kl) are the outer loop, so each is loaded once; the
     // bra's (the same for the whole group or warp) the inner one.
     const float qthf = qthr;
-    const float qb0 = jk_pp_q(bpp[0]);
+    const float qb0 = jk_pp_q(bpp[ab0]);
     int nprim = 0;
 #pragma unroll 1
     for (int kl = 0; kl < ncd; ++kl) {
-        const PPT kp = kpp[kl];
-        const float qk = jk_pp_q(kp);
+        const PPT kr = kpp[kl];
+        const float qk = jk_pp_q(kr);
         if (qb0 * qk <= qthf) break;
+        const JkPrim<R> kp = jk_prim<R>(kr);
 #pragma unroll 1
-        for (int ij = 0; ij < nab; ++ij) {
-            const PPT bp = bpp[ij];
-            if (jk_pp_q(bp) * qk <= qthf) break;
+        for (int ij = ab0; ij < nab; ij += dab) {
+            const PPT br = bpp[ij];
+            if (jk_pp_q(br) * qk <= qthf) break;
             ++nprim;
-            const R p = bp.p, q = kp.p;
-            const R rpq = jk_rsqrt(p + q);
-            const R inv_pq = rpq * rpq;
-            const R PQx = bp.Px - kp.Px, PQy = bp.Py - kp.Py, PQz = bp.Pz - kp.Pz;
-            const R rho = p * q * inv_pq;
-            const R Tt = rho * (PQx * PQx + PQy * PQy + PQz * PQz);
-            const R pref = (R)JK_TWO_PI_2_5 * bp.K * kp.K * rpq;
-            const R qf = q * inv_pq, pf = p * inv_pq;
-            if (S::G == 1) {
-#pragma unroll
+            const JkPrim<R> bp = jk_prim<R>(br);
+            const R rpq = jk_rsqrt(jk_norm(jk_add(bp.p, kp.p)));
+            const R inv_pq = jk_norm(jk_mul(rpq, rpq));
+            const R PQx = jk_norm(jk_sub(bp.Px, kp.Px)), PQy = jk_norm(jk_sub(bp.Py, kp.Py)),
+                    PQz = jk_norm(jk_sub(bp.Pz, kp.Pz));
+            const R qf = jk_norm(jk_mul(kp.p, inv_pq)), pf = jk_norm(jk_mul(bp.p, inv_pq));
+            const R rho = jk_norm(jk_mul(bp.p, qf));
+            R r2 = jk_mul(PQx, PQx);
+            jk_acc(r2, PQy, PQy);
+            jk_acc(r2, PQz, PQz);
+            const R Tt = jk_norm(jk_mul(rho, jk_norm(r2)));
+            const R pref = jk_norm(jk_mul(jk_norm(jk_mul(JkConst<R>::get(JK_TWO_PI_2_5), bp.K)),
+                                          jk_norm(jk_mul(kp.K, rpq))));
+            if constexpr (S::G == 1) {
+#pragma unroll(JkIsDf<R>::v ? 1 : NRE)
                 for (int r = 0; r < NRE; ++r) {
                     R u, wp;
                     jk_op_root<NR, OP, R>(Tt, rho, pref, omega, a64, r, rys, u, wp);
-                    const R b00 = (R)0.5 * u * inv_pq;
-                    const R b10 = bp.inv2p * ((R)1 - u * qf);
-                    const R b01 = kp.inv2p * ((R)1 - u * pf);
-                    const R uq = u * qf, up = u * pf;
+                    const R uq = jk_norm(jk_mul(u, qf)), up = jk_norm(jk_mul(u, pf));
+                    const R one = JkConst<R>::get(1.0);
+                    const R b00 = jk_scale(jk_norm(jk_mul(u, inv_pq)), 0.5f);
+                    R muq = one, mup = one;   // 1 - u qf, 1 - u pf, the product not rounded
+                    jk_acc(muq, jk_neg(u), qf);
+                    jk_acc(mup, jk_neg(u), pf);
+                    const R b10 = jk_norm(jk_mul(bp.inv2p, jk_norm(muq)));
+                    const R b01 = jk_norm(jk_mul(kp.inv2p, jk_norm(mup)));
+                    const R nuq = jk_neg(uq);
+                    R ax = bp.PAx, ay = bp.PAy, az = bp.PAz, cx = kp.PAx, cy = kp.PAy, cz = kp.PAz;
+                    jk_acc(ax, nuq, PQx); jk_acc(ay, nuq, PQy); jk_acc(az, nuq, PQz);
+                    jk_acc(cx, up, PQx); jk_acc(cy, up, PQy); jk_acc(cz, up, PQz);
                     R tx[S::NI], ty[S::NI], tz[S::NI];
-                    jk_build_2d<LA, LB, LC, LD, R>(bp.PAx - uq * PQx, kp.PAx + up * PQx, b10, b01, b00, (R)1, ABx, CDx, tx);
-                    jk_build_2d<LA, LB, LC, LD, R>(bp.PAy - uq * PQy, kp.PAy + up * PQy, b10, b01, b00, (R)1, ABy, CDy, ty);
-                    jk_build_2d<LA, LB, LC, LD, R>(bp.PAz - uq * PQz, kp.PAz + up * PQz, b10, b01, b00, wp, ABz, CDz, tz);
+                    jk_build_2d<LA, LB, LC, LD, true, R>(jk_norm(ax), jk_norm(cx), b10, b01, b00, one, ABx, CDx, tx);
+                    jk_build_2d<LA, LB, LC, LD, true, R>(jk_norm(ay), jk_norm(cy), b10, b01, b00, one, ABy, CDy, ty);
+                    jk_build_2d<LA, LB, LC, LD, false, R>(jk_norm(az), jk_norm(cz), b10, b01, b00, wp, ABz, CDz, tz);
 #pragma unroll
                     for (int ia = 0; ia < S::FA; ++ia)
 #pragma unroll
@@ -409,7 +595,11 @@ __device__ __forceinline__ int jk_quartet(const JkPair &bra, const JkPair &ket, 
                                     const int oz = jk_cart_exp(LA, ia, 2) * S::SA + jk_cart_exp(LB, ib, 2) * S::SB +
                                                    jk_cart_exp(LC, ic, 2) * S::SC + jk_cart_exp(LD, id, 2);
                                     const int k = ((ia * S::FB + ib) * S::FC + ic) * S::FD + id;
-                                    T[k] += tx[ox] * ty[oy] * tz[oz];
+                                    // entry 0 of the x and y tables is 1
+                                    if (ox == 0 && oy == 0) jk_addto(T[k], tz[oz]);
+                                    else if (oy == 0) jk_acc(T[k], tx[ox], tz[oz]);
+                                    else if (ox == 0) jk_acc(T[k], ty[oy], tz[oz]);
+                                    else jk_acc(T[k], jk_mul(tx[ox], ty[oy]), tz[oz]);
                                 }
                 }
             } else {
@@ -424,16 +614,22 @@ __device__ __forceinline__ int jk_quartet(const JkPair &bra, const JkPair &ket, 
                 for (int task = tg; task < 3 * NRE && tg < NT; task += NT) {
                     const int r = task / 3, dir = task - 3 * r;
                     const R u = roots[r];
-                    const R b00 = (R)0.5 * u * inv_pq;
-                    const R b10 = bp.inv2p * ((R)1 - u * qf);
-                    const R b01 = kp.inv2p * ((R)1 - u * pf);
-                    const R uq = u * qf, up = u * pf;
-                    R pa, qc, pqd, abd, cdd, i00 = (R)1;
+                    const R one = JkConst<R>::get(1.0);
+                    const R uq = jk_norm(jk_mul(u, qf)), up = jk_norm(jk_mul(u, pf));
+                    const R b00 = jk_scale(jk_norm(jk_mul(u, inv_pq)), 0.5f);
+                    R muq = one, mup = one;   // 1 - u qf, 1 - u pf, the product not rounded
+                    jk_acc(muq, jk_neg(u), qf);
+                    jk_acc(mup, jk_neg(u), pf);
+                    const R b10 = jk_norm(jk_mul(bp.inv2p, jk_norm(muq)));
+                    const R b01 = jk_norm(jk_mul(kp.inv2p, jk_norm(mup)));
+                    R pa, qc, pqd, abd, cdd, i00 = one;
                     if (dir == 0) { pa = bp.PAx; qc = kp.PAx; pqd = PQx; abd = ABx; cdd = CDx; }
                     else if (dir == 1) { pa = bp.PAy; qc = kp.PAy; pqd = PQy; abd = ABy; cdd = CDy; }
                     else { pa = bp.PAz; qc = kp.PAz; pqd = PQz; abd = ABz; cdd = CDz; i00 = roots[NRE + r]; }
-                    jk_build_2d<LA, LB, LC, LD, R>(pa - uq * pqd, qc + up * pqd, b10, b01, b00, i00, abd, cdd,
-                                                   grp + (r * 3 + dir) * S::NI);
+                    jk_acc(pa, jk_neg(uq), pqd);
+                    jk_acc(qc, up, pqd);
+                    jk_build_2d<LA, LB, LC, LD, false, R>(jk_norm(pa), jk_norm(qc), b10, b01, b00, i00, abd, cdd,
+                                                          grp + (r * 3 + dir) * S::NI);
                 }
                 jk_group_sync<S::G>(gmask);
                 if (act) {
@@ -449,27 +645,38 @@ __device__ __forceinline__ int jk_quartet(const JkPair &bra, const JkPair &ket, 
                                 const int oy = off.a[1][ia] + off.b[1][ib] + off.c[1][ic] + off.d[1][id];
                                 const int oz = off.a[2][ia] + off.b[2][ib] + off.c[2][ic] + off.d[2][id];
                                 const int k = ((ia * S::FB + ib) * S::FC + ic) * S::FD + id;
-                                R acc = (R)0;
+                                if constexpr (JkIsDf<R>::v) {
 #pragma unroll
-                                for (int r = 0; r < NRE; ++r)
-                                    acc += grp[(r * 3 + 0) * S::NI + ox] * grp[(r * 3 + 1) * S::NI + oy] *
-                                           grp[(r * 3 + 2) * S::NI + oz];
-                                T[k] += acc;
+                                    for (int r = 0; r < NRE; ++r)
+                                        jk_acc(T[k], jk_mul(grp[(r * 3 + 0) * S::NI + ox], grp[(r * 3 + 1) * S::NI + oy]),
+                                               grp[(r * 3 + 2) * S::NI + oz]);
+                                } else {
+                                    R acc = (R)0;
+#pragma unroll
+                                    for (int r = 0; r < NRE; ++r)
+                                        acc += grp[(r * 3 + 0) * S::NI + ox] * grp[(r * 3 + 1) * S::NI + oy] *
+                                               grp[(r * 3 + 2) * S::NI + oz];
+                                    T[k] += acc;
+                                }
                             }
                 }
                 jk_group_sync<S::G>(gmask);
             }
         }
     }
+#pragma unroll
+    for (int k = 0; k < S::EPT; ++k) T[k] = jk_norm(T[k]);
     return nprim;
 }
 
 template <typename R> __device__ __forceinline__ const typename JkPP<R>::T *jk_pp(const JkClassArgs &a);
 template <> __device__ __forceinline__ const JkPrimPair64 *jk_pp<double>(const JkClassArgs &a) { return a.pp64; }
 template <> __device__ __forceinline__ const JkPrimPair32 *jk_pp<float>(const JkClassArgs &a) { return a.pp32; }
-template <typename R> __device__ __forceinline__ const R *jk_rys(const JkClassArgs &a);
+template <> __device__ __forceinline__ const JkPrimPairDf *jk_pp<jkdf>(const JkClassArgs &a) { return a.ppdf; }
+template <typename R> __device__ __forceinline__ const typename JkTab<R>::T *jk_rys(const JkClassArgs &a);
 template <> __device__ __forceinline__ const double *jk_rys<double>(const JkClassArgs &a) { return a.rys64; }
 template <> __device__ __forceinline__ const float *jk_rys<float>(const JkClassArgs &a) { return a.rys32; }
+template <> __device__ __forceinline__ const float *jk_rys<jkdf>(const JkClassArgs &a) { return a.rysdf; }
 
 // ---------------------------------------------- routed builds: the FP64 tier
 // The FP64 tier of a routed build is the only tier that runs the router: the
@@ -497,16 +704,35 @@ __device__ __forceinline__ bool jk_route_out(const JkClassArgs &args, int launch
 }
 
 // ------------------------------------------------- screening of a candidate
+// The bounds of a tier for one molecule (FP64 and rounded to FP32): the split
+// threshold follows the molecule's largest density element, and is formed
+// alike by every launch of a build.
+struct JkBounds {
+    double lo, hi;
+    float lo32, hi32;
+};
+__device__ __forceinline__ JkBounds jk_bounds(const JkClassArgs &args, const JkMol &mol, double dmol)
+{
+    JkBounds b = {args.lo, args.hi, args.lo32, args.hi32};
+    if (args.split_side != 0) {
+        // (densities near the FP32 range, or not finite, stay in FP64)
+        const double th =
+            dmol < 1e15 ? fmax(args.split_min, __dmul_rn(__dmul_rn(args.split, mol.qmax2), dmol)) : 0.0;
+        if (args.split_side > 0 && th > b.lo) { b.lo = th; b.lo32 = (float)th; }
+        if (args.split_side < 0 && th < b.hi) { b.hi = th; b.hi32 = (float)th; }
+    }
+    return b;
+}
 template <int MODE>
-__device__ __forceinline__ void jk_screen_bound(const JkClassArgs &args, const JkPair *__restrict__ kets,
-                                                const JkPair &bra, const JkMol &mol,
+__device__ __forceinline__ void jk_screen_bound(const JkClassArgs &args, const JkBounds &bd,
+                                                const JkPair *__restrict__ kets, const JkPair &bra, const JkMol &mol,
                                                 const double *dmx, double dmol, float dmol32, int j, int ke,
                                                 bool &sig, bool &stop, bool &band, float &dmq, float &Bout);
 // Keep (bra, ket j) iff lo < Q_ab Q_cd Dmax <= hi; `stop` when even the
 // molecule's largest density element cannot lift this ket (and every later
 // one, kets being sorted by Q) above lo.
 template <int MODE>
-__device__ __forceinline__ void jk_screen(const JkClassArgs &args, const JkSub &sub, const JkPair &bra,
+__device__ __forceinline__ void jk_screen(const JkClassArgs &args, const JkBounds &bd, const JkSub &sub, const JkPair &bra,
                                           const JkPairFeat &braf, const JkMol &mol, const double *dmx, double dmol, float dmol32, int item,
                                           int j, int ke, bool &sig, bool &stop, bool &band, float &dmq,
                                           unsigned short *rsm)
@@ -516,7 +742,7 @@ __device__ __forceinline__ void jk_screen(const JkClassArgs &args, const JkSub &
     band = false;
     dmq = 1.0f;
     float B = 0.0f;
-    jk_screen_bound<MODE>(args, sub.ket, bra, mol, dmx, dmol, dmol32, j, ke, sig, stop, band, dmq, B);
+    jk_screen_bound<MODE>(args, bd, sub.ket, bra, mol, dmx, dmol, dmol32, j, ke, sig, stop, band, dmq, B);
     if (MODE == 1) {
         // learned router for the band candidates, all lanes together on the
         // tensor cores; `band` then marks the quartets released to FP32
@@ -541,8 +767,8 @@ __device__ __forceinline__ bool jk_near(float x, float y)
 }
 
 template <int MODE>
-__device__ __forceinline__ void jk_screen_bound(const JkClassArgs &args, const JkPair *__restrict__ kets,
-                                                const JkPair &bra, const JkMol &mol,
+__device__ __forceinline__ void jk_screen_bound(const JkClassArgs &args, const JkBounds &bd,
+                                                const JkPair *__restrict__ kets, const JkPair &bra, const JkMol &mol,
                                                 const double *dmx, double dmol, float dmol32, int j, int ke,
                                                 bool &sig, bool &stop, bool &band, float &dmq, float &Bout)
 {
@@ -557,8 +783,8 @@ __device__ __forceinline__ void jk_screen_bound(const JkClassArgs &args, const J
         // few are redone in FP64 (every tier decides alike, as in FP64).
         const float bq = bra.Qf * __ldg(&kt.Qf);
         const float s = bq * dmol32;
-        bool st = s <= args.lo32;
-        if (args.scr32 == 2 && jk_near(s, args.lo32)) st = (bra.Q * kt.Q) * dmol <= args.lo;
+        bool st = s <= bd.lo32;
+        if (args.scr32 == 2 && jk_near(s, bd.lo32)) st = (bra.Q * kt.Q) * dmol <= bd.lo;
         if (st) { stop = true; return; }
         float dm = 1.0f;
         const int c = __ldg(&kt.a_loc), d = __ldg(&kt.b_loc);
@@ -576,10 +802,10 @@ __device__ __forceinline__ void jk_screen_bound(const JkClassArgs &args, const J
         dmq = dm;
         const float B = bq * dm;
         Bout = B;
-        sig = (B > args.lo32) && (B <= args.hi32);
+        sig = (B > bd.lo32) && (B <= bd.hi32);
         band = MODE == 1 && sig && B > args.tau32 && B <= args.band_hi32;
         if (args.scr32 == 2 &&
-            (jk_near(B, args.lo32) || jk_near(B, args.hi32) ||
+            (jk_near(B, bd.lo32) || jk_near(B, bd.hi32) ||
              (MODE == 1 && (jk_near(B, args.tau32) || jk_near(B, args.band_hi32))))) {
             double dm64 = 1.0;
             if (args.use_dmax) {
@@ -591,13 +817,13 @@ __device__ __forceinline__ void jk_screen_bound(const JkClassArgs &args, const J
                 }
             }
             const double B64 = (bra.Q * kt.Q) * dm64;
-            sig = (B64 > args.lo) && (B64 <= args.hi);
+            sig = (B64 > bd.lo) && (B64 <= bd.hi);
             band = MODE == 1 && sig && B64 > args.tau && B64 <= args.band_hi;
         }
         return;
     }
     const double bq = bra.Q * kt.Q;
-    if (bq * dmol <= args.lo) { stop = true; return; }
+    if (bq * dmol <= bd.lo) { stop = true; return; }
     double dm = 1.0;
     if (args.use_dmax) {
         const int c = kt.a_loc, d = kt.b_loc;
@@ -614,7 +840,7 @@ __device__ __forceinline__ void jk_screen_bound(const JkClassArgs &args, const J
     dmq = (float)dm;
     const double B = bq * dm;
     Bout = (float)B;
-    sig = (B > args.lo) && (B <= args.hi);
+    sig = (B > bd.lo) && (B <= bd.hi);
     band = MODE == 1 && sig && B > args.tau && B <= args.band_hi;
 }
 
@@ -652,9 +878,17 @@ __device__ __forceinline__ void jk_log_sample(const JkClassArgs &args, const JkP
 // ------------------------------------------ contraction with the density
 // The thread's fragment T of (ab|cd), degeneracy f: J_ab partial kept in
 // jab (flushed once per bra pair), the other five blocks by FP64 atomics.
-template <typename R> __device__ __forceinline__ const R *jk_dens(const JkMol &mol);
-template <> __device__ __forceinline__ const double *jk_dens<double>(const JkMol &mol) { return mol.D; }
-template <> __device__ __forceinline__ const float *jk_dens<float>(const JkMol &mol) { return mol.D32; }
+template <typename R> struct JkDens;
+template <> struct JkDens<double> { typedef double T; __device__ static __forceinline__ const double *p(const JkMol &m) { return m.D; } };
+template <> struct JkDens<float> { typedef float T; __device__ static __forceinline__ const float *p(const JkMol &m) { return m.D32; } };
+template <> struct JkDens<jkdf> { typedef float2 T; __device__ static __forceinline__ const float2 *p(const JkMol &m) { return m.D2; } };
+__device__ __forceinline__ double jk_ldd(const double *p) { return __ldg(p); }
+__device__ __forceinline__ float jk_ldd(const float *p) { return __ldg(p); }
+__device__ __forceinline__ jkdf jk_ldd(const float2 *p)
+{
+    const float2 v = __ldg(p);
+    return {v.x, v.y};
+}
 
 // J and K accumulate by FP64 reductions that return nothing (RED): atomicAdd
 // on doubles issues ATOM, whose value the L2 sends back although nobody
@@ -666,7 +900,7 @@ __device__ __forceinline__ void jk_red_add(double *p, double v)
 }
 
 template <int FA, int FB, int FC, int FD, int NDM, int DOJ, int DOK, typename R>
-__device__ __forceinline__ void jk_contract(const R (&T)[FA * FB * FC * FD], R f, const JkMol &mol,
+__device__ __forceinline__ void jk_contract(const R (&T)[FA * FB * FC * FD], float f, const JkMol &mol,
                                             int a0, int b0, int c0, int d0, R (&jab)[NDM][FA][FB], int wi)
 {
     const long long nn = (long long)mol.nao * mol.nao;
@@ -674,73 +908,74 @@ __device__ __forceinline__ void jk_contract(const R (&T)[FA * FB * FC * FD], R f
 #pragma unroll
     for (int m = 0; m < NDM; ++m) {
         // the tier's own copy of D (the FP32 tier reads a pre-rounded one)
-        const R *D = jk_dens<R>(mol) + m * nn;
+        const typename JkDens<R>::T *D = JkDens<R>::p(mol) + m * nn;
         if (DOJ) {
             R Dcd[FC][FD], Dab[FA][FB];
 #pragma unroll
             for (int ic = 0; ic < FC; ++ic)
 #pragma unroll
-                for (int id = 0; id < FD; ++id) Dcd[ic][id] = (R)__ldg(D + (long long)(c0 + ic) * nao + d0 + id);
+                for (int id = 0; id < FD; ++id) Dcd[ic][id] = jk_ldd(D + (long long)(c0 + ic) * nao + d0 + id);
 #pragma unroll
             for (int ia = 0; ia < FA; ++ia)
 #pragma unroll
-                for (int ib = 0; ib < FB; ++ib) Dab[ia][ib] = (R)__ldg(D + (long long)(a0 + ia) * nao + b0 + ib);
+                for (int ib = 0; ib < FB; ++ib) Dab[ia][ib] = jk_ldd(D + (long long)(a0 + ia) * nao + b0 + ib);
             R jcd[FC][FD];
 #pragma unroll
             for (int ic = 0; ic < FC; ++ic)
 #pragma unroll
-                for (int id = 0; id < FD; ++id) jcd[ic][id] = (R)0;
+                for (int id = 0; id < FD; ++id) jcd[ic][id] = JkConst<R>::get(0.0);
 #pragma unroll
             for (int ia = 0; ia < FA; ++ia)
 #pragma unroll
                 for (int ib = 0; ib < FB; ++ib) {
-                    R sum = (R)0;
+                    R sum = JkConst<R>::get(0.0);
 #pragma unroll
                     for (int ic = 0; ic < FC; ++ic)
 #pragma unroll
                         for (int id = 0; id < FD; ++id) {
                             const R t = T[((ia * FB + ib) * FC + ic) * FD + id];
-                            sum += t * Dcd[ic][id];
-                            jcd[ic][id] += t * Dab[ia][ib];
+                            jk_acc(sum, t, Dcd[ic][id]);
+                            jk_acc(jcd[ic][id], t, Dab[ia][ib]);
                         }
-                    jab[m][ia][ib] += (R)2 * f * sum;
+                    jk_addto(jab[m][ia][ib], jk_scale(sum, 2.0f * f));
+                    jab[m][ia][ib] = jk_norm(jab[m][ia][ib]);
                 }
 #pragma unroll
             for (int ic = 0; ic < FC; ++ic)
 #pragma unroll
                 for (int id = 0; id < FD; ++id)
-                    jk_red_add(mol.J + m * nn + (long long)(c0 + ic) * nao + d0 + id, jk_wide((R)2 * f * jcd[ic][id], wi));
+                    jk_red_add(mol.J + m * nn + (long long)(c0 + ic) * nao + d0 + id, jk_wide(jk_scale(jcd[ic][id], 2.0f * f), wi));
         }
         if (DOK) {
             R Dbd[FB][FD], Dbc[FB][FC], Dad[FA][FD], Dac[FA][FC];
 #pragma unroll
             for (int ib = 0; ib < FB; ++ib) {
 #pragma unroll
-                for (int id = 0; id < FD; ++id) Dbd[ib][id] = (R)__ldg(D + (long long)(b0 + ib) * nao + d0 + id);
+                for (int id = 0; id < FD; ++id) Dbd[ib][id] = jk_ldd(D + (long long)(b0 + ib) * nao + d0 + id);
 #pragma unroll
-                for (int ic = 0; ic < FC; ++ic) Dbc[ib][ic] = (R)__ldg(D + (long long)(b0 + ib) * nao + c0 + ic);
+                for (int ic = 0; ic < FC; ++ic) Dbc[ib][ic] = jk_ldd(D + (long long)(b0 + ib) * nao + c0 + ic);
             }
 #pragma unroll
             for (int ia = 0; ia < FA; ++ia) {
 #pragma unroll
-                for (int id = 0; id < FD; ++id) Dad[ia][id] = (R)__ldg(D + (long long)(a0 + ia) * nao + d0 + id);
+                for (int id = 0; id < FD; ++id) Dad[ia][id] = jk_ldd(D + (long long)(a0 + ia) * nao + d0 + id);
 #pragma unroll
-                for (int ic = 0; ic < FC; ++ic) Dac[ia][ic] = (R)__ldg(D + (long long)(a0 + ia) * nao + c0 + ic);
+                for (int ic = 0; ic < FC; ++ic) Dac[ia][ic] = jk_ldd(D + (long long)(a0 + ia) * nao + c0 + ic);
             }
             R kac[FA][FC], kad[FA][FD], kbc[FB][FC], kbd[FB][FD];
 #pragma unroll
             for (int ia = 0; ia < FA; ++ia) {
 #pragma unroll
-                for (int ic = 0; ic < FC; ++ic) kac[ia][ic] = (R)0;
+                for (int ic = 0; ic < FC; ++ic) kac[ia][ic] = JkConst<R>::get(0.0);
 #pragma unroll
-                for (int id = 0; id < FD; ++id) kad[ia][id] = (R)0;
+                for (int id = 0; id < FD; ++id) kad[ia][id] = JkConst<R>::get(0.0);
             }
 #pragma unroll
             for (int ib = 0; ib < FB; ++ib) {
 #pragma unroll
-                for (int ic = 0; ic < FC; ++ic) kbc[ib][ic] = (R)0;
+                for (int ic = 0; ic < FC; ++ic) kbc[ib][ic] = JkConst<R>::get(0.0);
 #pragma unroll
-                for (int id = 0; id < FD; ++id) kbd[ib][id] = (R)0;
+                for (int id = 0; id < FD; ++id) kbd[ib][id] = JkConst<R>::get(0.0);
             }
 #pragma unroll
             for (int ia = 0; ia < FA; ++ia)
@@ -751,34 +986,37 @@ __device__ __forceinline__ void jk_contract(const R (&T)[FA * FB * FC * FD], R f
 #pragma unroll
                         for (int id = 0; id < FD; ++id) {
                             const R t = T[((ia * FB + ib) * FC + ic) * FD + id];
-                            kac[ia][ic] += t * Dbd[ib][id];
-                            kad[ia][id] += t * Dbc[ib][ic];
-                            kbc[ib][ic] += t * Dad[ia][id];
-                            kbd[ib][id] += t * Dac[ia][ic];
+                            jk_acc(kac[ia][ic], t, Dbd[ib][id]);
+                            jk_acc(kad[ia][id], t, Dbc[ib][ic]);
+                            jk_acc(kbc[ib][ic], t, Dad[ia][id]);
+                            jk_acc(kbd[ib][id], t, Dac[ia][ic]);
                         }
             double *K = mol.K + m * nn;
 #pragma unroll
             for (int ia = 0; ia < FA; ++ia) {
 #pragma unroll
                 for (int ic = 0; ic < FC; ++ic)
-                    jk_red_add(K + (long long)(a0 + ia) * nao + c0 + ic, jk_wide(f * kac[ia][ic], wi));
+                    jk_red_add(K + (long long)(a0 + ia) * nao + c0 + ic, jk_wide(jk_scale(kac[ia][ic], f), wi));
 #pragma unroll
                 for (int id = 0; id < FD; ++id)
-                    jk_red_add(K + (long long)(a0 + ia) * nao + d0 + id, jk_wide(f * kad[ia][id], wi));
+                    jk_red_add(K + (long long)(a0 + ia) * nao + d0 + id, jk_wide(jk_scale(kad[ia][id], f), wi));
             }
 #pragma unroll
             for (int ib = 0; ib < FB; ++ib) {
 #pragma unroll
                 for (int ic = 0; ic < FC; ++ic)
-                    jk_red_add(K + (long long)(b0 + ib) * nao + c0 + ic, jk_wide(f * kbc[ib][ic], wi));
+                    jk_red_add(K + (long long)(b0 + ib) * nao + c0 + ic, jk_wide(jk_scale(kbc[ib][ic], f), wi));
 #pragma unroll
                 for (int id = 0; id < FD; ++id)
-                    jk_red_add(K + (long long)(b0 + ib) * nao + d0 + id, jk_wide(f * kbd[ib][id], wi));
+                    jk_red_add(K + (long long)(b0 + ib) * nao + d0 + id, jk_wide(jk_scale(kbd[ib][id], f), wi));
             }
         }
     }
 }
 
+__device__ __forceinline__ bool jk_nonzero(double x) { return x != 0.0; }
+__device__ __forceinline__ bool jk_nonzero(float x) { return x != 0.0f; }
+__device__ __forceinline__ bool jk_nonzero(jkdf x) { return x.h != 0.0f; }
 template <int FA, int FB, int NDM, typename R>
 __device__ __forceinline__ void jk_flush_jab(R (&jab)[NDM][FA][FB], const JkMol &mol, int a0, int b0, int wi)
 {
@@ -789,7 +1027,7 @@ __device__ __forceinline__ void jk_flush_jab(R (&jab)[NDM][FA][FB], const JkMol 
         for (int ia = 0; ia < FA; ++ia)
 #pragma unroll
             for (int ib = 0; ib < FB; ++ib)
-                if (jab[m][ia][ib] != (R)0)
+                if (jk_nonzero(jab[m][ia][ib]))
                     jk_red_add(mol.J + m * nn + (long long)(a0 + ia) * mol.nao + b0 + ib, jk_wide(jab[m][ia][ib], wi));
 }
 
@@ -800,7 +1038,7 @@ struct JkCount {
 };
 __device__ __forceinline__ void jk_count_flush(const JkClassArgs &args, int launch, JkCount &c)
 {
-    if (launch >= 0 && (c.nq || c.nband)) {
+    if (launch >= 0 && (c.nq || c.nprim || c.nband)) {
         unsigned long long *st = args.stats + (long long)launch * args.stat_stride;
         atomicAdd(st, c.nq);
         atomicAdd(st + 1, c.nprim);
@@ -834,7 +1072,7 @@ jk_class_kernel(const JkClassArgs args)
     extern __shared__ __align__(16) double jk_smem_raw[];
     const int lane = threadIdx.x & 31;
     const typename JkPP<R>::T *pp = jk_pp<R>(args);
-    const R *rys = jk_rys<R>(args);
+    const typename JkTab<R>::T *rys = jk_rys<R>(args);
     const long long nitems = MODE == 3 ? 0 : (long long)*args.nitems;
     if (MODE != 3 && (long long)blockIdx.x * (G <= 32 ? 4 : 1) >= nitems * X) return;
     // The FP32 tier reads its Rys table from shared memory: lanes gather
@@ -852,6 +1090,18 @@ jk_class_kernel(const JkClassArgs args)
         __syncthreads();
         rys = reinterpret_cast<const R *>(jk_smem_raw);
         smem_groups = reinterpret_cast<R *>(jk_smem_raw) + NT;
+    }
+    if constexpr (JkIsDf<R>::v) {
+        constexpr int NT = JkRysTabDf<S::NR>::n;
+        rys = rys + rysdf_offset[S::NR];
+        if constexpr (NT > 0) {
+            float4 *dst = reinterpret_cast<float4 *>(jk_smem_raw);
+            const float4 *src = reinterpret_cast<const float4 *>(rys);
+            for (int i = threadIdx.x; i < NT / 4; i += blockDim.x) dst[i] = __ldg(src + i);
+            __syncthreads();
+            rys = reinterpret_cast<const float *>(jk_smem_raw);
+            smem_groups = reinterpret_cast<R *>(jk_smem_raw) + NT / 2;
+        }
     }
     JkCount cnt = {0, 0, 0};
     int cur = -1;   // class pair the counters belong to
@@ -903,21 +1153,21 @@ jk_class_kernel(const JkClassArgs args)
                         const JkMol mol = args.mols[bra.mol];
                         R T[S::EPT];
 #pragma unroll
-                        for (int k = 0; k < S::EPT; ++k) T[k] = (R)0;
+                        for (int k = 0; k < S::EPT; ++k) T[k] = JkConst<R>::get(0.0);
                         const int np = jk_quartet<LA, LB, LC, LD, GA, GB, GC, GD, R, OP>(
-                            bra, ket, sub.nab, sub.ncd, __fdiv_rn(args.prim_eps32, rq.dmq), args.omega, args.asym64,
+                            bra, ket, 0, 1, sub.nab, sub.ncd, __fdiv_rn(args.prim_eps32, rq.dmq), args.omega, args.asym64,
                             pp, rys, grp, gmask, tg, true, off, T);
-                        R f = (R)1;
-                        if (bra.a == bra.b) f *= (R)0.5;
-                        if (ket.a == ket.b) f *= (R)0.5;
-                        if (sub.same_class && rq.ket == rq.item) f *= (R)0.5;
+                        float f = 1.0f;
+                        if (bra.a == bra.b) f *= 0.5f;
+                        if (ket.a == ket.b) f *= 0.5f;
+                        if (sub.same_class && rq.ket == rq.item) f *= 0.5f;
                         R jab[NDM][FA][FB];
 #pragma unroll
                         for (int m = 0; m < NDM; ++m)
 #pragma unroll
                             for (int i = 0; i < FA; ++i)
 #pragma unroll
-                                for (int jj = 0; jj < FB; ++jj) jab[m][i][jj] = (R)0;
+                                for (int jj = 0; jj < FB; ++jj) jab[m][i][jj] = JkConst<R>::get(0.0);
                         const int a0 = bra.a_ao + ga * FA, b0 = bra.b_ao + gb * FB;
                         jk_contract<FA, FB, FC, FD, NDM, DOJ, DOK, R>(T, f, mol, a0, b0, ket.a_ao + gc * FC,
                                                                      ket.b_ao + gd * FD, jab, args.widen_int);
@@ -943,7 +1193,8 @@ jk_class_kernel(const JkClassArgs args)
             unsigned long long nx = 0;
             if (AHEAD && lane == 0) nx = atomicAdd(args.work, 1ull);
             const JkItem wi = args.items[t];
-            const JkSub &sub = args.subs[wi.sub];
+            const JkSub &sub = args.subs[wi.sub & 0xffff];
+            const int part = wi.sub >> 16, parts = sub.split;   // share of the bra's primitive pairs
             const JkPair *__restrict__ kets = sub.ket;
             const int item = wi.bra, nab = sub.nab, ncd = sub.ncd, same_class = sub.same_class;
             const int kb = wi.kb, ke = wi.ke;
@@ -956,6 +1207,7 @@ jk_class_kernel(const JkClassArgs args)
             const double *dmx = args.dmax + mol.dmax_off;
             const double dmol = args.use_dmax ? args.dmax_mol[bra.mol] : 1.0;
             const float dmol32 = (float)dmol;
+            const JkBounds bd = jk_bounds(args, mol, dmol);
             const int a0 = bra.a_ao + ga * FA, b0 = bra.b_ao + gb * FB;
             JkPairFeat braf;
             if (MODE != 0) braf = sub.bra_feat[item];
@@ -965,7 +1217,7 @@ jk_class_kernel(const JkClassArgs args)
 #pragma unroll
                 for (int i = 0; i < FA; ++i)
 #pragma unroll
-                    for (int j = 0; j < FB; ++j) jab[m][i][j] = (R)0;
+                    for (int j = 0; j < FB; ++j) jab[m][i][j] = JkConst<R>::get(0.0);
             int nq = 0, nband = 0, nprim = 0;
             // significant kets wait in a per-warp queue (in scan order) until
             // a round can give every group of the warp one; partial rounds
@@ -977,7 +1229,7 @@ jk_class_kernel(const JkClassArgs args)
             for (int base = kb; base < ke; base += 32) {
                 bool sig = false, stop = false, band = false;
                 float dmq = 1.0f, B = 0.0f;
-                jk_screen_bound<MODE>(args, kets, bra, mol, dmx, dmol, dmol32, base + lane, ke, sig, stop, band, dmq, B);
+                jk_screen_bound<MODE>(args, bd, kets, bra, mol, dmx, dmol, dmol32, base + lane, ke, sig, stop, band, dmq, B);
                 const unsigned lt = (1u << lane) - 1u;
                 const bool def = sig && !band;   // decided by the bounds alone
                 const unsigned mdef = __ballot_sync(0xffffffffu, def);
@@ -1049,21 +1301,21 @@ jk_class_kernel(const JkClassArgs args)
                         const JkPair ket = kets[myket];
                         R T[S::EPT];
 #pragma unroll
-                        for (int k = 0; k < S::EPT; ++k) T[k] = (R)0;
+                        for (int k = 0; k < S::EPT; ++k) T[k] = JkConst<R>::get(0.0);
                         const int np = jk_quartet<LA, LB, LC, LD, GA, GB, GC, GD, R, OP>(
-                            bra, ket, nab, ncd, __fdiv_rn(args.prim_eps32, dmk), args.omega, args.asym64, pp, rys, grp,
+                            bra, ket, part, parts, nab, ncd, __fdiv_rn(args.prim_eps32, dmk), args.omega, args.asym64, pp, rys, grp,
                             gmask, tg, true, off, T);
                         if (tg == 0) nprim += np;
-                        R f = (R)1;
-                        if (bra.a == bra.b) f *= (R)0.5;
-                        if (ket.a == ket.b) f *= (R)0.5;
-                        if (same_class && myket == item) f *= (R)0.5;
+                        float f = 1.0f;
+                        if (bra.a == bra.b) f *= 0.5f;
+                        if (ket.a == ket.b) f *= 0.5f;
+                        if (same_class && myket == item) f *= 0.5f;
                         jk_contract<FA, FB, FC, FD, NDM, DOJ, DOK, R>(T, f, mol, a0, b0, ket.a_ao + gc * FC,
                                                                      ket.b_ao + gd * FD, jab, args.widen_int);
                         if (MODE == 2) {
                             double tm = 0.0;
 #pragma unroll
-                            for (int k = 0; k < S::EPT; ++k) tm = fmax(tm, fabs((double)T[k]));
+                            for (int k = 0; k < S::EPT; ++k) tm = fmax(tm, fabs(jk_wide(T[k], 0)));
                             for (int q = 0; q < G; ++q) tm = fmax(tm, __shfl_sync(gmask, tm, (gw * G + q) & 31));
                             if (tg == 0)
                                 jk_log_sample(args, bra, ket, braf, sub.ket_feat[myket],
@@ -1084,7 +1336,7 @@ jk_class_kernel(const JkClassArgs args)
                 if (last) break;
             }
             if (DOJ && active) jk_flush_jab<FA, FB, NDM, R>(jab, mol, a0, b0, args.widen_int);
-            cnt.nq += nq;
+            if (part == 0) cnt.nq += nq;
             cnt.nband += nband;
             cnt.nprim += __reduce_add_sync(0xffffffffu, (unsigned)nprim);
             if (!AHEAD && lane == 0) nx = atomicAdd(args.work, 1ull);
@@ -1133,22 +1385,22 @@ jk_class_kernel(const JkClassArgs args)
                     const JkMol mol = args.mols[bra.mol];
                     R T[S::EPT];
 #pragma unroll
-                    for (int k = 0; k < S::EPT; ++k) T[k] = (R)0;
+                    for (int k = 0; k < S::EPT; ++k) T[k] = JkConst<R>::get(0.0);
                     const int np = jk_quartet<LA, LB, LC, LD, GA, GB, GC, GD, R, OP, NTC>(
-                        bra, ket, sub.nab, sub.ncd, __fdiv_rn(args.prim_eps32, rq.dmq), args.omega, args.asym64, pp,
+                        bra, ket, 0, 1, sub.nab, sub.ncd, __fdiv_rn(args.prim_eps32, rq.dmq), args.omega, args.asym64, pp,
                         rys, grp, 0u, tg, act, off, T);
                     if (act) {
-                        R f = (R)1;
-                        if (bra.a == bra.b) f *= (R)0.5;
-                        if (ket.a == ket.b) f *= (R)0.5;
-                        if (sub.same_class && rq.ket == rq.item) f *= (R)0.5;
+                        float f = 1.0f;
+                        if (bra.a == bra.b) f *= 0.5f;
+                        if (ket.a == ket.b) f *= 0.5f;
+                        if (sub.same_class && rq.ket == rq.item) f *= 0.5f;
                         R jab[NDM][FA][FB];
 #pragma unroll
                         for (int m = 0; m < NDM; ++m)
 #pragma unroll
                             for (int i = 0; i < FA; ++i)
 #pragma unroll
-                                for (int jj = 0; jj < FB; ++jj) jab[m][i][jj] = (R)0;
+                                for (int jj = 0; jj < FB; ++jj) jab[m][i][jj] = JkConst<R>::get(0.0);
                         const int a0 = bra.a_ao + ga * FA, b0 = bra.b_ao + gb * FB;
                         jk_contract<FA, FB, FC, FD, NDM, DOJ, DOK, R>(T, f, mol, a0, b0, ket.a_ao + gc * FC,
                                                                      ket.b_ao + gd * FD, jab, args.widen_int);
@@ -1174,7 +1426,8 @@ jk_class_kernel(const JkClassArgs args)
                 jk_make_offsets<LA, LB, LC, LD, GA, GB, GC, GD, S>(ga, gb, gc, gd, off);
             }
             const JkItem wi = args.items[t];
-            const JkSub &sub = args.subs[wi.sub];
+            const JkSub &sub = args.subs[wi.sub & 0xffff];
+            const int part = wi.sub >> 16, parts = sub.split;   // share of the bra's primitive pairs
             const int item = wi.bra, nab = sub.nab, ncd = sub.ncd, same_class = sub.same_class;
             const int kb = wi.kb, ke = wi.ke;
             if (sub.launch != cur) {
@@ -1186,6 +1439,7 @@ jk_class_kernel(const JkClassArgs args)
             const double *dmx = args.dmax + mol.dmax_off;
             const double dmol = args.use_dmax ? args.dmax_mol[bra.mol] : 1.0;
             const float dmol32 = (float)dmol;
+            const JkBounds bd = jk_bounds(args, mol, dmol);
             const int a0 = bra.a_ao + ga * FA, b0 = bra.b_ao + gb * FB;
             JkPairFeat braf;
             if (MODE != 0) braf = sub.bra_feat[item];
@@ -1195,13 +1449,13 @@ jk_class_kernel(const JkClassArgs args)
 #pragma unroll
                 for (int i = 0; i < FA; ++i)
 #pragma unroll
-                    for (int j = 0; j < FB; ++j) jab[m][i][j] = (R)0;
+                    for (int j = 0; j < FB; ++j) jab[m][i][j] = JkConst<R>::get(0.0);
             unsigned long long nq = 0, nband = 0, nprim = 0;
             for (int base = kb; base < ke; base += 32) {
                 if (threadIdx.x < 32) {
                     bool sig, stop, band;
                     float dmq;
-                    jk_screen<MODE>(args, sub, bra, braf, mol, dmx, dmol, dmol32, item, base + lane, ke, sig, stop, band,
+                    jk_screen<MODE>(args, bd, sub, bra, braf, mol, dmx, dmol, dmol32, item, base + lane, ke, sig, stop, band,
                                     dmq, s_rsm);
                     s_dm[lane] = dmq;
                     const unsigned msk = __ballot_sync(0xffffffffu, sig);
@@ -1220,16 +1474,16 @@ jk_class_kernel(const JkClassArgs args)
                     const JkPair ket = sub.ket[myket];
                     R T[S::EPT];
 #pragma unroll
-                    for (int k = 0; k < S::EPT; ++k) T[k] = (R)0;
+                    for (int k = 0; k < S::EPT; ++k) T[k] = JkConst<R>::get(0.0);
                     const int np = jk_quartet<LA, LB, LC, LD, GA, GB, GC, GD, R, OP, NTC>(
-                        bra, ket, nab, ncd, __fdiv_rn(args.prim_eps32, s_dm[myket - base]), args.omega, args.asym64, pp,
+                        bra, ket, part, parts, nab, ncd, __fdiv_rn(args.prim_eps32, s_dm[myket - base]), args.omega, args.asym64, pp,
                         rys, grp, 0u, tg, act, off, T);
                     nprim += np;
                     if (act) {
-                        R f = (R)1;
-                        if (bra.a == bra.b) f *= (R)0.5;
-                        if (ket.a == ket.b) f *= (R)0.5;
-                        if (same_class && myket == item) f *= (R)0.5;
+                        float f = 1.0f;
+                        if (bra.a == bra.b) f *= 0.5f;
+                        if (ket.a == ket.b) f *= 0.5f;
+                        if (same_class && myket == item) f *= 0.5f;
                         jk_contract<FA, FB, FC, FD, NDM, DOJ, DOK, R>(T, f, mol, a0, b0, ket.a_ao + gc * FC,
                                                                      ket.b_ao + gd * FD, jab, args.widen_int);
                     }
@@ -1238,7 +1492,7 @@ jk_class_kernel(const JkClassArgs args)
                         double tm = 0.0;
                         if (act) {
 #pragma unroll
-                            for (int k = 0; k < S::EPT; ++k) tm = fmax(tm, fabs((double)T[k]));
+                            for (int k = 0; k < S::EPT; ++k) tm = fmax(tm, fabs(jk_wide(T[k], 0)));
                         }
                         for (int o = 16; o > 0; o >>= 1) tm = fmax(tm, __shfl_xor_sync(0xffffffffu, tm, o));
                         if (lane == 0) s_tm[threadIdx.x >> 5] = tm;
@@ -1258,7 +1512,7 @@ jk_class_kernel(const JkClassArgs args)
                 if (stop) break;
             }
             if (DOJ && act) jk_flush_jab<FA, FB, NDM, R>(jab, mol, a0, b0, args.widen_int);
-            if (slab == 0) { cnt.nq += nq; cnt.nprim += nprim; cnt.nband += nband; }
+            if (slab == 0) { cnt.nq += part == 0 ? nq : 0; cnt.nprim += nprim; cnt.nband += nband; }
             if (threadIdx.x == 0) s_item = (long long)gridDim.x + (long long)atomicAdd(args.work, 1ull);
             __syncthreads();
             tt = s_item;
@@ -1307,7 +1561,7 @@ jk_schwarz_kernel(const JkSchwarzArgs args)
                 double T[S::EPT];
 #pragma unroll
                 for (int k = 0; k < S::EPT; ++k) T[k] = 0.0;
-                jk_quartet<LA, LB, LA, LB, GA, GB, GC, GD, double>(pr, pr, NPA * NPB, NPA * NPB, -1.0f, 0.0, 0, args.pp64, args.rys64, grp, gmask, tg, true, off, T);
+                jk_quartet<LA, LB, LA, LB, GA, GB, GC, GD, double>(pr, pr, 0, 1, NPA * NPB, NPA * NPB, -1.0f, 0.0, 0, args.pp64, args.rys64, grp, gmask, tg, true, off, T);
                 if (ga == gc && gb == gd) {
 #pragma unroll
                     for (int ia = 0; ia < FA; ++ia)
@@ -1343,7 +1597,7 @@ jk_schwarz_kernel(const JkSchwarzArgs args)
 #pragma unroll
             for (int k = 0; k < S::EPT; ++k) T[k] = 0.0;
             jk_quartet<LA, LB, LA, LB, GA, GB, GC, GD, double, 0, NTC>(
-                pr, pr, NPA * NPB, NPA * NPB, -1.0f, 0.0, 0, args.pp64, args.rys64, grp, 0u, tg, act, off, T);
+                pr, pr, 0, 1, NPA * NPB, NPA * NPB, -1.0f, 0.0, 0, args.pp64, args.rys64, grp, 0u, tg, act, off, T);
             double mx = 0.0;
             if (act && ga == gc && gb == gd) {
 #pragma unroll

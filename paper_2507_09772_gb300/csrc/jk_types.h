@@ -16,8 +16,7 @@ struct alignas(16) JkPair {
     int a_loc, b_loc;  // molecule-local shell indices (density-max table)
     double Q;          // Schwarz factor sqrt(max |(mu nu|mu nu)|)
     float ABxf, AByf, ABzf;  // A - B rounded to FP32 (the FP32 tier reads these, no conversion)
-    int pad0;
-    double pad1;
+    float ABxl, AByl, ABzl;  // what the rounding left (the split tier reads A - B as two floats)
     double ABx, ABy, ABz;  // A - B (horizontal recurrence)
     float Qf;              // Q rounded to FP32 (the FP32 screening path)
     float padf;
@@ -45,9 +44,18 @@ struct alignas(16) JkPrimPair32 {
     float inv2p, q, pad1, pad2;
 };
 
+// The same in two-float arithmetic (x = xh + xl, 48 bits): the split tier.
+struct alignas(16) JkPrimPairDf {
+    float Pxh, Pxl, Pyh, Pyl, Pzh, Pzl, ph, pl;
+    float PAxh, PAxl, PAyh, PAyl, PAzh, PAzl, Kh, Kl;
+    float i2ph, i2pl, q, pad;
+};
+
 // Per molecule of a handle.
 struct JkMol {
     const double *D;   // n_dm x nao x nao (Cartesian)
+    const float2 *D2;  // the same as two floats, read by the split tier (nullptr when it does not run)
+    double qmax2;      // largest Q squared
     const float *D32;  // the same rounded to FP32, read by the FP32 tier (nullptr when it does not run)
     double *J;         // half-matrix accumulator X, symmetrised after the build
     double *K;         // half-matrix accumulator Y
@@ -73,12 +81,14 @@ struct JkSub {
     int same_class;              // ket class == bra class: ket index >= bra index
     int nab, ncd;                // primitive pairs of a bra / ket pair
     int chunk;                   // kets per work item
+    int split;                   // work items that share a bra pair's primitive pairs
     int group;                   // launch it belongs to
     int launch;                  // class pair index: statistics, routed lists
-    int pad;
 };
 
-// A work item: the candidates [kb, ke) of the ket class for one bra pair.
+// A work item: the candidates [kb, ke) of the ket class for one bra pair, and
+// of the bra's primitive pairs number s, s + split, ... (J and K are linear in
+// them); sub = class pair + s * 65536.
 struct alignas(16) JkItem {
     int sub, bra, kb, ke;
 };
@@ -102,18 +112,25 @@ struct JkClassArgs {
     unsigned long long *work;    // work counter (zeroed before the launch)
     const JkPrimPair64 *pp64;
     const JkPrimPair32 *pp32;
+    const JkPrimPairDf *ppdf;
     const JkMol *mols;
     const double *dmax;          // block max |D| tables, all molecules
     const float *dmax32;         // the same rounded to FP32
     const double *dmax_mol;      // per molecule: max over its table
     const double *rys64;         // FP64 Rys tables
     const float *rys32;          // FP32 Rys tables
+    const float *rysdf;          // two-float Rys tables
     double prim_eps;             // skip primitive quartets with q_ij q_kl Dmax <= prim_eps
     double omega;                // |w| of the range-separated operator (OP 1, 2)
     unsigned long long *stats;   // per class pair (stride stat_stride): [0] quartets, [1] primitive quartets, [2] routed
     int stat_stride;
     int *err;                    // device error word
     double lo, hi;               // keep a quartet iff lo < Q_ab Q_cd Dmax <= hi
+    // the split threshold of a molecule, split x max Q^2 x max |D| and at least
+    // split_min, narrows that range: split_side 1 raises lo to it (the FP64
+    // tier), -1 lowers hi to it (the split tier), 0 leaves the range alone
+    double split, split_min;
+    int split_side;
     // FP32 screening (scr32 = 1, used when the build's cutoff is >= 1e-30 so
     // that no product of interest leaves the FP32 range): the same bounds and
     // the band in FP32; every tier of a build evaluates them identically

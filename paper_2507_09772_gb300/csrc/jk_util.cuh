@@ -3,6 +3,13 @@
 #pragma once
 #include "jk_types.h"
 
+// v as two floats, h + l.
+__device__ __forceinline__ void jk_two(double v, float &h, float &l)
+{
+    h = (float)v;
+    l = (float)(v - (double)h);
+}
+
 // Primitive-pair records of one shell pair per thread (Sec. 3, pair data
 // precomputed once per geometry; Table 2 lists the raw inputs).
 __global__ void jk_pairdata_kernel(int npair, const int *__restrict__ pa, const int *__restrict__ pb,
@@ -10,7 +17,7 @@ __global__ void jk_pairdata_kernel(int npair, const int *__restrict__ pa, const 
                                    const int *__restrict__ sh_nprim, const int *__restrict__ sh_prim,
                                    const double *__restrict__ coords, const double *__restrict__ exps,
                                    const double *__restrict__ coeffs, JkPrimPair64 *__restrict__ out64,
-                                   JkPrimPair32 *__restrict__ out32)
+                                   JkPrimPair32 *__restrict__ out32, JkPrimPairDf *__restrict__ outdf)
 {
     int t = blockIdx.x * blockDim.x + threadIdx.x;
     if (t >= npair) return;
@@ -44,6 +51,13 @@ __global__ void jk_pairdata_kernel(int npair, const int *__restrict__ pa, const 
             s.PAx = (float)r.PAx; s.PAy = (float)r.PAy; s.PAz = (float)r.PAz; s.K = (float)r.K;
             s.inv2p = (float)r.inv2p; s.q = 0.f; s.pad1 = s.pad2 = 0.f;
             out32[o] = s;
+            JkPrimPairDf d;
+            jk_two(r.Px, d.Pxh, d.Pxl); jk_two(r.Py, d.Pyh, d.Pyl); jk_two(r.Pz, d.Pzh, d.Pzl);
+            jk_two(r.p, d.ph, d.pl);
+            jk_two(r.PAx, d.PAxh, d.PAxl); jk_two(r.PAy, d.PAyh, d.PAyl); jk_two(r.PAz, d.PAzh, d.PAzl);
+            jk_two(r.K, d.Kh, d.Kl); jk_two(r.inv2p, d.i2ph, d.i2pl);
+            d.q = d.pad = 0.f;
+            outdf[o] = d;
         }
     }
 }
@@ -156,11 +170,13 @@ struct JkPlanTier {
     const long long *item_off;     // per launch group: where its items start
     unsigned long long *nitems;    // per launch group (zeroed before)
     double lo;
-    float lo32;
+    int split_side;                // 1: lo is raised to the molecule's split threshold
 };
 struct JkPlanArgs {
-    JkPlanTier tier[2];
+    JkPlanTier tier[3];
     const double *dmax_mol;
+    const JkMol *mols;
+    double split, split_min;
     int use_dmax, scr32;
     int part_index, part_count;
 };
@@ -177,7 +193,7 @@ struct JkPlanArgs {
 // class kernels decide each one exactly.
 __global__ void __launch_bounds__(256) jk_plan_kernel(const JkPlanArgs args)
 {
-    const JkPlanTier T = blockIdx.y == 0 ? args.tier[0] : args.tier[1];
+    const JkPlanTier T = blockIdx.y == 0 ? args.tier[0] : (blockIdx.y == 1 ? args.tier[1] : args.tier[2]);
     if ((int)blockIdx.x >= T.nblocks) return;
     const int2 blk = T.blocks[blockIdx.x];
     const JkSub &S = T.subs[blk.x];
@@ -189,8 +205,14 @@ __global__ void __launch_bounds__(256) jk_plan_kernel(const JkPlanArgs args)
         k0 = S.same_class ? i : S.ket_beg[m];
         int lo = k0, hi = S.ket_end[m];
         const double dm = args.use_dmax ? args.dmax_mol[m] : 1.0;
+        double tlo = T.lo;
+        if (T.split_side > 0) {   // as jk_bounds forms it
+            const double th =
+                dm < 1e15 ? fmax(args.split_min, __dmul_rn(__dmul_rn(args.split, args.mols[m].qmax2), dm)) : 0.0;
+            tlo = fmax(tlo, th);
+        }
         if (args.scr32) {
-            const float f = b.Qf * (float)dm, thr = T.lo32 * (1.0f - 4e-6f);
+            const float f = b.Qf * (float)dm, thr = (float)tlo * (1.0f - 4e-6f);
             while (lo < hi) {
                 const int mid = (lo + hi) >> 1;
                 if (f * S.ket[mid].Qf > thr) lo = mid + 1; else hi = mid;
@@ -198,7 +220,7 @@ __global__ void __launch_bounds__(256) jk_plan_kernel(const JkPlanArgs args)
         } else {
             while (lo < hi) {
                 const int mid = (lo + hi) >> 1;
-                if ((b.Q * S.ket[mid].Q) * dm > T.lo) lo = mid + 1; else hi = mid;
+                if ((b.Q * S.ket[mid].Q) * dm > tlo) lo = mid + 1; else hi = mid;
             }
         }
         n = lo - k0;
@@ -206,7 +228,7 @@ __global__ void __launch_bounds__(256) jk_plan_kernel(const JkPlanArgs args)
     const int c = S.chunk, nch = (n + c - 1) / c;
     // chunks of this part: c0, c0 + part_count, ...
     const int c0 = (args.part_index + args.part_count - (i + S.launch) % args.part_count) % args.part_count;
-    const int mine = nch > c0 ? (nch - c0 + args.part_count - 1) / args.part_count : 0;
+    const int mine = nch > c0 ? (nch - c0 + args.part_count - 1) / args.part_count * S.split : 0;
     int pre = mine;
 #pragma unroll
     for (int o = 1; o < 32; o <<= 1) {
@@ -219,9 +241,9 @@ __global__ void __launch_bounds__(256) jk_plan_kernel(const JkPlanArgs args)
     base = __shfl_sync(0xffffffffu, base, 31);
     JkItem *out = T.items + T.item_off[S.group] + base + (pre - mine);
     for (int k = 0; k < mine; ++k) {
-        const int kb = k0 + (c0 + k * args.part_count) * c;
+        const int kb = k0 + (c0 + k / S.split * args.part_count) * c;
         JkItem it;
-        it.sub = blk.x;
+        it.sub = blk.x + ((k % S.split) << 16);
         it.bra = i;
         it.kb = kb;
         it.ke = min(k0 + n, kb + c);
@@ -241,15 +263,23 @@ __global__ void jk_zero_kernel(const JkMol *__restrict__ mols, int ndm)
     }
 }
 
-// FP32 copy of every molecule's densities for the FP32 tier (one rounding
-// per element, as the tier would apply on every load).
+// Copies of every molecule's densities for the FP32 tier (one rounding per
+// element, as the tier would apply on every load) and the split tier (two
+// floats), where they run.
 __global__ void jk_d32_kernel(const JkMol *__restrict__ mols, int ndm)
 {
     const JkMol mol = mols[blockIdx.y];
     float *dst = const_cast<float *>(mol.D32);
+    float2 *dst2 = const_cast<float2 *>(mol.D2);
     const long long n = (long long)ndm * mol.nao * mol.nao;
     for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x)
-        dst[i] = (float)mol.D[i];
+    {
+        const double v = mol.D[i];
+        float2 t;
+        jk_two(v, t.x, t.y);
+        if (dst) dst[i] = t.x;
+        if (dst2) dst2[i] = t;
+    }
 }
 
 // Spherical <-> Cartesian transforms, one thread per (shell a, shell b)
@@ -329,8 +359,9 @@ __global__ void jk_sph_kernel(const JkSphMol *__restrict__ mols, const int *__re
 // primitive pairs reordered by q (largest first), one thread per shell pair.
 __global__ void jk_primsort_kernel(int npair, const int *__restrict__ pp_off, const int *__restrict__ pp_cnt,
                                    const double *__restrict__ qprim, const JkPrimPair64 *__restrict__ in64,
-                                   const JkPrimPair32 *__restrict__ in32, JkPrimPair64 *__restrict__ out64,
-                                   JkPrimPair32 *__restrict__ out32)
+                                   const JkPrimPair32 *__restrict__ in32, const JkPrimPairDf *__restrict__ indf,
+                                   JkPrimPair64 *__restrict__ out64, JkPrimPair32 *__restrict__ out32,
+                                   JkPrimPairDf *__restrict__ outdf)
 {
     const int t = blockIdx.x * blockDim.x + threadIdx.x;
     if (t >= npair) return;
@@ -350,5 +381,8 @@ __global__ void jk_primsort_kernel(int npair, const int *__restrict__ pp_off, co
         s.q = (float)qk;
         out64[o + rank] = r;
         out32[o + rank] = s;
+        JkPrimPairDf d = indf[o + k];
+        d.q = (float)qk;
+        outdf[o + rank] = d;
     }
 }

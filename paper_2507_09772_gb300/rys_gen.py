@@ -218,6 +218,8 @@ def write_sources(outdir: str) -> dict:
         f.write(f"static const int rys32_nint_host[{NMAX + 1}] = {{0,"
                 + ",".join(str(p['nint']) for p in p32) + "};\n")
         f.write(f"static const int rys32_deg_host = {p32[0]['deg']};\n")
+        f.write(f"static const int rys64_nint_host[{NMAX + 1}] = {{0,"
+                + ",".join(str(p['nint']) for p in p64) + "};\n")
         f.write(f"static const size_t rys_table32_size = {t32.size};\n")
         f.write("static const double rys_table32_src[] = {\n")
         for i in range(0, t32.size, 4):
@@ -246,6 +248,14 @@ def write_sources(outdir: str) -> dict:
         # compile-time interval counts of the FP32 tables (shared-memory sizing)
         f.write(f"constexpr int rys32_nint_c[{NMAX + 1}] = {{0,"
                 + ",".join(str(p['nint']) for p in p32) + "};\n")
+        f.write(f"constexpr int rys64_nint_c[{NMAX + 1}] = {{0,"
+                + ",".join(str(p['nint']) for p in p64) + "};\n")
+        # two-float tables: per interval 2 N functions x 16 floats and 4 floats of padding
+        offsdf, o = [], 0
+        for p in p64:
+            offsdf.append(o)
+            o += p["nint"] * (32 * p["N"] + 4)
+        f.write(f"constexpr int rysdf_offset[{NMAX + 1}] = {{0," + ",".join(str(x) for x in offsdf) + "};\n")
         # Gauss-Hermite limits, packed per N: x_r^2 then w_r
         offs, flat = [0], []
         for p in p64:
@@ -259,6 +269,12 @@ def write_sources(outdir: str) -> dict:
         # FP32 tier reads floats (no FP64 conversion on its path)
         f.write(f"__device__ __constant__ float rys_gh32[{len(flat)}] = {{"
                 + ",".join(_fmt(float(np.float32(v))) + "f" for v in flat) + "};\n")
+        # the same limits as two floats: (x_r^2 h, l, w_r h, l)
+        def two(v):
+            h = float(np.float32(v))
+            return f"{_fmt(h)}f,{_fmt(float(np.float32(v - h)))}f"
+        f.write(f"__device__ __constant__ float4 rys_ghdf[{len(flat) // 2}] = {{"
+                + ",".join("{" + two(x) + "," + two(w) + "}" for p in p64 for x, w in zip(p["x2"], p["wh"])) + "};\n")
         f.write(f"__device__ __constant__ float rys32_tmaxf[{NMAX + 1}] = {{0.0f,"
                 + ",".join(_fmt(float(np.float32(p['tmax']))) + "f" for p in p32) + "};\n")
     os.replace(os.path.join(outdir, "rys_params.cuh.tmp"), os.path.join(outdir, "rys_params.cuh"))

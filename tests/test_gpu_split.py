@@ -1,0 +1,97 @@
+"""GPU: the split tier (FP64-tier quartets below the split threshold evaluated
+in pairs of floats).
+
+Two floats carry 48 bits; the largest relative error of an integral is about
+2e-12 (the difference of two centres near 10 bohr, 2^-49 x 10, against the
+width of the tightest products, exponents up to 5,000), so with every quartet
+in two floats (split = 1) and |J|, |K| below 50 the result stays within 1e-10;
+at the default threshold, 1/8192 of the largest bound, within 1e-12 of the
+all-FP64 build.
+"""
+import numpy as np
+import pytest
+
+import oracle
+from paper_2507_09772_gb300 import jk, synth
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _gpu():
+    if not torch.cuda.is_available():
+        pytest.skip("needs a CUDA device")
+
+
+def build(mol, split, options=(), **kw):
+    eng = jk.JK(mol)
+    try:
+        eng.set_option("split", split)
+        for k, v in dict(options).items():
+            eng.set_option(k, v)
+        D = torch.tensor(mol.D, dtype=torch.float64, device="cuda")
+        J, K, st = eng.build(D, cutoff=1e-13, stats=True, **kw)
+        return [None if x is None else x.cpu().numpy() for x in (J, K)], st["quartets_fp64"]
+    finally:
+        eng.close()
+
+
+def one_l(l, seed):
+    """Two atoms with one shell type of angular momentum l and an s shell."""
+    rng = np.random.default_rng(seed)
+    xyz = np.array([[0.0, 0.1, -0.2], [1.1, -0.4, 0.7]])
+    return synth.custom_basis_molecule(xyz, [[(l, [2.3, 0.4][: 2 if l < 3 else 1]), (0, [30.0, 0.5])]] * 2, rng)
+
+
+CASES = {
+    "tiny": lambda: (synth.tiny_631gs(), {}, {}),
+    "two densities": lambda: (synth.random_small_molecule(5, natm=3, lmax=2, n_dm=2), {}, {}),
+    "j only": lambda: (synth.batched_molecule(4, natm=10), {}, {"with_k": False}),
+    "k only": lambda: (synth.batched_molecule(4, natm=10), {}, {"with_j": False}),
+    "erf": lambda: (synth.random_small_molecule(6, natm=3, lmax=2), {"omega": 0.4}, {}),
+    "erfc": lambda: (synth.random_small_molecule(6, natm=3, lmax=2), {"omega": -0.4}, {}),
+    "no dmax": lambda: (synth.random_small_molecule(8, natm=3, lmax=2), {"use_dmax": 0}, {}),
+    "spherical": lambda: (synth.random_small_molecule(9, natm=2, lmax=3, spherical=True), {}, {}),
+    "p": lambda: (one_l(1, 1), {}, {}), "d": lambda: (one_l(2, 2), {}, {}), "f": lambda: (one_l(3, 3), {}, {}),
+    "g": lambda: (one_l(4, 4), {}, {}),
+}
+
+
+@pytest.mark.parametrize("name", sorted(CASES))
+def test_two_float_quartets(name):
+    mol, options, kw = CASES[name]()
+    ref, n0 = build(mol, 0.0, options, **kw)
+    for split, tol in ((1.0, 1e-10), (1.0 / 8192, 1e-12)):
+        got, n = build(mol, split, options, **kw)
+        assert n == n0            # every quartet in exactly one of the tiers
+        for a, b in zip(got, ref):
+            if b is not None:
+                assert np.abs(a - b).max() <= tol * max(1.0, np.abs(b).max() / 50)
+
+
+def test_every_quartet_in_two_floats_against_the_oracle():
+    mol = synth.batched_molecule(2, natm=12)
+    (J, K), n = build(mol, 1.0)
+    Jr, Kr, nq = oracle.jk(mol, cutoff=1e-13)
+    assert n == nq
+    assert np.abs(J - Jr).max() <= 1e-10 and np.abs(K - Kr).max() <= 1e-10
+
+
+def test_scaled_density_keeps_the_relative_error():
+    """The threshold follows the density: a small change of it is built as
+    exactly, relative to its own size, as a whole density."""
+    mol = synth.tiny_631gs()
+    mol.D = mol.D * 2.0 ** -12
+    (J0, K0), _ = build(mol, 0.0)
+    (J1, K1), _ = build(mol, 1.0 / 8192)
+    assert np.abs(J1 - J0).max() <= 1e-12 * 2.0 ** -12 and np.abs(K1 - K0).max() <= 1e-12 * 2.0 ** -12
+
+
+def test_a_basis_outside_the_fp32_range_stays_in_fp64():
+    rng = np.random.default_rng(3)
+    mol = synth.custom_basis_molecule(np.array([[0.0, 0, 0], [1.2, 0, 0.3]]), [[(0, [3e8]), (0, [0.7]), (1, [1.1])]] * 2, rng)
+    (J0, K0), n0 = build(mol, 0.0)
+    (J1, K1), n1 = build(mol, 1.0)
+    assert n0 == n1
+    assert np.abs(J1 - J0).max() <= 1e-13 * np.abs(J0).max() and np.abs(K1 - K0).max() <= 1e-13 * np.abs(K0).max()
