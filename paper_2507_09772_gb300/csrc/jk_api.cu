@@ -105,7 +105,7 @@ Driver &drv()
 }
 
 static_assert(sizeof(JkPair) == 96 && sizeof(JkPrimPair64) == 96 && sizeof(JkPrimPair32) == 48 && sizeof(JkPrimPairDf) == 80 &&
-                  sizeof(JkPairFeat) == 32,
+                  sizeof(JkPairFeat) == 32 && sizeof(JkKetScr) == 16 && sizeof(JkRec) == 64,
               "record sizes are part of the device layout");
 
 // ------------------------------------------------------------ kernel spec
@@ -771,6 +771,8 @@ struct jk_handle {
     // device
     int *d_sh_mol = nullptr, *d_mol_sh0 = nullptr, *d_sh_ao = nullptr, *d_sh_nc = nullptr;
     JkPair *d_pairs = nullptr;
+    JkKetScr *d_scr = nullptr;             // aligned with d_pairs
+    JkRec *d_rec = nullptr;
     JkPrimPair64 *d_pp64 = nullptr;
     JkPrimPair32 *d_pp32 = nullptr;
     JkPrimPairDf *d_ppdf = nullptr;
@@ -868,7 +870,7 @@ void free_handle(jk_handle *h)
     for (auto &c : h->classes) { cudaFree(c.d_beg); cudaFree(c.d_end); }
     h->plans.clear();
     cudaFree(h->d_sh_mol); cudaFree(h->d_mol_sh0); cudaFree(h->d_sh_ao); cudaFree(h->d_sh_nc);
-    cudaFree(h->d_pairs); cudaFree(h->d_pp64); cudaFree(h->d_pp32); cudaFree(h->d_ppdf); cudaFree(h->d_rysdf); cudaFree(h->d_d2); cudaFree(h->d_mols);
+    cudaFree(h->d_pairs); cudaFree(h->d_scr); cudaFree(h->d_rec); cudaFree(h->d_pp64); cudaFree(h->d_pp32); cudaFree(h->d_ppdf); cudaFree(h->d_rysdf); cudaFree(h->d_d2); cudaFree(h->d_mols);
     cudaFree(h->d_dmax); cudaFree(h->d_dmax32); cudaFree(h->d_rys64); cudaFree(h->d_rys32);
     cudaFree(h->d_zero); cudaFree(h->d_err); cudaFree(h->d_tile_off);
     if (h->h_mols) cudaFreeHost(h->h_mols);
@@ -994,6 +996,8 @@ int tier_plan(jk_handle *h, int t, int hi, int merge, int whole, TierPlan **out)
                 memset(&S, 0, sizeof S);
                 S.bra = h->d_pairs + A.off;
                 S.ket = h->d_pairs + B.off;
+                S.ket_scr = h->d_scr + B.off;
+                S.ket_rec = h->d_rec + B.off;
                 S.ket_beg = B.d_beg;
                 S.ket_end = B.d_end;
                 S.bra_feat = h->d_pfeat + A.off;
@@ -1291,6 +1295,34 @@ int init_impl(int32_t nmol, const int32_t *mol_shell_off, const jk_shell *shells
     std::vector<double> q(ncand);
     CK(cudaMemcpy(q.data(), d_q, sizeof(double) * ncand, cudaMemcpyDeviceToHost));
 
+    // ---- prune, group by (class, molecule), sort by Q descending
+    std::vector<long long> order;
+    for (long long i = 0; i < ncand; ++i)
+        if (q[i] > h->pair_cutoff && std::isfinite(q[i])) order.push_back(i);
+    std::stable_sort(order.begin(), order.end(), [&](long long x, long long y) {
+        if (cand[x].cls != cand[y].cls) return cand[x].cls < cand[y].cls;
+        if (cp[x].mol != cp[y].mol) return cp[x].mol < cp[y].mol;
+        return q[x] > q[y];
+    });
+    h->h_pairs.resize(order.size());
+    // primitive pairs in the order of the sorted pairs
+    std::vector<int> new_off(ncand, -1);
+    int npp_kept = 0;
+    for (size_t k = 0; k < order.size(); ++k) {
+        h->h_pairs[k] = cp[order[k]];
+        new_off[order[k]] = h->h_pairs[k].pp_off = npp_kept;
+        npp_kept += shells[cp[order[k]].a].nprim * shells[cp[order[k]].b].nprim;
+        h->h_pairs[k].Q = q[order[k]];
+        h->h_pairs[k].Qf = (float)q[order[k]];
+    }
+    h->mol_qmax2.assign(nmol, 0.0);
+    for (auto &p : h->h_pairs) h->mol_qmax2[p.mol] = std::max(h->mol_qmax2[p.mol], p.Q * p.Q);
+    // two floats need every intermediate well inside the FP32 range
+    for (int i = 0; i < nprim_total; ++i) {
+        const double c = std::fabs(coeffs[i]);
+        h->df_ok = h->df_ok && exps[i] > 1e-6 && exps[i] < 1e8 && c < 1e8 && (c == 0 || c > 1e-8);
+    }
+    for (int i = 0; i < 3 * natm; ++i) h->df_ok = h->df_ok && std::fabs(coords[i]) < 1e5;
     // ---- primitive-pair Schwarz factors: the Schwarz kernel of each pair
     // class on single-primitive pseudo pairs (same centres, pp_off pointing
     // at one primitive pair), then every shell pair's primitive pairs sorted
@@ -1322,11 +1354,11 @@ int init_impl(int32_t nmol, const int32_t *mol_shell_off, const jk_shell *shells
         }
         JkPair *d_pseudo = nullptr;
         double *d_qp = nullptr;
-        int *d_cnt = nullptr;
+        int *d_cnt = nullptr, *d_new = nullptr;
         JkPrimPair64 *n64 = nullptr;
         JkPrimPair32 *n32 = nullptr;
         JkPrimPairDf *ndf = nullptr;
-        auto cl2 = [&]() { cudaFree(d_pseudo); cudaFree(d_qp); cudaFree(d_cnt); cudaFree(n64); cudaFree(n32); cudaFree(ndf); };
+        auto cl2 = [&]() { cudaFree(d_pseudo); cudaFree(d_qp); cudaFree(d_cnt); cudaFree(d_new); cudaFree(n64); cudaFree(n32); cudaFree(ndf); };
         struct G3 { std::function<void()> f; ~G3() { f(); } } g3{cl2};
         if ((rc = upload(&d_pseudo, pseudo))) return rc;
         CK(cudaMalloc(&d_qp, sizeof(double) * npp));
@@ -1353,11 +1385,12 @@ int init_impl(int32_t nmol, const int32_t *mol_shell_off, const jk_shell *shells
         }
         std::vector<int> cnt(ncand);
         for (long long i = 0; i < ncand; ++i) cnt[i] = shells[ca[i]].nprim * shells[cb[i]].nprim;
-        if ((rc = upload(&d_cnt, cnt))) return rc;
-        CK(cudaMalloc(&n64, sizeof(JkPrimPair64) * npp));
-        CK(cudaMalloc(&n32, sizeof(JkPrimPair32) * npp));
-        CK(cudaMalloc(&ndf, sizeof(JkPrimPairDf) * npp));
-        jk_primsort_kernel<<<(unsigned)((ncand + 127) / 128), 128>>>((int)ncand, d_cpp, d_cnt, d_qp, h->d_pp64,
+        if ((rc = upload(&d_cnt, cnt)) || (rc = upload(&d_new, new_off))) return rc;
+        const size_t nkeep = std::max(npp_kept, 1);
+        CK(cudaMalloc(&n64, sizeof(JkPrimPair64) * nkeep));
+        CK(cudaMalloc(&n32, sizeof(JkPrimPair32) * nkeep));
+        CK(cudaMalloc(&ndf, sizeof(JkPrimPairDf) * nkeep));
+        jk_primsort_kernel<<<(unsigned)((ncand + 127) / 128), 128>>>((int)ncand, d_cpp, d_cnt, d_new, d_qp, h->d_pp64,
                                                                       h->d_pp32, h->d_ppdf, n64, n32, ndf);
         CK(cudaGetLastError());
         CK(cudaDeviceSynchronize());
@@ -1366,29 +1399,6 @@ int init_impl(int32_t nmol, const int32_t *mol_shell_off, const jk_shell *shells
         std::swap(h->d_ppdf, ndf);
     }
 
-    // ---- prune, group by (class, molecule), sort by Q descending
-    std::vector<long long> order;
-    for (long long i = 0; i < ncand; ++i)
-        if (q[i] > h->pair_cutoff && std::isfinite(q[i])) order.push_back(i);
-    std::stable_sort(order.begin(), order.end(), [&](long long x, long long y) {
-        if (cand[x].cls != cand[y].cls) return cand[x].cls < cand[y].cls;
-        if (cp[x].mol != cp[y].mol) return cp[x].mol < cp[y].mol;
-        return q[x] > q[y];
-    });
-    h->h_pairs.resize(order.size());
-    for (size_t k = 0; k < order.size(); ++k) {
-        h->h_pairs[k] = cp[order[k]];
-        h->h_pairs[k].Q = q[order[k]];
-        h->h_pairs[k].Qf = (float)q[order[k]];
-    }
-    h->mol_qmax2.assign(nmol, 0.0);
-    for (auto &p : h->h_pairs) h->mol_qmax2[p.mol] = std::max(h->mol_qmax2[p.mol], p.Q * p.Q);
-    // two floats need every intermediate well inside the FP32 range
-    for (int i = 0; i < nprim_total; ++i) {
-        const double c = std::fabs(coeffs[i]);
-        h->df_ok = h->df_ok && exps[i] > 1e-6 && exps[i] < 1e8 && c < 1e8 && (c == 0 || c > 1e-8);
-    }
-    for (int i = 0; i < 3 * natm; ++i) h->df_ok = h->df_ok && std::fabs(coords[i]) < 1e5;
     size_t k0 = 0;
     while (k0 < order.size()) {
         size_t k1 = k0;
@@ -1411,7 +1421,16 @@ int init_impl(int32_t nmol, const int32_t *mol_shell_off, const jk_shell *shells
         h->classes.push_back(pc);
         k0 = k1;
     }
-    if ((rc = upload(&h->d_pairs, h->h_pairs))) return rc;
+    {
+        std::vector<JkKetScr> scr(h->h_pairs.size());
+        std::vector<JkRec> rec(h->h_pairs.size());
+        for (size_t k = 0; k < rec.size(); ++k) {
+            const JkPair &p = h->h_pairs[k];
+            scr[k] = JkKetScr{p.Qf, p.a_loc, p.b_loc, 0};
+            rec[k] = JkRec{p.pp_off, p.a_ao, p.b_ao, p.a == p.b, p.ABxf, p.AByf, p.ABzf, p.ABxl, p.AByl, p.ABzl, p.ABx, p.ABy, p.ABz};
+        }
+        if ((rc = upload(&h->d_pairs, h->h_pairs)) || (rc = upload(&h->d_scr, scr)) || (rc = upload(&h->d_rec, rec))) return rc;
+    }
     {
         // router features per pair: exponent-sum range, |A-B|, log10 Q, centre
         // of the most diffuse primitive pair, l_a + l_b

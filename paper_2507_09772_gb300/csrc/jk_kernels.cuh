@@ -144,17 +144,22 @@ template <> __device__ __forceinline__ JkPrim<jkdf> jk_prim<jkdf, JkPrimPairDf>(
 
 __device__ __forceinline__ double jk_rsqrt(double x) { return rsqrt(x); }
 
+__device__ __forceinline__ JkRec jk_rec(const JkPair &p)
+{
+    return {p.pp_off, p.a_ao, p.b_ao, p.a == p.b, p.ABxf, p.AByf, p.ABzf, p.ABxl, p.AByl, p.ABzl, p.ABx, p.ABy, p.ABz};
+}
+
 // A - B of a pair in the tier's precision (the FP32 copy is stored, so the
 // FP32 tier converts nothing on the FP64 pipe).
-__device__ __forceinline__ void jk_pair_ab(const JkPair &p, double &x, double &y, double &z)
+__device__ __forceinline__ void jk_pair_ab(const JkRec &p, double &x, double &y, double &z)
 {
     x = p.ABx; y = p.ABy; z = p.ABz;
 }
-__device__ __forceinline__ void jk_pair_ab(const JkPair &p, float &x, float &y, float &z)
+__device__ __forceinline__ void jk_pair_ab(const JkRec &p, float &x, float &y, float &z)
 {
     x = p.ABxf; y = p.AByf; z = p.ABzf;
 }
-__device__ __forceinline__ void jk_pair_ab(const JkPair &p, jkdf &x, jkdf &y, jkdf &z)
+__device__ __forceinline__ void jk_pair_ab(const JkRec &p, jkdf &x, jkdf &y, jkdf &z)
 {
     x = {p.ABxf, p.ABxl}; y = {p.AByf, p.AByl}; z = {p.ABzf, p.ABzl};
 }
@@ -510,7 +515,7 @@ __device__ __forceinline__ void jk_op_root(R Tt, R rho, R pref, double omega, in
 
 template <int LA, int LB, int LC, int LD, int GA, int GB, int GC, int GD, typename R, int OP = 0,
           int NT = JkShape<LA, LB, LC, LD, GA, GB, GC, GD, OP>::G>
-__device__ __forceinline__ int jk_quartet(const JkPair &bra, const JkPair &ket, int ab0, int dab, int nab, int ncd, float qthr, double omega, int a64,
+__device__ __forceinline__ int jk_quartet(const JkRec &bra, const JkRec &ket, int ab0, int dab, int nab, int ncd, float qthr, double omega, int a64,
                                            const typename JkPP<R>::T *__restrict__ pp,
                                            const typename JkTab<R>::T *__restrict__ rys, R *grp, unsigned gmask,
                                            int tg, bool act,
@@ -725,7 +730,7 @@ __device__ __forceinline__ JkBounds jk_bounds(const JkClassArgs &args, const JkM
 }
 template <int MODE>
 __device__ __forceinline__ void jk_screen_bound(const JkClassArgs &args, const JkBounds &bd,
-                                                const JkPair *__restrict__ kets, const JkPair &bra, const JkMol &mol,
+                                                const JkSub &sub, const JkPair &bra, const JkMol &mol,
                                                 const double *dmx, double dmol, float dmol32, int j, int ke,
                                                 bool &sig, bool &stop, bool &band, float &dmq, float &Bout);
 // Keep (bra, ket j) iff lo < Q_ab Q_cd Dmax <= hi; `stop` when even the
@@ -742,7 +747,7 @@ __device__ __forceinline__ void jk_screen(const JkClassArgs &args, const JkBound
     band = false;
     dmq = 1.0f;
     float B = 0.0f;
-    jk_screen_bound<MODE>(args, bd, sub.ket, bra, mol, dmx, dmol, dmol32, j, ke, sig, stop, band, dmq, B);
+    jk_screen_bound<MODE>(args, bd, sub, bra, mol, dmx, dmol, dmol32, j, ke, sig, stop, band, dmq, B);
     if (MODE == 1) {
         // learned router for the band candidates, all lanes together on the
         // tensor cores; `band` then marks the quartets released to FP32
@@ -768,26 +773,26 @@ __device__ __forceinline__ bool jk_near(float x, float y)
 
 template <int MODE>
 __device__ __forceinline__ void jk_screen_bound(const JkClassArgs &args, const JkBounds &bd,
-                                                const JkPair *__restrict__ kets, const JkPair &bra, const JkMol &mol,
+                                                const JkSub &sub, const JkPair &bra, const JkMol &mol,
                                                 const double *dmx, double dmol, float dmol32, int j, int ke,
                                                 bool &sig, bool &stop, bool &band, float &dmq, float &Bout)
 {
     if (j >= ke) return;
-    const JkPair &kt = kets[j];
     if (args.scr32) {
+        const JkKetScr ks = sub.ket_scr[j];
         // FP32 bounds: a handful of FP32 operations per candidate instead of
         // FP64-pipe work (an FP64 instruction costs the FP32 tier 64 FP32
         // ones on GB300). scr32 == 2 keeps the FP64 rule exact: the FP32
         // products carry at most 5 roundings, so only a bound within 2e-6 of
         // a threshold can compare differently from its FP64 value, and those
         // few are redone in FP64 (every tier decides alike, as in FP64).
-        const float bq = bra.Qf * __ldg(&kt.Qf);
+        const float bq = bra.Qf * ks.Qf;
         const float s = bq * dmol32;
         bool st = s <= bd.lo32;
-        if (args.scr32 == 2 && jk_near(s, bd.lo32)) st = (bra.Q * kt.Q) * dmol <= bd.lo;
+        if (args.scr32 == 2 && jk_near(s, bd.lo32)) st = (bra.Q * sub.ket[j].Q) * dmol <= bd.lo;
         if (st) { stop = true; return; }
         float dm = 1.0f;
-        const int c = __ldg(&kt.a_loc), d = __ldg(&kt.b_loc);
+        const int c = ks.a_loc, d = ks.b_loc;
         const int a = bra.a_loc, b = bra.b_loc, ns = mol.nsh;
         if (args.use_dmax) {
             const float *d32 = args.dmax32 + mol.dmax_off;
@@ -816,12 +821,13 @@ __device__ __forceinline__ void jk_screen_bound(const JkClassArgs &args, const J
                     dm64 = fmax(dm64, fmax(__ldg(dmx + b * ns + c), __ldg(dmx + b * ns + d)));
                 }
             }
-            const double B64 = (bra.Q * kt.Q) * dm64;
+            const double B64 = (bra.Q * sub.ket[j].Q) * dm64;
             sig = (B64 > bd.lo) && (B64 <= bd.hi);
             band = MODE == 1 && sig && B64 > args.tau && B64 <= args.band_hi;
         }
         return;
     }
+    const JkPair &kt = sub.ket[j];
     const double bq = bra.Q * kt.Q;
     if (bq * dmol <= bd.lo) { stop = true; return; }
     double dm = 1.0;
@@ -899,6 +905,18 @@ __device__ __forceinline__ void jk_red_add(double *p, double v)
     asm volatile("red.relaxed.gpu.global.add.f64 [%0], %1;" ::"l"(__cvta_generic_to_global(p)), "d"(v) : "memory");
 }
 
+// Adds the block v[F1][F2] times f to rows r0.., columns q0.. of the half matrix M.
+template <int F1, int F2, typename R>
+__device__ __forceinline__ void jk_store_block(double *__restrict__ M, int nao, int r0, int q0, const R (&v)[F1][F2],
+                                               float f, int wi)
+{
+#pragma unroll
+    for (int i = 0; i < F1; ++i)
+#pragma unroll
+        for (int j = 0; j < F2; ++j)
+            jk_red_add(M + (long long)(r0 + i) * nao + q0 + j, jk_wide(jk_scale(v[i][j], f), wi));
+}
+
 template <int FA, int FB, int FC, int FD, int NDM, int DOJ, int DOK, typename R>
 __device__ __forceinline__ void jk_contract(const R (&T)[FA * FB * FC * FD], float f, const JkMol &mol,
                                             int a0, int b0, int c0, int d0, R (&jab)[NDM][FA][FB], int wi)
@@ -940,11 +958,7 @@ __device__ __forceinline__ void jk_contract(const R (&T)[FA * FB * FC * FD], flo
                     jk_addto(jab[m][ia][ib], jk_scale(sum, 2.0f * f));
                     jab[m][ia][ib] = jk_norm(jab[m][ia][ib]);
                 }
-#pragma unroll
-            for (int ic = 0; ic < FC; ++ic)
-#pragma unroll
-                for (int id = 0; id < FD; ++id)
-                    jk_red_add(mol.J + m * nn + (long long)(c0 + ic) * nao + d0 + id, jk_wide(jk_scale(jcd[ic][id], 2.0f * f), wi));
+            jk_store_block<FC, FD>(mol.J + m * nn, nao, c0, d0, jcd, 2.0f * f, wi);
         }
         if (DOK) {
             R Dbd[FB][FD], Dbc[FB][FC], Dad[FA][FD], Dac[FA][FC];
@@ -992,24 +1006,10 @@ __device__ __forceinline__ void jk_contract(const R (&T)[FA * FB * FC * FD], flo
                             jk_acc(kbd[ib][id], t, Dac[ia][ic]);
                         }
             double *K = mol.K + m * nn;
-#pragma unroll
-            for (int ia = 0; ia < FA; ++ia) {
-#pragma unroll
-                for (int ic = 0; ic < FC; ++ic)
-                    jk_red_add(K + (long long)(a0 + ia) * nao + c0 + ic, jk_wide(jk_scale(kac[ia][ic], f), wi));
-#pragma unroll
-                for (int id = 0; id < FD; ++id)
-                    jk_red_add(K + (long long)(a0 + ia) * nao + d0 + id, jk_wide(jk_scale(kad[ia][id], f), wi));
-            }
-#pragma unroll
-            for (int ib = 0; ib < FB; ++ib) {
-#pragma unroll
-                for (int ic = 0; ic < FC; ++ic)
-                    jk_red_add(K + (long long)(b0 + ib) * nao + c0 + ic, jk_wide(jk_scale(kbc[ib][ic], f), wi));
-#pragma unroll
-                for (int id = 0; id < FD; ++id)
-                    jk_red_add(K + (long long)(b0 + ib) * nao + d0 + id, jk_wide(jk_scale(kbd[ib][id], f), wi));
-            }
+            jk_store_block<FA, FC>(K, nao, a0, c0, kac, f, wi);
+            jk_store_block<FA, FD>(K, nao, a0, d0, kad, f, wi);
+            jk_store_block<FB, FC>(K, nao, b0, c0, kbc, f, wi);
+            jk_store_block<FB, FD>(K, nao, b0, d0, kbd, f, wi);
         }
     }
 }
@@ -1149,17 +1149,17 @@ jk_class_kernel(const JkClassArgs args)
                     if (active && e < n) {
                         const JkRouted rq = list[e];
                         const JkPair bra = sub.bra[rq.item];
-                        const JkPair ket = sub.ket[rq.ket];
+                        const JkRec ket = jk_rec(sub.ket[rq.ket]);
                         const JkMol mol = args.mols[bra.mol];
                         R T[S::EPT];
 #pragma unroll
                         for (int k = 0; k < S::EPT; ++k) T[k] = JkConst<R>::get(0.0);
                         const int np = jk_quartet<LA, LB, LC, LD, GA, GB, GC, GD, R, OP>(
-                            bra, ket, 0, 1, sub.nab, sub.ncd, __fdiv_rn(args.prim_eps32, rq.dmq), args.omega, args.asym64,
+                            jk_rec(bra), ket, 0, 1, sub.nab, sub.ncd, __fdiv_rn(args.prim_eps32, rq.dmq), args.omega, args.asym64,
                             pp, rys, grp, gmask, tg, true, off, T);
                         float f = 1.0f;
                         if (bra.a == bra.b) f *= 0.5f;
-                        if (ket.a == ket.b) f *= 0.5f;
+                        if (ket.same) f *= 0.5f;
                         if (sub.same_class && rq.ket == rq.item) f *= 0.5f;
                         R jab[NDM][FA][FB];
 #pragma unroll
@@ -1195,7 +1195,7 @@ jk_class_kernel(const JkClassArgs args)
             const JkItem wi = args.items[t];
             const JkSub &sub = args.subs[wi.sub & 0xffff];
             const int part = wi.sub >> 16, parts = sub.split;   // share of the bra's primitive pairs
-            const JkPair *__restrict__ kets = sub.ket;
+            const JkRec *__restrict__ kets = sub.ket_rec;
             const int item = wi.bra, nab = sub.nab, ncd = sub.ncd, same_class = sub.same_class;
             const int kb = wi.kb, ke = wi.ke;
             if (sub.launch != cur) {
@@ -1203,6 +1203,7 @@ jk_class_kernel(const JkClassArgs args)
                 cur = sub.launch;
             }
             const JkPair bra = sub.bra[item];
+            const JkRec brec = jk_rec(bra);
             const JkMol mol = args.mols[bra.mol];
             const double *dmx = args.dmax + mol.dmax_off;
             const double dmol = args.use_dmax ? args.dmax_mol[bra.mol] : 1.0;
@@ -1229,7 +1230,7 @@ jk_class_kernel(const JkClassArgs args)
             for (int base = kb; base < ke; base += 32) {
                 bool sig = false, stop = false, band = false;
                 float dmq = 1.0f, B = 0.0f;
-                jk_screen_bound<MODE>(args, bd, kets, bra, mol, dmx, dmol, dmol32, base + lane, ke, sig, stop, band, dmq, B);
+                jk_screen_bound<MODE>(args, bd, sub, bra, mol, dmx, dmol, dmol32, base + lane, ke, sig, stop, band, dmq, B);
                 const unsigned lt = (1u << lane) - 1u;
                 const bool def = sig && !band;   // decided by the bounds alone
                 const unsigned mdef = __ballot_sync(0xffffffffu, def);
@@ -1291,35 +1292,30 @@ jk_class_kernel(const JkClassArgs args)
                     }
                     if (!full_round && !tail_round) break;
                     const int take = qn < NGW ? qn : NGW;
-                    int myket = -1;
-                    float dmk = 1.0f;
                     if (active && gw < take) {
-                        myket = s_qk[wib][gw];
-                        dmk = s_qd[wib][gw];
-                    }
-                    if (myket >= 0) {
-                        const JkPair ket = kets[myket];
+                        const int myket = s_qk[wib][gw];
+                        const JkRec ket = kets[myket];
                         R T[S::EPT];
 #pragma unroll
                         for (int k = 0; k < S::EPT; ++k) T[k] = JkConst<R>::get(0.0);
                         const int np = jk_quartet<LA, LB, LC, LD, GA, GB, GC, GD, R, OP>(
-                            bra, ket, part, parts, nab, ncd, __fdiv_rn(args.prim_eps32, dmk), args.omega, args.asym64, pp, rys, grp,
-                            gmask, tg, true, off, T);
+                            brec, ket, part, parts, nab, ncd, __fdiv_rn(args.prim_eps32, s_qd[wib][gw]), args.omega,
+                            args.asym64, pp, rys, grp, gmask, tg, true, off, T);
                         if (tg == 0) nprim += np;
                         float f = 1.0f;
-                        if (bra.a == bra.b) f *= 0.5f;
-                        if (ket.a == ket.b) f *= 0.5f;
+                        if (brec.same) f *= 0.5f;
+                        if (ket.same) f *= 0.5f;
                         if (same_class && myket == item) f *= 0.5f;
                         jk_contract<FA, FB, FC, FD, NDM, DOJ, DOK, R>(T, f, mol, a0, b0, ket.a_ao + gc * FC,
-                                                                     ket.b_ao + gd * FD, jab, args.widen_int);
+                                                                          ket.b_ao + gd * FD, jab, args.widen_int);
                         if (MODE == 2) {
                             double tm = 0.0;
 #pragma unroll
                             for (int k = 0; k < S::EPT; ++k) tm = fmax(tm, fabs(jk_wide(T[k], 0)));
                             for (int q = 0; q < G; ++q) tm = fmax(tm, __shfl_sync(gmask, tm, (gw * G + q) & 31));
                             if (tg == 0)
-                                jk_log_sample(args, bra, ket, braf, sub.ket_feat[myket],
-                                              jk_quartet_dmax(args, bra, ket, mol, dmx), tm);
+                                jk_log_sample(args, bra, sub.ket[myket], braf, sub.ket_feat[myket],
+                                              jk_quartet_dmax(args, bra, sub.ket[myket], mol, dmx), tm);
                         }
                     }
                     // drop the round's entries (at most 31 remain)
@@ -1381,18 +1377,18 @@ jk_class_kernel(const JkClassArgs args)
                     }
                     const JkRouted rq = list[e];
                     const JkPair bra = sub.bra[rq.item];
-                    const JkPair ket = sub.ket[rq.ket];
+                    const JkRec ket = jk_rec(sub.ket[rq.ket]);
                     const JkMol mol = args.mols[bra.mol];
                     R T[S::EPT];
 #pragma unroll
                     for (int k = 0; k < S::EPT; ++k) T[k] = JkConst<R>::get(0.0);
                     const int np = jk_quartet<LA, LB, LC, LD, GA, GB, GC, GD, R, OP, NTC>(
-                        bra, ket, 0, 1, sub.nab, sub.ncd, __fdiv_rn(args.prim_eps32, rq.dmq), args.omega, args.asym64, pp,
+                        jk_rec(bra), ket, 0, 1, sub.nab, sub.ncd, __fdiv_rn(args.prim_eps32, rq.dmq), args.omega, args.asym64, pp,
                         rys, grp, 0u, tg, act, off, T);
                     if (act) {
                         float f = 1.0f;
                         if (bra.a == bra.b) f *= 0.5f;
-                        if (ket.a == ket.b) f *= 0.5f;
+                        if (ket.same) f *= 0.5f;
                         if (sub.same_class && rq.ket == rq.item) f *= 0.5f;
                         R jab[NDM][FA][FB];
 #pragma unroll
@@ -1435,6 +1431,7 @@ jk_class_kernel(const JkClassArgs args)
                 cur = sub.launch;
             }
             const JkPair bra = sub.bra[item];
+            const JkRec brec = jk_rec(bra);
             const JkMol mol = args.mols[bra.mol];
             const double *dmx = args.dmax + mol.dmax_off;
             const double dmol = args.use_dmax ? args.dmax_mol[bra.mol] : 1.0;
@@ -1471,18 +1468,18 @@ jk_class_kernel(const JkClassArgs args)
                 while (mask) {
                     const int myket = base + __ffs(mask) - 1;
                     mask &= mask - 1;
-                    const JkPair ket = sub.ket[myket];
+                    const JkRec ket = sub.ket_rec[myket];
                     R T[S::EPT];
 #pragma unroll
                     for (int k = 0; k < S::EPT; ++k) T[k] = JkConst<R>::get(0.0);
                     const int np = jk_quartet<LA, LB, LC, LD, GA, GB, GC, GD, R, OP, NTC>(
-                        bra, ket, part, parts, nab, ncd, __fdiv_rn(args.prim_eps32, s_dm[myket - base]), args.omega, args.asym64, pp,
+                        brec, ket, part, parts, nab, ncd, __fdiv_rn(args.prim_eps32, s_dm[myket - base]), args.omega, args.asym64, pp,
                         rys, grp, 0u, tg, act, off, T);
                     nprim += np;
                     if (act) {
                         float f = 1.0f;
                         if (bra.a == bra.b) f *= 0.5f;
-                        if (ket.a == ket.b) f *= 0.5f;
+                        if (ket.same) f *= 0.5f;
                         if (same_class && myket == item) f *= 0.5f;
                         jk_contract<FA, FB, FC, FD, NDM, DOJ, DOK, R>(T, f, mol, a0, b0, ket.a_ao + gc * FC,
                                                                      ket.b_ao + gd * FD, jab, args.widen_int);
@@ -1499,8 +1496,8 @@ jk_class_kernel(const JkClassArgs args)
                         __syncthreads();
                         if (threadIdx.x == 0) {
                             for (int w = 1; w < (int)(blockDim.x >> 5); ++w) tm = fmax(tm, s_tm[w]);
-                            jk_log_sample(args, bra, ket, braf, sub.ket_feat[myket],
-                                          jk_quartet_dmax(args, bra, ket, mol, dmx), tm);
+                            jk_log_sample(args, bra, sub.ket[myket], braf, sub.ket_feat[myket],
+                                          jk_quartet_dmax(args, bra, sub.ket[myket], mol, dmx), tm);
                         }
                         __syncthreads();
                     }
@@ -1557,7 +1554,7 @@ jk_schwarz_kernel(const JkSchwarzArgs args)
             const bool mine = active && pi < args.npair;
             double mx = 0.0;
             if (mine) {
-                const JkPair pr = args.pairs[pi];
+                const JkRec pr = jk_rec(args.pairs[pi]);
                 double T[S::EPT];
 #pragma unroll
                 for (int k = 0; k < S::EPT; ++k) T[k] = 0.0;
@@ -1592,7 +1589,7 @@ jk_schwarz_kernel(const JkSchwarzArgs args)
                 gd = tgl % GD; gc = (tgl / GD) % GC; gb = (tgl / (GD * GC)) % GB; ga = tgl / (GD * GC * GB);
                 jk_make_offsets<LA, LB, LA, LB, GA, GB, GC, GD, S>(ga, gb, gc, gd, off);
             }
-            const JkPair pr = args.pairs[pi];
+            const JkRec pr = jk_rec(args.pairs[pi]);
             double T[S::EPT];
 #pragma unroll
             for (int k = 0; k < S::EPT; ++k) T[k] = 0.0;

@@ -22,6 +22,22 @@ struct alignas(16) JkPair {
     float padf;
 };
 
+// What a kernel reads of every candidate ket: one 16-byte vector for the
+// screening (32 candidates in a row are four lines; the JkPair records would be
+// 24), and a 64-byte record for a quartet, of which the FP32 tier touches the
+// first half and the split tier three quarters. Arrays aligned with the pairs.
+struct alignas(16) JkKetScr {
+    float Qf;
+    int a_loc, b_loc;
+    int pad;
+};
+struct alignas(16) JkRec {
+    int pp_off, a_ao, b_ao;
+    int same;                // a == b
+    float ABxf, AByf, ABzf, ABxl, AByl, ABzl;
+    double ABx, ABy, ABz;
+};
+
 // Per primitive pair (alpha_i on a, beta_j on b), p = alpha + beta:
 //   P    = (alpha A + beta B) / p
 //   PA   = P - A
@@ -73,6 +89,8 @@ struct JkPairFeat;
 struct JkSub {
     const JkPair *bra;           // pairs of the bra class
     const JkPair *ket;           // pairs of the ket class
+    const JkKetScr *ket_scr;     // aligned with ket
+    const JkRec *ket_rec;
     const int *ket_beg;          // per molecule: first ket index in the ket class
     const int *ket_end;          // per molecule: one past the last
     const JkPairFeat *bra_feat;  // aligned with bra / ket

@@ -212,10 +212,11 @@ __global__ void __launch_bounds__(256) jk_plan_kernel(const JkPlanArgs args)
             tlo = fmax(tlo, th);
         }
         if (args.scr32) {
+            const JkKetScr *ks = S.ket_scr;
             const float f = b.Qf * (float)dm, thr = (float)tlo * (1.0f - 4e-6f);
             while (lo < hi) {
                 const int mid = (lo + hi) >> 1;
-                if (f * S.ket[mid].Qf > thr) lo = mid + 1; else hi = mid;
+                if (f * ks[mid].Qf > thr) lo = mid + 1; else hi = mid;
             }
         } else {
             while (lo < hi) {
@@ -356,8 +357,11 @@ __global__ void jk_sph_kernel(const JkSphMol *__restrict__ mols, const int *__re
 }
 
 // Primitive Schwarz factors into the pair records, then each shell pair's
-// primitive pairs reordered by q (largest first), one thread per shell pair.
+// primitive pairs reordered by q (largest first), one thread per shell pair,
+// into the order of the sorted pairs (new_off; -1: a dropped pair): the lanes
+// of a round hold neighbouring kets, whose records then share lines.
 __global__ void jk_primsort_kernel(int npair, const int *__restrict__ pp_off, const int *__restrict__ pp_cnt,
+                                   const int *__restrict__ new_off,
                                    const double *__restrict__ qprim, const JkPrimPair64 *__restrict__ in64,
                                    const JkPrimPair32 *__restrict__ in32, const JkPrimPairDf *__restrict__ indf,
                                    JkPrimPair64 *__restrict__ out64, JkPrimPair32 *__restrict__ out32,
@@ -365,7 +369,8 @@ __global__ void jk_primsort_kernel(int npair, const int *__restrict__ pp_off, co
 {
     const int t = blockIdx.x * blockDim.x + threadIdx.x;
     if (t >= npair) return;
-    const int o = pp_off[t], n = pp_cnt[t];
+    const int o = pp_off[t], n = pp_cnt[t], w = new_off[t];
+    if (w < 0) return;
     for (int k = 0; k < n; ++k) {
         // rank of record k: how many records precede it (q descending, ties by index)
         const double qk = qprim[o + k];
@@ -379,10 +384,10 @@ __global__ void jk_primsort_kernel(int npair, const int *__restrict__ pp_off, co
         r.q = qk;
         r.qf = (float)qk;
         s.q = (float)qk;
-        out64[o + rank] = r;
-        out32[o + rank] = s;
+        out64[w + rank] = r;
+        out32[w + rank] = s;
         JkPrimPairDf d = indf[o + k];
         d.q = (float)qk;
-        outdf[o + rank] = d;
+        outdf[w + rank] = d;
     }
 }
