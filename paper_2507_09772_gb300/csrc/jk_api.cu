@@ -2102,24 +2102,22 @@ int check_blob(const jk_router_blob *w)
 }  // namespace
 
 // ============================================= no-allocation gradient variant
-// Fixed device scratch for jk_router_gradient_noalloc: the weight copies, the
-// row list and the two accumulators of jk_mlp_grad_kernel live in one
-// file-scope __device__ array (about 560 KB, held by every GPU that loads this
-// library until the process exits) instead of buffers from cudaMalloc.
-struct JkNoAllocScratch {   // JK_NOALLOC_MAX_ROWS comes from jk.h
-    float theta[JK_RT_NPARAM];
+// Fixed device scratch for jk_router_gradient_noalloc: the weight copies and the
+// two accumulators of jk_mlp_grad_kernel live in one file-scope __device__ array
+// (43 KB, held by every GPU that loads this library until the process exits)
+// instead of buffers from cudaMalloc.
+struct JkGradBuffers {   // mu, isd, theta as in jk_router_blob
     float mu[16], isd[16];
-    float grad[JK_RT_NPARAM];
+    float theta[JK_RT_NPARAM];
+    float pad;
     double loss;
-    long long idx[JK_NOALLOC_MAX_ROWS];
+    float grad[JK_RT_NPARAM];
 };
+static_assert(offsetof(jk_router_blob, theta) - offsetof(jk_router_blob, mu) == 32 * sizeof(float) &&
+                  offsetof(jk_router_blob, isd) - offsetof(jk_router_blob, mu) == 16 * sizeof(float),
+              "one copy takes the parameters");
+typedef JkGradBuffers JkNoAllocScratch;
 static __device__ __align__(256) unsigned char jk_noalloc_scratch[sizeof(JkNoAllocScratch)];
-
-__global__ void jk_noalloc_iota_kernel(long long *idx, long long n)
-{
-    const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (t < n) idx[t] = t;
-}
 
 namespace {
 std::mutex g_noalloc_mu;
@@ -2143,6 +2141,25 @@ int noalloc_scratch(JkNoAllocScratch **out)
         g_noalloc_ptr[dev] = p;
     }
     *out = (JkNoAllocScratch *)g_noalloc_ptr[dev];
+    return JK_OK;
+}
+
+// Gradient over rows 0 .. n-1 with the parameters in B; queued on st, the
+// results copied back, st synchronised.
+int grad_rows(JkGradBuffers *B, const jk_router_blob *w, const float *X, const float *y, int64_t n, float quantile,
+              float *grad_host, double *loss, cudaStream_t st)
+{
+    int dev = 0, sms = 0;
+    CK(cudaGetDevice(&dev));
+    CK(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
+    CK(cudaMemcpyAsync(B->mu, w->mu, sizeof(float) * (32 + JK_RT_NPARAM), cudaMemcpyHostToDevice, st));
+    CK(cudaMemsetAsync(&B->loss, 0, sizeof(double) + sizeof(float) * JK_RT_NPARAM, st));
+    CK(jk_mlp_grad(B->theta, B->mu, B->isd, X, y, (long long)n, (int)n, JK_GRAD_ROWS, quantile, B->grad, &B->loss, sms, st));
+    struct { double loss; float grad[JK_RT_NPARAM]; } out;
+    CK(cudaMemcpyAsync(&out, &B->loss, sizeof(double) + sizeof(float) * JK_RT_NPARAM, cudaMemcpyDeviceToHost, st));
+    CK(cudaStreamSynchronize(st));
+    *loss = out.loss;
+    memcpy(grad_host, out.grad, sizeof(float) * JK_RT_NPARAM);
     return JK_OK;
 }
 }  // namespace
@@ -2286,25 +2303,8 @@ int jk_router_gradient_noalloc(const jk_router_blob *w, const float *X, const fl
                     (long long)n, JK_NOALLOC_MAX_ROWS);
     JkNoAllocScratch *S = nullptr;
     if ((rc = noalloc_scratch(&S))) return rc;
-    cudaStream_t st = (cudaStream_t)stream;
-    CK(cudaMemcpyAsync(S->theta, w->theta, sizeof(float) * JK_RT_NPARAM, cudaMemcpyHostToDevice, st));
-    CK(cudaMemcpyAsync(S->mu, w->mu, sizeof(float) * 16, cudaMemcpyHostToDevice, st));
-    CK(cudaMemcpyAsync(S->isd, w->isd, sizeof(float) * 16, cudaMemcpyHostToDevice, st));
-    // the accumulators keep the previous call's values: clear them
-    CK(cudaMemsetAsync(S->grad, 0, sizeof(float) * JK_RT_NPARAM, st));
-    CK(cudaMemsetAsync(&S->loss, 0, sizeof(double), st));
-    jk_noalloc_iota_kernel<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(S->idx, (long long)n);
-    const size_t smem = 2 * JK_RT_NPARAM * sizeof(float);
-    jk_mlp_grad_kernel<<<(unsigned)((n + 255) / 256), 256, smem, st>>>(S->theta, S->mu, S->isd, X, y, (long long)n,
-                                                                       S->idx, (int)n, 0ull, quantile, S->grad,
-                                                                       &S->loss);
-    CK(cudaGetLastError());
-    CK(cudaMemcpyAsync(grad_host, S->grad, sizeof(float) * JK_RT_NPARAM, cudaMemcpyDeviceToHost, st));
-    CK(cudaMemcpyAsync(loss, &S->loss, sizeof(double), cudaMemcpyDeviceToHost, st));
-    CK(cudaStreamSynchronize(st));
-    return JK_OK;
+    return grad_rows(S, w, X, y, n, quantile, grad_host, loss, (cudaStream_t)stream);
 }
-
 
 int jk_init(const jk_shell *shells, int32_t nshell, const double *coords, int32_t natm, const double *exps,
             const double *coeffs, int32_t nprim_total, jk_handle **out)
@@ -2553,33 +2553,10 @@ int jk_router_gradient(const jk_router_blob *w, const float *X, const float *y, 
     if (rc) return rc;
     if (!X || !y || !grad_host || !loss || n < 1 || n > (1 << 30) || !(quantile > 0 && quantile < 1))
         return fail(JK_ERR_ARG, "bad arguments");
-    float *th = nullptr, *mu = nullptr, *isd = nullptr, *g = nullptr;
-    double *l = nullptr;
-    long long *idx = nullptr;
-    std::vector<long long> iota((size_t)n);
-    for (int64_t i = 0; i < n; ++i) iota[i] = i;
-    auto cleanup = [&]() { cudaFree(th); cudaFree(mu); cudaFree(isd); cudaFree(g); cudaFree(l); cudaFree(idx); };
-    struct Guard { std::function<void()> f; ~Guard() { f(); } } guard{cleanup};
-    CK(cudaMalloc(&th, sizeof(float) * JK_RT_NPARAM));
-    CK(cudaMalloc(&mu, sizeof(float) * 16));
-    CK(cudaMalloc(&isd, sizeof(float) * 16));
-    CK(cudaMalloc(&g, sizeof(float) * JK_RT_NPARAM));
-    CK(cudaMalloc(&l, sizeof(double)));
-    CK(cudaMalloc(&idx, sizeof(long long) * n));
-    CK(cudaMemcpy(th, w->theta, sizeof(float) * JK_RT_NPARAM, cudaMemcpyHostToDevice));
-    CK(cudaMemcpy(mu, w->mu, sizeof(float) * 16, cudaMemcpyHostToDevice));
-    CK(cudaMemcpy(isd, w->isd, sizeof(float) * 16, cudaMemcpyHostToDevice));
-    CK(cudaMemcpy(idx, iota.data(), sizeof(long long) * n, cudaMemcpyHostToDevice));
-    CK(cudaMemset(g, 0, sizeof(float) * JK_RT_NPARAM));
-    CK(cudaMemset(l, 0, sizeof(double)));
-    const size_t smem = 2 * JK_RT_NPARAM * sizeof(float);
-    jk_mlp_grad_kernel<<<(unsigned)((n + 255) / 256), 256, smem>>>(th, mu, isd, X, y, (long long)n, idx, (int)n, 0ull,
-                                                                 quantile, g, l);
-    CK(cudaGetLastError());
-    CK(cudaDeviceSynchronize());
-    CK(cudaMemcpy(grad_host, g, sizeof(float) * JK_RT_NPARAM, cudaMemcpyDeviceToHost));
-    CK(cudaMemcpy(loss, l, sizeof(double), cudaMemcpyDeviceToHost));
-    return JK_OK;
+    JkGradBuffers *B = nullptr;
+    struct Guard { JkGradBuffers *&p; ~Guard() { cudaFree(p); } } guard{B};
+    CK(cudaMalloc(&B, sizeof *B));
+    return grad_rows(B, w, X, y, n, quantile, grad_host, loss, 0);
 }
 
 int jk_router_train(const float *X, const float *y, int64_t n, const jk_train_opts *opts, jk_router_blob *out,
@@ -2649,13 +2626,14 @@ int jk_router_train(const float *X, const float *y, int64_t n, const jk_train_op
     CK(cudaMemset(m1, 0, sizeof(float) * JK_RT_NPARAM));
     CK(cudaMemset(m2, 0, sizeof(float) * JK_RT_NPARAM));
     CK(cudaMemset(lh, 0, sizeof(double) * opts->steps));
-    const size_t smem = 2 * JK_RT_NPARAM * sizeof(float);
-    const unsigned gb = (unsigned)((opts->batch + 255) / 256);
+    int dev = 0, sms = 0;
+    CK(cudaGetDevice(&dev));
+    CK(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
     for (int step = 1; step <= opts->steps; ++step) {
         CK(cudaMemsetAsync(g, 0, sizeof(float) * JK_RT_NPARAM));
-        jk_mlp_grad_kernel<<<gb, 256, smem>>>(dth, mu, isd, X, y, (long long)n, nullptr, opts->batch,
-                                               opts->seed * 1000003ull + (unsigned long long)step, opts->quantile, g,
-                                               lh + (step - 1));
+        unsigned long long seed = opts->seed * 1000003ull + (unsigned long long)step;
+        if (seed == JK_GRAD_ROWS) seed = 0;
+        CK(jk_mlp_grad(dth, mu, isd, X, y, (long long)n, opts->batch, seed, opts->quantile, g, lh + (step - 1), sms, 0));
         jk_adam_kernel<<<(JK_RT_NPARAM + 255) / 256, 256>>>(dth, g, m1, m2, step, opts->lr, 0.9f, 0.999f, 1e-8f);
     }
     CK(cudaGetLastError());
