@@ -461,7 +461,8 @@ std::vector<double> solid_harmonics(int l)
 // -------------------------------------------------------- fragment choice
 // Threads per quartet: G = ga*gb*gc*gd with each g dividing the Cartesian
 // size of its shell. G == 1 keeps the 2D tables in registers and is taken
-// when elements plus tables stay small; otherwise the smallest G whose
+// when elements plus tables stay small; otherwise the smallest G that fills
+// its warps with small fragments, else whose
 // per-thread fragment fits the register budget within one CTA (G <= 32: a
 // warp holds 32 / G groups; up to 256, or 1024 for the Schwarz kernels: one
 // group per CTA), else the smallest G that fits when the group is split
@@ -476,9 +477,24 @@ void choose_fragments(KSpec &s, bool symmetric)
     const int reg_cap = 48;                   // per-thread fragment budget (reals)
     const int gmax = symmetric ? 1024 : 256;  // threads per quartet in one CTA
     const int gsplit = 256;                   // threads per CTA of a group split over CTAs
-    const int g1_cap = s.fp32 == 1 ? 128 : 64;     // register-mode budget: fragment + 3 tables
     s.gx = 1;
-    if (ne + 3 * ni <= g1_cap) { s.ga = s.gb = s.gc = s.gd = 1; return; }
+    // One thread per quartet: fragment + 3 tables in registers (FP64, FP32);
+    // two floats take several instructions per operation, so that beyond 18
+    // elements the unrolled code leaves the instruction cache ((pp|ps) with one
+    // thread: 63 % of its issue slots stalled on instruction fetch).
+    const int g1_cap = symmetric ? 64 : (s.fp32 == 1 ? 135 : 90);
+    if (s.fp32 == 2 ? ne <= 18 : ne + 3 * ni <= g1_cap) { s.ga = s.gb = s.gc = s.gd = 1; return; }
+    // The fragment of the other classes' threads: small enough that registers
+    // leave several warps per SM, in groups that fill their warps. Summed launch
+    // times of 8 molecules of the 6-31G*-shaped batch, by threads per quartet:
+    // FP64 (pp|pp) 3: 12.9, 9: 9.0, 27: 11.4 ms; (dd|pp) 9: 3.6, 27: 2.9, 18: 3.6;
+    // two floats (dd|dp) 18: 6.2, 54: 2.9; (dp|dp) 9: 11.1, 27: 6.5; (pp|ps) 1:
+    // 23.2, 3: 21.4; FP32 (pp|pp) 1: 2.2, 3: 2.9; (dd|pp) 9: 1.2, 12: 1.1.
+    // with f or g shells small fragments lose (6 atoms of s p d f shells: 3.1 ->
+    // 4.0 ms): few quartets per SM, whose larger tables only some threads build
+    const bool fshell = std::max(std::max(s.la, s.lb), std::max(s.lc, s.ld)) > 2;
+    const int small_cap = symmetric || fshell ? 0 : (s.fp32 == 1 ? 27 : 12);
+    auto fill = [](int g) { return g <= 32 ? (32 / g) * g / 32.0 : g / (32.0 * ((g + 31) / 32)); };
     // CTAs for a group of g threads: 1 if it fits one CTA, else the fewest
     // x (<= 16) dividing g with g / x <= gsplit, 0 if there is none
     auto split = [&](int g) {
@@ -506,7 +522,8 @@ void choose_fragments(KSpec &s, bool symmetric)
                     // smallest fragment in one CTA; fewest idle lanes last
                     const long idle = gc <= 32 ? 32 % gc : (32 - gc % 32) % 32;
                     long score;
-                    if (ept <= reg_cap && x == 1) score = 300000000L + (4096L - g) * 1000L;
+                    if (ept <= small_cap && x == 1 && fill(g) >= 0.75) score = 400000000L + (4096L - g) * 1000L;
+                    else if (ept <= reg_cap && x == 1) score = 300000000L + (4096L - g) * 1000L;
                     else if (ept <= reg_cap) score = 200000000L + (65536L - g) * 1000L / 16;
                     else if (x == 1) score = 100000000L - (long)ept * 10L;
                     else continue;

@@ -565,7 +565,8 @@ __device__ __forceinline__ int jk_quartet(const JkRec &bra, const JkRec &ket, in
             const R pref = jk_norm(jk_mul(jk_norm(jk_mul(JkConst<R>::get(JK_TWO_PI_2_5), bp.K)),
                                           jk_norm(jk_mul(kp.K, rpq))));
             if constexpr (S::G == 1) {
-#pragma unroll(JkIsDf<R>::v ? 1 : NRE)
+                // large blocks: one copy of the root's code (compiling FP32 (dp|ps) 41 -> 6 s)
+#pragma unroll(JkIsDf<R>::v || S::EPT * NRE > 100 ? 1 : NRE)
                 for (int r = 0; r < NRE; ++r) {
                     R u, wp;
                     jk_op_root<NR, OP, R>(Tt, rho, pref, omega, a64, r, rys, u, wp);
