@@ -210,12 +210,12 @@ int jk_build_batch(jk_handle *h, const double *const *D, int32_t n_dm, int with_
  * in FP32 and is redone in FP64 when the two sides are within a relative
  * 2e-6 of each other; 0 keeps the plain FP32 compare when the cutoff is
  * >= 1e-30),
- * "split" (0..1, default 1/8192: FP64-tier quartets whose bound Q_ab Q_cd Dmax
- * is at most split x max Q^2 x max |D| of their molecule, and in mixed and
- * routed builds at least those up to 4,096 tau32, are evaluated in pairs of FP32
- * numbers (48 bits, relative error about 1e-14, 1e-12 at worst for the tightest
- * functions), which the GPU does several times faster; the error this adds is
- * below the one the result has from the cutoff. They count as FP64 quartets.
+ * "split" (0..1, default 1/128: FP64-tier quartets whose bound Q_ab Q_cd Dmax
+ * is at most split (with f or g shells split / 64) x max Q^2 x max |D| of their
+ * molecule, and in mixed and routed builds at least those up to 4,096 tau32, are
+ * evaluated in pairs of FP32 numbers (48 bits, relative error about 1e-14), which
+ * the GPU does several times faster; the error this adds is below the one the
+ * result has from the cutoff. They count as FP64 quartets.
  * 0: FP64 instructions for every FP64-tier quartet, as for cutoffs below 1e-30
  * and for bases with exponents outside (1e-6, 1e8)),
  * "route_cap" (default 16777216: initial entries of the per-class-pair lists

@@ -104,7 +104,7 @@ Driver &drv()
     return d;
 }
 
-static_assert(sizeof(JkPair) == 96 && sizeof(JkPrimPair64) == 96 && sizeof(JkPrimPair32) == 48 && sizeof(JkPrimPairDf) == 80 &&
+static_assert(sizeof(JkPair) == 96 && sizeof(JkPrimPair64) == 96 && sizeof(JkPrimPair32) == 48 && sizeof(JkPrimPairDf) == 64 &&
                   sizeof(JkPairFeat) == 32 && sizeof(JkKetScr) == 16 && sizeof(JkRec) == 64,
               "record sizes are part of the device layout");
 
@@ -752,18 +752,27 @@ struct TierPlan {
 // Small systems: an item is a serial chain of primitive quartets, about
 // JK_LAT_* seconds per modelled FLOP of a lane when few warps share an SM
 // ((ss|ss) of six-primitive s shells: 1,296 primitive quartets, 1.8 ms). Where
-// the chain would exceed both JK_CHAIN_MIN and a quarter of the build's
-// estimated time (modelled FLOPs at JK_RATE_*), the chunk goes down to one
+// the chain would exceed both JK_CHAIN_MIN and 2 % of the build's estimated
+// time (modelled FLOPs at JK_RATE_*; 25 %: erfc of 14 atoms 4.3 instead of 3.9
+// ms, 9 atoms of s p d f shells mixed 6.5 instead of 4.4), the chunk goes down to one
 // round of the warp, then the bra's primitive pairs are shared out over
 // several items, each of which contracts its part with the density by itself.
 #define JK_CHAIN_MIN 30e-6
+#define JK_CHAIN_SHARE 0.02
 static const double JK_LAT[3] = {20e-9, 5e-9, 20e-9};      // FP64, FP32, two floats
 static const double JK_RATE[3] = {0.8e12, 6e12, 2e12};
 #define JK_ITEM_EPS 1e-15
 // Quartets of the FP64 tier whose bound is at most JK_SPLIT x (max Q)^2 x
 // max |D| are evaluated in two-float arithmetic (relative error about 1e-14),
-// the few above it, which carry the result, in FP64 instructions.
-#define JK_SPLIT (1.0 / 8192)
+// the few above it, which carry the result, in FP64 instructions; classes with
+// f or g shells, whose recurrences lose more, from JK_SPLIT_F of that on.
+// Relative error of K against a 64-bit reference (FP64 instructions alone first;
+// the cutoff sets it): 20 atoms 6.58e-13, 6.58e-13 at 2^-7 and at 1; erfc on 14
+// atoms 1.46e-13, 1.46e-13, 1.46e-13; 6 atoms of s p d f shells 6.59e-14, 7.2e-14
+// at 2^-7, 6.59e-14 at 2^-13, 1.6e-13 at 1. 8 molecules, ms: 0: 598, 2^-13: 253,
+// 2^-10: 239, 2^-7: 231, 1: 225.
+#define JK_SPLIT (1.0 / 128)
+#define JK_SPLIT_F (1.0 / 64)
 #define JK_SPLIT_TAU 4096.0
 
 }  // namespace
@@ -950,6 +959,11 @@ void drop_graphs(jk_handle *h)
     h->graphs.clear();
 }
 
+double split_factor(const KSpec &s)
+{
+    return std::max(std::max(s.la, s.lb), std::max(s.lc, s.ld)) > 2 ? JK_SPLIT_F : 1.0;
+}
+
 // The launches of a tier (t = 0 FP64 shapes, 1 FP32, 2 two-float; hi: the chunk of
 // the FP64 tier of two-tier builds; merge: class pairs that share a kernel in
 // one launch; whole: items never share a quartet's primitives, for the kernels
@@ -990,7 +1004,7 @@ int tier_plan(jk_handle *h, int t, int hi, int merge, int whole, TierPlan **out)
     double total_cost = 0;
     for (auto &L : h->launches) total_cost += L.cost;
     const double kept = hi ? 0.3 : 1.0;   // share of the candidates the tier evaluates
-    const double chain_max = std::max(JK_CHAIN_MIN, 0.25 * kept * total_cost / JK_RATE[t]) / JK_LAT[t];
+    const double chain_max = std::max(JK_CHAIN_MIN, JK_CHAIN_SHARE * kept * total_cost / JK_RATE[t]) / JK_LAT[t];
     std::vector<JkSub> subs;
     std::vector<long long> cap;
     for (long long f = 1;; f *= 2) {
@@ -1015,6 +1029,7 @@ int tier_plan(jk_handle *h, int t, int hi, int merge, int whole, TierPlan **out)
                 S.ket = h->d_pairs + B.off;
                 S.ket_scr = h->d_scr + B.off;
                 S.ket_rec = h->d_rec + B.off;
+                S.bra_rec = h->d_rec + A.off;
                 S.ket_beg = B.d_beg;
                 S.ket_end = B.d_end;
                 S.bra_feat = h->d_pfeat + A.off;
@@ -1036,6 +1051,7 @@ int tier_plan(jk_handle *h, int t, int hi, int merge, int whole, TierPlan **out)
                 S.chunk = (int)c;
                 S.group = (int)k;
                 S.launch = l;
+                S.tight = split_factor(L.spec[t]);
                 for (int m = 0; m < h->nmol; ++m) {
                     const long long nb = A.end[m] - A.beg[m], nk = B.end[m] - B.beg[m];
                     // same class: bra i has nk - i kets
@@ -1444,7 +1460,17 @@ int init_impl(int32_t nmol, const int32_t *mol_shell_off, const jk_shell *shells
         for (size_t k = 0; k < rec.size(); ++k) {
             const JkPair &p = h->h_pairs[k];
             scr[k] = JkKetScr{p.Qf, p.a_loc, p.b_loc, 0};
-            rec[k] = JkRec{p.pp_off, p.a_ao, p.b_ao, p.a == p.b, p.ABxf, p.AByf, p.ABzf, p.ABxl, p.AByl, p.ABzl, p.ABx, p.ABy, p.ABz};
+            JkRec &r = rec[k];
+            memset(&r, 0, sizeof r);
+            r.pp_off = p.pp_off; r.a_ao = p.a_ao; r.b_ao = p.b_ao; r.same = p.a == p.b;
+            r.ABxf = p.ABxf; r.AByf = p.AByf; r.ABzf = p.ABzf;
+            r.ABxl = p.ABxl; r.AByl = p.AByl; r.ABzl = p.ABzl;
+            const double *A = coords + 3 * shells[p.a].atom;
+            float *c = &r.Axh;   // h, l per axis
+            for (int ax = 0; ax < 3; ++ax) {
+                c[2 * ax] = (float)A[ax];
+                c[2 * ax + 1] = (float)(A[ax] - (double)c[2 * ax]);
+            }
         }
         if ((rc = upload(&h->d_pairs, h->h_pairs)) || (rc = upload(&h->d_scr, scr)) || (rc = upload(&h->d_rec, rec))) return rc;
     }
@@ -1910,7 +1936,7 @@ int build_impl(jk_handle *h, const double *const *D, int32_t ndm, int with_j, in
                 a.rys64 = h->d_rys64;
                 a.rys32 = h->d_rys32;
                 a.rysdf = h->d_rysdf;
-                a.split = h->split;
+                a.split = h->split * split_factor(G.spec);
                 a.split_min = split_min;
                 a.split_side = side_of(T.t);
                 a.stats = h->d_stats + 3 * T.t;

@@ -97,18 +97,20 @@ template <typename R> struct JkConst {
 template <> struct JkConst<jkdf> {   // compile-time constants only
     __device__ static __forceinline__ jkdf get(double c) { return {(float)c, (float)(c - (double)(float)c)}; }
 };
-// 1 / sqrt(x): the FP32 estimate y and its residual r = 1 - x y^2 in two
-// floats, y (1 + r/2 + 3 r^2 / 8) (normalised)
+// 1 / sqrt(x): the FP32 estimate y and its residual r = 1 - x y^2 = d - t (d =
+// 1 - fl(x y^2) has a few bits, t the rest), y (1 + r/2 + 3 r^2 / 8) with the
+// product y d / 2 kept exact (normalised; 5e-15 at most)
 __device__ __forceinline__ jkdf jk_rsqrt(jkdf x)
 {
     const float y = rsqrtf(x.h);
     const float p = __fmul_rn(y, y), e = __fmaf_rn(y, y, -p);
-    const jkdf m = jk_mul(x, jkdf{p, e});
-    const float r = __fadd_rn(__fadd_rn(1.0f, -m.h), -m.l);   // m.h is within an ulp or two of 1: exact difference
-    const float c = __fmaf_rn(__fmul_rn(0.375f, r), r, __fmul_rn(0.5f, r));
-    const float q = __fmul_rn(y, c);
+    const float h = __fmul_rn(x.h, p);
+    const float t = __fmaf_rn(x.h, e, __fmaf_rn(x.l, p, __fmaf_rn(x.h, p, -h)));
+    const float d = __fadd_rn(1.0f, -h), hd = __fmul_rn(0.5f, d), r = __fadd_rn(d, -t);
+    const float q = __fmul_rn(y, hd);
+    const float w = __fmaf_rn(y, __fmaf_rn(-0.5f, t, __fmul_rn(__fmul_rn(0.375f, r), r)), __fmaf_rn(y, hd, -q));
     const float s = __fadd_rn(y, q);
-    return {s, __fadd_rn(q, -__fadd_rn(s, -y))};
+    return {s, __fadd_rn(__fadd_rn(q, -__fadd_rn(s, -y)), w)};
 }
 // the same names for the machine types
 template <typename T> __device__ __forceinline__ T jk_norm(T a) { return a; }
@@ -138,20 +140,54 @@ template <typename R, typename T> __device__ __forceinline__ JkPrim<R> jk_prim(c
 }
 template <> __device__ __forceinline__ JkPrim<jkdf> jk_prim<jkdf, JkPrimPairDf>(const JkPrimPairDf &r)
 {
-    return {{r.Pxh, r.Pxl}, {r.Pyh, r.Pyl}, {r.Pzh, r.Pzl}, {r.ph, r.pl}, {r.PAxh, r.PAxl}, {r.PAyh, r.PAyl},
+    return {{0.f, 0.f}, {0.f, 0.f}, {0.f, 0.f}, {r.ph, r.pl}, {r.PAxh, r.PAxl}, {r.PAyh, r.PAyl},
             {r.PAzh, r.PAzl}, {r.Kh, r.Kl}, {r.i2ph, r.i2pl}};
 }
 
 __device__ __forceinline__ double jk_rsqrt(double x) { return rsqrt(x); }
 
-__device__ __forceinline__ JkRec jk_rec(const JkPair &p)
+// The same of a pair for the FP64 kernels.
+struct JkRec64 {
+    int pp_off, a_ao, b_ao, same;
+    double ABx, ABy, ABz;
+};
+__device__ __forceinline__ JkRec64 jk_rec64(const JkPair &p)
 {
-    return {p.pp_off, p.a_ao, p.b_ao, p.a == p.b, p.ABxf, p.AByf, p.ABzf, p.ABxl, p.AByl, p.ABzl, p.ABx, p.ABy, p.ABz};
+    return {p.pp_off, p.a_ao, p.b_ao, p.a == p.b, p.ABx, p.ABy, p.ABz};
 }
+template <typename R> struct JkRecOf {
+    typedef JkRec T;
+    __device__ static __forceinline__ T bra(const JkSub &s, int i) { return s.bra_rec[i]; }
+    __device__ static __forceinline__ T ket(const JkSub &s, int i) { return s.ket_rec[i]; }
+};
+template <> struct JkRecOf<double> {
+    typedef JkRec64 T;
+    __device__ static __forceinline__ T bra(const JkSub &s, int i) { return jk_rec64(s.bra[i]); }
+    __device__ static __forceinline__ T ket(const JkSub &s, int i) { return jk_rec64(s.ket[i]); }
+};
+
+// A - C of a quartet, read by the split tier alone.
+template <typename R, typename T> __device__ __forceinline__ void jk_centres(const T &, const T &, R &, R &, R &) {}
+template <> __device__ __forceinline__ void jk_centres<jkdf, JkRec>(const JkRec &b, const JkRec &k, jkdf &x, jkdf &y, jkdf &z)
+{
+    x = jk_norm(jk_sub(jkdf{b.Axh, b.Axl}, jkdf{k.Axh, k.Axl}));
+    y = jk_norm(jk_sub(jkdf{b.Ayh, b.Ayl}, jkdf{k.Ayh, k.Ayl}));
+    z = jk_norm(jk_sub(jkdf{b.Azh, b.Azl}, jkdf{k.Azh, k.Azl}));
+}
+// P - Q = (P - A) + W with W = (A - C) - (Q - C), kept in the ket's P field.
+template <typename R> __device__ __forceinline__ void jk_ket_w(JkPrim<R> &, R, R, R) {}
+template <> __device__ __forceinline__ void jk_ket_w<jkdf>(JkPrim<jkdf> &k, jkdf x, jkdf y, jkdf z)
+{
+    k.Px = jk_norm(jk_sub(x, k.PAx));
+    k.Py = jk_norm(jk_sub(y, k.PAy));
+    k.Pz = jk_norm(jk_sub(z, k.PAz));
+}
+template <typename R> __device__ __forceinline__ R jk_pq(R P, R Q, R) { return P - Q; }
+__device__ __forceinline__ jkdf jk_pq(jkdf, jkdf w, jkdf pa) { return jk_norm(jk_add(pa, w)); }
 
 // A - B of a pair in the tier's precision (the FP32 copy is stored, so the
 // FP32 tier converts nothing on the FP64 pipe).
-__device__ __forceinline__ void jk_pair_ab(const JkRec &p, double &x, double &y, double &z)
+__device__ __forceinline__ void jk_pair_ab(const JkRec64 &p, double &x, double &y, double &z)
 {
     x = p.ABx; y = p.ABy; z = p.ABz;
 }
@@ -515,7 +551,7 @@ __device__ __forceinline__ void jk_op_root(R Tt, R rho, R pref, double omega, in
 
 template <int LA, int LB, int LC, int LD, int GA, int GB, int GC, int GD, typename R, int OP = 0,
           int NT = JkShape<LA, LB, LC, LD, GA, GB, GC, GD, OP>::G>
-__device__ __forceinline__ int jk_quartet(const JkRec &bra, const JkRec &ket, int ab0, int dab, int nab, int ncd, float qthr, double omega, int a64,
+__device__ __forceinline__ int jk_quartet(const typename JkRecOf<R>::T &bra, const typename JkRecOf<R>::T &ket, int ab0, int dab, int nab, int ncd, float qthr, double omega, int a64,
                                            const typename JkPP<R>::T *__restrict__ pp,
                                            const typename JkTab<R>::T *__restrict__ rys, R *grp, unsigned gmask,
                                            int tg, bool act,
@@ -529,6 +565,8 @@ __device__ __forceinline__ int jk_quartet(const JkRec &bra, const JkRec &ket, in
     R ABx, ABy, ABz, CDx, CDy, CDz;
     jk_pair_ab(bra, ABx, ABy, ABz);
     jk_pair_ab(ket, CDx, CDy, CDz);
+    R ACx, ACy, ACz;
+    jk_centres<R>(bra, ket, ACx, ACy, ACz);
     const PPT *bpp = pp + bra.pp_off;
     const PPT *kpp = pp + ket.pp_off;
     // primitive pairs are sorted by their Schwarz factor q (largest first):
@@ -545,7 +583,8 @@ __device__ __forceinline__ int jk_quartet(const JkRec &bra, const JkRec &ket, in
         const PPT kr = kpp[kl];
         const float qk = jk_pp_q(kr);
         if (qb0 * qk <= qthf) break;
-        const JkPrim<R> kp = jk_prim<R>(kr);
+        JkPrim<R> kp = jk_prim<R>(kr);
+        jk_ket_w<R>(kp, ACx, ACy, ACz);
 #pragma unroll 1
         for (int ij = ab0; ij < nab; ij += dab) {
             const PPT br = bpp[ij];
@@ -554,8 +593,7 @@ __device__ __forceinline__ int jk_quartet(const JkRec &bra, const JkRec &ket, in
             const JkPrim<R> bp = jk_prim<R>(br);
             const R rpq = jk_rsqrt(jk_norm(jk_add(bp.p, kp.p)));
             const R inv_pq = jk_norm(jk_mul(rpq, rpq));
-            const R PQx = jk_norm(jk_sub(bp.Px, kp.Px)), PQy = jk_norm(jk_sub(bp.Py, kp.Py)),
-                    PQz = jk_norm(jk_sub(bp.Pz, kp.Pz));
+            const R PQx = jk_pq(bp.Px, kp.Px, bp.PAx), PQy = jk_pq(bp.Py, kp.Py, bp.PAy), PQz = jk_pq(bp.Pz, kp.Pz, bp.PAz);
             const R qf = jk_norm(jk_mul(kp.p, inv_pq)), pf = jk_norm(jk_mul(bp.p, inv_pq));
             const R rho = jk_norm(jk_mul(bp.p, qf));
             R r2 = jk_mul(PQx, PQx);
@@ -1150,13 +1188,13 @@ jk_class_kernel(const JkClassArgs args)
                     if (active && e < n) {
                         const JkRouted rq = list[e];
                         const JkPair bra = sub.bra[rq.item];
-                        const JkRec ket = jk_rec(sub.ket[rq.ket]);
+                        const typename JkRecOf<R>::T ket = JkRecOf<R>::ket(sub, rq.ket);
                         const JkMol mol = args.mols[bra.mol];
                         R T[S::EPT];
 #pragma unroll
                         for (int k = 0; k < S::EPT; ++k) T[k] = JkConst<R>::get(0.0);
                         const int np = jk_quartet<LA, LB, LC, LD, GA, GB, GC, GD, R, OP>(
-                            jk_rec(bra), ket, 0, 1, sub.nab, sub.ncd, __fdiv_rn(args.prim_eps32, rq.dmq), args.omega, args.asym64,
+                            JkRecOf<R>::bra(sub, rq.item), ket, 0, 1, sub.nab, sub.ncd, __fdiv_rn(args.prim_eps32, rq.dmq), args.omega, args.asym64,
                             pp, rys, grp, gmask, tg, true, off, T);
                         float f = 1.0f;
                         if (bra.a == bra.b) f *= 0.5f;
@@ -1196,7 +1234,6 @@ jk_class_kernel(const JkClassArgs args)
             const JkItem wi = args.items[t];
             const JkSub &sub = args.subs[wi.sub & 0xffff];
             const int part = wi.sub >> 16, parts = sub.split;   // share of the bra's primitive pairs
-            const JkRec *__restrict__ kets = sub.ket_rec;
             const int item = wi.bra, nab = sub.nab, ncd = sub.ncd, same_class = sub.same_class;
             const int kb = wi.kb, ke = wi.ke;
             if (sub.launch != cur) {
@@ -1204,7 +1241,7 @@ jk_class_kernel(const JkClassArgs args)
                 cur = sub.launch;
             }
             const JkPair bra = sub.bra[item];
-            const JkRec brec = jk_rec(bra);
+            const typename JkRecOf<R>::T brec = JkRecOf<R>::bra(sub, item);
             const JkMol mol = args.mols[bra.mol];
             const double *dmx = args.dmax + mol.dmax_off;
             const double dmol = args.use_dmax ? args.dmax_mol[bra.mol] : 1.0;
@@ -1295,7 +1332,7 @@ jk_class_kernel(const JkClassArgs args)
                     const int take = qn < NGW ? qn : NGW;
                     if (active && gw < take) {
                         const int myket = s_qk[wib][gw];
-                        const JkRec ket = kets[myket];
+                        const typename JkRecOf<R>::T ket = JkRecOf<R>::ket(sub, myket);
                         R T[S::EPT];
 #pragma unroll
                         for (int k = 0; k < S::EPT; ++k) T[k] = JkConst<R>::get(0.0);
@@ -1378,13 +1415,13 @@ jk_class_kernel(const JkClassArgs args)
                     }
                     const JkRouted rq = list[e];
                     const JkPair bra = sub.bra[rq.item];
-                    const JkRec ket = jk_rec(sub.ket[rq.ket]);
+                    const typename JkRecOf<R>::T ket = JkRecOf<R>::ket(sub, rq.ket);
                     const JkMol mol = args.mols[bra.mol];
                     R T[S::EPT];
 #pragma unroll
                     for (int k = 0; k < S::EPT; ++k) T[k] = JkConst<R>::get(0.0);
                     const int np = jk_quartet<LA, LB, LC, LD, GA, GB, GC, GD, R, OP, NTC>(
-                        jk_rec(bra), ket, 0, 1, sub.nab, sub.ncd, __fdiv_rn(args.prim_eps32, rq.dmq), args.omega, args.asym64, pp,
+                        JkRecOf<R>::bra(sub, rq.item), ket, 0, 1, sub.nab, sub.ncd, __fdiv_rn(args.prim_eps32, rq.dmq), args.omega, args.asym64, pp,
                         rys, grp, 0u, tg, act, off, T);
                     if (act) {
                         float f = 1.0f;
@@ -1432,7 +1469,7 @@ jk_class_kernel(const JkClassArgs args)
                 cur = sub.launch;
             }
             const JkPair bra = sub.bra[item];
-            const JkRec brec = jk_rec(bra);
+            const typename JkRecOf<R>::T brec = JkRecOf<R>::bra(sub, item);
             const JkMol mol = args.mols[bra.mol];
             const double *dmx = args.dmax + mol.dmax_off;
             const double dmol = args.use_dmax ? args.dmax_mol[bra.mol] : 1.0;
@@ -1469,7 +1506,7 @@ jk_class_kernel(const JkClassArgs args)
                 while (mask) {
                     const int myket = base + __ffs(mask) - 1;
                     mask &= mask - 1;
-                    const JkRec ket = sub.ket_rec[myket];
+                    const typename JkRecOf<R>::T ket = JkRecOf<R>::ket(sub, myket);
                     R T[S::EPT];
 #pragma unroll
                     for (int k = 0; k < S::EPT; ++k) T[k] = JkConst<R>::get(0.0);
@@ -1555,7 +1592,7 @@ jk_schwarz_kernel(const JkSchwarzArgs args)
             const bool mine = active && pi < args.npair;
             double mx = 0.0;
             if (mine) {
-                const JkRec pr = jk_rec(args.pairs[pi]);
+                const JkRec64 pr = jk_rec64(args.pairs[pi]);
                 double T[S::EPT];
 #pragma unroll
                 for (int k = 0; k < S::EPT; ++k) T[k] = 0.0;
@@ -1590,7 +1627,7 @@ jk_schwarz_kernel(const JkSchwarzArgs args)
                 gd = tgl % GD; gc = (tgl / GD) % GC; gb = (tgl / (GD * GC)) % GB; ga = tgl / (GD * GC * GB);
                 jk_make_offsets<LA, LB, LA, LB, GA, GB, GC, GD, S>(ga, gb, gc, gd, off);
             }
-            const JkRec pr = jk_rec(args.pairs[pi]);
+            const JkRec64 pr = jk_rec64(args.pairs[pi]);
             double T[S::EPT];
 #pragma unroll
             for (int k = 0; k < S::EPT; ++k) T[k] = 0.0;

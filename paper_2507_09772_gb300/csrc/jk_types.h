@@ -24,8 +24,8 @@ struct alignas(16) JkPair {
 
 // What a kernel reads of every candidate ket: one 16-byte vector for the
 // screening (32 candidates in a row are four lines; the JkPair records would be
-// 24), and a 64-byte record for a quartet, of which the FP32 tier touches the
-// first half and the split tier three quarters. Arrays aligned with the pairs.
+// 24), and a 64-byte record for a quartet in FP32 (the first half) or two
+// floats. Arrays aligned with the pairs.
 struct alignas(16) JkKetScr {
     float Qf;
     int a_loc, b_loc;
@@ -35,7 +35,7 @@ struct alignas(16) JkRec {
     int pp_off, a_ao, b_ao;
     int same;                // a == b
     float ABxf, AByf, ABzf, ABxl, AByl, ABzl;
-    double ABx, ABy, ABz;
+    float Axh, Axl, Ayh, Ayl, Azh, Azl;   // centre A in two floats
 };
 
 // Per primitive pair (alpha_i on a, beta_j on b), p = alpha + beta:
@@ -60,11 +60,14 @@ struct alignas(16) JkPrimPair32 {
     float inv2p, q, pad1, pad2;
 };
 
-// The same in two-float arithmetic (x = xh + xl, 48 bits): the split tier.
+// The same in two-float arithmetic (x = xh + xl, 48 bits): the split tier,
+// which forms P - Q as (P - A) + (A - C) - (Q - C): the difference of the
+// absolute centres would carry 2^-49 of their distance from the origin, which
+// the tightest products (exponents of thousands) turn into 1e-12 of the integral.
 struct alignas(16) JkPrimPairDf {
-    float Pxh, Pxl, Pyh, Pyl, Pzh, Pzl, ph, pl;
-    float PAxh, PAxl, PAyh, PAyl, PAzh, PAzl, Kh, Kl;
-    float i2ph, i2pl, q, pad;
+    float ph, pl, Kh, Kl;
+    float PAxh, PAxl, PAyh, PAyl, PAzh, PAzl;
+    float i2ph, i2pl, q, pad[3];
 };
 
 // Per molecule of a handle.
@@ -90,7 +93,7 @@ struct JkSub {
     const JkPair *bra;           // pairs of the bra class
     const JkPair *ket;           // pairs of the ket class
     const JkKetScr *ket_scr;     // aligned with ket
-    const JkRec *ket_rec;
+    const JkRec *ket_rec, *bra_rec;
     const int *ket_beg;          // per molecule: first ket index in the ket class
     const int *ket_end;          // per molecule: one past the last
     const JkPairFeat *bra_feat;  // aligned with bra / ket
@@ -102,6 +105,7 @@ struct JkSub {
     int split;                   // work items that share a bra pair's primitive pairs
     int group;                   // launch it belongs to
     int launch;                  // class pair index: statistics, routed lists
+    double tight;                // factor of the split threshold for its angular momenta
 };
 
 // A work item: the candidates [kb, ke) of the ket class for one bra pair, and

@@ -52,11 +52,10 @@ __global__ void jk_pairdata_kernel(int npair, const int *__restrict__ pa, const 
             s.inv2p = (float)r.inv2p; s.q = 0.f; s.pad1 = s.pad2 = 0.f;
             out32[o] = s;
             JkPrimPairDf d;
-            jk_two(r.Px, d.Pxh, d.Pxl); jk_two(r.Py, d.Pyh, d.Pyl); jk_two(r.Pz, d.Pzh, d.Pzl);
             jk_two(r.p, d.ph, d.pl);
             jk_two(r.PAx, d.PAxh, d.PAxl); jk_two(r.PAy, d.PAyh, d.PAyl); jk_two(r.PAz, d.PAzh, d.PAzl);
             jk_two(r.K, d.Kh, d.Kl); jk_two(r.inv2p, d.i2ph, d.i2pl);
-            d.q = d.pad = 0.f;
+            d.q = d.pad[0] = d.pad[1] = d.pad[2] = 0.f;
             outdf[o] = d;
         }
     }
@@ -208,7 +207,7 @@ __global__ void __launch_bounds__(256) jk_plan_kernel(const JkPlanArgs args)
         double tlo = T.lo;
         if (T.split_side > 0) {   // as jk_bounds forms it
             const double th =
-                dm < 1e15 ? fmax(args.split_min, __dmul_rn(__dmul_rn(args.split, args.mols[m].qmax2), dm)) : 0.0;
+                dm < 1e15 ? fmax(args.split_min, __dmul_rn(__dmul_rn(args.split * S.tight, args.mols[m].qmax2), dm)) : 0.0;
             tlo = fmax(tlo, th);
         }
         if (args.scr32) {

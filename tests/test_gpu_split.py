@@ -1,12 +1,11 @@
 """GPU: the split tier (FP64-tier quartets below the split threshold evaluated
 in pairs of floats).
 
-Two floats carry 48 bits; the largest relative error of an integral is about
-2e-12 (the difference of two centres near 10 bohr, 2^-49 x 10, against the
-width of the tightest products, exponents up to 5,000), so with every quartet
-in two floats (split = 1) and |J|, |K| below 50 the result stays within 1e-10;
-at the default threshold, 1/8192 of the largest bound, within 1e-12 of the
-all-FP64 build.
+Two floats carry 48 bits; an integral takes some hundred operations, each
+within 2^-46 of its result, a relative error of at most 2e-12, so with every
+quartet in two floats (split = 1) and |J|, |K| below 50 the result stays within
+1e-10; at the default threshold, 1/128 of the largest bound, within 1e-12 of
+the all-FP64 build.
 """
 import numpy as np
 import pytest
@@ -62,7 +61,7 @@ CASES = {
 def test_two_float_quartets(name):
     mol, options, kw = CASES[name]()
     ref, n0 = build(mol, 0.0, options, **kw)
-    for split, tol in ((1.0, 1e-10), (1.0 / 8192, 1e-12)):
+    for split, tol in ((1.0, 1e-10), (1.0 / 128, 1e-12)):
         got, n = build(mol, split, options, **kw)
         assert n == n0            # every quartet in exactly one of the tiers
         for a, b in zip(got, ref):
@@ -84,7 +83,7 @@ def test_scaled_density_keeps_the_relative_error():
     mol = synth.tiny_631gs()
     mol.D = mol.D * 2.0 ** -12
     (J0, K0), _ = build(mol, 0.0)
-    (J1, K1), _ = build(mol, 1.0 / 8192)
+    (J1, K1), _ = build(mol, 1.0 / 128)
     assert np.abs(J1 - J0).max() <= 1e-12 * 2.0 ** -12 and np.abs(K1 - K0).max() <= 1e-12 * 2.0 ** -12
 
 
