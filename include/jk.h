@@ -93,7 +93,7 @@ typedef struct {
 /* Per-launch record of the last build made with option "profile" = 1. */
 typedef struct {
     int32_t la, lb, lc, ld, na, nb, nc, nd;  /* class: angular momenta, primitive counts */
-    int32_t tier;                            /* 0 FP64, 1 FP32 */
+    int32_t tier;                            /* 0 FP64, 1 FP32, 2 FP64-tier quartets in two floats (option split) */
     int32_t threads_per_quartet;             /* fragmentation (1 = one quartet per thread) */
     int32_t regs, local_bytes;               /* registers per thread, local (spill) bytes */
     int64_t quartets, prim_quartets;         /* significant quartets it evaluated */
@@ -195,13 +195,14 @@ int jk_build_batch(jk_handle *h, const double *const *D, int32_t n_dm, int with_
  * kernels; other builds spread them over 24),
  * "chunk" (32..65536, default 64: candidate kets per work item of the
  * persistent class kernels for classes with one thread per quartet; classes
- * with G threads per quartet take 1/G of it, at least 4, and systems with more
- * than 8 million items larger ones; changing it re-plans the work items),
+ * with G threads per quartet take 1/G of it, and systems with more than 8
+ * million items larger ones; changing it re-plans the work items),
  * "asym64" (0/1, default 0: the FP32 tier evaluates the large-T
  * Gauss-Hermite limit of the Rys roots and weights in FP64 and rounds the
  * result to FP32, instead of evaluating it in FP32),
- * "chunk_fp64tier" (default 512: the same for the FP64 tier of mixed and
- * routed builds, whose kernels keep only the candidates above tau32),
+ * "chunk_fp64tier" (default 512: the most candidate kets per work item of the
+ * FP64 tiers of mixed and routed builds and of an FP64 build above its split
+ * threshold, whose kernels keep few of the candidates),
  * "widen_int" (0/1, default 0: the FP32 tier widens its contributions to
  * FP64 for the J/K reductions with the conversion instruction, which runs on the
  * FP64 pipe; 1 builds the FP64 bit pattern with integer operations),

@@ -744,10 +744,14 @@ struct TierPlan {
 // 2 ms on its own. Systems whose items would exceed JK_ITEMS_MAX get larger
 // chunks.
 #define JK_CHUNK 64
-// The FP64 tier of a mixed build keeps ~7 % of the candidates; with 512 per
-// item the batched mixed build ran 5 % faster than with 64 (and than 2,048).
+// Tiers that keep few of the candidates they scan; the FP64 and split tiers of a
+// mixed build (~7 %) as many as leave every resident warp JK_ITEMS_PER_WARP items
+// of the launch, between JK_CHUNK and this. 33 atoms mixed, two densities: 13.6 ms
+// with 512 throughout, 12.9 with the rule; 45 atoms routed 18.3 and 17.0. (The
+// other tiers lose with more than 64: 8 molecules FP64 224 ms, 236 with 256.)
 #define JK_CHUNK_HI 512
 #define JK_CHUNK_MIN 4
+#define JK_ITEMS_PER_WARP 32.0
 #define JK_ITEMS_MAX 8000000LL
 // Small systems: an item is a serial chain of primitive quartets, about
 // JK_LAT_* seconds per modelled FLOP of a lane when few warps share an SM
@@ -755,8 +759,8 @@ struct TierPlan {
 // the chain would exceed both JK_CHAIN_MIN and 2 % of the build's estimated
 // time (modelled FLOPs at JK_RATE_*; 25 %: erfc of 14 atoms 4.3 instead of 3.9
 // ms, 9 atoms of s p d f shells mixed 6.5 instead of 4.4), the chunk goes down to one
-// round of the warp, then the bra's primitive pairs are shared out over
-// several items, each of which contracts its part with the density by itself.
+// round of the warp, then the bra's and the ket's primitive pairs are shared out
+// over several items, each of which contracts its part with the density by itself.
 #define JK_CHAIN_MIN 30e-6
 #define JK_CHAIN_SHARE 0.02
 static const double JK_LAT[3] = {20e-9, 5e-9, 20e-9};      // FP64, FP32, two floats
@@ -964,14 +968,14 @@ double split_factor(const KSpec &s)
     return std::max(std::max(s.la, s.lb), std::max(s.lc, s.ld)) > 2 ? JK_SPLIT_F : 1.0;
 }
 
-// The launches of a tier (t = 0 FP64 shapes, 1 FP32, 2 two-float; hi: the chunk of
-// the FP64 tier of two-tier builds; merge: class pairs that share a kernel in
+// The launches of a tier (t = 0 FP64 shapes, 1 FP32, 2 two-float; hi: the chunk of tiers
+// that keep few candidates, 2 in builds with an FP32 tier; merge: class pairs that share a kernel in
 // one launch; whole: items never share a quartet's primitives, for the kernels
 // that log or route quartets), made on first use and kept until the shapes or
 // chunks change.
 int tier_plan(jk_handle *h, int t, int hi, int merge, int whole, TierPlan **out)
 {
-    const int key = t + 4 * hi + 8 * merge + 16 * whole;
+    const int key = t + 4 * hi + 16 * merge + 32 * whole;
     auto it = h->plans.find(key);
     if (it != h->plans.end()) { *out = it->second.get(); return JK_OK; }
     std::unique_ptr<TierPlan> P(new TierPlan());
@@ -1000,7 +1004,6 @@ int tier_plan(jk_handle *h, int t, int hi, int merge, int whole, TierPlan **out)
         std::stable_sort(members[g].begin(), members[g].end(), [&](int x, int y) { return prims(x) > prims(y); });
     }
     std::stable_sort(gord.begin(), gord.end(), [&](int x, int y) { return cost[x] > cost[y]; });
-    const long long base = hi ? h->chunk_hi : h->chunk;
     double total_cost = 0;
     for (auto &L : h->launches) total_cost += L.cost;
     const double kept = hi ? 0.3 : 1.0;   // share of the candidates the tier evaluates
@@ -1020,6 +1023,13 @@ int tier_plan(jk_handle *h, int t, int hi, int merge, int whole, TierPlan **out)
             G.sub0 = (int)subs.size();
             G.nsub = (int)mem.size();
             const int ngw = G.spec.G() <= 32 ? 32 / G.spec.G() : 1;
+            double cand = 0;
+            for (int l : mem) cand += h->launches[l].cand;
+            // kets per item for one thread per quartet
+            const long long base =
+                hi < 2 ? (hi ? h->chunk_hi : h->chunk)
+                       : (long long)std::min<double>(h->chunk_hi, std::max<double>(std::min(h->chunk, h->chunk_hi),
+                                                                                   cand / (8.0 * h->num_sms * JK_ITEMS_PER_WARP)));
             for (int l : mem) {
                 const Launch &L = h->launches[l];
                 const PairClass &A = h->classes[L.c1], &B = h->classes[L.c2];
@@ -1044,9 +1054,16 @@ int tier_plan(jk_handle *h, int t, int hi, int merge, int whole, TierPlan **out)
                 const double round = class_flops(one, 1) / one.G() * S.nab * S.ncd;
                 long long c = std::max<long long>(JK_CHUNK_MIN, base * ngw / 32);
                 while (c > ngw && round * std::max(1.0, kept * c / ngw) > chain_max) c = (c + 1) / 2;
-                S.split = 1;
-                if (!whole)
-                    S.split = (int)std::min<double>(S.nab, std::max(1.0, std::ceil(round * std::max(1.0, kept * c / ngw) / chain_max)));
+                S.split = S.split_ab = 1;
+                if (!whole) {
+                    const double want = std::max(1.0, std::ceil(round * std::max(1.0, kept * c / ngw) / chain_max));
+                    S.split_ab = (int)std::min<double>(S.nab, want);
+                    // the ket's where the chain is still twice too long and a
+                    // share keeps eight times the work of contracting its part
+                    const double prim = class_flops(one, 0) * S.nab * S.ncd, contract = class_flops(one, 1) - class_flops(one, 0);
+                    const double most = std::min(std::floor(256.0 / S.split_ab), prim / (8.0 * contract * S.split_ab));
+                    S.split = S.split_ab * (int)std::max(1.0, std::min({(double)S.ncd, std::ceil(want / (2.0 * S.split_ab)), most}));
+                }
                 c = std::min<long long>(1 << 24, c * f);
                 S.chunk = (int)c;
                 S.group = (int)k;
@@ -1674,7 +1691,7 @@ int build_impl(jk_handle *h, const double *const *D, int32_t ndm, int with_j, in
         if (!use) continue;
         Tier T{t, nullptr, nullptr};
         // tiers that keep few of the candidates they scan take longer items
-        const int hi = (t == 0 && (two || usedf)) || (t == 3 && two) ? 1 : 0;
+        const int hi = two && (t == 0 || t == 3) ? 2 : (t == 0 && usedf ? 1 : 0);
         const int whole = logs || (routed && t != 1) ? 1 : 0;
         if ((rc = tier_plan(h, spec_of[t], hi, merge, t == 2 ? 0 : whole, &T.P))) return rc;
         const int kmode = logs ? 2 : (routed ? (t == 2 ? 3 : (t == 1 ? 0 : 1)) : 0);
@@ -2071,7 +2088,7 @@ int build_impl(jk_handle *h, const double *const *D, int32_t ndm, int with_j, in
                         jk_launch_prof p;
                         p.la = x.la; p.lb = x.lb; p.lc = x.lc; p.ld = x.ld;
                         p.na = x.na; p.nb = x.nb; p.nc = x.nc; p.nd = x.nd;
-                        p.tier = T.t == 0 || T.t == 3 ? 0 : 1;
+                        p.tier = T.t == 0 ? 0 : (T.t == 3 ? 2 : 1);
                         p.threads_per_quartet = x.G();
                         p.regs = ki.regs;
                         p.local_bytes = ki.local_bytes;

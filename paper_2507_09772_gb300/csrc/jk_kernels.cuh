@@ -549,9 +549,15 @@ __device__ __forceinline__ void jk_op_root(R Tt, R rho, R pref, double omega, in
     }
 }
 
+// A work item's share of a quartet's primitive quartets: bra pairs ab, ab + dab,
+// ..., ket pairs cd, cd + dcd, ...
+struct JkShare {
+    int ab, dab, cd, dcd;
+};
+
 template <int LA, int LB, int LC, int LD, int GA, int GB, int GC, int GD, typename R, int OP = 0,
           int NT = JkShape<LA, LB, LC, LD, GA, GB, GC, GD, OP>::G>
-__device__ __forceinline__ int jk_quartet(const typename JkRecOf<R>::T &bra, const typename JkRecOf<R>::T &ket, int ab0, int dab, int nab, int ncd, float qthr, double omega, int a64,
+__device__ __forceinline__ int jk_quartet(const typename JkRecOf<R>::T &bra, const typename JkRecOf<R>::T &ket, JkShare sh, int nab, int ncd, float qthr, double omega, int a64,
                                            const typename JkPP<R>::T *__restrict__ pp,
                                            const typename JkTab<R>::T *__restrict__ rys, R *grp, unsigned gmask,
                                            int tg, bool act,
@@ -576,17 +582,17 @@ __device__ __forceinline__ int jk_quartet(const typename JkRecOf<R>::T &bra, con
     // record per lane and kl) are the outer loop, so each is loaded once; the
     // bra's (the same for the whole group or warp) the inner one.
     const float qthf = qthr;
-    const float qb0 = jk_pp_q(bpp[ab0]);
+    const float qb0 = jk_pp_q(bpp[sh.ab]);
     int nprim = 0;
 #pragma unroll 1
-    for (int kl = 0; kl < ncd; ++kl) {
+    for (int kl = sh.cd; kl < ncd; kl += sh.dcd) {
         const PPT kr = kpp[kl];
         const float qk = jk_pp_q(kr);
         if (qb0 * qk <= qthf) break;
         JkPrim<R> kp = jk_prim<R>(kr);
         jk_ket_w<R>(kp, ACx, ACy, ACz);
 #pragma unroll 1
-        for (int ij = ab0; ij < nab; ij += dab) {
+        for (int ij = sh.ab; ij < nab; ij += sh.dab) {
             const PPT br = bpp[ij];
             if (jk_pp_q(br) * qk <= qthf) break;
             ++nprim;
@@ -759,9 +765,9 @@ __device__ __forceinline__ JkBounds jk_bounds(const JkClassArgs &args, const JkM
 {
     JkBounds b = {args.lo, args.hi, args.lo32, args.hi32};
     if (args.split_side != 0) {
-        // (densities near the FP32 range, or not finite, stay in FP64)
+        // (densities near the ends of the FP32 range, or not finite, stay in FP64)
         const double th =
-            dmol < 1e15 ? fmax(args.split_min, __dmul_rn(__dmul_rn(args.split, mol.qmax2), dmol)) : 0.0;
+            dmol > 1e-15 && dmol < 1e15 ? fmax(args.split_min, __dmul_rn(__dmul_rn(args.split, mol.qmax2), dmol)) : 0.0;
         if (args.split_side > 0 && th > b.lo) { b.lo = th; b.lo32 = (float)th; }
         if (args.split_side < 0 && th < b.hi) { b.hi = th; b.hi32 = (float)th; }
     }
@@ -1194,7 +1200,7 @@ jk_class_kernel(const JkClassArgs args)
 #pragma unroll
                         for (int k = 0; k < S::EPT; ++k) T[k] = JkConst<R>::get(0.0);
                         const int np = jk_quartet<LA, LB, LC, LD, GA, GB, GC, GD, R, OP>(
-                            JkRecOf<R>::bra(sub, rq.item), ket, 0, 1, sub.nab, sub.ncd, __fdiv_rn(args.prim_eps32, rq.dmq), args.omega, args.asym64,
+                            JkRecOf<R>::bra(sub, rq.item), ket, JkShare{0, 1, 0, 1}, sub.nab, sub.ncd, __fdiv_rn(args.prim_eps32, rq.dmq), args.omega, args.asym64,
                             pp, rys, grp, gmask, tg, true, off, T);
                         float f = 1.0f;
                         if (bra.a == bra.b) f *= 0.5f;
@@ -1232,8 +1238,9 @@ jk_class_kernel(const JkClassArgs args)
             unsigned long long nx = 0;
             if (AHEAD && lane == 0) nx = atomicAdd(args.work, 1ull);
             const JkItem wi = args.items[t];
-            const JkSub &sub = args.subs[wi.sub & 0xffff];
-            const int part = wi.sub >> 16, parts = sub.split;   // share of the bra's primitive pairs
+            const JkSub &sub = args.subs[wi.sub & 0x7fffff];
+            const int part = wi.sub >> 23;   // share of the primitive quartets
+            const JkShare sh = {part % sub.split_ab, sub.split_ab, part / sub.split_ab, sub.split / sub.split_ab};
             const int item = wi.bra, nab = sub.nab, ncd = sub.ncd, same_class = sub.same_class;
             const int kb = wi.kb, ke = wi.ke;
             if (sub.launch != cur) {
@@ -1337,7 +1344,7 @@ jk_class_kernel(const JkClassArgs args)
 #pragma unroll
                         for (int k = 0; k < S::EPT; ++k) T[k] = JkConst<R>::get(0.0);
                         const int np = jk_quartet<LA, LB, LC, LD, GA, GB, GC, GD, R, OP>(
-                            brec, ket, part, parts, nab, ncd, __fdiv_rn(args.prim_eps32, s_qd[wib][gw]), args.omega,
+                            brec, ket, sh, nab, ncd, __fdiv_rn(args.prim_eps32, s_qd[wib][gw]), args.omega,
                             args.asym64, pp, rys, grp, gmask, tg, true, off, T);
                         if (tg == 0) nprim += np;
                         float f = 1.0f;
@@ -1421,7 +1428,7 @@ jk_class_kernel(const JkClassArgs args)
 #pragma unroll
                     for (int k = 0; k < S::EPT; ++k) T[k] = JkConst<R>::get(0.0);
                     const int np = jk_quartet<LA, LB, LC, LD, GA, GB, GC, GD, R, OP, NTC>(
-                        JkRecOf<R>::bra(sub, rq.item), ket, 0, 1, sub.nab, sub.ncd, __fdiv_rn(args.prim_eps32, rq.dmq), args.omega, args.asym64, pp,
+                        JkRecOf<R>::bra(sub, rq.item), ket, JkShare{0, 1, 0, 1}, sub.nab, sub.ncd, __fdiv_rn(args.prim_eps32, rq.dmq), args.omega, args.asym64, pp,
                         rys, grp, 0u, tg, act, off, T);
                     if (act) {
                         float f = 1.0f;
@@ -1460,8 +1467,9 @@ jk_class_kernel(const JkClassArgs args)
                 jk_make_offsets<LA, LB, LC, LD, GA, GB, GC, GD, S>(ga, gb, gc, gd, off);
             }
             const JkItem wi = args.items[t];
-            const JkSub &sub = args.subs[wi.sub & 0xffff];
-            const int part = wi.sub >> 16, parts = sub.split;   // share of the bra's primitive pairs
+            const JkSub &sub = args.subs[wi.sub & 0x7fffff];
+            const int part = wi.sub >> 23;   // share of the primitive quartets
+            const JkShare sh = {part % sub.split_ab, sub.split_ab, part / sub.split_ab, sub.split / sub.split_ab};
             const int item = wi.bra, nab = sub.nab, ncd = sub.ncd, same_class = sub.same_class;
             const int kb = wi.kb, ke = wi.ke;
             if (sub.launch != cur) {
@@ -1511,7 +1519,7 @@ jk_class_kernel(const JkClassArgs args)
 #pragma unroll
                     for (int k = 0; k < S::EPT; ++k) T[k] = JkConst<R>::get(0.0);
                     const int np = jk_quartet<LA, LB, LC, LD, GA, GB, GC, GD, R, OP, NTC>(
-                        brec, ket, part, parts, nab, ncd, __fdiv_rn(args.prim_eps32, s_dm[myket - base]), args.omega, args.asym64, pp,
+                        brec, ket, sh, nab, ncd, __fdiv_rn(args.prim_eps32, s_dm[myket - base]), args.omega, args.asym64, pp,
                         rys, grp, 0u, tg, act, off, T);
                     nprim += np;
                     if (act) {
@@ -1596,7 +1604,7 @@ jk_schwarz_kernel(const JkSchwarzArgs args)
                 double T[S::EPT];
 #pragma unroll
                 for (int k = 0; k < S::EPT; ++k) T[k] = 0.0;
-                jk_quartet<LA, LB, LA, LB, GA, GB, GC, GD, double>(pr, pr, 0, 1, NPA * NPB, NPA * NPB, -1.0f, 0.0, 0, args.pp64, args.rys64, grp, gmask, tg, true, off, T);
+                jk_quartet<LA, LB, LA, LB, GA, GB, GC, GD, double>(pr, pr, JkShare{0, 1, 0, 1}, NPA * NPB, NPA * NPB, -1.0f, 0.0, 0, args.pp64, args.rys64, grp, gmask, tg, true, off, T);
                 if (ga == gc && gb == gd) {
 #pragma unroll
                     for (int ia = 0; ia < FA; ++ia)
@@ -1632,7 +1640,7 @@ jk_schwarz_kernel(const JkSchwarzArgs args)
 #pragma unroll
             for (int k = 0; k < S::EPT; ++k) T[k] = 0.0;
             jk_quartet<LA, LB, LA, LB, GA, GB, GC, GD, double, 0, NTC>(
-                pr, pr, 0, 1, NPA * NPB, NPA * NPB, -1.0f, 0.0, 0, args.pp64, args.rys64, grp, 0u, tg, act, off, T);
+                pr, pr, JkShare{0, 1, 0, 1}, NPA * NPB, NPA * NPB, -1.0f, 0.0, 0, args.pp64, args.rys64, grp, 0u, tg, act, off, T);
             double mx = 0.0;
             if (act && ga == gc && gb == gd) {
 #pragma unroll

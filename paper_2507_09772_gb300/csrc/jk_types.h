@@ -102,15 +102,17 @@ struct JkSub {
     int same_class;              // ket class == bra class: ket index >= bra index
     int nab, ncd;                // primitive pairs of a bra / ket pair
     int chunk;                   // kets per work item
-    int split;                   // work items that share a bra pair's primitive pairs
+    int split, split_ab;         // work items that share the primitive quartets: in all, and by the bra's pairs
     int group;                   // launch it belongs to
     int launch;                  // class pair index: statistics, routed lists
     double tight;                // factor of the split threshold for its angular momenta
 };
 
 // A work item: the candidates [kb, ke) of the ket class for one bra pair, and
-// of the bra's primitive pairs number s, s + split, ... (J and K are linear in
-// them); sub = class pair + s * 65536.
+// of the primitive pairs of the bra number s % split_ab, + split_ab, ... and of
+// the ket number s / split_ab, + split / split_ab, ... (J and K are linear in
+// them); sub = class pair + s * 2^23 (at most 80 shell types, 5.2 million class
+// pairs, and 256 shares).
 struct alignas(16) JkItem {
     int sub, bra, kb, ke;
 };

@@ -207,7 +207,7 @@ __global__ void __launch_bounds__(256) jk_plan_kernel(const JkPlanArgs args)
         double tlo = T.lo;
         if (T.split_side > 0) {   // as jk_bounds forms it
             const double th =
-                dm < 1e15 ? fmax(args.split_min, __dmul_rn(__dmul_rn(args.split * S.tight, args.mols[m].qmax2), dm)) : 0.0;
+                dm > 1e-15 && dm < 1e15 ? fmax(args.split_min, __dmul_rn(__dmul_rn(args.split * S.tight, args.mols[m].qmax2), dm)) : 0.0;
             tlo = fmax(tlo, th);
         }
         if (args.scr32) {
@@ -243,7 +243,7 @@ __global__ void __launch_bounds__(256) jk_plan_kernel(const JkPlanArgs args)
     for (int k = 0; k < mine; ++k) {
         const int kb = k0 + (c0 + k / S.split * args.part_count) * c;
         JkItem it;
-        it.sub = blk.x + ((k % S.split) << 16);
+        it.sub = blk.x + ((k % S.split) << 23);
         it.bra = i;
         it.kb = kb;
         it.ke = min(k0 + n, kb + c);
