@@ -39,6 +39,15 @@ WORKLOAD = "batched-631gs-64mol"
 # the 1.25 TFLOP/s nominal figure; FP32: 152 x 256 FLOP/clk x 2.07 GHz.
 PEAK_FP64_NOMINAL = 152 * 4 * 2.07e9
 PEAK_FP32_NOMINAL = 152 * 256 * 2.07e9
+# two-float arithmetic (the split tier of FP64): a multiply-add is 12 FP32
+# instructions, 128 lanes per SM
+PEAK_SPLIT_NOMINAL = 2 * 152 * 128 * 2.07e9 / 12
+TIER_PEAK = {0: PEAK_FP64_NOMINAL, 1: PEAK_FP32_NOMINAL, 2: PEAK_SPLIT_NOMINAL}
+TIER_TYPE = {0: "double", 1: "float", 2: "jkdf"}
+TIER_PEAK_SOURCE = {
+    0: "nominal FP64 FMA rate: 152 SMs x 4 FLOP/clk x 2.07 GHz (MEASURED_PEAKS.json has no FP64 figure)",
+    1: "nominal FP32 FMA rate: 152 SMs x 256 FLOP/clk x 2.07 GHz (MEASURED_PEAKS.json has no FP32 figure)",
+    2: "two-float multiply-adds of 12 FP32 instructions each: 152 SMs x 128 lanes x 2.07 GHz / 12 x 2 FLOP"}
 
 # DRAM traffic of the integral kernel family (dram__bytes_read.sum +
 # dram__bytes_write.sum summed over every jk_class_kernel launch of one
@@ -100,7 +109,7 @@ def family_roofline(prof_rows, tier, probe, ms_serial):
     fl = sum(v["flops_model"] for v in rows)
     q = sum(v["quartets"] for v in rows)
     n = sum(v["launches"] for v in rows)
-    peak = PEAK_FP64_NOMINAL if tier == 0 else PEAK_FP32_NOMINAL
+    peak = TIER_PEAK[tier]
     ach = fl / (ms * 1e-3) if ms > 0 else 0.0
     dom = max(rows, key=lambda v: v["ms"])
     traffic = traffic_for(tier, q)
@@ -117,15 +126,12 @@ def family_roofline(prof_rows, tier, probe, ms_serial):
                     "hash %s, now %s), scaled by this step's quartets; not the traffic of the kernels timed here"
                     % (TRAFFIC_CAPTURES[tier][1], sources_sha())} if earlier is not None else None),
         "kernel": "jk_class_kernel<..., %s> (all %d class instantiations of the tier)"
-                  % ("double" if tier == 0 else "float", n),
+                  % (TIER_TYPE[tier], n),
         "launches": n, "launch_ms": ms / n, "kernel_ms": ms,
         "kernel_share": ms / ms_serial if ms_serial else None,
         "flops_per_launch": fl / n,
         "timing": "CUDA events around each launch, serialised replay after the timed region",
-        "peak_source": ("nominal FP64 FMA rate: 152 SMs x 4 FLOP/clk x 2.07 GHz (MEASURED_PEAKS.json has no FP64 "
-                        "figure)" if tier == 0 else
-                        "nominal FP32 FMA rate: 152 SMs x 256 FLOP/clk x 2.07 GHz (MEASURED_PEAKS.json has no FP32 "
-                        "figure)"),
+        "peak_source": TIER_PEAK_SOURCE[tier],
         "peak_probe_tflops": probe / 1e12 if probe else None,
         "frac_of_probe": ach / probe if probe else None,
         "largest_class": {"class": "(%d%d|%d%d)/%d%d%d%d" % (dom["la"], dom["lb"], dom["lc"], dom["ld"], dom["na"],
@@ -352,18 +358,19 @@ def tier_split(eng, Ds, Js, Ks, args, precision):
         eng.set_option("profile", 1)
         eng.set_option("branches", 1)
         _, _, st = eng.build(Ds, cutoff=args.cutoff, precision=precision, J=Js, K=Ks, stats=True)
-        ms = {0: 0.0, 1: 0.0}
-        q = {0: 0, 1: 0}
+        ms = {0: 0.0, 1: 0.0, 2: 0.0}
+        q = {0: 0, 1: 0, 2: 0}
         rows = []
         for p in jk.jk_profile(eng.h):
             ms[p["tier"]] += p["ms"]
             q[p["tier"]] += p["quartets"]
             rows.append(dict(p, launches=1))
-        out = {"fp64_kernels_ms": ms[0], "fp32_kernels_ms": ms[1], "fp64_quartets": q[0], "fp32_quartets": q[1],
+        out = {"fp64_kernels_ms": ms[0], "fp32_kernels_ms": ms[1], "split_kernels_ms": ms[2], "fp64_quartets": q[0],
+               "fp32_quartets": q[1], "split_quartets": q[2],
                "serial_build_ms": st["ms"], "timing": "serialised replay, CUDA events around each class launch"}
         probes = {0: getattr(args, "probe64", None), 1: getattr(args, "probe32", None)}
-        for t, name in ((0, "fp64_tier_roofline"), (1, "fp32_tier_roofline")):
-            out[name] = family_roofline(rows, t, probes[t], st["ms"])
+        for t, name in ((0, "fp64_tier_roofline"), (1, "fp32_tier_roofline"), (2, "split_tier_roofline")):
+            out[name] = family_roofline(rows, t, probes.get(t), st["ms"])
         return out
     except Exception as e:   # a diagnostic, never the reason a run fails
         return {"error": str(e)[:200]}
@@ -642,13 +649,17 @@ def run_ours(args):
         ms_max, q_all = ms_total, float(quartets)
     value = q_all / (ms_max * 1e-3)
 
-    # roofline of the integral kernel family (FP64 FMA pipe)
+    # roofline of the integral kernel family: of an FP64 build, the one of its
+    # two (FP64 instructions, two floats) that takes longer
     args.probe64 = None if args.no_probe else jk.jk_measure_peak("fp64", 100.0)
     args.probe32 = None if args.no_probe else jk.jk_measure_peak("fp32", 100.0)
-    tier = 0 if args.precision == "fp64" else 1
-    roofline = family_roofline(list(prof.values()), tier, args.probe64 if tier == 0 else args.probe32,
-                               ms_serial / args.prof_steps)
-    if args.precision == "mixed":
+    tier = 1
+    if args.precision == "fp64":
+        ms_of = {t: sum(v["ms"] for v in prof.values() if v["tier"] == t) for t in (0, 2)}
+        tier = 2 if ms_of[2] > ms_of[0] else 0
+    probe = {0: args.probe64, 1: args.probe32, 2: None}[tier]
+    roofline = family_roofline(list(prof.values()), tier, probe, ms_serial / args.prof_steps)
+    if args.precision == "mixed" or tier == 2:
         roofline["fp64_tier"] = family_roofline(list(prof.values()), 0, args.probe64, ms_serial / args.prof_steps)
     total_kernel_ms = sum(v["ms"] for v in prof.values())
     all_flops = sum(v["flops_model"] for v in prof.values())
