@@ -287,7 +287,7 @@ int jk_router_gradient(const jk_router_blob *w, const float *X, const float *y, 
  * start-up) owns every byte of device memory and forbids libraries to take
  * more, and training loops that cannot afford cudaMalloc / cudaFree in the
  * step (cudaFree synchronises the whole device).
- *   - Scratch: one fixed __device__ array in the library (about 43 KB,
+ *   - Scratch: one fixed __device__ array in the library (about 65 KB,
  *     present on every GPU that loads the library until the process exits),
  *     holding the weight copies and the accumulators. At most
  *     JK_NOALLOC_MAX_ROWS rows per call; larger n returns JK_ERR_UNSUPPORTED

@@ -2164,14 +2164,14 @@ int check_blob(const jk_router_blob *w)
 // ============================================= no-allocation gradient variant
 // Fixed device scratch for jk_router_gradient_noalloc: the weight copies and the
 // two accumulators of jk_mlp_grad_kernel live in one file-scope __device__ array
-// (43 KB, held by every GPU that loads this library until the process exits)
+// (65 KB, held by every GPU that loads this library until the process exits)
 // instead of buffers from cudaMalloc.
 struct JkGradBuffers {   // mu, isd, theta as in jk_router_blob
     float mu[16], isd[16];
     float theta[JK_RT_NPARAM];
     float pad;
     double loss;
-    float grad[JK_RT_NPARAM];
+    double grad[JK_RT_NPARAM];
 };
 static_assert(offsetof(jk_router_blob, theta) - offsetof(jk_router_blob, mu) == 32 * sizeof(float) &&
                   offsetof(jk_router_blob, isd) - offsetof(jk_router_blob, mu) == 16 * sizeof(float),
@@ -2213,13 +2213,13 @@ int grad_rows(JkGradBuffers *B, const jk_router_blob *w, const float *X, const f
     CK(cudaGetDevice(&dev));
     CK(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
     CK(cudaMemcpyAsync(B->mu, w->mu, sizeof(float) * (32 + JK_RT_NPARAM), cudaMemcpyHostToDevice, st));
-    CK(cudaMemsetAsync(&B->loss, 0, sizeof(double) + sizeof(float) * JK_RT_NPARAM, st));
+    CK(cudaMemsetAsync(&B->loss, 0, sizeof(double) * (1 + JK_RT_NPARAM), st));
     CK(jk_mlp_grad(B->theta, B->mu, B->isd, X, y, (long long)n, (int)n, JK_GRAD_ROWS, quantile, B->grad, &B->loss, sms, st));
-    struct { double loss; float grad[JK_RT_NPARAM]; } out;
-    CK(cudaMemcpyAsync(&out, &B->loss, sizeof(double) + sizeof(float) * JK_RT_NPARAM, cudaMemcpyDeviceToHost, st));
+    struct { double loss, grad[JK_RT_NPARAM]; } out;
+    CK(cudaMemcpyAsync(&out, &B->loss, sizeof out, cudaMemcpyDeviceToHost, st));
     CK(cudaStreamSynchronize(st));
     *loss = out.loss;
-    memcpy(grad_host, out.grad, sizeof(float) * JK_RT_NPARAM);
+    for (int i = 0; i < JK_RT_NPARAM; ++i) grad_host[i] = (float)out.grad[i];
     return JK_OK;
 }
 }  // namespace
@@ -2669,12 +2669,12 @@ int jk_router_train(const float *X, const float *y, int64_t n, const jk_train_op
         for (auto v : hy) m += v;
         th[JK_RT_OFF_B3] = (float)(m / n);
     }
-    float *dth = nullptr, *mu = nullptr, *isd = nullptr, *g = nullptr, *m1 = nullptr, *m2 = nullptr;
-    double *lh = nullptr;
+    float *dth = nullptr, *mu = nullptr, *isd = nullptr, *m1 = nullptr, *m2 = nullptr;
+    double *lh = nullptr, *g = nullptr;
     auto cleanup = [&]() { cudaFree(dth); cudaFree(mu); cudaFree(isd); cudaFree(g); cudaFree(m1); cudaFree(m2); cudaFree(lh); };
     struct Guard { std::function<void()> f; ~Guard() { f(); } } guard{cleanup};
     CK(cudaMalloc(&dth, sizeof(float) * JK_RT_NPARAM));
-    CK(cudaMalloc(&g, sizeof(float) * JK_RT_NPARAM));
+    CK(cudaMalloc(&g, sizeof(double) * JK_RT_NPARAM));
     CK(cudaMalloc(&m1, sizeof(float) * JK_RT_NPARAM));
     CK(cudaMalloc(&m2, sizeof(float) * JK_RT_NPARAM));
     CK(cudaMalloc(&mu, sizeof(float) * 16));
@@ -2690,7 +2690,7 @@ int jk_router_train(const float *X, const float *y, int64_t n, const jk_train_op
     CK(cudaGetDevice(&dev));
     CK(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
     for (int step = 1; step <= opts->steps; ++step) {
-        CK(cudaMemsetAsync(g, 0, sizeof(float) * JK_RT_NPARAM));
+        CK(cudaMemsetAsync(g, 0, sizeof(double) * JK_RT_NPARAM));
         unsigned long long seed = opts->seed * 1000003ull + (unsigned long long)step;
         if (seed == JK_GRAD_ROWS) seed = 0;
         CK(jk_mlp_grad(dth, mu, isd, X, y, (long long)n, opts->batch, seed, opts->quantile, g, lh + (step - 1), sms, 0));

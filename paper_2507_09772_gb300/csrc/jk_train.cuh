@@ -52,7 +52,7 @@ __device__ __forceinline__ unsigned long long jk_mix64(unsigned long long z)
 // Persistent CTAs of 256 threads take tiles of ROWS samples. The three 64 x 64
 // products of a tile (hidden layer 2, its backward pass, the gradient of W2) are
 // FP32 register tiles over shared memory, and the gradients stay in registers
-// (22 per thread) until the CTA's last tile, one atomic per parameter and CTA.
+// (20 per thread) until the CTA's last tile, one FP64 atomic per parameter and CTA.
 // Bound by FP32 FMA issue and shared-memory reads: 50,000 rows are 1.5 GFLOP, 20
 // us at the FP32 peak. A thread per sample, adding each of its 5,313 products to
 // shared memory by atomics that all lanes of a warp aimed at one word, took
@@ -70,7 +70,7 @@ template <int ROWS>
 __global__ void __launch_bounds__(256) jk_mlp_grad_kernel(const float *__restrict__ theta, const float *__restrict__ mu,
                                                           const float *__restrict__ isd, const float *__restrict__ X,
                                                           const float *__restrict__ y, long long n, int batch,
-                                                          unsigned long long seed, float q, float *__restrict__ grad,
+                                                          unsigned long long seed, float q, double *__restrict__ grad,
                                                           double *__restrict__ loss)
 {
     constexpr int H = JK_RT_NH, RT = ROWS / 16;   // rows of a thread's tile
@@ -89,9 +89,12 @@ __global__ void __launch_bounds__(256) jk_mlp_grad_kernel(const float *__restric
         S.b2[tid] = theta[JK_RT_OFF_B2 + tid];
         if (tid == 0) S.b3[0] = theta[JK_RT_OFF_B3];
     }
-    float gw2[4][4] = {}, gw1[3] = {}, gv = 0.0f;   // gv: w3, b2, b1 or (one thread) b3
+    float gw2[4][4] = {}, gw1[3] = {};
+    double gvd = 0.0;   // w3, b2 or b1, summed tile by tile
+    int below = 0, above = 0;   // one thread: rows with a negative residual and the others (b3)
     double lsum = 0.0;
     for (int t0 = blockIdx.x * ROWS; t0 < batch; t0 += gridDim.x * ROWS) {
+        float gv = 0.0f;
         __syncthreads();
         // normalised features, rounded to BF16 (rows past the batch are zero and carry no weight)
         for (int i = tid; i < ROWS * JK_RT_NINP; i += 256) {
@@ -225,7 +228,10 @@ __global__ void __launch_bounds__(256) jk_mlp_grad_kernel(const float *__restric
             for (int r = 0; r < ROWS; ++r) gv += S.d[r][tid - 64];
         } else if (tid == 192) {
 #pragma unroll 4
-            for (int r = 0; r < ROWS; ++r) gv += S.g[r];
+            for (int r = 0; r < ROWS; ++r) {
+                below += S.g[r] > 0.0f;
+                above += S.g[r] < 0.0f;
+            }
         }
         // delta of layer 1, into h2
         float dh[RT][4] = {};
@@ -263,20 +269,24 @@ __global__ void __launch_bounds__(256) jk_mlp_grad_kernel(const float *__restric
                 if (tid >= 128 && tid < 192) gv += d;
             }
         }
+        gvd += (double)gv;
     }
-    // one atomic per parameter and CTA
+    // b3: the derivative has two values, 1 - q and -q over the batch, which FP32
+    // would add with the same rounding error every time
+    if (tid == 192) gvd = (double)below * (double)((1.0f - q) / (float)batch) - (double)above * (double)(q / (float)batch);
+    // one FP64 atomic per parameter and CTA
 #pragma unroll
     for (int i = 0; i < 4; ++i)
 #pragma unroll
         for (int j = 0; j < 4; ++j)
-            if (gw2[i][j] != 0.0f) atomicAdd(&grad[JK_RT_OFF_W2 + (4 * ty + i) * H + 4 * tx + j], gw2[i][j]);
+            if (gw2[i][j] != 0.0f) atomicAdd(&grad[JK_RT_OFF_W2 + (4 * ty + i) * H + 4 * tx + j], (double)gw2[i][j]);
 #pragma unroll
     for (int k = 0; k < 3; ++k)
-        if (gw1[k] != 0.0f) atomicAdd(&grad[JK_RT_OFF_W1 + (3 * (tid >> 6) + k) * H + (tid & 63)], gw1[k]);
-    if (gv != 0.0f) {
+        if (gw1[k] != 0.0f) atomicAdd(&grad[JK_RT_OFF_W1 + (3 * (tid >> 6) + k) * H + (tid & 63)], (double)gw1[k]);
+    if (gvd != 0.0) {
         const int at = tid < 64 ? JK_RT_OFF_W3 + tid
                                 : (tid < 128 ? JK_RT_OFF_B2 + tid - 64 : (tid < 192 ? JK_RT_OFF_B1 + tid - 128 : JK_RT_OFF_B3));
-        atomicAdd(&grad[at], gv);
+        atomicAdd(&grad[at], gvd);
     }
     for (int o = 16; o > 0; o >>= 1) lsum += __shfl_xor_sync(0xffffffffu, lsum, o);
     if ((tid & 31) == 0 && lsum != 0.0) atomicAdd(loss, lsum / batch);
@@ -285,7 +295,7 @@ __global__ void __launch_bounds__(256) jk_mlp_grad_kernel(const float *__restric
 // Tiles of 64 rows where they fill the GPU (more arithmetic per shared-memory
 // read), of 16 below (a training step of 4,096 samples is 256 of them).
 static cudaError_t jk_mlp_grad(const float *theta, const float *mu, const float *isd, const float *X, const float *y,
-                               long long n, int batch, unsigned long long seed, float q, float *grad, double *loss,
+                               long long n, int batch, unsigned long long seed, float q, double *grad, double *loss,
                                int sms, cudaStream_t st)
 {
     if ((batch + 63) / 64 >= sms) {
@@ -304,12 +314,12 @@ static cudaError_t jk_mlp_grad(const float *theta, const float *mu, const float 
     return cudaGetLastError();
 }
 
-__global__ void jk_adam_kernel(float *__restrict__ theta, const float *__restrict__ grad, float *__restrict__ m1,
+__global__ void jk_adam_kernel(float *__restrict__ theta, const double *__restrict__ grad, float *__restrict__ m1,
                                float *__restrict__ m2, int step, float lr, float b1, float b2, float eps)
 {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= JK_RT_NPARAM) return;
-    const float g = grad[i];
+    const float g = (float)grad[i];
     const float a = b1 * m1[i] + (1.0f - b1) * g;
     const float v = b2 * m2[i] + (1.0f - b2) * g * g;
     m1[i] = a;
