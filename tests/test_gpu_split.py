@@ -94,3 +94,26 @@ def test_a_basis_outside_the_fp32_range_stays_in_fp64():
     (J1, K1), n1 = build(mol, 1.0)
     assert n0 == n1
     assert np.abs(J1 - J0).max() <= 1e-13 * np.abs(J0).max() and np.abs(K1 - K0).max() <= 1e-13 * np.abs(K0).max()
+
+
+@pytest.mark.parametrize("split", [1.0, 1.0 / 128])
+def test_a_nan_in_the_density_stays_one(split):
+    """A queued build of a density with a NaN leaves NaN wherever the all-FP64
+    build does, nothing finite in its place, and the error word is raised."""
+    mol = synth.batched_molecule(4, natm=10)
+    mol.D = mol.D.copy()
+    mol.D[0, 5, 11] = mol.D[0, 11, 5] = np.nan
+    got = []
+    for s in (0.0, split):
+        eng = jk.JK(mol)
+        eng.set_option("split", s)
+        J, K, _ = eng.build(torch.tensor(mol.D, dtype=torch.float64, device="cuda"), cutoff=1e-13, check=False)
+        with pytest.raises(jk.JKError):
+            jk.jk_check(eng.h)
+        got.append((J.cpu().numpy(), K.cpu().numpy()))
+        eng.close()
+    for a, b in zip(*got):
+        assert not np.isfinite(a).all()
+        assert (np.isfinite(a) == np.isfinite(b)).all()
+        m = np.isfinite(a)
+        assert np.abs(a - b)[m].max(initial=0.0) <= 1e-10
