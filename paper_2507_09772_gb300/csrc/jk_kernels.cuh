@@ -761,18 +761,17 @@ __device__ __forceinline__ bool jk_route_out(const JkClassArgs &args, int launch
 // ------------------------------------------------- screening of a candidate
 // The bounds of a tier for one molecule (FP64 and rounded to FP32): the split
 // threshold follows the molecule's largest density element, and is formed
-// alike by every launch of a build.
+// alike by every launch of a build. dreal: the largest |D|, also where the
+// screening takes 1 for it (dmol).
 struct JkBounds {
     double lo, hi;
     float lo32, hi32;
 };
-__device__ __forceinline__ JkBounds jk_bounds(const JkClassArgs &args, const JkMol &mol, double dmol)
+__device__ __forceinline__ JkBounds jk_bounds(const JkClassArgs &args, const JkMol &mol, double dmol, double dreal)
 {
     JkBounds b = {args.lo, args.hi, args.lo32, args.hi32};
     if (args.split_side != 0) {
-        // (densities near the ends of the FP32 range, or not finite, stay in FP64)
-        const double th =
-            dmol > 1e-15 && dmol < 1e15 ? fmax(args.split_min, __dmul_rn(__dmul_rn(args.split, mol.qmax2), dmol)) : 0.0;
+        const double th = jk_split_threshold(args.split, args.split_min, mol.qmax2, dmol, dreal);
         if (args.split_side > 0 && th > b.lo) { b.lo = th; b.lo32 = (float)th; }
         if (args.split_side < 0 && th < b.hi) { b.hi = th; b.hi32 = (float)th; }
     }
@@ -1256,9 +1255,9 @@ jk_class_kernel(const JkClassArgs args)
             const typename JkRecOf<R>::T brec = JkRecOf<R>::bra(sub, item);
             const JkMol mol = args.mols[bra.mol];
             const double *dmx = args.dmax + mol.dmax_off;
-            const double dmol = args.use_dmax ? args.dmax_mol[bra.mol] : 1.0;
+            const double dreal = args.dmax_mol[bra.mol], dmol = args.use_dmax ? dreal : 1.0;
             const float dmol32 = (float)dmol;
-            const JkBounds bd = jk_bounds(args, mol, dmol);
+            const JkBounds bd = jk_bounds(args, mol, dmol, dreal);
             const int a0 = bra.a_ao + ga * FA, b0 = bra.b_ao + gb * FB;
             JkPairFeat braf;
             if (MODE != 0) braf = sub.bra_feat[item];
@@ -1485,9 +1484,9 @@ jk_class_kernel(const JkClassArgs args)
             const typename JkRecOf<R>::T brec = JkRecOf<R>::bra(sub, item);
             const JkMol mol = args.mols[bra.mol];
             const double *dmx = args.dmax + mol.dmax_off;
-            const double dmol = args.use_dmax ? args.dmax_mol[bra.mol] : 1.0;
+            const double dreal = args.dmax_mol[bra.mol], dmol = args.use_dmax ? dreal : 1.0;
             const float dmol32 = (float)dmol;
-            const JkBounds bd = jk_bounds(args, mol, dmol);
+            const JkBounds bd = jk_bounds(args, mol, dmol, dreal);
             const int a0 = bra.a_ao + ga * FA, b0 = bra.b_ao + gb * FB;
             JkPairFeat braf;
             if (MODE != 0) braf = sub.bra_feat[item];

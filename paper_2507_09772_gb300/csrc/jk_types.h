@@ -86,6 +86,19 @@ struct JkMol {
 struct JkRouterDev;
 struct JkPairFeat;
 
+// Bound up to which a molecule's FP64-tier quartets run in two floats: split x
+// max Q^2 x the largest density element the screening uses (dmol), at least
+// split_min; 0 (none) where the largest |D| itself (dreal; infinite for a
+// density that is not finite) or the largest product with an integral is not
+// well inside the FP32 range: sums of products of integrals and density
+// elements are formed in it, and halves below 1.2e-38 are lost.
+__device__ __forceinline__ double jk_split_threshold(double split, double split_min, double qmax2, double dmol, double dreal)
+{
+    const double s = qmax2 * dreal;
+    if (!(dreal > 1e-15 && dreal < 1e15 && s > 1e-20 && s < 1e30)) return 0.0;
+    return fmax(split_min, __dmul_rn(__dmul_rn(split, qmax2), dmol));
+}
+
 // One class pair (bra pair class, ket pair class) of a launch. A launch runs
 // every class pair that shares a kernel (angular momenta and fragment shape),
 // whatever its primitive counts.

@@ -89,7 +89,8 @@ __global__ void jk_dmax_kernel(const JkMol *__restrict__ mols, const int *__rest
                     bad = bad || !(v <= 1.7976931348623157e308);   // NaN or infinity
                     mx = fmax(mx, v);
                 }
-        if (bad) atomicOr(err, JK_ERR_DEV_NAN);
+        // (the maxima drop NaN: an infinite molecule maximum keeps it in sight of the split tier)
+        if (bad) { atomicOr(err, JK_ERR_DEV_NAN); rowmax = __longlong_as_double(0x7ff0000000000000ll); }
         dmax[mol.dmax_off + (long long)a * mol.nsh + b] = mx;
         dmax32[mol.dmax_off + (long long)a * mol.nsh + b] = (float)mx;
         rowmax = fmax(rowmax, mx);
@@ -205,11 +206,8 @@ __global__ void __launch_bounds__(256) jk_plan_kernel(const JkPlanArgs args)
         int lo = k0, hi = S.ket_end[m];
         const double dm = args.use_dmax ? args.dmax_mol[m] : 1.0;
         double tlo = T.lo;
-        if (T.split_side > 0) {   // as jk_bounds forms it
-            const double th =
-                dm > 1e-15 && dm < 1e15 ? fmax(args.split_min, __dmul_rn(__dmul_rn(args.split * S.tight, args.mols[m].qmax2), dm)) : 0.0;
-            tlo = fmax(tlo, th);
-        }
+        if (T.split_side > 0)   // as jk_bounds forms it
+            tlo = fmax(tlo, jk_split_threshold(args.split * S.tight, args.split_min, args.mols[m].qmax2, dm, args.dmax_mol[m]));
         if (args.scr32) {
             const JkKetScr *ks = S.ket_scr;
             const float f = b.Qf * (float)dm, thr = (float)tlo * (1.0f - 4e-6f);

@@ -117,3 +117,25 @@ def test_a_nan_in_the_density_stays_one(split):
         assert (np.isfinite(a) == np.isfinite(b)).all()
         m = np.isfinite(a)
         assert np.abs(a - b)[m].max(initial=0.0) <= 1e-10
+
+
+@pytest.mark.parametrize("scale", [1e-34, 1e-22, 1e18, 1e37])
+@pytest.mark.parametrize("use_dmax", [0, 1])
+def test_densities_near_the_ends_of_the_fp32_range(scale, use_dmax):
+    """Whatever the screening takes for the density's size, a density outside
+    1e-15 .. 1e15 is built in FP64 instructions: the same result but for the
+    order of the sums (1e-13 of the largest element)."""
+    mol = synth.tiny_631gs()
+    mol.D = mol.D * scale
+    eng = jk.JK(mol)
+    D = torch.tensor(mol.D, dtype=torch.float64, device="cuda")
+    eng.set_option("use_dmax", use_dmax)
+    got = []
+    for split in (0.0, 1.0):
+        eng.set_option("split", split)
+        J, K, st = eng.build(D, cutoff=1e-13 if scale > 1 or not use_dmax else 1e-28, stats=True)
+        got.append((J.cpu().numpy() / scale, K.cpu().numpy() / scale, st["quartets_fp64"]))
+    eng.close()
+    assert got[0][2] == got[1][2]
+    for a, b in zip(got[0][:2], got[1][:2]):
+        assert np.isfinite(b).all() and np.abs(a - b).max() <= 1e-13 * max(1.0, np.abs(a).max())
