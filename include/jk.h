@@ -217,8 +217,9 @@ int jk_build_batch(jk_handle *h, const double *const *D, int32_t n_dm, int with_
  * evaluated in pairs of FP32 numbers (48 bits, relative error about 1e-14), which
  * the GPU does several times faster; the error this adds is below the one the
  * result has from the cutoff. They count as FP64 quartets.
- * 0: FP64 instructions for every FP64-tier quartet, as for cutoffs below 1e-30
- * and for bases with exponents outside (1e-6, 1e8)),
+ * 0: FP64 instructions for every FP64-tier quartet, as for cutoffs below 1e-30,
+ * for |omega| outside 1e-6 .. 1e6 (and not 0), and for bases with exponents
+ * outside (1e-6, 1e8)),
  * "route_cap" (default 16777216: initial entries of the per-class-pair lists
  * of quartets the router releases from the FP64 tier, shared out by
  * candidate count; a list that overflowed in a build with stats is grown

@@ -963,6 +963,16 @@ void drop_graphs(jk_handle *h)
     h->graphs.clear();
 }
 
+// Whether a build evaluates FP64-tier quartets in two floats: not where its
+// cutoff or its operator leave the FP32 range. theta = w^2 / (w^2 + rho), with
+// rho in 1e-6 .. 1e8, keeps 48 bits for |w| in 1e-6 .. 1e6; w^2 overflows from
+// 1.9e19 on, and the residual of the square root's estimate is lost from 1e16.
+bool uses_two_floats(const jk_handle *h, int mode, double cutoff)
+{
+    const double w = std::fabs(h->omega);
+    return mode != JK_PREC_FP32 && h->split > 0 && h->df_ok && cutoff >= 1e-30 && (w == 0 || (w >= 1e-6 && w <= 1e6));
+}
+
 double split_factor(const KSpec &s)
 {
     return std::max(std::max(s.la, s.lb), std::max(s.lc, s.ld)) > 2 ? JK_SPLIT_F : 1.0;
@@ -1681,7 +1691,7 @@ int build_impl(jk_handle *h, const double *const *D, int32_t ndm, int with_j, in
     const int merge = prof ? 0 : 1;
     const int op = h->omega == 0.0 ? 0 : (h->omega > 0.0 ? 1 : 2);
     const bool use32 = mode != JK_PREC_FP64;
-    const bool usedf = mode != JK_PREC_FP32 && h->split > 0 && h->df_ok && !logs && cutoff >= 1e-30;
+    const bool usedf = !logs && uses_two_floats(h, mode, cutoff);
     static const int spec_of[4] = {0, 1, 1, 2}, ctr_of[4] = {0, 1, 1, 2};
     struct Tier { int t; TierPlan *P; std::vector<KInfo> *ki; };
     std::vector<Tier> tiers;
@@ -2241,7 +2251,7 @@ int tune_impl(jk_handle *h, const double *const *D, int32_t ndm, int with_j, int
     if (ndm < 1 || ndm > JK_NDM_MAX) return fail(JK_ERR_ARG, "bad n_dm");
     const auto t0 = std::chrono::steady_clock::now();
     const bool two = mode == JK_PREC_MIXED || mode == JK_PREC_MIXED_ROUTED;
-    const bool usedf = mode != JK_PREC_FP32 && h->split > 0 && h->df_ok && cutoff >= 1e-30;
+    const bool usedf = uses_two_floats(h, mode, cutoff);
     std::vector<int> tiers;   // shapes: FP64, FP32, two floats
     if (mode == JK_PREC_FP64 || two) tiers.push_back(0);
     if (mode == JK_PREC_FP32 || two) tiers.push_back(1);

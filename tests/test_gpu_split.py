@@ -139,3 +139,18 @@ def test_densities_near_the_ends_of_the_fp32_range(scale, use_dmax):
     assert got[0][2] == got[1][2]
     for a, b in zip(got[0][:2], got[1][:2]):
         assert np.isfinite(b).all() and np.abs(a - b).max() <= 1e-13 * max(1.0, np.abs(a).max())
+
+
+@pytest.mark.parametrize("omega", [1e-40, 1e-9, 1e-6, 1e6, -1e6, 1e16, 1e17, 2e19, -2e19, 1e100])
+def test_range_separation_at_the_ends_of_the_fp32_range(omega):
+    """omega^2 enters the roots of erf(omega r)/r: where FP32 cannot hold it to
+    48 bits the build takes FP64 instructions."""
+    mol = synth.tiny_631gs()
+    (J0, K0), n0 = build(mol, 0.0, {"omega": omega})
+    (J1, K1), n1 = build(mol, 1.0, {"omega": omega})
+    assert n0 == n1
+    for a, b in ((J0, J1), (K0, K1)):
+        # erfc is the difference of 1/r (|J| and |K| up to 50) and erf
+        top = 50.0 if omega < 0 else np.abs(a).max()
+        # in range: two floats (1e-10 of |J| up to 50); outside: the order of the sums
+        assert np.isfinite(b).all() and np.abs(a - b).max() <= (2e-12 if 1e-6 <= abs(omega) <= 1e6 else 1e-13) * top
