@@ -218,8 +218,9 @@ int jk_build_batch(jk_handle *h, const double *const *D, int32_t n_dm, int with_
  * the GPU does several times faster; the error this adds is below the one the
  * result has from the cutoff. They count as FP64 quartets.
  * 0: FP64 instructions for every FP64-tier quartet, as for cutoffs below 1e-30,
- * for |omega| outside 1e-6 .. 1e6 (and not 0), and for bases with exponents
- * outside (1e-6, 1e8)),
+ * for |omega| outside 1e-6 .. 1e6 (and not 0), and for molecules whose
+ * exponents lie outside (1e-6, 1e8) or whose integrals pass through numbers far
+ * from 1 (diffuse g shells with unnormalised coefficients, for instance)),
  * "route_cap" (default 16777216: initial entries of the per-class-pair lists
  * of quartets the router releases from the FP64 tier, shared out by
  * candidate count; a list that overflowed in a build with stats is grown

@@ -795,7 +795,7 @@ struct jk_handle {
     std::vector<jk_shell> shells;
     std::vector<int> mol_sh0;              // nmol + 1
     std::vector<int> nao_cart, nao_user;   // per molecule
-    std::vector<double> mol_qmax2;         // largest Q squared
+    std::vector<double> mol_qmax2;         // largest Q squared (0: the molecule stays out of the split tier)
     std::vector<int> sh_ao_cart;           // molecule-local Cartesian AO offset per shell
     bool spherical = false;
     // device
@@ -872,7 +872,7 @@ struct jk_handle {
     std::vector<long long> rl_need;        // entries each list needed in the last build with stats
     double route_cap = 16777216.0;         // list entries over all launches
     double split = JK_SPLIT;               // split threshold; 0: every quartet of the FP64 tier in FP64 instructions
-    bool df_ok = true;                     // the basis stays far inside the FP32 range
+    bool df_ok = false;                    // some molecule's basis stays far inside the FP32 range
     int asym64 = 0;                        // FP32 tier: large-T roots and weights in FP64
     int chunk = JK_CHUNK;                  // kets per work item
     // FP32 tier: float-to-double by integer operations (1) or by the
@@ -1134,6 +1134,45 @@ int plan_kernels(jk_handle *h, TierPlan *P, int ndm, int doj, int dok, int mode,
     return JK_OK;
 }
 
+// Clears the largest Q of the molecules whose integrals two floats cannot hold
+// (all their quartets then stay in FP64 instructions). A table entry of a pair
+// is a product of at most l_a + l_b lengths, |A - B| and a few 1/sqrt(p), and
+// a prefactor 35 K K' / sqrt(p + q) at most f f' with f = 5 K / p^(1/4), so an
+// intermediate of a quartet is at most about size size' with size = max(1, f)
+// max(1, length)^(l_a + l_b). It must stay below 1e30, and what an underflow
+// loses (1.4e-45, times at most size size') below 2^-53 of the largest integral.
+// size size' is 1e14 for 6-31G* shapes, 6e15 with f shells, 4e23 for g shells of exponent 0.3.
+void two_float_range(jk_handle *h, const double *coords, const double *exps, const double *coeffs)
+{
+    struct Shell { double amin = INFINITY, cmax = 0; bool ok = true; };
+    std::vector<Shell> sh(h->nshell);
+    for (int s = 0; s < h->nshell; ++s) {
+        const jk_shell &x = h->shells[s];
+        for (int i = x.prim_off; i < x.prim_off + x.nprim; ++i) {
+            const double c = std::fabs(coeffs[i]);
+            sh[s].amin = std::min(sh[s].amin, exps[i]);
+            sh[s].cmax = std::max(sh[s].cmax, c);
+            sh[s].ok = sh[s].ok && exps[i] > 1e-6 && exps[i] < 1e8 && c < 1e8 && (c == 0 || c > 1e-8);
+        }
+        for (int ax = 0; ax < 3; ++ax) sh[s].ok = sh[s].ok && std::fabs(coords[3 * x.atom + ax]) < 1e5;
+    }
+    std::vector<double> size(h->nmol, 1.0);
+    for (auto &p : h->h_pairs) {
+        const Shell &A = sh[p.a], &B = sh[p.b];
+        const double pmin = A.amin + B.amin, f = 5.0 * A.cmax * B.cmax / (pmin * std::sqrt(std::sqrt(pmin)));
+        const double ab = std::sqrt(p.ABx * p.ABx + p.ABy * p.ABy + p.ABz * p.ABz);
+        const double len = 1.2 * ab + 4.0 / std::sqrt(pmin);
+        const double v = std::max(1.0, f) * std::pow(std::max(1.0, len), h->shells[p.a].l + h->shells[p.b].l);
+        size[p.mol] = std::max(size[p.mol], A.ok && B.ok ? v : INFINITY);
+    }
+    h->df_ok = false;
+    for (int m = 0; m < h->nmol; ++m) {
+        const double u = size[m] * size[m];
+        if (!(u < 1e30 && u < 1e27 * h->mol_qmax2[m])) h->mol_qmax2[m] = 0;
+        h->df_ok = h->df_ok || h->mol_qmax2[m] > 0;
+    }
+}
+
 int init_impl(int32_t nmol, const int32_t *mol_shell_off, const jk_shell *shells, int32_t nshell,
               const double *coords, int32_t natm, const double *exps, const double *coeffs,
               int32_t nprim_total, jk_handle **out)
@@ -1377,12 +1416,7 @@ int init_impl(int32_t nmol, const int32_t *mol_shell_off, const jk_shell *shells
     }
     h->mol_qmax2.assign(nmol, 0.0);
     for (auto &p : h->h_pairs) h->mol_qmax2[p.mol] = std::max(h->mol_qmax2[p.mol], p.Q * p.Q);
-    // two floats need every intermediate well inside the FP32 range
-    for (int i = 0; i < nprim_total; ++i) {
-        const double c = std::fabs(coeffs[i]);
-        h->df_ok = h->df_ok && exps[i] > 1e-6 && exps[i] < 1e8 && c < 1e8 && (c == 0 || c > 1e-8);
-    }
-    for (int i = 0; i < 3 * natm; ++i) h->df_ok = h->df_ok && std::fabs(coords[i]) < 1e5;
+    two_float_range(h.get(), coords, exps, coeffs);
     // ---- primitive-pair Schwarz factors: the Schwarz kernel of each pair
     // class on single-primitive pseudo pairs (same centres, pp_off pointing
     // at one primitive pair), then every shell pair's primitive pairs sorted

@@ -74,7 +74,7 @@ struct alignas(16) JkPrimPairDf {
 struct JkMol {
     const double *D;   // n_dm x nao x nao (Cartesian)
     const float2 *D2;  // the same as two floats, read by the split tier (nullptr when it does not run)
-    double qmax2;      // largest Q squared
+    double qmax2;      // largest Q squared (0: no quartets in two floats)
     const float *D32;  // the same rounded to FP32, read by the FP32 tier (nullptr when it does not run)
     double *J;         // half-matrix accumulator X, symmetrised after the build
     double *K;         // half-matrix accumulator Y

@@ -154,3 +154,43 @@ def test_range_separation_at_the_ends_of_the_fp32_range(omega):
         top = 50.0 if omega < 0 else np.abs(a).max()
         # in range: two floats (1e-10 of |J| up to 50); outside: the order of the sums
         assert np.isfinite(b).all() and np.abs(a - b).max() <= (2e-12 if 1e-6 <= abs(omega) <= 1e6 else 1e-13) * top
+
+
+def two_float_quartets(mol):
+    eng = jk.JK(mol)
+    try:
+        eng.set_option("profile", 1)
+        eng.build(torch.tensor(mol.D, dtype=torch.float64, device="cuda"), cutoff=1e-13, stats=True)
+        return sum(p["quartets"] for p in jk.jk_profile(eng.h) if p["tier"] == 2)
+    finally:
+        eng.close()
+
+
+@pytest.mark.parametrize("alpha,coef", [(1.1e-5, 2e-8), (1.1e-5, 1e-7), (3e-6, 9e7)])
+def test_intermediates_beyond_the_fp32_range_stay_in_fp64(alpha, coef):
+    """A diffuse g shell passes (1 / 2p)^8 in one table entry, 3e41 here, although
+    its integrals and the products with the density are in range."""
+    rng = np.random.default_rng(8)
+    mol = synth.custom_basis_molecule(np.array([[0.0, 0, 0], [40.0, 5.0, -9.0]]), [[(4, [alpha]), (0, [0.4])]] * 2, rng)
+    mol.coeffs = np.where(mol.exps < 1e-3, coef, mol.coeffs)
+    (J0, K0), n0 = build(mol, 0.0)
+    (J1, K1), n1 = build(mol, 1.0)
+    assert n0 == n1 and two_float_quartets(mol) == 0
+    for a, b in ((J0, J1), (K0, K1)):
+        assert np.isfinite(b).all() and np.abs(a - b).max() <= 1e-13 * np.abs(a).max()
+
+
+@pytest.mark.parametrize("name", ["tiny", "spherical", "g", "batch"])
+def test_ordinary_bases_take_two_floats(name):
+    mol = synth.batched_molecule(3, natm=12) if name == "batch" else CASES[name]()[0]
+    assert two_float_quartets(mol) > 0
+
+
+def test_the_range_is_judged_molecule_by_molecule():
+    rng = np.random.default_rng(8)
+    wide = synth.custom_basis_molecule(np.array([[0.0, 0, 0], [1.2, 0, 0.3]]), [[(0, [3e8]), (0, [0.7]), (1, [1.1])]] * 2, rng)
+    eng = jk.JK([wide, synth.batched_molecule(3, natm=6)])
+    eng.set_option("profile", 1)
+    eng.build([torch.tensor(m.D, dtype=torch.float64, device="cuda") for m in (wide, synth.batched_molecule(3, natm=6))], stats=True)
+    assert sum(p["quartets"] for p in jk.jk_profile(eng.h) if p["tier"] == 2) > 0
+    eng.close()
