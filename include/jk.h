@@ -188,9 +188,10 @@ int jk_build_batch(jk_handle *h, const double *const *D, int32_t n_dm, int with_
  * "prim_eps" (primitive quartets with q_ij q_kl Dmax <= min(prim_eps,
  * cutoff) are skipped; q is the primitive-pair Schwarz factor; default 1e-16),
  * "part_count", "part_index" (a build computes only part part_index of
- * part_count of every class kernel's work, every part_count-th work item; J and K are then partial sums
- * whose sum over the parts is the full result, i.e. one sum all-reduce
- * combines GPUs that split one batch),
+ * part_count of every class kernel's work, every part_count-th bra pair; J and
+ * K are then partial sums whose sum over the parts is the full result, i.e.
+ * one sum all-reduce combines GPUs that split one batch. Ranks may tune, chunk
+ * and profile by themselves; tau32, split, cutoff and the like must agree),
  * "branches" (1..8: streams / graph branches of a profiled build's class
  * kernels; other builds spread them over 24),
  * "chunk" (32..65536, default 64: candidate kets per work item of the

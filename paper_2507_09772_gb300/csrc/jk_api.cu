@@ -1078,6 +1078,7 @@ int tier_plan(jk_handle *h, int t, int hi, int merge, int whole, TierPlan **out)
                 S.chunk = (int)c;
                 S.group = (int)k;
                 S.launch = l;
+                S.seed = (L.c1 + L.c2) % 65536;   // of the basis alone; not the order by cost
                 S.tight = split_factor(L.spec[t]);
                 for (int m = 0; m < h->nmol; ++m) {
                     const long long nb = A.end[m] - A.beg[m], nk = B.end[m] - B.beg[m];

@@ -118,6 +118,7 @@ struct JkSub {
     int split, split_ab;         // work items that share the primitive quartets: in all, and by the bra's pairs
     int group;                   // launch it belongs to
     int launch;                  // class pair index: statistics, routed lists
+    int seed;                    // bra i belongs to part (i + seed) % part_count of a partitioned build
     double tight;                // factor of the split threshold for its angular momenta
 };
 

@@ -187,10 +187,11 @@ struct JkPlanArgs {
 // does the list). Listing the items per build, from this build's density and
 // thresholds, instead of once from Q alone leaves no empty items: in the FP64
 // tier of a mixed build most (bra, chunk) combinations have no candidate. A
-// partitioned build keeps every part_count-th chunk, counted so that the
-// choice depends on the pair indices only. The FP32 bound is taken 4e-6 low
-// (it carries at most four roundings, 2.4e-7), so no candidate is lost; the
-// class kernels decide each one exactly.
+// partitioned build keeps every part_count-th bra of a class pair: which part
+// a quartet belongs to depends on the sorted pair lists alone, not on chunks
+// or fragment shapes, which ranks that tuned by themselves do not share. The
+// FP32 bound is taken 4e-6 low (it carries at most four roundings, 2.4e-7), so
+// no candidate is lost; the class kernels decide each one exactly.
 __global__ void __launch_bounds__(256) jk_plan_kernel(const JkPlanArgs args)
 {
     const JkPlanTier T = blockIdx.y == 0 ? args.tier[0] : (blockIdx.y == 1 ? args.tier[1] : args.tier[2]);
@@ -199,7 +200,7 @@ __global__ void __launch_bounds__(256) jk_plan_kernel(const JkPlanArgs args)
     const JkSub &S = T.subs[blk.x];
     const int i = blk.y + threadIdx.x, lane = threadIdx.x & 31;
     int k0 = 0, n = 0;
-    if (i < S.nbra) {
+    if (i < S.nbra && (i + S.seed) % args.part_count == args.part_index) {
         const JkPair &b = S.bra[i];
         const int m = b.mol;
         k0 = S.same_class ? i : S.ket_beg[m];
@@ -223,10 +224,7 @@ __global__ void __launch_bounds__(256) jk_plan_kernel(const JkPlanArgs args)
         }
         n = lo - k0;
     }
-    const int c = S.chunk, nch = (n + c - 1) / c;
-    // chunks of this part: c0, c0 + part_count, ...
-    const int c0 = (args.part_index + args.part_count - (i + S.launch) % args.part_count) % args.part_count;
-    const int mine = nch > c0 ? (nch - c0 + args.part_count - 1) / args.part_count * S.split : 0;
+    const int c = S.chunk, mine = (n + c - 1) / c * S.split;
     int pre = mine;
 #pragma unroll
     for (int o = 1; o < 32; o <<= 1) {
@@ -239,7 +237,7 @@ __global__ void __launch_bounds__(256) jk_plan_kernel(const JkPlanArgs args)
     base = __shfl_sync(0xffffffffu, base, 31);
     JkItem *out = T.items + T.item_off[S.group] + base + (pre - mine);
     for (int k = 0; k < mine; ++k) {
-        const int kb = k0 + (c0 + k / S.split * args.part_count) * c;
+        const int kb = k0 + k / S.split * c;
         JkItem it;
         it.sub = blk.x + ((k % S.split) << 23);
         it.bra = i;

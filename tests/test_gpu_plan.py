@@ -1,6 +1,8 @@
 """GPU: the work items of a build (jk_plan_kernel) cover every candidate once,
 whatever the chunk, the partition and the grouping of class pairs into
 launches, at the edges of their ranges."""
+import itertools
+
 import numpy as np
 import pytest
 
@@ -71,3 +73,44 @@ def test_item_bound_follows_the_density(case, scale, use_dmax):
     assert st["quartets_fp64"] == nq
     assert np.abs(J.cpu().numpy() - Jr).max() <= 1e-10 * max(scale, 1e-3)
     assert np.abs(K.cpu().numpy() - Kr).max() <= 1e-10 * max(scale, 1e-3)
+
+
+def tuning_table(path):
+    """Other shapes for the s and p classes than the built-in rule's, as another rank's autotuner might have stored."""
+    p = torch.cuda.get_device_properties(0)
+    name = "".join(c if c.isalnum() and c.isascii() else "_" for c in p.name)
+    shape = {"1010": "3 1 1 1", "1011": "1 1 3 1", "1110": "3 1 1 1", "1100": "3 1 1 1", "1000": "3 1 1 1"}
+    prims = [1, 3, 6]
+    with open(path / f"tune_{name}_sm{p.major}{p.minor}_{p.multi_processor_count}.txt", "w") as f:
+        for k, v in shape.items():
+            for n in itertools.product(prims, repeat=4):
+                for t in (0, 1, 2):
+                    f.write("%s/%d_%d_%d_%d/%d %s\n" % (k, *n, t, v))
+
+
+@pytest.mark.parametrize("precision", ["fp64", "mixed"])
+def test_parts_of_differently_tuned_handles_sum_to_the_build(case, precision, tmp_path, monkeypatch):
+    """Ranks tune, chunk and profile by themselves: the parts still hold every quartet once."""
+    mol, Jr, Kr, nq = case
+    J = K = n = 0
+    shapes = []
+    for part in range(3):
+        where = tmp_path / str(part)
+        where.mkdir()
+        if part == 1:
+            tuning_table(where)
+        monkeypatch.setenv("JK_TUNING_DIR", str(where))
+        eng = jk.JK(mol)
+        for k, v in {"part_count": 3, "part_index": part, "profile": int(part == 2), "chunk": 41 if part == 2 else 64}.items():
+            eng.set_option(k, v)
+        j, k, st = eng.build(torch.tensor(mol.D, dtype=torch.float64, device="cuda"), cutoff=1e-13, precision=precision,
+                             stats=True)
+        J, K, n = J + j.cpu().numpy(), K + k.cpu().numpy(), n + st["quartets_fp64"] + st["quartets_fp32"]
+        eng.set_option("profile", 1)
+        eng.build(torch.tensor(mol.D, dtype=torch.float64, device="cuda"), precision=precision, stats=True)
+        shapes.append({(p["la"], p["lb"], p["lc"], p["ld"], p["tier"]): p["threads_per_quartet"] for p in jk.jk_profile(eng.h)})
+        eng.close()
+    assert shapes[1] != shapes[0]     # the table took effect
+    assert n == nq
+    tol = 1e-10 if precision == "fp64" else 1e-8
+    assert np.abs(J - Jr).max() <= tol and np.abs(K - Kr).max() <= tol
