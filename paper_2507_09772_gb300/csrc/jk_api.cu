@@ -9,6 +9,7 @@
 // coefficients, D) are device arrays. Screening (eq:schwartz, and the
 // density-matrix bound of Sec. 2) happens inside the kernels.
 #include "jk.h"
+#include "jk_grow.h"
 #include "jk_types.h"
 #include "jk_util.cuh"
 #include "jk_train.cuh"
@@ -851,15 +852,13 @@ struct jk_handle {
     std::vector<int> sh_ao_user;           // molecule-local AO offset in the caller's basis
     int *d_sh_l = nullptr, *d_sh_sph = nullptr, *d_sh_aou = nullptr, *d_c2s_off = nullptr;
     double *d_c2s = nullptr;
-    double *d_cart = nullptr;              // scratch: per spherical molecule 3 x ndm x nao_c^2
-    size_t cart_ndm = 0;
-    std::vector<size_t> cart_off;          // per molecule offset into d_cart
+    JkPerMol<double> cart;                 // 3 x ndm x nao_c^2 per spherical molecule
+    std::vector<size_t> cart_unit;         // nmol + 1: elements per density before each molecule
     JkSphMol *d_sph = nullptr, *h_sph = nullptr;  // [0, nmol): to Cartesian, [nmol, 2 nmol): back
     size_t cart_gen = 0;                   // bumps when the scratch moves (invalidates graphs)
-    float *d_d32 = nullptr;                // FP32 copies of D for the FP32 tier: ndm x nao_c^2 per molecule
-    float2 *d_d2 = nullptr;                // ... as two floats for the split tier
-    size_t d32_ndm = 0, d2_ndm = 0;
-    std::vector<size_t> d32_off;
+    JkPerMol<float> d32;                   // FP32 copies of D for the FP32 tier: ndm x nao_c^2 per molecule
+    JkPerMol<float2> d2;                   // ... as two floats for the split tier
+    std::vector<size_t> dens_unit;         // nmol + 1: elements per density before each molecule
     // learned router
     JkPairFeat *d_pfeat = nullptr;         // aligned with d_pairs
     JkRouterDev *d_router = nullptr;
@@ -900,7 +899,7 @@ void free_handle(jk_handle *h)
     for (auto &c : h->classes) { cudaFree(c.d_beg); cudaFree(c.d_end); }
     h->plans.clear();
     cudaFree(h->d_sh_mol); cudaFree(h->d_mol_sh0); cudaFree(h->d_sh_ao); cudaFree(h->d_sh_nc);
-    cudaFree(h->d_pairs); cudaFree(h->d_scr); cudaFree(h->d_rec); cudaFree(h->d_pp64); cudaFree(h->d_pp32); cudaFree(h->d_ppdf); cudaFree(h->d_rysdf); cudaFree(h->d_d2); cudaFree(h->d_mols);
+    cudaFree(h->d_pairs); cudaFree(h->d_scr); cudaFree(h->d_rec); cudaFree(h->d_pp64); cudaFree(h->d_pp32); cudaFree(h->d_ppdf); cudaFree(h->d_rysdf); cudaFree(h->d2.base); cudaFree(h->d_mols);
     cudaFree(h->d_dmax); cudaFree(h->d_dmax32); cudaFree(h->d_rys64); cudaFree(h->d_rys32);
     cudaFree(h->d_zero); cudaFree(h->d_err); cudaFree(h->d_tile_off);
     if (h->h_mols) cudaFreeHost(h->h_mols);
@@ -911,7 +910,7 @@ void free_handle(jk_handle *h)
     if (h->ev1) cudaEventDestroy(h->ev1);
     for (auto e : h->prof_ev) cudaEventDestroy(e);
     cudaFree(h->d_sh_l); cudaFree(h->d_sh_sph); cudaFree(h->d_sh_aou); cudaFree(h->d_c2s_off);
-    cudaFree(h->d_c2s); cudaFree(h->d_cart); cudaFree(h->d_sph); cudaFree(h->d_d32);
+    cudaFree(h->d_c2s); cudaFree(h->cart.base); cudaFree(h->d_sph); cudaFree(h->d32.base);
     cudaFree(h->d_pfeat); cudaFree(h->d_router); cudaFree(h->d_logn);
     cudaFree(h->d_rlist); cudaFree(h->d_rl);
     for (auto &g : h->graphs) cudaGraphExecDestroy(g.second.first);
@@ -1232,6 +1231,13 @@ int init_impl(int32_t nmol, const int32_t *mol_shell_off, const jk_shell *shells
         h->nao_user.push_back(ou);
         h->mol_sph.push_back(sph ? 1 : 0);
         h->spherical = h->spherical || sph;
+    }
+    h->dens_unit.assign(nmol + 1, 0);
+    h->cart_unit.assign(nmol + 1, 0);
+    for (int m = 0; m < nmol; ++m) {
+        const size_t nn = (size_t)h->nao_cart[m] * h->nao_cart[m];
+        h->dens_unit[m + 1] = h->dens_unit[m] + nn;
+        h->cart_unit[m + 1] = h->cart_unit[m] + (h->mol_sph[m] ? 3 * nn : 0);
     }
 
     // ---- shell types and pair classes
@@ -1746,41 +1752,18 @@ int build_impl(jk_handle *h, const double *const *D, int32_t ndm, int with_j, in
     size_t nlaunch_class = 0;
     for (auto &T : tiers) nlaunch_class += T.P->groups.size();
 
-    // Cartesian scratch for spherical molecules (3 x ndm x nao_c^2 each)
-    if (h->spherical && h->cart_ndm < (size_t)ndm) {
+    // Cartesian scratch for spherical molecules (3 x ndm x nao_c^2 each), copies
+    // of the densities for the FP32 and split tiers
+    const bool grow_cart = h->spherical && h->cart.ndm < (size_t)ndm;
+    const bool grow_32 = use32 && h->d32.ndm < (size_t)ndm, grow_2 = usedf && h->d2.ndm < (size_t)ndm;
+    if (grow_cart || grow_32 || grow_2) {
         CK(cudaStreamSynchronize(st));
-        cudaFree(h->d_cart);
-        h->d_cart = nullptr;
-        h->cart_off.assign(h->nmol, 0);
-        size_t tot = 0;
-        for (int m = 0; m < h->nmol; ++m)
-            if (h->mol_sph[m]) { h->cart_off[m] = tot; tot += 3 * (size_t)ndm * h->nao_cart[m] * h->nao_cart[m]; }
-        CK(cudaMalloc(&h->d_cart, sizeof(double) * std::max<size_t>(tot, 1)));
-        h->cart_ndm = ndm;
         ++h->cart_gen;
-    }
-    // copies of the densities for the FP32 and split tiers
-    if ((use32 && h->d32_ndm < (size_t)ndm) || (usedf && h->d2_ndm < (size_t)ndm)) {
-        CK(cudaStreamSynchronize(st));
-        h->d32_off.assign(h->nmol, 0);
-        const size_t n = std::max({h->d32_ndm, h->d2_ndm, (size_t)ndm});
-        size_t tot = 0;
-        for (int m = 0; m < h->nmol; ++m) { h->d32_off[m] = tot; tot += n * h->nao_cart[m] * h->nao_cart[m]; }
-        if (use32 || h->d_d32) {
-            cudaFree(h->d_d32);
-            h->d_d32 = nullptr;
-            h->d32_ndm = 0;
-            CK(cudaMalloc(&h->d_d32, sizeof(float) * std::max<size_t>(tot, 1)));
-            h->d32_ndm = n;
-        }
-        if (usedf || h->d_d2) {
-            cudaFree(h->d_d2);
-            h->d_d2 = nullptr;
-            h->d2_ndm = 0;
-            CK(cudaMalloc(&h->d_d2, sizeof(float2) * std::max<size_t>(tot, 1)));
-            h->d2_ndm = n;
-        }
-        ++h->cart_gen;
+        auto alloc = [](size_t bytes, void **p) { return (int)cudaMalloc(p, bytes); };
+        auto release = [](void *p) { cudaFree(p); };
+        if (grow_cart) CK((cudaError_t)h->cart.grow(ndm, h->cart_unit.back(), alloc, release));
+        if (grow_32) CK((cudaError_t)h->d32.grow(ndm, h->dens_unit.back(), alloc, release));
+        if (grow_2) CK((cudaError_t)h->d2.grow(ndm, h->dens_unit.back(), alloc, release));
     }
     // routed builds: one list per class pair for the quartets the router
     // releases from the FP64 tier, first sized by the pair's share of the
@@ -1790,7 +1773,7 @@ int build_impl(jk_handle *h, const double *const *D, int32_t ndm, int with_j, in
     bool grow = false;
     if (routed && h->d_rlist)
         for (size_t i = 0; i < h->rl_need.size(); ++i) grow = grow || h->rl_need[i] > h->rl_cap[i];
-    if (routed && (!h->d_rlist || grow)) {
+    if (routed && (!h->d_rlist || !h->d_rl || grow)) {
         CK(cudaStreamSynchronize(st));
         cudaFree(h->d_rlist); cudaFree(h->d_rl);
         h->d_rlist = nullptr; h->d_rl = nullptr;
@@ -1825,7 +1808,7 @@ int build_impl(jk_handle *h, const double *const *D, int32_t ndm, int with_j, in
         x.nao = h->nao_cart[m];
         if (h->mol_sph[m]) {
             const size_t nn = (size_t)ndm * x.nao * x.nao;
-            double *base = h->d_cart + h->cart_off[m];
+            double *base = h->cart.at(h->cart_unit[m]);
             x.D = base;
             x.J = with_j ? base + nn : nullptr;
             x.K = with_k ? base + 2 * nn : nullptr;
@@ -1847,8 +1830,8 @@ int build_impl(jk_handle *h, const double *const *D, int32_t ndm, int with_j, in
                 b = JkSphMol{};
             }
         }
-        x.D32 = use32 ? h->d_d32 + h->d32_off[m] : nullptr;
-        x.D2 = usedf ? h->d_d2 + h->d32_off[m] : nullptr;
+        x.D32 = use32 ? h->d32.at(h->dens_unit[m]) : nullptr;
+        x.D2 = usedf ? h->d2.at(h->dens_unit[m]) : nullptr;
         x.qmax2 = h->mol_qmax2[m];
         x.nsh = h->mol_sh0[m + 1] - h->mol_sh0[m];
         x.dmax_off = off;
