@@ -174,7 +174,7 @@ def parse():
     ap.add_argument("--form-steps", type=int, default=2)
     ap.add_argument("--tau32", type=float, default=1e-4)
     ap.add_argument("--graph", type=int, default=1, help="replay each build as one CUDA graph")
-    ap.add_argument("--branches", type=int, default=4, help="class kernels forked over this many graph branches")
+    ap.add_argument("--branches", type=int, default=4, help="1: the class kernels in one chain of the graph; more: spread over up to 24 branches")
     ap.add_argument("--micro", action="store_true", help="appendix-style micro-benchmarks instead of the workload")
     ap.add_argument("--micro-units", type=int, default=64,
                     help="triatomic units of the d-only / f-only n_dm sweep geometry (3 atoms each)")

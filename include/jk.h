@@ -192,8 +192,10 @@ int jk_build_batch(jk_handle *h, const double *const *D, int32_t n_dm, int with_
  * K are then partial sums whose sum over the parts is the full result, i.e.
  * one sum all-reduce combines GPUs that split one batch. Ranks may tune, chunk
  * and profile by themselves; tau32, split, cutoff and the like must agree),
- * "branches" (1..8: streams / graph branches of a profiled build's class
- * kernels; other builds spread them over 24),
+ * "branches" (1..8, reads 1 until it is set: 1 keeps every kernel of a build
+ * on the caller's stream, or in one chain of its graph; not set, or more: a
+ * build spreads its class kernels over up to 24 streams or graph branches. A
+ * profiled build takes exactly this many, one if it is not set),
  * "chunk" (32..65536, default 64: candidate kets per work item of the
  * persistent class kernels for classes with one thread per quartet; classes
  * with G threads per quartet take 1/G of it, and systems with more than 8
@@ -235,8 +237,9 @@ int jk_set_option(jk_handle *h, const char *key, double value);
 /* Reads any option above, and the read-only figures "graphs" (captured
  * graphs held), "init_ms" (jk_init wall time), "compile_ms" (NVRTC time spent
  * by this handle), "npairs", "nclasses", "nlaunches" (significant shell
- * pairs, pair classes, class-pair launches per tier). JK_ERR_ARG for an
- * unknown key. */
+ * pairs, pair classes, class-pair launches per tier), "streams" (streams or
+ * graph branches that the class kernels of the last build were spread over).
+ * JK_ERR_ARG for an unknown key. */
 int jk_get_option(jk_handle *h, const char *key, double *value);
 
 /* Number of molecules, basis functions of molecule m (in the basis D is

@@ -783,10 +783,11 @@ static const double JK_RATE[3] = {0.8e12, 6e12, 2e12};
 }  // namespace
 
 #define JK_MAX_BRANCHES 7        // option "branches" less one
-// Streams the launches of a build are spread over unless they are profiled: the
-// tail of one launch is filled by the next ones (s, p, d shells: 21 per tier; s
-// to f: 55). 45 functions in FP64: 1.74 ms on 4 streams, 1.17 on 8, 0.98 on 14,
-// 0.76 on 24; 8 molecules 280, 282, 286, 279 ms; 24 mixed 314, 314, 317, 300.
+// Streams the launches of a build are spread over unless they are profiled or
+// the caller set branches to 1: the tail of one launch is filled by the next
+// ones (s, p, d shells: 21 per tier; s to f: 55). ms on 1, 4, 8 and 24 streams:
+// 45 functions in FP64 2.00, 0.67, 0.48, 0.39; 20 atoms 7.0, 4.5, 4.1, 4.1; 33
+// atoms mixed 15.9, 12.8, 12.6, 12.6; 8 molecules 276, 258, 256, 257.
 #define JK_SIDE_STREAMS 23
 
 struct jk_handle {
@@ -884,7 +885,8 @@ struct jk_handle {
     // costs about 2 % of a mixed build of the batched workload
     int screen64 = 1;
     // graphs and branch streams
-    int branches = 1;
+    int branches = 0;                      // option; 0: not set
+    int last_streams = 0;                  // streams of the last build's class kernels
     cudaStream_t cap = nullptr;
     cudaStream_t side[JK_SIDE_STREAMS] = {};
     cudaEvent_t ev_fork = nullptr, ev_join[JK_SIDE_STREAMS] = {};
@@ -1854,8 +1856,10 @@ int build_impl(jk_handle *h, const double *const *D, int32_t ndm, int with_j, in
         h->prof_ev.resize(2 * nlaunch_class);
         for (size_t e = have; e < h->prof_ev.size(); ++e) CK(cudaEventCreate(&h->prof_ev[e]));
     }
-    const int nbranch = prof ? h->branches
-                             : std::min(JK_SIDE_STREAMS + 1, (int)nlaunch_class);
+    // option branches = 1 keeps a build on the caller's stream
+    const int nbranch = prof ? std::max(1, h->branches)
+                             : (h->branches == 1 ? 1 : std::min(JK_SIDE_STREAMS + 1, (int)nlaunch_class));
+    h->last_streams = nbranch;
     int nlaunch_aux = 0;
 
     // Everything a build does on the device, in order, on stream s (and, for
@@ -2516,7 +2520,8 @@ int jk_get_option(jk_handle *h, const char *key, double *value)
     else if (k == "use_graph") *value = h->use_graph;
     else if (k == "use_dmax") *value = h->use_dmax;
     else if (k == "profile") *value = h->profile;
-    else if (k == "branches") *value = h->branches;
+    else if (k == "branches") *value = std::max(1, h->branches);
+    else if (k == "streams") *value = h->last_streams;
     else if (k == "part_count") *value = h->part_count;
     else if (k == "prim_eps") *value = h->prim_eps;
     else if (k == "omega") *value = h->omega;

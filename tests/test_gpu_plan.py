@@ -114,3 +114,22 @@ def test_parts_of_differently_tuned_handles_sum_to_the_build(case, precision, tm
     assert n == nq
     tol = 1e-10 if precision == "fp64" else 1e-8
     assert np.abs(J - Jr).max() <= tol and np.abs(K - Kr).max() <= tol
+
+
+@pytest.mark.parametrize("precision", ["fp64", "mixed"])
+@pytest.mark.parametrize("use_graph", [0, 1])
+def test_branches_1_keeps_the_build_on_the_callers_stream(case, precision, use_graph):
+    mol, Jr, Kr, _ = case
+    eng = jk.JK(mol)
+    eng.set_option("use_graph", use_graph)
+    assert eng.get_option("branches") == 1
+    D = torch.tensor(mol.D, dtype=torch.float64, device="cuda")
+    tol = 1e-10 if precision == "fp64" else 1e-8
+    for branches, streams in ((None, 24), (1, 1), (4, 24), (1, 1)):
+        if branches:
+            eng.set_option("branches", branches)
+        J, K, st = eng.build(D, precision=precision, stats=True)
+        assert eng.get_option("streams") == min(streams, st["kernel_launches"])
+        assert np.abs(J.cpu().numpy() - Jr).max() <= tol and np.abs(K.cpu().numpy() - Kr).max() <= tol
+    assert eng.get_option("graphs") == 2 * use_graph
+    eng.close()
