@@ -238,8 +238,9 @@ int jk_set_option(jk_handle *h, const char *key, double value);
  * graphs held), "init_ms" (jk_init wall time), "compile_ms" (NVRTC time spent
  * by this handle), "npairs", "nclasses", "nlaunches" (significant shell
  * pairs, pair classes, class-pair launches per tier), "streams" (streams or
- * graph branches that the class kernels of the last build were spread over).
- * JK_ERR_ARG for an unknown key. */
+ * graph branches that the class kernels of the last build were spread over),
+ * "stream_priority" (their priority: the caller's stream's, or the default
+ * one in a graph). JK_ERR_ARG for an unknown key. */
 int jk_get_option(jk_handle *h, const char *key, double *value);
 
 /* Number of molecules, basis functions of molecule m (in the basis D is

@@ -888,7 +888,9 @@ struct jk_handle {
     int branches = 0;                      // option; 0: not set
     int last_streams = 0;                  // streams of the last build's class kernels
     cudaStream_t cap = nullptr;
-    cudaStream_t side[JK_SIDE_STREAMS] = {};
+    // by priority: eager builds fork with the caller's, graphs are captured with the default one
+    std::map<int, std::array<cudaStream_t, JK_SIDE_STREAMS>> side;
+    int last_priority = 0;                 // of the streams the last build forked over
     cudaEvent_t ev_fork = nullptr, ev_join[JK_SIDE_STREAMS] = {};
     std::map<std::string, std::pair<cudaGraphExec_t, int>> graphs;
 };
@@ -917,10 +919,11 @@ void free_handle(jk_handle *h)
     cudaFree(h->d_rlist); cudaFree(h->d_rl);
     for (auto &g : h->graphs) cudaGraphExecDestroy(g.second.first);
     if (h->cap) cudaStreamDestroy(h->cap);
-    for (int b = 0; b < JK_SIDE_STREAMS; ++b) {
-        if (h->side[b]) cudaStreamDestroy(h->side[b]);
+    for (auto &p : h->side)
+        for (cudaStream_t s : p.second)
+            if (s) cudaStreamDestroy(s);
+    for (int b = 0; b < JK_SIDE_STREAMS; ++b)
         if (h->ev_join[b]) cudaEventDestroy(h->ev_join[b]);
-    }
     if (h->ev_fork) cudaEventDestroy(h->ev_fork);
     if (h->h_sph) cudaFreeHost(h->h_sph);
     delete h;
@@ -956,6 +959,22 @@ void estimate_costs(jk_handle *h)
         L.cand = work;
         L.cost = work * class_flops(L.spec[0], 1);
     }
+}
+
+// The streams a build of this priority forks over, made on first use.
+int side_streams(jk_handle *h, int priority)
+{
+    if (h->side.count(priority)) return JK_OK;
+    std::array<cudaStream_t, JK_SIDE_STREAMS> v{};
+    for (int b = 0; b < JK_SIDE_STREAMS; ++b) {
+        const cudaError_t e = cudaStreamCreateWithPriority(&v[b], cudaStreamNonBlocking, priority);
+        if (e != cudaSuccess) {
+            for (int k = 0; k < b; ++k) cudaStreamDestroy(v[k]);
+            CK(e);
+        }
+    }
+    h->side[priority] = v;
+    return JK_OK;
 }
 
 void drop_graphs(jk_handle *h)
@@ -1659,10 +1678,8 @@ int init_impl(int32_t nmol, const int32_t *mol_shell_off, const jk_shell *shells
     CK(cudaEventCreate(&h->ev1));
     CK(cudaStreamCreateWithFlags(&h->cap, cudaStreamNonBlocking));
     CK(cudaEventCreateWithFlags(&h->ev_fork, cudaEventDisableTiming));
-    for (int b = 0; b < JK_SIDE_STREAMS; ++b) {
-        CK(cudaStreamCreateWithFlags(&h->side[b], cudaStreamNonBlocking));
-        CK(cudaEventCreateWithFlags(&h->ev_join[b], cudaEventDisableTiming));
-    }
+    if ((rc = side_streams(h.get(), 0))) return rc;
+    for (int b = 0; b < JK_SIDE_STREAMS; ++b) CK(cudaEventCreateWithFlags(&h->ev_join[b], cudaEventDisableTiming));
     CK(cudaDeviceSynchronize());
     h->init_ms = std::chrono::duration<double, std::milli>(std::chrono::steady_clock::now() - t_start).count();
     *out = h.release();
@@ -1860,6 +1877,11 @@ int build_impl(jk_handle *h, const double *const *D, int32_t ndm, int with_j, in
     const int nbranch = prof ? std::max(1, h->branches)
                              : (h->branches == 1 ? 1 : std::min(JK_SIDE_STREAMS + 1, (int)nlaunch_class));
     h->last_streams = nbranch;
+    int priority = 0;
+    if (!h->use_graph || logs) CK(cudaStreamGetPriority(st, &priority));
+    if (nbranch > 1 && (rc = side_streams(h, priority))) return rc;
+    const auto &side = h->side[nbranch > 1 ? priority : 0];
+    h->last_priority = priority;
     int nlaunch_aux = 0;
 
     // Everything a build does on the device, in order, on stream s (and, for
@@ -1945,12 +1967,12 @@ int build_impl(jk_handle *h, const double *const *D, int32_t ndm, int with_j, in
         auto fork = [&]() -> int {
             if (nbranch < 2) return JK_OK;
             CK(cudaEventRecord(h->ev_fork, s0));
-            for (int b = 1; b < nbranch; ++b) CK(cudaStreamWaitEvent(h->side[b - 1], h->ev_fork, 0));
+            for (int b = 1; b < nbranch; ++b) CK(cudaStreamWaitEvent(side[b - 1], h->ev_fork, 0));
             return JK_OK;
         };
         auto join = [&]() -> int {
             for (int b = 1; b < nbranch; ++b) {
-                CK(cudaEventRecord(h->ev_join[b - 1], h->side[b - 1]));
+                CK(cudaEventRecord(h->ev_join[b - 1], side[b - 1]));
                 CK(cudaStreamWaitEvent(s0, h->ev_join[b - 1], 0));
             }
             return JK_OK;
@@ -1966,7 +1988,7 @@ int build_impl(jk_handle *h, const double *const *D, int32_t ndm, int with_j, in
             for (size_t g = 0; g < T.P->groups.size(); ++g, ++k) {
                 const LaunchGroup &G = T.P->groups[g];
                 const KInfo &ki = (*T.ki)[g];
-                cudaStream_t sk = k % nbranch ? h->side[k % nbranch - 1] : s0;
+                cudaStream_t sk = k % nbranch ? side[k % nbranch - 1] : s0;
                 JkClassArgs a;
                 memset(&a, 0, sizeof a);
                 a.subs = T.P->d_subs + (T.t == 2 ? G.sub0 : 0);   // items index the plan's whole table
@@ -2522,6 +2544,7 @@ int jk_get_option(jk_handle *h, const char *key, double *value)
     else if (k == "profile") *value = h->profile;
     else if (k == "branches") *value = std::max(1, h->branches);
     else if (k == "streams") *value = h->last_streams;
+    else if (k == "stream_priority") *value = h->last_priority;
     else if (k == "part_count") *value = h->part_count;
     else if (k == "prim_eps") *value = h->prim_eps;
     else if (k == "omega") *value = h->omega;

@@ -133,3 +133,18 @@ def test_branches_1_keeps_the_build_on_the_callers_stream(case, precision, use_g
         assert np.abs(J.cpu().numpy() - Jr).max() <= tol and np.abs(K.cpu().numpy() - Kr).max() <= tol
     assert eng.get_option("graphs") == 2 * use_graph
     eng.close()
+
+
+def test_an_eager_build_keeps_the_priority_of_the_callers_stream(case):
+    mol, Jr, Kr, _ = case
+    eng = jk.JK(mol)
+    D = torch.tensor(mol.D, dtype=torch.float64, device="cuda")
+    torch.cuda.synchronize()
+    for priority in (0, -1, 0):
+        s = torch.cuda.Stream(priority=priority)
+        with torch.cuda.stream(s):
+            J, K, _ = eng.build(D)
+        s.synchronize()
+        assert eng.get_option("stream_priority") == priority
+        assert np.abs(J.cpu().numpy() - Jr).max() <= 1e-10 and np.abs(K.cpu().numpy() - Kr).max() <= 1e-10
+    eng.close()
