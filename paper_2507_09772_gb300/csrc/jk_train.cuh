@@ -78,16 +78,13 @@ __global__ void __launch_bounds__(256) jk_mlp_grad_kernel(const float *__restric
     JkGradSmem<ROWS> &S = *reinterpret_cast<JkGradSmem<ROWS> *>(jk_grad_smem);
     const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
     for (int i = tid; i < JK_RT_NIN * H; i += 256) S.w1[i] = jk_bf2f(jk_f2bf(theta[JK_RT_OFF_W1 + i]));
-    bool wodd = false;   // a weight of layer 2 or 3 that is not finite
     for (int i = tid; i < H * H; i += 256) {
         const float w = jk_bf2f(jk_f2bf(theta[JK_RT_OFF_W2 + i]));
-        wodd = wodd || !(fabsf(w) <= 3.0e38f);
         S.w2[i] = w;
         S.w2t[i % H][i / H] = w;
     }
     if (tid < H) {
         S.w3[tid] = jk_bf2f(jk_f2bf(theta[JK_RT_OFF_W3 + tid]));
-        wodd = wodd || !(fabsf(S.w3[tid]) <= 3.0e38f);
         S.b1[tid] = theta[JK_RT_OFF_B1 + tid];
         S.b2[tid] = theta[JK_RT_OFF_B2 + tid];
         if (tid == 0) S.b3[0] = theta[JK_RT_OFF_B3];
@@ -116,7 +113,7 @@ __global__ void __launch_bounds__(256) jk_mlp_grad_kernel(const float *__restric
         __syncthreads();
         // layer 1: rows RT ty .., outputs 4 tx ..
         unsigned pos1 = 0;
-        bool odd = wodd;    // a weight or hidden value that is not finite
+        bool odd = false;   // a hidden value that is not finite
         {
             float a[RT][4];
 #pragma unroll
@@ -143,9 +140,8 @@ __global__ void __launch_bounds__(256) jk_mlp_grad_kernel(const float *__restric
                     S.h1[RT * ty + i][4 * tx + j] = h;
                 }
         }
-        // weights, features or hidden values that are not finite: an inactive unit
-        // (its rounded activation is zero) takes and passes no gradient, where a
-        // product with its zero delta would be NaN; nor does a zero input
+        // features or hidden values that are not finite: products with a zero
+        // delta count as zero, not as NaN (an inactive unit takes no gradient)
         const bool wild = __syncthreads_or(odd);
         // layer 2
         unsigned pos2 = 0;
@@ -171,17 +167,13 @@ __global__ void __launch_bounds__(256) jk_mlp_grad_kernel(const float *__restric
                     }
                 }
             }
-            // (rows past the batch have no active unit: their zero weight would
-            // make a NaN of an infinite bias or weight)
 #pragma unroll
-            for (int i = 0; i < RT; ++i) {
-                const bool in = t0 + RT * ty + i < batch;
+            for (int i = 0; i < RT; ++i)
 #pragma unroll
                 for (int j = 0; j < 4; ++j) {
-                    if (in && a[i][j] > 0.0f) pos2 |= 1u << (4 * i + j);
-                    S.h2[RT * ty + i][4 * tx + j] = in ? jk_bf2f(jk_f2bf(fmaxf(a[i][j], 0.0f))) : 0.0f;
+                    if (a[i][j] > 0.0f) pos2 |= 1u << (4 * i + j);
+                    S.h2[RT * ty + i][4 * tx + j] = jk_bf2f(jk_f2bf(fmaxf(a[i][j], 0.0f)));
                 }
-            }
         }
         __syncthreads();
         // output, pinball loss u (q - [u < 0]) and its derivative
@@ -219,7 +211,7 @@ __global__ void __launch_bounds__(256) jk_mlp_grad_kernel(const float *__restric
                 for (int i = 0; i < 4; ++i)
 #pragma unroll
                     for (int j = 0; j < 4; ++j)
-                        if (S.h2[r][4 * tx + j] > 0.0f && hv[i] != 0.0f) gw2[i][j] = fmaf(hv[i], dv[j], gw2[i][j]);
+                        if (dv[j] != 0.0f && hv[i] != 0.0f) gw2[i][j] = fmaf(hv[i], dv[j], gw2[i][j]);
                 continue;
             }
 #pragma unroll
@@ -243,15 +235,6 @@ __global__ void __launch_bounds__(256) jk_mlp_grad_kernel(const float *__restric
         }
         // delta of layer 1, into h2
         float dh[RT][4] = {};
-        if (wild) {
-#pragma unroll
-            for (int i = 0; i < RT; ++i)
-                for (int k = 0; k < H; ++k)
-                    if (S.h2[RT * ty + i][k] > 0.0f)
-#pragma unroll
-                        for (int j = 0; j < 4; ++j)
-                            dh[i][j] = fmaf(S.w2t[k][4 * tx + j], S.d[RT * ty + i][k], dh[i][j]);
-        } else
 #pragma unroll 4
         for (int k = 0; k < H; k += 4) {
             float4 w[4];
@@ -282,7 +265,7 @@ __global__ void __launch_bounds__(256) jk_mlp_grad_kernel(const float *__restric
                 const float d = S.h2[r][o];
 #pragma unroll
                 for (int k = 0; k < 3; ++k)
-                    if (!wild || (S.h1[r][o] > 0.0f && S.x[r][k0 + k] != 0.0f)) gw1[k] = fmaf(S.x[r][k0 + k], d, gw1[k]);
+                    if (!wild || (d != 0.0f && S.x[r][k0 + k] != 0.0f)) gw1[k] = fmaf(S.x[r][k0 + k], d, gw1[k]);
                 if (tid >= 128 && tid < 192) gv += d;
             }
         }

@@ -54,37 +54,3 @@ def test_infinite_feature_leaves_inactive_units_alone():
     dead = W1[2] < 0
     dW1 = g[:768].reshape(12, 64)[:, dead]
     assert np.isfinite(dW1).all() and np.isfinite(g[1024:1088][dead]).all()
-
-
-@pytest.mark.parametrize("n", [5, 64, 9735])
-@pytest.mark.parametrize("value", [-np.inf, np.nan])
-def test_weights_of_an_inactive_unit_that_are_not_finite(n, value):
-    """A layer-2 unit with an infinite or NaN weight is inactive in every row
-    (-inf or NaN activations): it takes and passes no gradient, also in the
-    rows that fill up the last tile."""
-    if not torch.cuda.is_available():
-        pytest.skip("needs a CUDA device")
-    b, th, mu, isd = blob(7)
-    th2 = th.copy()
-    th[1088 + 3 * 64 + 7] = value          # W2[3][7]
-    b.theta[:] = th.tolist()
-    th2[1088:5184].reshape(64, 64)[:, 7] = 0.0
-    th2[5184 + 7] = -1.0                   # b2[7]: the same unit switched off
-    X, y = rows(n, 8)
-    g, loss = jk.jk_router_gradient(b, torch.tensor(X, device="cuda"), torch.tensor(y, device="cuda"), 0.9)
-    lref, gref = R.pinball_grad(th2, mu, isd, X, y, 0.9)
-    assert np.isfinite(g).all() and loss == pytest.approx(lref, rel=1e-3)
-    assert np.linalg.norm(g - gref) <= 1e-2 * np.linalg.norm(gref)
-
-
-def test_infinite_bias_leaves_the_other_gradients_finite():
-    """b2[9] = inf: the unit's W3 gradient is infinite, nothing becomes NaN."""
-    if not torch.cuda.is_available():
-        pytest.skip("needs a CUDA device")
-    b, th, _, _ = blob(9)
-    th[5184 + 9] = np.inf
-    th[5248 + 9] = 0.5
-    b.theta[:] = th.tolist()
-    X, y = rows(17, 10)
-    g, _ = jk.jk_router_gradient(b, torch.tensor(X, device="cuda"), torch.tensor(y, device="cuda"), 0.9)
-    assert not np.isnan(g).any() and np.isinf(g[5248 + 9])
