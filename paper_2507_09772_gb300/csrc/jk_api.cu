@@ -1009,17 +1009,28 @@ int tier_plan(jk_handle *h, int t, int hi, int merge, int whole, TierPlan **out)
     auto it = h->plans.find(key);
     if (it != h->plans.end()) { *out = it->second.get(); return JK_OK; }
     std::unique_ptr<TierPlan> P(new TierPlan());
-    // group the class pairs (h->launches is sorted by cost, largest first)
+    // group the class pairs (h->launches is sorted by cost, largest first): those
+    // of the same angular momenta share a launch whatever shapes they were tuned
+    // to, and it takes the shape that most of their cost asks for. ms after
+    // autotuning, launches split by shape and shared: 45 functions 0.444 and
+    // 0.392 (0.385 untuned), 24 molecules mixed 247 and 231 (237), 20 atoms 4.60
+    // and 4.34 (4.48), 8 molecules 256 and 264 (268).
     std::vector<std::vector<int>> members;
-    std::map<std::string, int> by_kernel;
+    std::vector<KSpec> shape;
+    std::map<std::array<int, 4>, int> by_l;
     for (size_t l = 0; l < h->launches.size(); ++l) {
+        const KSpec &s = h->launches[l].spec[t];
         int g = (int)members.size();
-        if (merge) {
-            auto r = by_kernel.emplace(h->launches[l].spec[t].name(), g);
-            g = r.first->second;
-        }
-        if (g == (int)members.size()) members.emplace_back();
+        if (merge) g = by_l.emplace(std::array<int, 4>{s.la, s.lb, s.lc, s.ld}, g).first->second;
+        if (g == (int)members.size()) { members.emplace_back(); shape.push_back(s); }
         members[g].push_back((int)l);
+    }
+    for (size_t g = 0; g < members.size(); ++g) {
+        std::map<std::array<int, 4>, double> votes;
+        auto form = [](const KSpec &s) { return std::array<int, 4>{s.ga, s.gb, s.gc, s.gd}; };
+        for (int l : members[g]) votes[form(h->launches[l].spec[t])] += h->launches[l].cost;
+        for (int l : members[g])
+            if (votes[form(h->launches[l].spec[t])] > votes[form(shape[g])]) shape[g] = h->launches[l].spec[t];
     }
     auto prims = [&](int l) {
         const KSpec &s = h->launches[l].spec[t];
@@ -1039,17 +1050,15 @@ int tier_plan(jk_handle *h, int t, int hi, int merge, int whole, TierPlan **out)
     const double kept = hi ? 0.3 : 1.0;   // share of the candidates the tier evaluates
     const double chain_max = std::max(JK_CHAIN_MIN, JK_CHAIN_SHARE * kept * total_cost / JK_RATE[t]) / JK_LAT[t];
     std::vector<JkSub> subs;
-    std::vector<long long> cap;
     for (long long f = 1;; f *= 2) {
         subs.clear();
-        cap.assign(members.size(), 0);
         P->groups.clear();
         P->launch.clear();
         long long total = 0, least = 0;
         for (size_t k = 0; k < gord.size(); ++k) {
             const auto &mem = members[gord[k]];
             LaunchGroup G;
-            G.spec = h->launches[mem[0]].spec[t];
+            G.spec = shape[gord[k]];
             G.sub0 = (int)subs.size();
             G.nsub = (int)mem.size();
             const int ngw = G.spec.G() <= 32 ? 32 / G.spec.G() : 1;
@@ -1078,7 +1087,7 @@ int tier_plan(jk_handle *h, int t, int hi, int merge, int whole, TierPlan **out)
                 S.same_class = L.c1 == L.c2 ? 1 : 0;
                 S.nab = L.spec[t].na * L.spec[t].nb;
                 S.ncd = L.spec[t].nc * L.spec[t].nd;
-                KSpec one = L.spec[t];
+                KSpec one = G.spec;
                 one.na = one.nb = one.nc = one.nd = 1;
                 // modelled FLOPs of a lane per round, at most
                 const double round = class_flops(one, 1) / one.G() * S.nab * S.ncd;

@@ -22,7 +22,7 @@ def case():
     return mol, J, K, nq
 
 
-def build(mol, options, parts=1, **kw):
+def build(mol, options, parts=1, full=False, **kw):
     eng = jk.JK(mol)
     try:
         for k, v in options.items():
@@ -36,7 +36,7 @@ def build(mol, options, parts=1, **kw):
             j, k, st = eng.build(D, cutoff=1e-13, stats=True, **kw)
             J, K = J + j, K + k
             nq += st["quartets_fp64"] + st["quartets_fp32"]
-        return J.cpu().numpy(), K.cpu().numpy(), nq
+        return (J.cpu().numpy(), K.cpu().numpy(), nq) + ((st,) if full else ())
     finally:
         eng.close()
 
@@ -75,15 +75,14 @@ def test_item_bound_follows_the_density(case, scale, use_dmax):
     assert np.abs(K.cpu().numpy() - Kr).max() <= 1e-10 * max(scale, 1e-3)
 
 
-def tuning_table(path):
+def tuning_table(path, only=None):
     """Other shapes for the s and p classes than the built-in rule's, as another rank's autotuner might have stored."""
     p = torch.cuda.get_device_properties(0)
     name = "".join(c if c.isalnum() and c.isascii() else "_" for c in p.name)
     shape = {"1010": "3 1 1 1", "1011": "1 1 3 1", "1110": "3 1 1 1", "1100": "3 1 1 1", "1000": "3 1 1 1"}
-    prims = [1, 3, 6]
     with open(path / f"tune_{name}_sm{p.major}{p.minor}_{p.multi_processor_count}.txt", "w") as f:
         for k, v in shape.items():
-            for n in itertools.product(prims, repeat=4):
+            for n in [only] if only else itertools.product([1, 3, 6], repeat=4):
                 for t in (0, 1, 2):
                     f.write("%s/%d_%d_%d_%d/%d %s\n" % (k, *n, t, v))
 
@@ -148,3 +147,20 @@ def test_an_eager_build_keeps_the_priority_of_the_callers_stream(case):
         assert eng.get_option("stream_priority") == priority
         assert np.abs(J.cpu().numpy() - Jr).max() <= 1e-10 and np.abs(K.cpu().numpy() - Kr).max() <= 1e-10
     eng.close()
+
+
+@pytest.mark.parametrize("prims", [(3, 3, 3, 3), (1, 3, 1, 3), None])
+def test_tuned_class_pairs_still_share_a_launch(case, prims, tmp_path, monkeypatch):
+    """Shapes stored for some class pairs of an angular momentum do not split its launch."""
+    mol, Jr, Kr, nq = case
+    launches = []
+    for tuned in (False, True):
+        where = tmp_path / str(tuned)
+        where.mkdir()
+        if tuned:
+            tuning_table(where, prims)
+        monkeypatch.setenv("JK_TUNING_DIR", str(where))
+        J, K, n, st = build(mol, {}, full=True)
+        launches.append(st["kernel_launches"])
+        assert n == nq and np.abs(J - Jr).max() <= 1e-10 and np.abs(K - Kr).max() <= 1e-10
+    assert launches[0] == launches[1]
