@@ -170,3 +170,25 @@ def test_trained_router_moves_more_than_a_constant_router(trained):
     for Jx, Kx in ((Jt, Kt), (Jc, Kc)):
         assert np.abs(Jx - Jo).max() <= 1e-8 and np.abs(Kx - Ko).max() <= 1e-8
     assert st_t["quartets_routed"] > st_c["quartets_routed"], (st_t["quartets_routed"], st_c["quartets_routed"])
+
+
+@pytest.mark.parametrize("nprim", [1, 2])
+def test_quartets_split_over_ctas_are_evaluated_once(nprim):
+    """(gg|gg) quartets take more threads than one CTA has, and every CTA of
+    such a group screens: a router that releases every band quartet must not
+    make it one quartet per CTA. They stay in FP64, the other classes' move."""
+    rng = np.random.default_rng(17)
+    xyz = np.array([[0.0, 0.0, 0.0], [1.3, 0.2, -0.5]])
+    mol = synth.custom_basis_molecule(xyz, [[(4, [1.1, 0.5][:nprim]), (0, [0.6])]] * 2, rng)
+    assert jk.jk_compile_class(4, 4, 4, 4, nprim, nprim, nprim, nprim)[0] > 256
+    eng = jk.JK(mol)
+    eng.set_option("tau32", 1e-4)
+    J64, K64, s64 = _gpu_build(eng, mol, cutoff=1e-13, precision="fp64")
+    eng.load_router(constant_blob(-10.0, 0.0))
+    Jr, Kr, sr = _gpu_build(eng, mol, cutoff=1e-13, precision="routed")
+    eng.close()
+    assert sr["quartets_fp64"] + sr["quartets_fp32"] == s64["quartets_fp64"]
+    assert sr["quartets_routed"] > 0
+    # FP32 quartets up to 100 tau32 = 1e-2 (the band), relative error 1e-5 at most in g classes,
+    # a few hundred quartets; an integral taken twice would be off by 1e-2
+    assert np.abs(Jr - J64).max() <= 1e-5 and np.abs(Kr - K64).max() <= 1e-5
