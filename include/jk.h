@@ -217,9 +217,12 @@ int jk_build_batch(jk_handle *h, const double *const *D, int32_t n_dm, int with_
  * "split" (0..1, default 1/128: FP64-tier quartets whose bound Q_ab Q_cd Dmax
  * is at most split (with f or g shells split / 64) x max Q^2 x max |D| of their
  * molecule, and in mixed and routed builds at least those up to 4,096 tau32, are
- * evaluated in pairs of FP32 numbers (48 bits, relative error about 1e-14), which
- * the GPU does several times faster; the error this adds is below the one the
- * result has from the cutoff. They count as FP64 quartets.
+ * evaluated in pairs of FP32 numbers (48 bits), which the GPU does several times
+ * faster. With every quartet in them J and K were within 1e-14 of FP64 (2-norm)
+ * for s, p, d shells and 4e-13 with f shells; at the default the error against a
+ * 64-bit reference is the one of FP64 instructions, set by the cutoff. They
+ * count as FP64 quartets. With a cutoff below 1e-13 FP64-mode builds, and mixed
+ * ones with tau32 below 1e-8, take FP64 instructions unless this option is set.
  * 0: FP64 instructions for every FP64-tier quartet, as for cutoffs below 1e-30,
  * for |omega| outside 1e-6 .. 1e6 (and not 0), and for molecules whose
  * exponents lie outside (1e-6, 1e8) or whose integrals pass through numbers far

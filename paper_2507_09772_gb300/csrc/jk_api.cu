@@ -779,6 +779,15 @@ static const double JK_RATE[3] = {0.8e12, 6e12, 2e12};
 #define JK_SPLIT (1.0 / 128)
 #define JK_SPLIT_F (1.0 / 64)
 #define JK_SPLIT_TAU 4096.0
+// Below this cutoff the error of the cutoff no longer covers the one of two
+// floats and of the sums in two passes (1e-15 of J and K). Errors of J and K
+// against a 64-bit reference, default split over split = 0, 3, 8 and 14 atoms,
+// erfc on 14, 3 and 6 atoms of s p d f shells, three inputs each: at 1e-13
+// 1.000 to 1.004 times, at 1e-14 1.00 to 1.17, at 1e-15 1.04 to 1.79.
+// The FP32 tier's own error is 3.6e-11 at tau32 = 1e-4 (14 atoms) and follows
+// tau32: mixed builds keep two floats at any cutoff from JK_SPLIT_TAU32 on.
+#define JK_SPLIT_CUTOFF 1e-13
+#define JK_SPLIT_TAU32 1e-8
 
 }  // namespace
 
@@ -872,6 +881,7 @@ struct jk_handle {
     std::vector<long long> rl_need;        // entries each list needed in the last build with stats
     double route_cap = 16777216.0;         // list entries over all launches
     double split = JK_SPLIT;               // split threshold; 0: every quartet of the FP64 tier in FP64 instructions
+    bool split_set = false;                // by the caller: then for every cutoff
     bool df_ok = false;                    // some molecule's basis stays far inside the FP32 range
     int asym64 = 0;                        // FP32 tier: large-T roots and weights in FP64
     int chunk = JK_CHUNK;                  // kets per work item
@@ -987,9 +997,12 @@ void drop_graphs(jk_handle *h)
 // cutoff or its operator leave the FP32 range. theta = w^2 / (w^2 + rho), with
 // rho in 1e-6 .. 1e8, keeps 48 bits for |w| in 1e-6 .. 1e6; w^2 overflows from
 // 1.9e19 on, and the residual of the square root's estimate is lost from 1e16.
+// Nor, unless the caller sets the option, where the cutoff is below
+// JK_SPLIT_CUTOFF and no FP32 tier of more error covers it either.
 bool uses_two_floats(const jk_handle *h, int mode, double cutoff)
 {
     const double w = std::fabs(h->omega);
+    if (cutoff < JK_SPLIT_CUTOFF && !h->split_set && (mode == JK_PREC_FP64 || h->tau32 < JK_SPLIT_TAU32)) return false;
     return mode != JK_PREC_FP32 && h->split > 0 && h->df_ok && cutoff >= 1e-30 && (w == 0 || (w >= 1e-6 && w <= 1e6));
 }
 
@@ -1941,7 +1954,8 @@ int build_impl(jk_handle *h, const double *const *D, int32_t ndm, int with_j, in
         auto hi_of = [&](int t) { return two && (t == 1 || t == 2) ? tau : inf; };
         // the split threshold divides the FP64 tier's range (per molecule); a
         // build with an FP32 tier (relative error 6e-8 up to tau) takes two
-        // floats (1e-12 at worst) up to 4,096 tau, a sixteenth of that error
+        // floats (2e-12 by the operations' bounds, 4e-13 seen) up to 4,096 tau, at
+        // most a seventh of that error
         const double split_min = two ? JK_SPLIT_TAU * tau : 0.0;
         auto side_of = [&](int t) { return !usedf ? 0 : (t == 0 ? 1 : (t == 3 ? -1 : 0)); };
         {
@@ -2091,7 +2105,7 @@ int build_impl(jk_handle *h, const double *const *D, int32_t ndm, int with_j, in
                  h->part_count, h->prim_eps, h->asym64, h->screen64 + 2 * h->widen_int);
         std::string key = keyb;
         char ob[80];
-        snprintf(ob, sizeof ob, "/%a/%a", h->omega, h->split);
+        snprintf(ob, sizeof ob, "/%a/%a/%d", h->omega, h->split, usedf ? 1 : 0);
         key += ob;
         auto it = h->graphs.find(key);
         if (it == h->graphs.end()) {
@@ -2511,6 +2525,7 @@ int jk_set_option(jk_handle *h, const char *key, double value)
     else if (k == "split") {
         if (!(value >= 0 && value <= 1)) return fail(JK_ERR_ARG, "split must be in [0, 1]");
         h->split = value;
+        h->split_set = true;
     }
     else if (k == "asym64") h->asym64 = value != 0;
     else if (k == "widen_int") h->widen_int = value != 0;

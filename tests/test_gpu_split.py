@@ -2,10 +2,11 @@
 in pairs of floats).
 
 Two floats carry 48 bits; an integral takes some hundred operations, each
-within 2^-46 of its result, a relative error of at most 2e-12, so with every
-quartet in two floats (split = 1) and |J|, |K| below 50 the result stays within
-1e-10; at the default threshold, 1/128 of the largest bound, within 1e-12 of
-the all-FP64 build.
+within 2^-46 of its result, a relative error of at most 2e-12 (J and K so built
+were 1e-14 off for s, p, d shells, 4e-13 with f shells), so with every quartet
+in two floats (split = 1) and |J|, |K| below 50 the result stays within 1e-10;
+at the default threshold, 1/128 of the largest bound, within 1e-12 of the
+all-FP64 build.
 """
 import numpy as np
 import pytest
@@ -193,4 +194,21 @@ def test_the_range_is_judged_molecule_by_molecule():
     eng.set_option("profile", 1)
     eng.build([torch.tensor(m.D, dtype=torch.float64, device="cuda") for m in (wide, synth.batched_molecule(3, natm=6))], stats=True)
     assert sum(p["quartets"] for p in jk.jk_profile(eng.h) if p["tier"] == 2) > 0
+    eng.close()
+
+
+@pytest.mark.parametrize("cutoff,precision,tau32,set_split,taken", [
+    (1e-13, "fp64", 1e-4, False, True), (9.9e-14, "fp64", 1e-4, False, False), (1e-15, "fp64", 1e-4, False, False),
+    (1e-15, "fp64", 1e-4, True, True), (1e-15, "mixed", 1e-4, False, True), (1e-15, "mixed", 9e-9, False, False),
+    (1e-13, "mixed", 1e-12, False, True), (1e-12, "fp64", 1e-4, False, True)])
+def test_two_floats_only_where_the_cutoff_covers_their_error(cutoff, precision, tau32, set_split, taken):
+    mol = synth.tiny_631gs()
+    eng = jk.JK(mol)
+    eng.set_option("tau32", tau32)
+    D = torch.tensor(mol.D, dtype=torch.float64, device="cuda")
+    if set_split:
+        eng.set_option("split", eng.get_option("split"))
+    eng.set_option("profile", 1)
+    eng.build(D, cutoff=cutoff, precision=precision, stats=True)
+    assert (sum(p["quartets"] for p in jk.jk_profile(eng.h) if p["tier"] == 2) > 0) == taken
     eng.close()
