@@ -105,7 +105,7 @@ Driver &drv()
     return d;
 }
 
-static_assert(sizeof(JkPair) == 96 && sizeof(JkPrimPair64) == 96 && sizeof(JkPrimPair32) == 48 && sizeof(JkPrimPairDf) == 64 &&
+static_assert(sizeof(JkPair) == 80 && sizeof(JkPrimPair64) == 96 && sizeof(JkPrimPair32) == 48 && sizeof(JkPrimPairDf) == 64 &&
                   sizeof(JkPairFeat) == 32 && sizeof(JkKetScr) == 16 && sizeof(JkRec) == 64,
               "record sizes are part of the device layout");
 
@@ -1391,8 +1391,6 @@ int init_impl(int32_t nmol, const int32_t *mol_shell_off, const jk_shell *shells
         p.a_loc = a - mol_shell_off[p.mol]; p.b_loc = b - mol_shell_off[p.mol];
         const double *A = coords + 3 * shells[a].atom, *B = coords + 3 * shells[b].atom;
         p.ABx = A[0] - B[0]; p.ABy = A[1] - B[1]; p.ABz = A[2] - B[2];
-        p.ABxf = (float)p.ABx; p.AByf = (float)p.ABy; p.ABzf = (float)p.ABz;
-        p.ABxl = (float)(p.ABx - (double)p.ABxf); p.AByl = (float)(p.ABy - (double)p.AByf); p.ABzl = (float)(p.ABz - (double)p.ABzf);
         p.Q = 0; p.Qf = 0.f; p.padf = 0.f;
     }
     JkPair *d_cp = nullptr;
@@ -1574,8 +1572,8 @@ int init_impl(int32_t nmol, const int32_t *mol_shell_off, const jk_shell *shells
             JkRec &r = rec[k];
             memset(&r, 0, sizeof r);
             r.pp_off = p.pp_off; r.a_ao = p.a_ao; r.b_ao = p.b_ao; r.same = p.a == p.b;
-            r.ABxf = p.ABxf; r.AByf = p.AByf; r.ABzf = p.ABzf;
-            r.ABxl = p.ABxl; r.AByl = p.AByl; r.ABzl = p.ABzl;
+            r.ABxf = (float)p.ABx; r.AByf = (float)p.ABy; r.ABzf = (float)p.ABz;
+            r.ABxl = (float)(p.ABx - (double)r.ABxf); r.AByl = (float)(p.ABy - (double)r.AByf); r.ABzl = (float)(p.ABz - (double)r.ABzf);
             const double *A = coords + 3 * shells[p.a].atom;
             float *c = &r.Axh;   // h, l per axis
             for (int ax = 0; ax < 3; ++ax) {

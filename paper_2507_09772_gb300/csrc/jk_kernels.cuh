@@ -99,7 +99,8 @@ template <> struct JkConst<jkdf> {   // compile-time constants only
 };
 // 1 / sqrt(x): the FP32 estimate y and its residual r = 1 - x y^2 = d - t (d =
 // 1 - fl(x y^2) has a few bits, t the rest), y (1 + r/2 + 3 r^2 / 8) with the
-// product y d / 2 kept exact (normalised; 5e-15 at most)
+// product y d / 2 kept exact (normalised; relative error 1.7e-14 at most and
+// 1.3e-15 rms over 4e6 arguments with estimates within 2 ulp, emulated)
 __device__ __forceinline__ jkdf jk_rsqrt(jkdf x)
 {
     const float y = rsqrtf(x.h);

@@ -15,8 +15,6 @@ struct alignas(16) JkPair {
     int a_ao, b_ao;    // molecule-local Cartesian AO offsets
     int a_loc, b_loc;  // molecule-local shell indices (density-max table)
     double Q;          // Schwarz factor sqrt(max |(mu nu|mu nu)|)
-    float ABxf, AByf, ABzf;  // A - B rounded to FP32 (the FP32 tier reads these, no conversion)
-    float ABxl, AByl, ABzl;  // what the rounding left (the split tier reads A - B as two floats)
     double ABx, ABy, ABz;  // A - B (horizontal recurrence)
     float Qf;              // Q rounded to FP32 (the FP32 screening path)
     float padf;
@@ -24,7 +22,7 @@ struct alignas(16) JkPair {
 
 // What a kernel reads of every candidate ket: one 16-byte vector for the
 // screening (32 candidates in a row are four lines; the JkPair records would be
-// 24), and a 64-byte record for a quartet in FP32 (the first half) or two
+// 20), and a 64-byte record for a quartet in FP32 (the first half) or two
 // floats. Arrays aligned with the pairs.
 struct alignas(16) JkKetScr {
     float Qf;
@@ -34,7 +32,7 @@ struct alignas(16) JkKetScr {
 struct alignas(16) JkRec {
     int pp_off, a_ao, b_ao;
     int same;                // a == b
-    float ABxf, AByf, ABzf, ABxl, AByl, ABzl;
+    float ABxf, AByf, ABzf, ABxl, AByl, ABzl;   // A - B rounded to FP32, and what the rounding left
     float Axh, Axl, Ayh, Ayl, Azh, Azl;   // centre A in two floats
 };
 
