@@ -60,14 +60,15 @@ TIER_PEAK_SOURCE = {
 TRAFFIC_SOURCES = ["paper_2507_09772_gb300/csrc/jk_kernels.cuh", "paper_2507_09772_gb300/csrc/jk_types.h",
                    "paper_2507_09772_gb300/csrc/jk_router.cuh"]
 # Captures of the 8-molecule case (profiles/jk_class_kernel_dram_traffic_batched8.md),
-# both over 287,529,305 quartets, with the hash of the comment-free kernel
-# sources they ran:
-#   tier 0 (FP64 build): 1,715,792,896 B read + 3,408,896 B written, on the
-#     kernels just before J and K moved from ATOM to RED accumulation;
-#   tier 1 (FP32 build): 1,289,914,624 B read + 0 B written, on the RED
-#     kernels.
-TRAFFIC_CAPTURES = {0: (1719201792 / 287529305, "f7bad00fedd57b74"),
-                    1: (1289914624 / 287529305, "83e18b6215b51bc2")}
+# with the hash of the comment-free kernel sources they ran:
+#   tier 0 (FP64 instructions, 339,618 quartets of an FP64 build): 75,833,344 B
+#     read, 0 B written;
+#   tier 1 (FP32 build, 287,529,305 quartets): 305,786,880 B + 909,056 B;
+#   tier 2 (two floats, 287,189,687 quartets of the FP64 build): 396,905,984 B
+#     + 560,640 B.
+TRAFFIC_CAPTURES = {0: (75833344 / 339618, "37b0ca6ca3087761"),
+                    1: (306695936 / 287529305, "37b0ca6ca3087761"),
+                    2: (397466624 / 287189687, "37b0ca6ca3087761")}
 
 
 def sources_sha():
@@ -617,6 +618,7 @@ def run_ours(args):
     if pg:
         pg.barrier()
     clocks = sampler.stop()
+    streams = int(eng.get_option("streams"))
     ms_total = e0.elapsed_time(e1)
     step_ms = [(e0 if i == 0 else step_ev[i - 1]).elapsed_time(step_ev[i]) for i in range(args.steps)]
 
@@ -723,19 +725,26 @@ def run_ours(args):
 
     if rank == 0:
         nbf = sum(m.nao for m in mols)
+        # the arithmetic of the timed quartets: FP64 instructions, pairs of FP32
+        # numbers (48 bits; the part of the FP64 tier below the split threshold), FP32
+        by_tier = {t: sum(v["quartets"] for v in prof.values() if v["tier"] == t) for t in TIER_PEAK}
+        dtype = "+".join(n for t, n in ((0, "f64"), (2, "2xf32"), (1, "f32")) if by_tier[t] or t == 0 and args.precision != "fp32")
         wl = WORKLOAD if args.workload == "batch" else {
             "cluster": "water-like-cluster-768atm-631gs", "highl": "tzvpp-shaped-60atm-spherical",
             "router": "router-cluster-1024atm-631gs"}[args.workload]
         out = {
             "metric": METRIC, "value": value, "unit": UNIT, "n_gpus": ws, "steps": args.steps,
             "warmup": args.warmup, "ms_per_step": ms_max / args.steps, "higher_is_better": True,
-            "scaling": "weak", "vs_baseline": None, "dtype": "f64" if args.precision == "fp64" else "f64+f32",
+            "scaling": "weak", "vs_baseline": None, "dtype": dtype,
             "data": "synthetic",
             "config": {"workload": wl, "nmol": len(mols), "nbf_total": nbf,
                        "natm_range": [min(m.natm for m in mols), max(m.natm for m in mols)],
                        "precision": args.precision, "cutoff": args.cutoff,
                        "l2": "flushed before every step (256 MiB write)",
-                       "graph": args.graph, "branches": args.branches,
+                       "graph": args.graph, "branches": args.branches, "streams": streams,
+                       "split": eng.get_option("split"),
+                       "quartet_share": {n: by_tier[t] / max(1, sum(by_tier.values()))
+                                         for t, n in ((0, "f64"), (2, "2xf32"), (1, "f32"))},
                        "chunk": eng.get_option("chunk"), "chunk_fp64tier": eng.get_option("chunk_fp64tier"),
                        "screen64": eng.get_option("screen64"), "widen_int": eng.get_option("widen_int"),
                        "options": args.opt,

@@ -794,7 +794,7 @@ static const double JK_RATE[3] = {0.8e12, 6e12, 2e12};
 #define JK_MAX_BRANCHES 7        // option "branches" less one
 // Streams the launches of a build are spread over unless they are profiled or
 // the caller set branches to 1: the tail of one launch is filled by the next
-// ones (s, p, d shells: 21 per tier; s to f: 55). ms on 1, 4, 8 and 24 streams:
+// ones (6-31G* shapes: 22 per tier; s to f: 55). ms on 1, 4, 8 and 24 streams:
 // 45 functions in FP64 2.00, 0.67, 0.48, 0.39; 20 atoms 7.0, 4.5, 4.1, 4.1; 33
 // atoms mixed 15.9, 12.8, 12.6, 12.6; 8 molecules 276, 258, 256, 257.
 #define JK_SIDE_STREAMS 23

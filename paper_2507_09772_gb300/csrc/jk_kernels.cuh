@@ -1108,7 +1108,7 @@ __device__ __forceinline__ void jk_count_flush(const JkClassArgs &args, int laun
 // the elements of its G / X threads.
 //
 // Why class pairs share a launch: a 6-31G*-shaped basis has 231 class pairs
-// (21 angular momenta); launched one by one, most of them were too small to
+// (22 kernels); launched one by one, most of them were too small to
 // fill the GPU and ended in a tail of a few long items each.
 template <int LA, int LB, int LC, int LD, int GA, int GB, int GC, int GD, int X, int NDM, int DOJ, int DOK,
           typename R, int MODE, int OP>
