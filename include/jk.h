@@ -270,7 +270,9 @@ int jk_destroy(jk_handle *h);
  * K): for every quartet the build evaluates inside the band (tau32, K tau32]
  * it writes the 12 features to X[i*12..] and the label y = log10(max|T| /
  * (Q_ab Q_cd)) to y[i] (X, y: device, capacity cap); *n receives the number
- * of band quartets seen (only the first cap are written). Synchronises. */
+ * of band quartets seen. Where that is more than cap, a second build writes a
+ * sample of cap of them, drawn by a hash of their shells: every quartet has the
+ * same chance, whatever the order of the launches. Synchronises. */
 int jk_router_collect(jk_handle *h, const double *const *D, int32_t n_dm, double cutoff, double *const *J,
                       double *const *K, float *X, float *y, int64_t cap, int64_t *n, void *stream);
 

@@ -1613,7 +1613,7 @@ int init_impl(int32_t nmol, const int32_t *mol_shell_off, const jk_shell *shells
         }
         if ((rc = upload(&h->d_pfeat, pf))) return rc;
         CK(cudaMalloc(&h->d_router, sizeof(JkRouterDev)));
-        CK(cudaMalloc(&h->d_logn, sizeof(unsigned long long)));
+        CK(cudaMalloc(&h->d_logn, 2 * sizeof(unsigned long long)));
     }
     for (auto &c : h->classes) {
         if ((rc = upload(&c.d_beg, c.beg)) || (rc = upload(&c.d_end, c.end))) return rc;
@@ -1709,6 +1709,8 @@ int init_impl(int32_t nmol, const int32_t *mol_shell_off, const jk_shell *shells
 struct LogSpec {
     float *x, *y;
     long long cap;
+    unsigned long long keep = ~0ull;     // keys up to this one
+    unsigned long long *key = nullptr;   // of the written samples
 };
 
 // The device error word (set by the kernels: a non-finite density element)
@@ -2055,6 +2057,8 @@ int build_impl(jk_handle *h, const double *const *D, int32_t ndm, int with_j, in
                 a.log_y = logs ? logs->y : nullptr;
                 a.log_n = h->d_logn;
                 a.log_cap = logs ? logs->cap : 0;
+                a.log_keep = logs ? logs->keep : 0;
+                a.log_key = logs ? logs->key : nullptr;
                 a.prim_eps = std::min(cutoff, h->prim_eps);
                 a.prim_eps32 = (float)a.prim_eps;
                 a.omega = std::fabs(h->omega);
@@ -2092,7 +2096,7 @@ int build_impl(jk_handle *h, const double *const *D, int32_t ndm, int with_j, in
         return JK_OK;
     };
 
-    if (logs) CK(cudaMemsetAsync(h->d_logn, 0, sizeof(unsigned long long), st));
+    if (logs) CK(cudaMemsetAsync(h->d_logn, 0, 2 * sizeof(unsigned long long), st));
     if (h->use_graph && !logs) {
         // one CUDA graph per flag combination, captured on the handle's own
         // stream and replayed on the caller's; per-call pointers live in the
@@ -2295,6 +2299,80 @@ int grad_rows(JkGradBuffers *B, const jk_router_blob *w, const float *X, const f
     CK(cudaStreamSynchronize(st));
     *loss = out.loss;
     for (int i = 0; i < JK_RT_NPARAM; ++i) grad_host[i] = (float)out.grad[i];
+    return JK_OK;
+}
+}  // namespace
+
+// Rows of a sample gathered into the caller's arrays.
+__global__ void jk_gather_samples_kernel(const long long *__restrict__ row, long long n, const float *__restrict__ X,
+                                         const float *__restrict__ y, float *__restrict__ Xo, float *__restrict__ yo)
+{
+    const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+    if (t >= n * JK_RT_NIN) return;
+    const long long i = t / JK_RT_NIN;
+    const int c = (int)(t - i * JK_RT_NIN);
+    Xo[t] = X[row[i] * JK_RT_NIN + c];
+    if (c == 0) yo[i] = y[row[i]];
+}
+
+namespace {
+// Router labels. Where more band quartets are seen than fit, a second build
+// keeps those whose key lies below a threshold a little above cap of them, and
+// the cap smallest keys of these are the sample: every quartet has the same
+// chance, whatever the order of the launches. (The first ones seen are all of
+// one angular momentum: a network trained on 2 of 63 million quartets, all with
+// l_a + l_b + l_c + l_d = 3, released 24 % of them wrongly, up to 100 tau32; of a
+// random sample 0.06 %.)
+int collect_impl(jk_handle *h, const double *const *D, int32_t n_dm, double cutoff, double *const *J, double *const *K,
+                 float *X, float *y, int64_t cap, int64_t *n, void *stream)
+{
+    jk_stats st;
+    unsigned long long cnt[2] = {0, 0};
+    auto build = [&](const LogSpec &ls) -> int {
+        if (int rc = build_impl(h, D, n_dm, 1, 1, cutoff, JK_PREC_FP64, J, K, stream, &st, &ls)) return rc;
+        CK(cudaMemcpy(cnt, h->d_logn, sizeof cnt, cudaMemcpyDeviceToHost));
+        return JK_OK;
+    };
+    LogSpec all;
+    all.x = X; all.y = y; all.cap = (long long)cap;
+    if (int rc = build(all)) return rc;
+    *n = (int64_t)cnt[0];
+    if (cnt[0] <= (unsigned long long)cap) return JK_OK;
+    // five standard deviations above cap on average, room for ten
+    const double sd = std::sqrt((double)cap), want = (double)cap + 5.0 * sd + 32.0;
+    LogSpec part;
+    part.cap = (long long)((double)cap + 10.0 * sd + 64.0);
+    float *kx = nullptr, *ky = nullptr;
+    long long *d_row = nullptr;
+    struct Guard { std::function<void()> f; ~Guard() { f(); } } guard{
+        [&]() { cudaFree(kx); cudaFree(ky); cudaFree(part.key); cudaFree(d_row); }};
+    CK(cudaMalloc(&kx, sizeof(float) * JK_RT_NIN * part.cap));
+    CK(cudaMalloc(&ky, sizeof(float) * part.cap));
+    CK(cudaMalloc(&part.key, sizeof(unsigned long long) * part.cap));
+    part.x = kx;
+    part.y = ky;
+    double share = want / (double)cnt[0];
+    for (int tries = 0;; ++tries) {
+        part.keep = share >= 1.0 ? ~0ull : (unsigned long long)std::ldexp(share, 64);
+        if (int rc = build(part)) return rc;
+        const bool fits = (long long)cnt[1] >= (long long)cap && (long long)cnt[1] <= part.cap;
+        if (fits) break;
+        if (tries == 3) return fail(JK_ERR_CUDA, "sample of %lld band quartets: %llu kept", (long long)cap, cnt[1]);
+        share *= want / (double)std::max(cnt[1], 1ull);
+    }
+    std::vector<unsigned long long> key(cnt[1]);
+    CK(cudaMemcpy(key.data(), part.key, sizeof(unsigned long long) * cnt[1], cudaMemcpyDeviceToHost));
+    std::vector<long long> row(cnt[1]);
+    for (size_t i = 0; i < row.size(); ++i) row[i] = (long long)i;
+    if ((size_t)cap < row.size())
+        std::nth_element(row.begin(), row.begin() + cap, row.end(), [&](long long a, long long b) { return key[a] < key[b]; });
+    row.resize((size_t)cap);
+    std::sort(row.begin(), row.end());
+    if (int rc = upload(&d_row, row)) return rc;
+    const long long work = (long long)cap * JK_RT_NIN;
+    jk_gather_samples_kernel<<<(unsigned)((work + 255) / 256), 256, 0, (cudaStream_t)stream>>>(d_row, (long long)cap, kx, ky, X, y);
+    CK(cudaGetLastError());
+    CK(cudaStreamSynchronize((cudaStream_t)stream));
     return JK_OK;
 }
 }  // namespace
@@ -2651,19 +2729,11 @@ int jk_router_collect(jk_handle *h, const double *const *D, int32_t n_dm, double
                       double *const *K, float *X, float *y, int64_t cap, int64_t *n, void *stream)
 {
     if (!h || !X || !y || !n || cap < 1 || !J || !K) return fail(JK_ERR_ARG, "NULL argument or cap < 1");
-    LogSpec ls{X, y, (long long)cap};
-    jk_stats st;
-    int rc;
     try {
-        rc = build_impl(h, D, n_dm, 1, 1, cutoff, JK_PREC_FP64, J, K, stream, &st, &ls);
+        return collect_impl(h, D, n_dm, cutoff, J, K, X, y, cap, n, stream);
     } catch (const std::exception &e) {
         return fail(JK_ERR_OOM, "host exception: %s", e.what());
     }
-    if (rc) return rc;
-    unsigned long long cnt = 0;
-    CK(cudaMemcpy(&cnt, h->d_logn, sizeof cnt, cudaMemcpyDeviceToHost));
-    *n = (int64_t)cnt;
-    return JK_OK;
 }
 
 int jk_router_forward(const jk_router_blob *w, const float *X, int64_t n, float *y_out)

@@ -916,14 +916,21 @@ __device__ __forceinline__ double jk_quartet_dmax(const JkClassArgs &args, const
 }
 
 // MODE 2: one training sample (features, label) for a band quartet, written
-// by the group's first thread. tmax is the group's max |T|.
+// by the group's first thread. tmax is the group's max |T|. Which quartets are
+// kept of too many follows a hash of their shells, not the order of the launches,
+// which run one angular momentum after the other.
 __device__ __forceinline__ void jk_log_sample(const JkClassArgs &args, const JkPair &bra, const JkPair &ket,
                                               const JkPairFeat &braf, const JkPairFeat &ketf, double dm, double tmax)
 {
     const double B = bra.Q * ket.Q * dm;
     if (!(B > args.tau && B <= args.band_hi)) return;
-    const unsigned long long idx = atomicAdd(args.log_n, 1ull);
+    atomicAdd(args.log_n, 1ull);
+    const unsigned long long key = jk_mix64(jk_mix64((unsigned long long)bra.a << 32 | (unsigned)bra.b) ^
+                                            ((unsigned long long)ket.a << 32 | (unsigned)ket.b));
+    if (key > args.log_keep) return;
+    const unsigned long long idx = atomicAdd(args.log_n + 1, 1ull);
     if ((long long)idx >= args.log_cap) return;
+    if (args.log_key) args.log_key[idx] = key;
     float x[JK_RT_NIN];
     // the bound as the FP32 screening path forms it
     jk_router_features(braf, ketf, (bra.Qf * ket.Qf) * (float)dm, (float)dm, args.tau32, x);

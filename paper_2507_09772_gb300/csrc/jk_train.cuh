@@ -37,15 +37,6 @@ __host__ __device__ inline float jk_bf2f(unsigned short b)
     return f;
 }
 
-// splitmix64: counter-based sample picker
-__device__ __forceinline__ unsigned long long jk_mix64(unsigned long long z)
-{
-    z += 0x9e3779b97f4a7c15ull;
-    z = (z ^ (z >> 30)) * 0xbf58476d1ce4e5b9ull;
-    z = (z ^ (z >> 27)) * 0x94d049bb133111ebull;
-    return z ^ (z >> 31);
-}
-
 // One mini-batch: forward, pinball loss, backward. Sample t of the batch is row
 // t of X (seed == JK_GRAD_ROWS) or a hashed one.
 //

@@ -97,6 +97,15 @@ __device__ __forceinline__ double jk_split_threshold(double split, double split_
     return fmax(split_min, __dmul_rn(__dmul_rn(split, qmax2), dmol));
 }
 
+// splitmix64 (Steele, Lea and Flood, OOPSLA 2014): counter-based random bits.
+__host__ __device__ __forceinline__ unsigned long long jk_mix64(unsigned long long z)
+{
+    z += 0x9e3779b97f4a7c15ull;
+    z = (z ^ (z >> 30)) * 0xbf58476d1ce4e5b9ull;
+    z = (z ^ (z >> 27)) * 0x94d049bb133111ebull;
+    return z ^ (z >> 31);
+}
+
 // One class pair (bra pair class, ket pair class) of a launch. A launch runs
 // every class pair that shares a kernel (angular momenta and fragment shape),
 // whatever its primitive counts.
@@ -182,8 +191,10 @@ struct JkClassArgs {
     int tier;                    // 0: this launch is the FP64 tier, 1: FP32
     float *log_x;                // MODE 2: features (12 per sample)
     float *log_y;                // MODE 2: labels
-    unsigned long long *log_n;   // MODE 2: samples written (may exceed log_cap)
+    unsigned long long *log_n;   // MODE 2: band quartets seen; those with a key up to log_keep (may exceed log_cap)
     long long log_cap;
+    unsigned long long log_keep; // a band quartet is written iff the key of its shells is at most this
+    unsigned long long *log_key; // the keys of the written ones, or nullptr
     // routed builds: the FP64 tier (MODE 1) appends the band quartets the
     // router releases to their class pair's list (rlist + roff[launch], while
     // it has room: rcap[launch]; a quartet that finds it full stays in FP64);

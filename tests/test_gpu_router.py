@@ -192,3 +192,38 @@ def test_quartets_split_over_ctas_are_evaluated_once(nprim):
     # FP32 quartets up to 100 tau32 = 1e-2 (the band), relative error 1e-5 at most in g classes,
     # a few hundred quartets; an integral taken twice would be off by 1e-2
     assert np.abs(Jr - J64).max() <= 1e-5 and np.abs(Kr - K64).max() <= 1e-5
+
+
+@pytest.mark.parametrize("share", [0.6, 0.05])
+def test_a_sample_of_the_labels_has_every_class(share):
+    """More band quartets than the arrays hold: the kept ones are a random
+    sample of all (each angular momentum within five standard deviations of its
+    share), the same in every call, and each is one of the whole collection."""
+    mol = synth.batched_molecule(6, natm=14)
+    eng = jk.JK(mol)
+    D = torch.tensor(mol.D, dtype=torch.float64, device="cuda")
+    J, K = torch.empty_like(D), torch.empty_like(D)
+
+    def collect(cap):
+        X = torch.full((cap, 12), np.nan, dtype=torch.float32, device="cuda")
+        y = torch.full((cap,), np.nan, dtype=torch.float32, device="cuda")
+        n = jk.jk_router_collect(eng.h, [D], 1, 1e-13, [J], [K], X, y)
+        return n, np.column_stack([X.cpu().numpy(), y.cpu().numpy()])[:min(n, cap)]
+
+    n, full = collect(400000)
+    assert 1000 < n < 400000 and np.isfinite(full).all()
+    cap = int(share * n)
+    seen, part = collect(cap)
+    again = collect(cap)[1]
+    eng.close()
+    assert seen == n and len(part) == cap
+    count = {}
+    for r in full:
+        count[r.tobytes()] = count.get(r.tobytes(), 0) + 1
+    for r in part:
+        count[r.tobytes()] -= 1
+    assert min(count.values()) >= 0                       # every row is one of the whole, once
+    assert sorted(r.tobytes() for r in part) == sorted(r.tobytes() for r in again)
+    want = np.bincount(full[:, 10].astype(int), minlength=9) * (cap / n)
+    got = np.bincount(part[:, 10].astype(int), minlength=9)
+    assert (np.abs(got - want) <= 5 * np.sqrt(want) + 1).all(), (got, want)
