@@ -61,14 +61,14 @@ TRAFFIC_SOURCES = ["paper_2507_09772_gb300/csrc/jk_kernels.cuh", "paper_2507_097
                    "paper_2507_09772_gb300/csrc/jk_router.cuh"]
 # Captures of the 8-molecule case (profiles/jk_class_kernel_dram_traffic_batched8.md),
 # with the hash of the comment-free kernel sources they ran:
-#   tier 0 (FP64 instructions, 339,618 quartets of an FP64 build): 75,833,344 B
+#   tier 0 (FP64 instructions, 339,618 quartets of an FP64 build): 75,765,760 B
 #     read, 0 B written;
-#   tier 1 (FP32 build, 287,529,305 quartets): 305,786,880 B + 909,056 B;
-#   tier 2 (two floats, 287,189,687 quartets of the FP64 build): 396,905,984 B
-#     + 560,640 B.
-TRAFFIC_CAPTURES = {0: (75833344 / 339618, "37b0ca6ca3087761"),
-                    1: (306695936 / 287529305, "37b0ca6ca3087761"),
-                    2: (397466624 / 287189687, "37b0ca6ca3087761")}
+#   tier 1 (FP32 build, 287,529,305 quartets): 306,904,064 B + 1,044,480 B;
+#   tier 2 (two floats, 287,189,687 quartets of the FP64 build): 396,560,640 B
+#     + 550,656 B.
+TRAFFIC_CAPTURES = {0: (75765760 / 339618, "e18c2948e4d36e23"),
+                    1: (307948544 / 287529305, "e18c2948e4d36e23"),
+                    2: (397111296 / 287189687, "e18c2948e4d36e23")}
 
 
 def sources_sha():
@@ -164,8 +164,9 @@ def parse():
     ap.add_argument("--no-forms", action="store_true", help="skip the mixed / routed comparison")
     ap.add_argument("--forms", default="mixed,routed", help="accelerated forms timed against the FP64 build")
     ap.add_argument("--chunk", type=int, default=0, help="candidate kets per work item (0: the library default)")
-    ap.add_argument("--router-margin", type=float, default=0.0,
-                    help="added to the trained router's margin (log10 units; larger releases fewer quartets)")
+    ap.add_argument("--router-margin", type=float, default=0.5,
+                    help="added to the trained router's margin (log10 units; larger releases fewer quartets; 0 leaves "
+                         "the routed build of the batch 1.6e-8 off in J, 0.5 6.7e-9)")
     ap.add_argument("--opt", action="append", default=[],
                     help="library option KEY=VALUE set on the handle before the run (repeatable)")
     ap.add_argument("--chunk-fp64tier", type=int, default=0,
