@@ -164,9 +164,9 @@ def parse():
     ap.add_argument("--no-forms", action="store_true", help="skip the mixed / routed comparison")
     ap.add_argument("--forms", default="mixed,routed", help="accelerated forms timed against the FP64 build")
     ap.add_argument("--chunk", type=int, default=0, help="candidate kets per work item (0: the library default)")
-    ap.add_argument("--router-margin", type=float, default=0.5,
-                    help="added to the trained router's margin (log10 units; larger releases fewer quartets; 0 leaves "
-                         "the routed build of the batch 1.6e-8 off in J, 0.5 6.7e-9)")
+    ap.add_argument("--router-margin", type=float, default=1.0,
+                    help="added to the trained router's margin (log10 units; larger releases fewer quartets and keeps "
+                         "the routed build closer to the mixed one)")
     ap.add_argument("--opt", action="append", default=[],
                     help="library option KEY=VALUE set on the handle before the run (repeatable)")
     ap.add_argument("--chunk-fp64tier", type=int, default=0,

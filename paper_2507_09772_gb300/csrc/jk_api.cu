@@ -749,7 +749,8 @@ struct TierPlan {
 // mixed build (~7 %) as many as leave every resident warp JK_ITEMS_PER_WARP items
 // of the launch, between JK_CHUNK and this. 33 atoms mixed, two densities: 13.6 ms
 // with 512 throughout, 12.9 with the rule; 45 atoms routed 18.3 and 17.0. (The
-// other tiers lose with more than 64: 8 molecules FP64 224 ms, 236 with 256.)
+// other tiers lose with more than 64: 8 molecules FP64 224 ms, 236 with 256, on the
+// same box.)
 #define JK_CHUNK_HI 512
 #define JK_CHUNK_MIN 4
 #define JK_ITEMS_PER_WARP 32.0
@@ -768,13 +769,13 @@ static const double JK_LAT[3] = {20e-9, 5e-9, 20e-9};      // FP64, FP32, two fl
 static const double JK_RATE[3] = {0.8e12, 6e12, 2e12};
 #define JK_ITEM_EPS 1e-15
 // Quartets of the FP64 tier whose bound is at most JK_SPLIT x (max Q)^2 x
-// max |D| are evaluated in two-float arithmetic (relative error about 1e-14),
-// the few above it, which carry the result, in FP64 instructions; classes with
+// max |D| are evaluated in two-float arithmetic (48 bits), the few above it, which carry the result, in FP64 instructions; classes with
 // f or g shells, whose recurrences lose more, from JK_SPLIT_F of that on.
 // Relative error of K against a 64-bit reference (FP64 instructions alone first;
 // the cutoff sets it): 20 atoms 6.58e-13, 6.58e-13 at 2^-7 and at 1; erfc on 14
 // atoms 1.46e-13, 1.46e-13, 1.46e-13; 6 atoms of s p d f shells 6.59e-14, 7.2e-14
-// at 2^-7, 6.59e-14 at 2^-13, 1.6e-13 at 1. 8 molecules, ms: 0: 598, 2^-13: 253,
+// at 2^-7, 6.59e-14 at 2^-13, 1.6e-13 at 1 (no system with g shells was measured).
+// 8 molecules, ms on one box (others take 245 to 262 at 2^-7): 0: 598, 2^-13: 253,
 // 2^-10: 239, 2^-7: 231, 1: 225.
 #define JK_SPLIT (1.0 / 128)
 #define JK_SPLIT_F (1.0 / 64)
