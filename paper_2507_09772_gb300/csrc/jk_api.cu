@@ -742,8 +742,13 @@ struct TierPlan {
 // quartet takes G threads gets proportionally fewer (at least JK_CHUNK_MIN),
 // so that an item is the same number of rounds of a warp: with 64 kets for
 // every class, a (dd|dp) item (18 threads, one quartet per warp at a time) ran
-// 2 ms on its own. Systems whose items would exceed JK_ITEMS_MAX get larger
-// chunks.
+// 2 ms on its own. Launches that leave every resident warp JK_ITEMS_PER_WARP items
+// (a CTA of a larger group JK_ITEMS_PER_CTA) keep up to JK_CHUNK: an item's own work
+// (its records, its J block) is that of several quartets. 150 p shells in FP64: 73 ms
+// with 6 kets per item, 16.9 with 64; 60 d shells in FP32: 10.5 and 5.8. An item
+// has at least JK_CHUNK_OWN primitive quartets' kets where that leaves four for every
+// warp or CTA: 14 g shells in FP32 with 2, 4, 8, 16 kets per item 4.95, 2.98, 2.17,
+// 1.92 ms. Systems whose items would exceed JK_ITEMS_MAX get larger chunks.
 #define JK_CHUNK 64
 // Tiers that keep few of the candidates they scan; the FP64 and split tiers of a
 // mixed build (~7 %) as many as leave every resident warp JK_ITEMS_PER_WARP items
@@ -754,6 +759,8 @@ struct TierPlan {
 #define JK_CHUNK_HI 512
 #define JK_CHUNK_MIN 4
 #define JK_ITEMS_PER_WARP 32.0
+#define JK_ITEMS_PER_CTA 16.0
+#define JK_CHUNK_OWN 16.0
 #define JK_ITEMS_MAX 8000000LL
 // Small systems: an item is a serial chain of primitive quartets, about
 // JK_LAT_* seconds per modelled FLOP of a lane when few warps share an SM
@@ -1078,11 +1085,14 @@ int tier_plan(jk_handle *h, int t, int hi, int merge, int whole, TierPlan **out)
             const int ngw = G.spec.G() <= 32 ? 32 / G.spec.G() : 1;
             double cand = 0;
             for (int l : mem) cand += h->launches[l].cand;
-            // kets per item for one thread per quartet
-            const long long base =
-                hi < 2 ? (hi ? h->chunk_hi : h->chunk)
-                       : (long long)std::min<double>(h->chunk_hi, std::max<double>(std::min(h->chunk, h->chunk_hi),
-                                                                                   cand / (8.0 * h->num_sms * JK_ITEMS_PER_WARP)));
+            // kets per item
+            const double workers = h->num_sms * (G.spec.G() <= 32 ? 8.0 : 2.0 / G.spec.gx);   // resident warps or groups
+            const long long rounds = hi < 2 ? (hi ? h->chunk_hi : h->chunk)
+                                            : (long long)std::min<double>(h->chunk_hi, std::max<double>(std::min(h->chunk, h->chunk_hi),
+                                                                                                        cand / (8.0 * h->num_sms * JK_ITEMS_PER_WARP)));
+            long long base = std::max<long long>(JK_CHUNK_MIN, rounds * ngw / 32);
+            if (hi == 0)
+                base = std::max(base, std::min(rounds, (long long)(cand / (workers * (G.spec.G() <= 32 ? JK_ITEMS_PER_WARP : JK_ITEMS_PER_CTA)))));
             for (int l : mem) {
                 const Launch &L = h->launches[l];
                 const PairClass &A = h->classes[L.c1], &B = h->classes[L.c2];
@@ -1105,8 +1115,11 @@ int tier_plan(jk_handle *h, int t, int hi, int merge, int whole, TierPlan **out)
                 one.na = one.nb = one.nc = one.nd = 1;
                 // modelled FLOPs of a lane per round, at most
                 const double round = class_flops(one, 1) / one.G() * S.nab * S.ncd;
-                long long c = std::max<long long>(JK_CHUNK_MIN, base * ngw / 32);
-                while (c > ngw && round * std::max(1.0, kept * c / ngw) > chain_max) c = (c + 1) / 2;
+                // an item's own work is that of some uncontracted quartets
+                const double own = hi == 0 ? std::min(JK_CHUNK_OWN / (S.nab * S.ncd), cand / (4.0 * workers)) : 0.0;
+                const long long least_c = std::max<long long>(ngw, (long long)own);
+                long long c = std::max(base, least_c);
+                while (c > least_c && round * std::max(1.0, kept * c / ngw) > chain_max) c = (c + 1) / 2;
                 S.split = S.split_ab = 1;
                 if (!whole) {
                     const double want = std::max(1.0, std::ceil(round * std::max(1.0, kept * c / ngw) / chain_max));
