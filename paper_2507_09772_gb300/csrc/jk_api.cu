@@ -121,6 +121,7 @@ struct KSpec {
     int fp32 = 0;  // 0 FP64, 1 FP32, 2 two floats (the split tier)
     int mode = 0;  // 0 plain, 1 routed (learned router in the band), 2 label logging
     int op = 0;    // 0 1/r, 1 erf(w r)/r, 2 erfc(w r)/r
+    int p1 = 0;    // every class pair it runs is uncontracted
 
     std::string name() const
     {
@@ -128,8 +129,8 @@ struct KSpec {
         if (kind == 1)
             snprintf(b, sizeof b, "jk_schwarz_kernel<%d,%d,%d,%d,%d,%d,%d,%d,%d>", la, lb, na, nb, ga, gb, gc, gd, gx);
         else
-            snprintf(b, sizeof b, "jk_class_kernel<%d,%d,%d,%d,%d,%d,%d,%d,%d,%d,%d,%d,%s,%d,%d>", la, lb, lc, ld, ga,
-                     gb, gc, gd, gx, ndm, doj, dok, fp32 == 2 ? "jkdf" : (fp32 ? "float" : "double"), mode, op);
+            snprintf(b, sizeof b, "jk_class_kernel<%d,%d,%d,%d,%d,%d,%d,%d,%d,%d,%d,%d,%s,%d,%d,%d>", la, lb, lc, ld, ga,
+                     gb, gc, gd, gx, ndm, doj, dok, fp32 == 2 ? "jkdf" : (fp32 ? "float" : "double"), mode, op, p1);
         return b;
     }
     int G() const { return ga * gb * gc * gd; }
@@ -154,6 +155,7 @@ struct KSpec {
         const size_t groups = G() <= 32 ? (size_t)4 * (32 / G()) : 1;
         return rys_table_bytes() + groups * smem_group_reals() * (fp32 == 1 ? 4 : 8);
     }
+    bool uncontracted() const { return na * nb * nc * nd == 1; }
     int groups_per_cta() const { return G() <= 32 ? 4 * (32 / G()) : 1; }
 };
 
@@ -1080,6 +1082,8 @@ int tier_plan(jk_handle *h, int t, int hi, int merge, int whole, TierPlan **out)
             const auto &mem = members[gord[k]];
             LaunchGroup G;
             G.spec = shape[gord[k]];
+            G.spec.p1 = 1;
+            for (int l : mem) G.spec.p1 = G.spec.p1 && h->launches[l].spec[t].uncontracted();
             G.sub0 = (int)subs.size();
             G.nsub = (int)mem.size();
             const int ngw = G.spec.G() <= 32 ? 32 / G.spec.G() : 1;
@@ -2440,6 +2444,7 @@ int tune_impl(jk_handle *h, const double *const *D, int32_t ndm, int with_j, int
         for (auto &it : items)
             for (auto c : it.c) {
                 c.ndm = ndm; c.doj = with_j ? 1 : 0; c.dok = with_k ? 1 : 0;
+                c.p1 = c.uncontracted();
                 c.mode = (mode == JK_PREC_MIXED_ROUTED && it.t != 1) ? 1 : 0;
                 c.op = h->omega == 0.0 ? 0 : (h->omega > 0.0 ? 1 : 2);
                 all.push_back(c);
@@ -2938,6 +2943,7 @@ int jk_compile_class(int32_t la, int32_t lb, int32_t lc, int32_t ld, int32_t na,
     s.ndm = n_dm; s.doj = with_j ? 1 : 0; s.dok = with_k ? 1 : 0; s.fp32 = fp32;
     s.mode = mode;
     s.op = op;
+    s.p1 = s.uncontracted();
     choose_fragments(s, false);
     if (threads_per_quartet) *threads_per_quartet = s.G();
     try {
@@ -2991,6 +2997,12 @@ int jk_compile_basis(const jk_shell *shells, int32_t nshell, int32_t n_dm, int32
             choose_fragments(s, false);
             specs.push_back(s);
         }
+    // one kernel per angular momenta, without primitive loops where none is contracted
+    for (auto &s : specs) {
+        s.p1 = s.kind == 0;
+        for (auto &x : specs)
+            if (x.kind == 0 && x.la == s.la && x.lb == s.lb && x.lc == s.lc && x.ld == s.ld) s.p1 = s.p1 && x.uncontracted();
+    }
     if (nkernels) *nkernels = (int32_t)specs.size();
     try {
         return compile_to_disk(specs, compile_ms);

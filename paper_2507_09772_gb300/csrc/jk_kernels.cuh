@@ -1114,11 +1114,16 @@ __device__ __forceinline__ void jk_count_flush(const JkClassArgs &args, int laun
 // item t / X, each CTA builds the roots and 2D tables itself and evaluates
 // the elements of its G / X threads.
 //
+// P1: every class pair of the launch is uncontracted. The primitive loops are then
+// known to be one pass, so that the block is not live while the tables are built
+// (FP32 (ff|ff) 112 -> 0 bytes of spills): 6 and 9 atoms of s p d f shells 2.05 -> 1.99
+// and 2.90 -> 2.81 ms, 6 of f and g shells in FP32 2.08 -> 1.49.
+//
 // Why class pairs share a launch: a 6-31G*-shaped basis has 231 class pairs
 // (22 kernels); launched one by one, most of them were too small to
 // fill the GPU and ended in a tail of a few long items each.
 template <int LA, int LB, int LC, int LD, int GA, int GB, int GC, int GD, int X, int NDM, int DOJ, int DOK,
-          typename R, int MODE, int OP>
+          typename R, int MODE, int OP, int P1>
 __global__ void __launch_bounds__(JkShape<LA, LB, LC, LD, GA, GB, GC, GD>::G <= 32 ? 128
                                   : ((JkShape<LA, LB, LC, LD, GA, GB, GC, GD>::G / X + 31) / 32) * 32)
 jk_class_kernel(const JkClassArgs args)
@@ -1212,7 +1217,7 @@ jk_class_kernel(const JkClassArgs args)
 #pragma unroll
                         for (int k = 0; k < S::EPT; ++k) T[k] = JkConst<R>::get(0.0);
                         const int np = jk_quartet<LA, LB, LC, LD, GA, GB, GC, GD, R, OP>(
-                            JkRecOf<R>::bra(sub, rq.item), ket, JkShare{0, 1, 0, 1}, sub.nab, sub.ncd, __fdiv_rn(args.prim_eps32, rq.dmq), args.omega, args.asym64,
+                            JkRecOf<R>::bra(sub, rq.item), ket, JkShare{0, 1, 0, 1}, P1 ? 1 : sub.nab, P1 ? 1 : sub.ncd, __fdiv_rn(args.prim_eps32, rq.dmq), args.omega, args.asym64,
                             pp, rys, grp, gmask, tg, true, off, T);
                         float f = 1.0f;
                         if (bra.a == bra.b) f *= 0.5f;
@@ -1252,8 +1257,9 @@ jk_class_kernel(const JkClassArgs args)
             const JkItem wi = args.items[t];
             const JkSub &sub = args.subs[wi.sub & 0x7fffff];
             const int part = wi.sub >> 23;   // share of the primitive quartets
-            const JkShare sh = {part % sub.split_ab, sub.split_ab, part / sub.split_ab, sub.split / sub.split_ab};
-            const int item = wi.bra, nab = sub.nab, ncd = sub.ncd, same_class = sub.same_class;
+            const JkShare sh = P1 ? JkShare{0, 1, 0, 1}
+                                  : JkShare{part % sub.split_ab, sub.split_ab, part / sub.split_ab, sub.split / sub.split_ab};
+            const int item = wi.bra, nab = P1 ? 1 : sub.nab, ncd = P1 ? 1 : sub.ncd, same_class = sub.same_class;
             const int kb = wi.kb, ke = wi.ke;
             if (sub.launch != cur) {
                 if (lane == 0) jk_count_flush(args, cur, cnt);
@@ -1440,7 +1446,7 @@ jk_class_kernel(const JkClassArgs args)
 #pragma unroll
                     for (int k = 0; k < S::EPT; ++k) T[k] = JkConst<R>::get(0.0);
                     const int np = jk_quartet<LA, LB, LC, LD, GA, GB, GC, GD, R, OP, NTC>(
-                        JkRecOf<R>::bra(sub, rq.item), ket, JkShare{0, 1, 0, 1}, sub.nab, sub.ncd, __fdiv_rn(args.prim_eps32, rq.dmq), args.omega, args.asym64, pp,
+                        JkRecOf<R>::bra(sub, rq.item), ket, JkShare{0, 1, 0, 1}, P1 ? 1 : sub.nab, P1 ? 1 : sub.ncd, __fdiv_rn(args.prim_eps32, rq.dmq), args.omega, args.asym64, pp,
                         rys, grp, 0u, tg, act, off, T);
                     if (act) {
                         float f = 1.0f;
@@ -1481,8 +1487,9 @@ jk_class_kernel(const JkClassArgs args)
             const JkItem wi = args.items[t];
             const JkSub &sub = args.subs[wi.sub & 0x7fffff];
             const int part = wi.sub >> 23;   // share of the primitive quartets
-            const JkShare sh = {part % sub.split_ab, sub.split_ab, part / sub.split_ab, sub.split / sub.split_ab};
-            const int item = wi.bra, nab = sub.nab, ncd = sub.ncd, same_class = sub.same_class;
+            const JkShare sh = P1 ? JkShare{0, 1, 0, 1}
+                                  : JkShare{part % sub.split_ab, sub.split_ab, part / sub.split_ab, sub.split / sub.split_ab};
+            const int item = wi.bra, nab = P1 ? 1 : sub.nab, ncd = P1 ? 1 : sub.ncd, same_class = sub.same_class;
             const int kb = wi.kb, ke = wi.ke;
             if (sub.launch != cur) {
                 if (threadIdx.x == 0) jk_count_flush(args, cur, cnt);
