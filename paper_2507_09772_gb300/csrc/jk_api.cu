@@ -496,7 +496,9 @@ void choose_fragments(KSpec &s, bool symmetric)
     // with f or g shells small fragments lose (6 atoms of s p d f shells: 3.1 ->
     // 4.0 ms): few quartets per SM, whose larger tables only some threads build
     const bool fshell = std::max(std::max(s.la, s.lb), std::max(s.lc, s.ld)) > 2;
-    const int small_cap = symmetric || fshell ? 0 : (s.fp32 == 1 ? 27 : 12);
+    // (FP32 (dd|dd) of 60 d shells, threads per quartet: 27: 4.2 ms, 48: 6.0, 108: 3.9;
+    // (dd|dp) of 30 atoms of s p d shells 24: 2.5, 54: 1.4; smaller blocks: 12 elements lose)
+    const int small_cap = symmetric || fshell ? 0 : (s.fp32 == 1 && ne < 600 ? 27 : 12);
     auto fill = [](int g) { return g <= 32 ? (32 / g) * g / 32.0 : g / (32.0 * ((g + 31) / 32)); };
     // CTAs for a group of g threads: 1 if it fits one CTA, else the fewest
     // x (<= 16) dividing g with g / x <= gsplit, 0 if there is none

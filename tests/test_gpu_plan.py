@@ -164,3 +164,20 @@ def test_tuned_class_pairs_still_share_a_launch(case, prims, tmp_path, monkeypat
         launches.append(st["kernel_launches"])
         assert n == nq and np.abs(J - Jr).max() <= 1e-10 and np.abs(K - Kr).max() <= 1e-10
     assert launches[0] == launches[1]
+
+
+@pytest.mark.parametrize("shells", [
+    [(1, [0.3])], [(2, [0.4])], [(0, [2.0, 0.3]), (1, [0.4])], [(2, [0.6]), (2, [0.25])], [(0, [0.4]), (3, [0.7])]])
+@pytest.mark.parametrize("precision", ["fp64", "mixed", "fp32"])
+def test_uncontracted_and_mixed_launches_of_many_quartets(shells, precision):
+    """Launches whose items keep many kets, with the primitive loops and (all
+    class pairs uncontracted) without them, against the oracle."""
+    rng = np.random.default_rng(3)
+    natm = 10 if shells[-1][0] == 3 else 22
+    xyz = synth._rejection_box(rng, natm, (natm / 0.08) ** (1.0 / 3.0), 0.9)
+    mol = synth.custom_basis_molecule(xyz, [shells] * natm, rng)
+    Jr, Kr, nq = oracle.jk(mol, cutoff=1e-13)
+    J, K, n = build(mol, {}, precision=precision)
+    assert n == nq
+    tol = {"fp64": 1e-10, "mixed": 1e-8, "fp32": 1e-3}[precision]
+    assert np.abs(J - Jr).max() <= tol and np.abs(K - Kr).max() <= tol
