@@ -61,14 +61,14 @@ TRAFFIC_SOURCES = ["paper_2507_09772_gb300/csrc/jk_kernels.cuh", "paper_2507_097
                    "paper_2507_09772_gb300/csrc/jk_router.cuh"]
 # Captures of the 8-molecule case (profiles/jk_class_kernel_dram_traffic_batched8.md),
 # with the hash of the comment-free kernel sources they ran:
-#   tier 0 (FP64 instructions, 339,618 quartets of an FP64 build): 75,765,760 B
+#   tier 0 (FP64 instructions, 339,618 quartets of an FP64 build): 76,140,544 B
 #     read, 0 B written;
-#   tier 1 (FP32 build, 287,529,305 quartets): 306,904,064 B + 1,044,480 B;
-#   tier 2 (two floats, 287,189,687 quartets of the FP64 build): 396,560,640 B
-#     + 550,656 B.
-TRAFFIC_CAPTURES = {0: (75765760 / 339618, "e18c2948e4d36e23"),
-                    1: (307948544 / 287529305, "e18c2948e4d36e23"),
-                    2: (397111296 / 287189687, "e18c2948e4d36e23")}
+#   tier 1 (FP32 build, 287,529,305 quartets): 340,203,008 B + 1,379,840 B;
+#   tier 2 (two floats, 287,189,687 quartets of the FP64 build): 399,649,024 B
+#     + 612,864 B.
+TRAFFIC_CAPTURES = {0: (76140544 / 339618, "74bc642657b5cc7e"),
+                    1: (341582848 / 287529305, "74bc642657b5cc7e"),
+                    2: (400261888 / 287189687, "74bc642657b5cc7e")}
 
 
 def sources_sha():
