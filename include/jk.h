@@ -198,8 +198,9 @@ int jk_build_batch(jk_handle *h, const double *const *D, int32_t n_dm, int with_
  * profiled build takes exactly this many, one if it is not set),
  * "chunk" (32..65536, default 64: candidate kets per work item of the
  * persistent class kernels for classes with one thread per quartet; classes
- * with G threads per quartet take 1/G of it, and systems with more than 8
- * million items larger ones; changing it re-plans the work items),
+ * with G threads per quartet take from 1/G of it, in launches that would leave
+ * warps without items, up to all of it, and systems with more than 8 million
+ * items larger ones; changing it re-plans the work items),
  * "asym64" (0/1, default 0: the FP32 tier evaluates the large-T
  * Gauss-Hermite limit of the Rys roots and weights in FP64 and rounds the
  * result to FP32, instead of evaluating it in FP32),
